@@ -44,10 +44,10 @@ __device__ __forceinline__ uint32_t relu_mask(uint32_t v, uint32_t m)
     return r;
 }
 
-template <int CIN, int COUT, bool MASK>
+template <int CIN, int COUT>
 constexpr size_t conv_smem()
 {
-    return ((size_t)(MASK ? 4 : 2) * (CH + 2) * (CW + 2) * (CIN + 8) + (size_t)COUT * (9 * CIN + 8)) * 2;
+    return ((size_t)2 * (CH + 2) * (CW + 2) * (CIN + 8) + (size_t)COUT * (9 * CIN + 8)) * 2;
 }
 
 // 16-byte asynchronous copy (both addresses 16-byte aligned); src-size 0 writes zeros.
@@ -75,25 +75,29 @@ __device__ __forceinline__ const bf16 *in_chunk(const bf16 *x, const bf16 *xu, i
     return x + (((long)bz * H + gy) * W + gx) * (CIN - CUP) + 8 * q - CUP;
 }
 
-// y = act(conv3x3(x * [xmask > 0]) + bias), NHWC, zero padding.
+// y = act(conv3x3(x) + bias) * [ymask > 0], NHWC, zero padding.
 // w: [COUT][9][CIN] (tap = 3 dy + dx multiplies x[i + dy - 1, j + dx - 1]).
 // Persistent: each CTA stages all weights once, then walks output tiles of
-// 8 x 16 pixels; the next tile (and its mask) is copied into the other
-// shared buffer with cp.async while the current one is on the tensor cores.
-// CUP > 0: the input is up2(xu) ++ x (see in_chunk).
-template <int CIN, int COUT, int CUP, bool MASK>
+// 8 x 16 pixels; the next tile is copied into the other shared buffer with
+// cp.async while the current one is on the tensor cores.
+// CUP > 0: the input is up2(xu) ++ x (see in_chunk).  ymask (NULL: none; the
+// backward-data passes): the ReLU mask of the gradient written, so that its
+// two readers, the next layer's weight gradient and backward-data pass, take
+// it as it is (masking at the reader loaded the mask with its halo twice and
+// selected it nine times, once per tap).
+template <int CIN, int COUT, int CUP>
 __global__ void __launch_bounds__(128)
 k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restrict__ xu,
-           const bf16 *__restrict__ xmask,
+           const bf16 *__restrict__ ymask,
            const bf16 *__restrict__ w, const float *__restrict__ bias, int relu,
            bf16 *__restrict__ y, float *__restrict__ y32)
 {
     constexpr int XS = CIN + 8, WS = 9 * CIN + 8, NT = COUT / 8;
     constexpr int TP = (CH + 2) * (CW + 2);       // pixels of a haloed tile
-    static_assert(CIN % 16 == 0 && CUP % 8 == 0 && (CUP == 0 || !MASK), "channel layout");
+    static_assert(CIN % 16 == 0 && CUP % 8 == 0, "channel layout");
     extern __shared__ __align__(16) unsigned char conv_sm[];
     bf16 *ws = (bf16 *)conv_sm;
-    bf16 *xs0 = ws + COUT * WS;                    // 2 input buffers, then 2 mask buffers
+    bf16 *xs0 = ws + COUT * WS;                    // 2 input buffers
     const int tw = (W + CW - 1) / CW, th = (H + CH - 1) / CH, ntiles = B * tw * th;
     for (int k = threadIdx.x; k < COUT * (9 * CIN / 2); k += 128) {
         const int co = k / (9 * CIN / 2), q = k - co * (9 * CIN / 2);
@@ -103,16 +107,12 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
         const int bz = tl / (tw * th), rem = tl - bz * tw * th;
         const int ty0 = (rem / tw) * CH, tx0 = (rem - (rem / tw) * tw) * CW;
         bf16 *xs = xs0 + buf * TP * XS;
-        bf16 *ms = xs0 + (2 + buf) * TP * XS;
         for (int k = threadIdx.x; k < TP * (CIN / 8); k += 128) {
             const int pix = k / (CIN / 8), q = k - pix * (CIN / 8);
             const int r = pix / (CW + 2), c = pix - r * (CW + 2);
             const int gy = ty0 + r - 1, gx = tx0 + c - 1;
             const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
             cp_async16(xs + pix * XS + 8 * q, in ? in_chunk<CIN, CUP>(x, xu, bz, H, W, gy, gx, q) : x, in);
-            if (MASK)
-                cp_async16(ms + pix * XS + 8 * q,
-                           xmask + (in ? (((long)bz * H + gy) * W + gx) * CIN + 8 * q : 0), in);
         }
         cp_async_commit();
     };
@@ -125,7 +125,6 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
         else cp_async_wait<0>();
         __syncthreads();
         const bf16 *xs = xs0 + buf * TP * XS;
-        const bf16 *ms = xs0 + (2 + buf) * TP * XS;
         float acc[2][NT][4];
 #pragma unroll
         for (int a = 0; a < 2; a++)
@@ -154,12 +153,6 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
                     af[1] = *(const uint32_t *)(xs + o1);
                     af[2] = *(const uint32_t *)(xs + o0 + 8);
                     af[3] = *(const uint32_t *)(xs + o1 + 8);
-                    if (MASK) {
-                        af[0] = relu_mask(af[0], *(const uint32_t *)(ms + o0));
-                        af[1] = relu_mask(af[1], *(const uint32_t *)(ms + o1));
-                        af[2] = relu_mask(af[2], *(const uint32_t *)(ms + o0 + 8));
-                        af[3] = relu_mask(af[3], *(const uint32_t *)(ms + o1 + 8));
-                    }
 #pragma unroll
                     for (int nt = 0; nt < NT; nt++) mma_bf16(acc[mt][nt], af, bf[nt]);
                 }
@@ -182,7 +175,10 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
                     float v0 = acc[mt][nt][2 * half] + b0, v1 = acc[mt][nt][2 * half + 1] + b1;
                     if (relu) { v0 = fmaxf(v0, 0.0f); v1 = fmaxf(v1, 0.0f); }
                     const long off = (((long)bz * H + oy) * W + ox) * COUT + co;
-                    *(__nv_bfloat162 *)(y + off) = __floats2bfloat162_rn(v0, v1);
+                    __nv_bfloat162 o2 = __floats2bfloat162_rn(v0, v1);
+                    uint32_t o = *(uint32_t *)&o2;
+                    if (ymask) o = relu_mask(o, *(const uint32_t *)(ymask + off));
+                    *(uint32_t *)(y + off) = o;
                     if (y32 && co == 0) y32[off / COUT] = v0;  // channel 0 only
                 }
             }
@@ -432,163 +428,269 @@ k_conv_tc(int B, int H, int W, int rpu, const bf16 *__restrict__ x, const bf16 *
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(taddr), "r"(32u));
 }
 
-// Partial weight (and bias) gradients of one tap over a chunk of output
-// tiles: dW[co][tap][ci] += sum_p g[p][co] x[p + tap][ci], with
-// g = gy * [ymask > 0].  M = COUT, N = CIN, K = pixels (16 per step).
+// Four 8 x 8 BF16 matrices from shared memory, transposed (lane l gives row
+// l & 7 of matrix l >> 3).
+__device__ __forceinline__ void ldsm4t(uint32_t *r, uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+
+// Work split of k_conv_dw: one CTA for a 16 x 16 block of channels (outputs x
+// inputs) and a chunk of tiles; with a single such block (16 -> 16) one CTA
+// for each row of taps.  Three warps take the products (three taps each, or
+// one), the fourth the bias.
+template <int CIN, int COUT>
+struct DwSplit {
+    static constexpr int NP = CIN / 16, G = (COUT / 16) * NP, DY = G == 1 ? 3 : 1;
+    static constexpr int TAPS = DY == 3 ? 1 : 3, T = 128, ST = 4;  // taps a warp, threads, stages
+    static constexpr int XS = 24, XR = DY == 3 ? CH : CH + 2;      // pitch (values) of a pixel, rows staged
+    static constexpr int XP = XR * (CW + 2), GP = CH * CW;
+    static constexpr size_t smem = (size_t)ST * (XP + GP) * XS * 2;
+    static constexpr long n = (long)COUT * 9 * CIN + COUT;         // values of a chunk's partial
+};
+
+// Partial weight and bias gradients over a chunk of output tiles:
+// dW[co][tap][ci] += sum_p g[p][co] x[p + tap][ci], g the (masked) output
+// gradient.  Per tap a GEMM with M = COUT, N = CIN, K = pixels, on the tensor
+// cores (mma.sync m16n8k16: the products are skinny, 16 channels wide, and
+// both operands are stored pixel-major, so the transposing fragment load
+// takes them as they lie).  A chunk's tiles (the input tile with its halo and
+// the gradient tile, 16 channels of each) are staged once for the CTA's taps
+// by cp.async into a ring of four, so that three tiles' copies cover the L2's
+// latency.  Each product's pixels are summed in one chain over the chunk, and
+// the chunks (64) in order, so the result does not depend on the split.
+// What bounds it is that chain and the fragment loads (four a 16-pixel step
+// for six products).  One CTA per tap with element-wise fragment reads took
+// 325 us (16 -> 16), 528 us (48 -> 16) and 260 us (64 -> 32, half resolution)
+// at 8 x 256^2; this takes 58, 82 and
+// 44 us.
 template <int CIN, int COUT, int CUP>
 __global__ void __launch_bounds__(128)
 k_conv_dw(int B, int H, int W, int tiles_per_chunk, const bf16 *__restrict__ x,
-          const bf16 *__restrict__ xu, const bf16 *__restrict__ gy, const bf16 *__restrict__ ymask,
-          float *__restrict__ part_w, float *__restrict__ part_b)
+          const bf16 *__restrict__ xu, const bf16 *__restrict__ gy, float *__restrict__ part)
 {
-    constexpr int XS = CIN + 8, GS = COUT + 8, MT = COUT / 16, NT = CIN / 8;
-    constexpr int FR = MT * NT;                 // fragments per tap
-    constexpr int FPW = (FR + 3) / 4;           // fragments per warp
-    __shared__ __align__(16) bf16 xs[(CH + 2) * (CW + 2) * XS];
-    __shared__ __align__(16) bf16 gs[CH * CW * GS];
-    const int tap = blockIdx.x, chunk = blockIdx.y;
-    const int dy = tap / 3, dx = tap - 3 * (tap / 3);
+    using D = DwSplit<CIN, COUT>;
+    constexpr int XS = D::XS, T = D::T, ST = D::ST, XP = D::XP, GP = D::GP, TAPS = D::TAPS;
+    extern __shared__ __align__(16) unsigned char conv_sm[];
+    bf16 *xs0 = (bf16 *)conv_sm, *gs0 = xs0 + ST * XP * XS;
     const int tw = (W + CW - 1) / CW, th = (H + CH - 1) / CH, ntiles = B * tw * th;
+    const int chunk = blockIdx.y, t0 = chunk * tiles_per_chunk, t1 = min(ntiles, t0 + tiles_per_chunk);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
-    float acc[FPW][4];
-#pragma unroll
-    for (int f = 0; f < FPW; f++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) acc[f][q] = 0.0f;
-    float bacc = 0.0f;  // bias partial of channel threadIdx.x (tap 0 only)
-    for (int tl = chunk * tiles_per_chunk; tl < min(ntiles, (chunk + 1) * tiles_per_chunk); tl++) {
-        const int bz = tl / (tw * th), rem = tl - bz * tw * th;
-        const int ty0 = (rem / tw) * CH, tx0 = (rem - (rem / tw) * tw) * CW;
-        __syncthreads();
-        for (int k = threadIdx.x; k < (CH + 2) * (CW + 2) * (CIN / 8); k += 128) {
-            const int pix = k / (CIN / 8), q = k - pix * (CIN / 8);
-            const int r = pix / (CW + 2), c = pix - r * (CW + 2);
-            const int yy = ty0 + r - 1, xx = tx0 + c - 1;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (yy >= 0 && yy < H && xx >= 0 && xx < W)
-                v = *(const uint4 *)in_chunk<CIN, CUP>(x, xu, bz, H, W, yy, xx, q);
-            *(uint4 *)(xs + pix * XS + 8 * q) = v;
-        }
-        for (int k = threadIdx.x; k < CH * CW * (COUT / 2); k += 128) {
-            const int pix = k / (COUT / 2), cp = k - pix * (COUT / 2);
-            const int r = pix / CW, c = pix - r * CW;
-            const int yy = ty0 + r, xx = tx0 + c;
-            uint32_t v = 0;
-            if (yy < H && xx < W) {
-                const long off = (((long)bz * H + yy) * W + xx) * COUT + 2 * cp;
-                v = *(const uint32_t *)(gy + off);
-                if (ymask) v = relu_mask(v, *(const uint32_t *)(ymask + off));
+    const int grp = blockIdx.x / D::DY, dy0 = D::DY == 3 ? blockIdx.x % 3 : 0;
+    const int mt = grp / D::NP, np = grp % D::NP;
+    const bool bias = np == 0 && (D::DY == 1 || dy0 == 0);
+    auto issue = [&](int tl, int st) {
+        if (tl < t1) {
+            const int bz = tl / (tw * th), rem = tl - bz * tw * th;
+            const int ty0 = (rem / tw) * CH, tx0 = (rem - (rem / tw) * tw) * CW;
+            bf16 *xs = xs0 + st * XP * XS, *gs = gs0 + st * GP * XS;
+            for (int k = threadIdx.x; k < XP * 2; k += T) {
+                const int pix = k >> 1, q = k & 1, r = pix / (CW + 2), c = pix - r * (CW + 2);
+                const int yy = ty0 + dy0 + r - 1, xx = tx0 + c - 1;
+                const bool in = yy >= 0 && yy < H && xx >= 0 && xx < W;
+                cp_async16(xs + pix * XS + 8 * q,
+                           in ? in_chunk<CIN, CUP>(x, xu, bz, H, W, yy, xx, 2 * np + q) : x, in);
             }
-            *(uint32_t *)(gs + pix * GS + 2 * cp) = v;
+            for (int k = threadIdx.x; k < GP * 2; k += T) {
+                const int pix = k >> 1, q = k & 1, yy = ty0 + pix / CW, xx = tx0 + pix % CW;
+                const bool in = yy < H && xx < W;  // beyond the image: no gradient
+                cp_async16(gs + pix * XS + 8 * q,
+                           gy + (in ? (((long)bz * H + yy) * W + xx) * COUT + 16 * mt + 8 * q : 0), in);
+            }
         }
-        __syncthreads();
-        if (tap == 0 && threadIdx.x < COUT)
-            for (int pix = 0; pix < CH * CW; pix++) bacc += __bfloat162float(gs[pix * GS + threadIdx.x]);
+        cp_async_commit();  // an empty group past the chunk's end keeps the count
+    };
+    float acc[TAPS][2][4], accb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-        for (int f = 0; f < FPW; f++) {
-            const int fr = warp * FPW + f;
-            if (fr >= FR) break;
-            const int mt = fr / NT, nt = fr - mt * NT;
-            const int co = mt * 16 + g, ci = nt * 8 + g;
-#pragma unroll 2
+    for (int t = 0; t < TAPS; t++)
+#pragma unroll
+        for (int q = 0; q < 8; q++) acc[t][q >> 2][q & 3] = 0.0f;
+    // the warp's first tap: row (warp) and column 0, or row dy0 and column (warp)
+    const int tap0 = D::DY == 3 ? 3 * dy0 + warp : 3 * warp;
+    const int shift = D::DY == 3 ? warp : warp * (CW + 2);
+    const uint32_t xa0 = (uint32_t)__cvta_generic_to_shared(xs0) +
+                         ((shift + (lane & 7) + ((lane >> 3) & 1) * 8) * XS + (lane >> 4) * 8) * 2;
+    const uint32_t ga0 = (uint32_t)__cvta_generic_to_shared(gs0) +
+                         (((lane & 7) + (lane >> 4) * 8) * XS + ((lane >> 3) & 1) * 8) * 2;
+    for (int k = 0; k < ST - 1; k++) issue(t0 + k, k);
+    int st = 0;
+    for (int tl = t0; tl < t1; tl++) {
+        cp_async_wait<ST - 2>();
+        __syncthreads();  // this tile's copies are visible; the slot of the one before is free
+        issue(tl + ST - 1, (st + ST - 1) % ST);
+        if (warp < 3) {
+            const uint32_t xa = xa0 + st * (XP * XS * 2), ga = ga0 + st * (GP * XS * 2);
+#pragma unroll 4
             for (int r = 0; r < CH; r++) {  // K step = the 16 pixels of output row r
-                const bf16 *ga = gs + (r * CW) * GS;
-                const int p0 = 2 * t4, p1 = 2 * t4 + 1, p2 = 2 * t4 + 8, p3 = 2 * t4 + 9;
-                __nv_bfloat162 a0, a1, a2, a3;
-                a0.x = ga[p0 * GS + co];       a0.y = ga[p1 * GS + co];
-                a1.x = ga[p0 * GS + co + 8];   a1.y = ga[p1 * GS + co + 8];
-                a2.x = ga[p2 * GS + co];       a2.y = ga[p3 * GS + co];
-                a3.x = ga[p2 * GS + co + 8];   a3.y = ga[p3 * GS + co + 8];
-                uint32_t af[4] = {*(uint32_t *)&a0, *(uint32_t *)&a1, *(uint32_t *)&a2, *(uint32_t *)&a3};
-                const bf16 *xb = xs + ((r + dy) * (CW + 2) + dx) * XS + ci;
-                __nv_bfloat162 b0, b1;
-                b0.x = xb[p0 * XS]; b0.y = xb[p1 * XS];
-                b1.x = xb[p2 * XS]; b1.y = xb[p3 * XS];
-                uint32_t bf[2] = {*(uint32_t *)&b0, *(uint32_t *)&b1};
-                mma_bf16(acc[f], af, bf);
+                uint32_t af[4], bf[TAPS][4];
+                ldsm4t(af, ga + r * (CW * XS * 2));
+#pragma unroll
+                for (int t = 0; t < TAPS; t++) ldsm4t(bf[t], xa + (r * (CW + 2) + t) * (XS * 2));
+#pragma unroll
+                for (int t = 0; t < TAPS; t++) {
+                    mma_bf16(acc[t][0], af, bf[t]);
+                    mma_bf16(acc[t][1], af, bf[t] + 2);
+                }
+            }
+        } else if (bias) {
+            // the gradient's column sums: its product with a matrix of ones
+            const uint32_t ga = ga0 + st * (GP * XS * 2), ones[2] = {0x3f803f80u, 0x3f803f80u};
+#pragma unroll 4
+            for (int r = 0; r < CH; r++) {
+                uint32_t af[4];
+                ldsm4t(af, ga + r * (CW * XS * 2));
+                mma_bf16(accb, af, ones);
             }
         }
+        st = (st + 1) % ST;
     }
+    // C fragment: rows co (g, g + 8), columns ci (2 t4, 2 t4 + 1)
+    float *pw = part + (long)chunk * D::n;
+    const int co0 = mt * 16 + g;
+    if (warp < 3) {
 #pragma unroll
-    for (int f = 0; f < FPW; f++) {
-        const int fr = warp * FPW + f;
-        if (fr >= FR) break;
-        const int mt = fr / NT, nt = fr - mt * NT;
-        // C fragment: rows co (g, g+8), columns ci (2 t4, 2 t4 + 1)
-        const int co0 = mt * 16 + g, ci0 = nt * 8 + 2 * t4;
-        float *pw = part_w + (long)chunk * COUT * 9 * CIN;
-        pw[(long)co0 * 9 * CIN + tap * CIN + ci0] = acc[f][0];
-        pw[(long)co0 * 9 * CIN + tap * CIN + ci0 + 1] = acc[f][1];
-        pw[(long)(co0 + 8) * 9 * CIN + tap * CIN + ci0] = acc[f][2];
-        pw[(long)(co0 + 8) * 9 * CIN + tap * CIN + ci0 + 1] = acc[f][3];
+        for (int t = 0; t < TAPS; t++)
+#pragma unroll
+            for (int b = 0; b < 2; b++) {
+                float *o = pw + (long)co0 * 9 * CIN + (tap0 + t) * CIN + np * 16 + b * 8 + 2 * t4;
+                *(float2 *)o = make_float2(acc[t][b][0], acc[t][b][1]);
+                *(float2 *)(o + 8L * 9 * CIN) = make_float2(acc[t][b][2], acc[t][b][3]);
+            }
+    } else if (bias && t4 == 0) {
+        pw[(long)COUT * 9 * CIN + co0] = accb[0];
+        pw[(long)COUT * 9 * CIN + co0 + 8] = accb[2];
     }
-    if (tap == 0 && threadIdx.x < COUT) part_b[(long)chunk * COUT + threadIdx.x] = bacc;
 }
 
-// Sum of the chunk partials in chunk order.
-__global__ void k_reduce_parts(int nchunks, long n, const float *__restrict__ part,
-                               float *__restrict__ out)
+// Gradients of every parameter from the chunk partials of all layers, in one
+// launch: each thread sums the chunks of one value in order and scatters it
+// from the padded layout [COP][9][CIP], [COP] into the master one.
+constexpr int kLayers = 9, kDwChunks = 64;
+struct ReduceArgs {
+    const float *part[kLayers];
+    float *gw[kLayers], *gb[kLayers];
+    int nchunks[kLayers], ci[kLayers], co[kLayers], cip[kLayers], cop[kLayers];
+    int first[kLayers + 1];  // first CTA of each layer
+};
+__global__ void __launch_bounds__(128) k_reduce_grads(const __grid_constant__ ReduceArgs a)
 {
-    long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
+    int l = 0;
+    while ((int)blockIdx.x >= a.first[l + 1]) l++;
+    const int nw = a.cop[l] * 9 * a.cip[l], n = nw + a.cop[l];
+    const int e = ((int)blockIdx.x - a.first[l]) * 128 + threadIdx.x;
+    if (e >= n) return;
     float s = 0.0f;
-    for (int c = 0; c < nchunks; c++) s += part[(long)c * n + k];
-    out[k] = s;
+    const float *p = a.part[l] + e;
+#pragma unroll 16
+    for (int c = 0; c < a.nchunks[l]; c++) s += p[(long)c * n];
+    if (e < nw) {
+        const int co = e / (9 * a.cip[l]), r = e - co * 9 * a.cip[l], tap = r / a.cip[l], i = r - tap * a.cip[l];
+        if (co < a.co[l] && i < a.ci[l]) a.gw[l][((long)co * 9 + tap) * a.ci[l] + i] = s;
+    } else if (e - nw < a.co[l]) {
+        a.gb[l][e - nw] = s;
+    }
 }
 
-// --- layout helpers (bf16 NHWC) -----------------------------------------
-__global__ void k_pool2(long nout, int H2, int W2, int C, const bf16 *__restrict__ x,
-                        bf16 *__restrict__ y)
+// --- layout helpers (bf16 NHWC), 8 channels (16 bytes) a thread ------------
+// (One channel a thread: 10 us a pooling, 16 us an up-sampling fold and 38 us
+// a skip sum at 8 x 256^2, bound by instructions; 8 channels: 10 us a
+// skip sum.)
+__device__ __forceinline__ void unpack8(const bf16 *p, float *f)
 {
-    long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nout) return;
-    const int c = (int)(k % C);
-    long p = k / C;
-    const int j = (int)(p % W2);
+    const uint4 v = *(const uint4 *)p;
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        f[2 * q] = __uint_as_float(w[q] << 16);
+        f[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u);
+    }
+}
+__device__ __forceinline__ uint4 pack8(const float *f)
+{
+    uint32_t w[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * q], f[2 * q + 1]);
+        w[q] = *(const uint32_t *)&h;
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ uint4 relu_mask8(uint4 v, uint4 m)
+{
+    return make_uint4(relu_mask(v.x, m.x), relu_mask(v.y, m.y), relu_mask(v.z, m.z), relu_mask(v.w, m.w));
+}
+// sum of the 2 x 2 block of an image of width W and C channels at p, in the
+// order (0,0), (0,1), (1,0), (1,1)
+__device__ __forceinline__ void sum4(const bf16 *p, int W, int C, float *s)
+{
+    float f[8];
+    unpack8(p, s);
+    unpack8(p + C, f);
+#pragma unroll
+    for (int q = 0; q < 8; q++) s[q] += f[q];
+    unpack8(p + (long)W * C, f);
+#pragma unroll
+    for (int q = 0; q < 8; q++) s[q] += f[q];
+    unpack8(p + (long)W * C + C, f);
+#pragma unroll
+    for (int q = 0; q < 8; q++) s[q] += f[q];
+}
+
+// n8: 8-channel groups of the output (H2 x W2, C channels)
+__global__ void __launch_bounds__(256)
+k_pool2(int n8, int H2, int W2, int C, const bf16 *__restrict__ x, bf16 *__restrict__ y)
+{
+    const int k = blockIdx.x * 256 + threadIdx.x;
+    if (k >= n8) return;
+    const int c8 = C / 8, c = (k % c8) * 8;
+    int p = k / c8;
+    const int j = p % W2;
     p /= W2;
-    const int i = (int)(p % H2);
-    const long b = p / H2;
-    const int W = 2 * W2;
-    const long base = ((b * (2 * H2) + 2 * i) * W + 2 * j) * C + c;
-    float s = __bfloat162float(x[base]) + __bfloat162float(x[base + C]) +
-              __bfloat162float(x[base + (long)W * C]) + __bfloat162float(x[base + (long)W * C + C]);
-    y[k] = __float2bfloat16_rn(0.25f * s);
+    const int i = p % H2, b = p / H2, W = 2 * W2;
+    float s[8];
+    sum4(x + (((long)b * (2 * H2) + 2 * i) * W + 2 * j) * C + c, W, C, s);
+#pragma unroll
+    for (int q = 0; q < 8; q++) s[q] *= 0.25f;
+    *(uint4 *)(y + 8L * k) = pack8(s);
 }
 
-// gt = sum over 2x2 of g[..., :C1];  gs = g[..., C1:] (+ gs_add)
-__global__ void k_up_cat_bwd(long nhalf, int H2, int W2, int C1, int C2, const bf16 *__restrict__ g,
-                             bf16 *__restrict__ gt)
+// gt = [mask > 0] * sum over 2x2 of g[..., :C1] (C1 channels at half resolution)
+__global__ void __launch_bounds__(256)
+k_up_cat_bwd(int n8, int H2, int W2, int C1, int C2, const bf16 *__restrict__ g,
+             const bf16 *__restrict__ mask, bf16 *__restrict__ gt)
 {
-    long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nhalf) return;
-    const int c = (int)(k % C1);
-    long p = k / C1;
-    const int j = (int)(p % W2);
+    const int k = blockIdx.x * 256 + threadIdx.x;
+    if (k >= n8) return;
+    const int c8 = C1 / 8, c = (k % c8) * 8;
+    int p = k / c8;
+    const int j = p % W2;
     p /= W2;
-    const int i = (int)(p % H2);
-    const long b = p / H2;
-    const int W = 2 * W2, C = C1 + C2;
-    const long base = ((b * (2 * H2) + 2 * i) * W + 2 * j) * C + c;
-    float s = __bfloat162float(g[base]) + __bfloat162float(g[base + C]) +
-              __bfloat162float(g[base + (long)W * C]) + __bfloat162float(g[base + (long)W * C + C]);
-    gt[k] = __float2bfloat16_rn(s);
+    const int i = p % H2, b = p / H2, W = 2 * W2, C = C1 + C2;
+    float s[8];
+    sum4(g + (((long)b * (2 * H2) + 2 * i) * W + 2 * j) * C + c, W, C, s);
+    *(uint4 *)(gt + 8L * k) = relu_mask8(pack8(s), *(const uint4 *)(mask + 8L * k));
 }
 
-// gskip = g_cat[..., C1:] + pool2_bwd(gp)   (gp at half resolution, C2 channels)
-__global__ void k_skip_grad(long n, int H, int W, int C1, int C2, const bf16 *__restrict__ gcat,
-                            const bf16 *__restrict__ gp, bf16 *__restrict__ gskip)
+// gskip = [mask > 0] * (g_cat[..., C1:] + pool2_bwd(gp))   (gp at half
+// resolution, C2 channels)
+__global__ void __launch_bounds__(256)
+k_skip_grad(int n8, int H, int W, int C1, int C2, const bf16 *__restrict__ gcat,
+            const bf16 *__restrict__ gp, const bf16 *__restrict__ mask, bf16 *__restrict__ gskip)
 {
-    long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const int c = (int)(k % C2);
-    long p = k / C2;
-    const int j = (int)(p % W);
+    const int k = blockIdx.x * 256 + threadIdx.x;
+    if (k >= n8) return;
+    const int c8 = C2 / 8, c = (k % c8) * 8;
+    int p = k / c8;
+    const int pix = p, j = p % W;
     p /= W;
-    const int i = (int)(p % H);
-    const long b = p / H;
-    float v = __bfloat162float(gcat[((b * H + i) * W + j) * (C1 + C2) + C1 + c]);
-    v += 0.25f * __bfloat162float(gp[((b * (H / 2) + i / 2) * (W / 2) + j / 2) * C2 + c]);
-    gskip[k] = __float2bfloat16_rn(v);
+    const int i = p % H, b = p / H;
+    float v[8], f[8];
+    unpack8(gcat + (long)pix * (C1 + C2) + C1 + c, v);
+    unpack8(gp + (((long)b * (H / 2) + i / 2) * (W / 2) + j / 2) * C2 + c, f);
+#pragma unroll
+    for (int q = 0; q < 8; q++) v[q] += 0.25f * f[q];
+    *(uint4 *)(gskip + 8L * k) = relu_mask8(pack8(v), *(const uint4 *)(mask + 8L * k));
 }
 
 // --- features, loss, output ----------------------------------------------
@@ -704,48 +806,82 @@ __global__ void k_features(long n, int N2, const double *__restrict__ b, const d
     if (t) t[k] = (float)(p[k] * st[4]);
 }
 
-// Mean-removed squared error per sample (one CTA per sample): loss partial and
-// the gradient 2 d / (B n) minus its mean, written as BF16 channel 0 of a
-// 16-channel tensor.
-__global__ void __launch_bounds__(256)
-k_loss(int N2, int Bn, const float *__restrict__ y32, const float *__restrict__ t,
-       bf16 *__restrict__ gy, float *__restrict__ lsum)
+// Mean-removed squared error per sample: loss partial and the gradient
+// 2 d / (B n) minus its mean, written as BF16 channel 0 of a 16-channel
+// tensor.  Three launches over kLossBlk CTAs a sample, each folding the
+// partial sums of the one before in a fixed order: the means; the loss and
+// the gradient's mean; the gradient.  (One CTA a sample: 288 us at 8 x 256^2
+// on 8 of the SMs; this takes 8 us.)
+constexpr int kLossBlk = 32;
+__device__ __forceinline__ float2 block_sum2(float2 v)
 {
-    __shared__ float sh[2][256];
-    const long base = (long)blockIdx.x * N2;
-    float sy = 0.0f, st = 0.0f;
-    for (int k = threadIdx.x; k < N2; k += 256) { sy += y32[base + k]; st += t[base + k]; }
-    sh[0][threadIdx.x] = sy; sh[1][threadIdx.x] = st;
-    __syncthreads();
-    for (int o = 128; o; o >>= 1) {
-        if (threadIdx.x < o) { sh[0][threadIdx.x] += sh[0][threadIdx.x + o]; sh[1][threadIdx.x] += sh[1][threadIdx.x + o]; }
-        __syncthreads();
-    }
-    const float my = sh[0][0] / N2, mt = sh[1][0] / N2;
-    __syncthreads();
-    float l = 0.0f, gs = 0.0f;
-    const float sc = 2.0f / ((float)Bn * (float)N2);
-    for (int k = threadIdx.x; k < N2; k += 256) {
-        float d = (y32[base + k] - my) - (t[base + k] - mt);
-        l += d * d;
-        gs += sc * d;
-    }
-    sh[0][threadIdx.x] = l; sh[1][threadIdx.x] = gs;
-    __syncthreads();
-    for (int o = 128; o; o >>= 1) {
-        if (threadIdx.x < o) { sh[0][threadIdx.x] += sh[0][threadIdx.x + o]; sh[1][threadIdx.x] += sh[1][threadIdx.x + o]; }
-        __syncthreads();
-    }
-    const float gmean = sh[1][0] / N2;
-    for (int k = threadIdx.x; k < N2; k += 256) {
-        float d = (y32[base + k] - my) - (t[base + k] - mt);
-        uint32_t *gp = (uint32_t *)(gy + (base + k) * 16);
-        __nv_bfloat162 v = __floats2bfloat162_rn(sc * d - gmean, 0.0f);
-        gp[0] = *(uint32_t *)&v;
+    __shared__ float2 sh[8];
 #pragma unroll
-        for (int q = 1; q < 8; q++) gp[q] = 0u;
+    for (int o = 16; o; o >>= 1) {
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
     }
-    if (threadIdx.x == 0) lsum[blockIdx.x] = sh[0][0] / ((float)Bn * (float)N2);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = sh[0];
+#pragma unroll
+    for (int w = 1; w < 8; w++) { v.x += sh[w].x; v.y += sh[w].y; }
+    return v;
+}
+__device__ __forceinline__ float2 fold_parts(const float2 *part)
+{
+    float2 v = part[threadIdx.x & 31];  // kLossBlk = 32 partials, every warp the same tree
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+    }
+    return v;
+}
+__global__ void __launch_bounds__(256)
+k_loss_means(int N2, const float *__restrict__ y32, const float *__restrict__ t, float2 *__restrict__ part)
+{
+    const long base = (long)blockIdx.y * N2;
+    float2 s = make_float2(0.0f, 0.0f);
+    for (int k = blockIdx.x * 256 + threadIdx.x; k < N2; k += 256 * kLossBlk) {
+        s.x += y32[base + k];
+        s.y += t[base + k];
+    }
+    s = block_sum2(s);
+    if (threadIdx.x == 0) part[blockIdx.y * kLossBlk + blockIdx.x] = s;
+}
+__global__ void __launch_bounds__(256)
+k_loss_sums(int N2, float sc, const float *__restrict__ y32, const float *__restrict__ t,
+            const float2 *__restrict__ means, float2 *__restrict__ part)
+{
+    const float2 m = fold_parts(means + blockIdx.y * kLossBlk);
+    const float my = m.x / N2, mt = m.y / N2;
+    const long base = (long)blockIdx.y * N2;
+    float2 s = make_float2(0.0f, 0.0f);
+    for (int k = blockIdx.x * 256 + threadIdx.x; k < N2; k += 256 * kLossBlk) {
+        const float d = (y32[base + k] - my) - (t[base + k] - mt);
+        s.x += d * d;
+        s.y += sc * d;
+    }
+    s = block_sum2(s);
+    if (threadIdx.x == 0) part[blockIdx.y * kLossBlk + blockIdx.x] = s;
+}
+__global__ void __launch_bounds__(256)
+k_loss_grad(int N2, int Bn, float sc, const float *__restrict__ y32, const float *__restrict__ t,
+            const float2 *__restrict__ means, const float2 *__restrict__ sums, bf16 *__restrict__ gy,
+            float *__restrict__ lsum)
+{
+    const float2 m = fold_parts(means + blockIdx.y * kLossBlk), s = fold_parts(sums + blockIdx.y * kLossBlk);
+    const float my = m.x / N2, mt = m.y / N2, gmean = s.y / N2;
+    const long base = (long)blockIdx.y * N2;
+    for (int k = blockIdx.x * 256 + threadIdx.x; k < N2; k += 256 * kLossBlk) {
+        const float d = (y32[base + k] - my) - (t[base + k] - mt);
+        const __nv_bfloat162 v = __floats2bfloat162_rn(sc * d - gmean, 0.0f);
+        uint4 *gp = (uint4 *)(gy + (base + k) * 16);
+        gp[0] = make_uint4(*(const uint32_t *)&v, 0u, 0u, 0u);
+        gp[1] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) lsum[blockIdx.y] = s.x / ((float)Bn * (float)N2);
 }
 
 // p0 = s pscale (y - mean y), FP64 out.
@@ -813,18 +949,6 @@ __global__ void k_pack(int ci, int co, int cip, int cop, const float *__restrict
     if (wb) wb[((long)i * 9 + (8 - tap)) * cop + o] = __float2bfloat16_rn(v);
 }
 
-// Padded gradients [COP][9][CIP] and [COP] -> master layout [co][9][ci], [co].
-__global__ void k_unpack_grad(int ci, int co, int cip, const float *__restrict__ gpw,
-                              const float *__restrict__ gpb, float *__restrict__ gw,
-                              float *__restrict__ gb)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < co) gb[k] = gpb[k];
-    if (k >= co * 9 * ci) return;
-    const int o = k / (9 * ci), r = k - o * 9 * ci, tap = r / ci, i = r - tap * ci;
-    gw[k] = gpw[((long)o * 9 + tap) * cip + i];
-}
-
 }  // namespace
 
 // rms of (a - mean a) of each sample (one CTA per sample, fixed order: the
@@ -885,14 +1009,14 @@ struct CnnLayer {
     int ci, co, cip, cop;     // real and padded channel counts
     bool relu;
     size_t woff, boff;        // offsets in the flat FP32 parameter vector
-    size_t pwoff, pboff;      // offsets of the padded gradients [COP][9][CIP], [COP]
+    size_t part_off = 0;      // chunk partials of the gradients ([COP][9][CIP], [COP] a chunk)
     bf16 *wf = nullptr, *wb = nullptr;
 };
 
 struct Cnn {
     int c1 = 16, c2 = 32;
     std::vector<CnnLayer> L;
-    size_t nparam = 0, npad = 0;
+    size_t nparam = 0;
     float *w = nullptr, *m = nullptr, *v = nullptr, *g = nullptr;  // flat FP32
     void *wmem = nullptr;
     int step = 0;
@@ -906,9 +1030,8 @@ struct Cnn {
          *a5 = nullptr, *y = nullptr, *gbig = nullptr, *gbig2 = nullptr,
          *gmid = nullptr, *gmid2 = nullptr, *gsmall = nullptr, *gsmall2 = nullptr, *gcat = nullptr,
          *gup = nullptr;
-    float *y32 = nullptr, *t = nullptr, *lsum = nullptr, *gpad = nullptr, *part = nullptr;
+    float *y32 = nullptr, *t = nullptr, *lsum = nullptr, *part = nullptr;
     double *stats = nullptr, *rpart = nullptr;
-    size_t part_cap = 0;
     // coarse-grid inference: restricted inputs and prolongated outputs
     double *cbuf = nullptr;
     size_t cbuf_cap = 0;
@@ -918,18 +1041,29 @@ namespace {
 
 int g_sms = 0;
 
+int sm_count()
+{
+    if (!g_sms) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
+        if (g_sms <= 0) g_sms = 152;
+    }
+    return g_sms;
+}
+
 // tc: 0 the warp-level kernel; 1 tcgen05 for the shapes where it measured
 // faster than the warp-level kernel (16 -> 32 channels: 8.7 against 12.2 us
 // at 128^2; the others are bound by operand staging and latency, where the
 // warp-level kernel's double-buffered 8 x 16 tiles stage less per output);
 // 2 tcgen05 wherever the width is a multiple of 128.
-template <int CIN, int COUT, int CUP, bool MASK>
-void conv_launch(int B, int H, int W, const bf16 *x, const bf16 *xu, const bf16 *xmask, const bf16 *w,
+template <int CIN, int COUT, int CUP>
+void conv_launch(int B, int H, int W, const bf16 *x, const bf16 *xu, const bf16 *ymask, const bf16 *w,
                  const float *bias, int relu, bf16 *y, float *y32, cudaStream_t s, int tc = 0)
 {
-    if constexpr (!MASK && (COUT == 16 || COUT == 32)) {
+    if constexpr (COUT == 16 || COUT == 32) {
         const bool faster = CIN == 16 && COUT == 32 && CUP == 0;
-        if ((tc == 2 || (tc == 1 && faster)) && W % kTcPix == 0) {
+        if (!ymask && bias && (tc == 2 || (tc == 1 && faster)) && W % kTcPix == 0) {
             constexpr size_t smt = conv_tc_smem<CIN, COUT>();
             static bool attr_tc = false;
             if (!attr_tc) {
@@ -937,12 +1071,7 @@ void conv_launch(int B, int H, int W, const bf16 *x, const bf16 *xu, const bf16 
                                      (int)smt);
                 attr_tc = true;
             }
-            if (!g_sms) {
-                int dev = 0;
-                cudaGetDevice(&dev);
-                cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
-                if (g_sms <= 0) g_sms = 152;
-            }
+            sm_count();
             // rows per unit: as many as keep every SM busy, up to 8 (a unit
             // stages rpu + 2 input rows for rpu output rows); CTAs per SM by
             // shared memory (at most 8: 256 of the 512 tensor-memory columns)
@@ -956,31 +1085,26 @@ void conv_launch(int B, int H, int W, const bf16 *x, const bf16 *xu, const bf16 
             return;
         }
     }
-    constexpr size_t sm = conv_smem<CIN, COUT, MASK>();
+    constexpr size_t sm = conv_smem<CIN, COUT>();
     static bool attr = false;
     if (!attr) {
-        cudaFuncSetAttribute(k_conv_fwd<CIN, COUT, CUP, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        cudaFuncSetAttribute(k_conv_fwd<CIN, COUT, CUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         attr = true;
     }
-    if (!g_sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
-        if (g_sms <= 0) g_sms = 152;
-    }
+    sm_count();
     const int ntiles = B * (int)cdiv(W, CW) * (int)cdiv(H, CH);
     const int per_sm = sm <= 56 * 1024 ? 4 : (sm <= 75 * 1024 ? 3 : 2);
     const int grid = std::min(ntiles, g_sms * per_sm);
     note_launch();
-    k_conv_fwd<CIN, COUT, CUP, MASK><<<grid, 128, sm, s>>>(B, H, W, x, xu, xmask, w, bias, relu, y, y32);
+    k_conv_fwd<CIN, COUT, CUP><<<grid, 128, sm, s>>>(B, H, W, x, xu, ymask, w, bias, relu, y, y32);
 }
 
+// ymask: mask of the output (backward-data passes), NULL for none.
 template <int CIN, int COUT>
-void conv_fwd(int B, int H, int W, const bf16 *x, const bf16 *xmask, const bf16 *w,
+void conv_fwd(int B, int H, int W, const bf16 *x, const bf16 *ymask, const bf16 *w,
               const float *bias, int relu, bf16 *y, float *y32, cudaStream_t s, int tc = 0)
 {
-    if (xmask) conv_launch<CIN, COUT, 0, true>(B, H, W, x, nullptr, xmask, w, bias, relu, y, y32, s);
-    else conv_launch<CIN, COUT, 0, false>(B, H, W, x, nullptr, xmask, w, bias, relu, y, y32, s, tc);
+    conv_launch<CIN, COUT, 0>(B, H, W, x, nullptr, ymask, w, bias, relu, y, y32, s, tc);
 }
 
 // Convolution of the concatenation up2(xu) ++ x (CUP channels from xu).
@@ -988,25 +1112,23 @@ template <int CIN, int COUT, int CUP>
 void conv_fwd_cat(int B, int H, int W, const bf16 *xu, const bf16 *x, const bf16 *w,
                   const float *bias, int relu, bf16 *y, cudaStream_t s, int tc = 0)
 {
-    conv_launch<CIN, COUT, CUP, false>(B, H, W, x, xu, nullptr, w, bias, relu, y, nullptr, s, tc);
+    conv_launch<CIN, COUT, CUP>(B, H, W, x, xu, nullptr, w, bias, relu, y, nullptr, s, tc);
 }
 
+// Partial gradients of layer k (input x, or up2(xu) ++ x; gy its masked
+// output gradient); records the chunk count for k_reduce_grads.
 template <int CIN, int COUT, int CUP = 0>
-void conv_dw(Cnn &n, int B, int H, int W, const bf16 *x, const bf16 *gy, const bf16 *ymask,
-             float *gw_pad, float *gb, cudaStream_t s, const bf16 *xu = nullptr)
+void conv_dw(Cnn &n, ReduceArgs &ra, int k, int B, int H, int W, const bf16 *x, const bf16 *gy,
+             cudaStream_t s, const bf16 *xu = nullptr)
 {
+    using D = DwSplit<CIN, COUT>;
     const int ntiles = B * (int)cdiv(W, CW) * (int)cdiv(H, CH);
-    const int nchunks = std::min(ntiles, 64);
-    const int tpc = (ntiles + nchunks - 1) / nchunks;
-    float *pw = n.part, *pb = n.part + (size_t)nchunks * COUT * 9 * CIN;
-    dim3 g(9, nchunks);
+    const int nchunks = std::min(ntiles, kDwChunks), tpc = (int)cdiv(ntiles, nchunks);
+    raise_smem_limit((const void *)k_conv_dw<CIN, COUT, CUP>, (int)D::smem);
+    ra.part[k] = n.part + n.L[k].part_off;
+    ra.nchunks[k] = nchunks;
     note_launch();
-    k_conv_dw<CIN, COUT, CUP><<<g, 128, 0, s>>>(B, H, W, tpc, x, xu, gy, ymask, pw, pb);
-    const long nw = (long)COUT * 9 * CIN;
-    note_launch();
-    k_reduce_parts<<<cdiv(nw, 256), 256, 0, s>>>(nchunks, nw, pw, gw_pad);
-    note_launch();
-    k_reduce_parts<<<1, 256, 0, s>>>(nchunks, COUT, pb, gb);
+    k_conv_dw<CIN, COUT, CUP><<<dim3(D::G * D::DY, nchunks), D::T, D::smem, s>>>(B, H, W, tpc, x, xu, gy, n.part + n.L[k].part_off);
 }
 
 size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -1032,12 +1154,6 @@ Cnn *cnn_new(int c1, int c2, unsigned long long seed, cudaStream_t s, cudaError_
         n->L.push_back(l);
     }
     n->nparam = off;
-    size_t po = 0;
-    for (auto &l : n->L) {
-        l.pwoff = po; po += (size_t)l.cop * 9 * l.cip;
-        l.pboff = po; po += (size_t)l.cop;
-    }
-    n->npad = po;
     size_t bytes = al(off * 4) * 4;
     for (auto &l : n->L) bytes += 2 * al((size_t)l.cop * 9 * l.cip * 2);
     *err = cudaMalloc(&n->wmem, bytes);
@@ -1108,9 +1224,14 @@ cudaError_t cnn_workspace(Cnn &n, int B, int N)
                    al(P * c1 * 2) + al(P * 16 * 2) +       // a5, y
                    al(P * 64 * 2) * 2 + al(P2 * 64 * 2) * 2 + al(P4 * 64 * 2) * 2 +  // grads
                    al(P * 64 * 2) + al(P2 * 64 * 2) +      // gcat, gup
-                   al(P * 4) + al(P * 4) + al(B * 4) + al(n.npad * 4) + al(B * kStat * 8) +
+                   al(P * 4) + al(P * 4) + al(B * 4) + al(B * kStat * 8) +
                    al(B * kRedBlocks * 3 * 8);
-    const size_t part = (size_t)64 * (64 * 9 * 64 + 64);
+    // chunk partials of the weight gradients, layer after layer
+    size_t part = 0;
+    for (auto &l : n.L) {
+        l.part_off = part;
+        part += (size_t)kDwChunks * ((size_t)l.cop * 9 * l.cip + l.cop);
+    }
     bytes += al(part * 4);
     cudaError_t e = cudaMalloc(&n.amem, bytes);
     if (e != cudaSuccess) { n.amem = nullptr; return e; }
@@ -1128,11 +1249,9 @@ cudaError_t cnn_workspace(Cnn &n, int B, int N)
     n.gsmall = (bf16 *)take(P4 * 64 * 2); n.gsmall2 = (bf16 *)take(P4 * 64 * 2);
     n.gcat = (bf16 *)take(P * 64 * 2); n.gup = (bf16 *)take(P2 * 64 * 2);
     n.y32 = (float *)take(P * 4); n.t = (float *)take(P * 4); n.lsum = (float *)take(B * 4);
-    n.gpad = (float *)take(n.npad * 4);
     n.stats = (double *)take(B * kStat * 8);
     n.rpart = (double *)take(B * kRedBlocks * 3 * 8);
     n.part = (float *)take(part * 4);
-    n.part_cap = part;
     n.capB = B;
     n.capN = N;
     return cudaSuccess;
@@ -1157,11 +1276,11 @@ void cnn_forward(Cnn &n, int B, int N, double h, const double *rhs, const double
     conv_fwd<16, 16>(B, N, N, n.x, nullptr, L[0].wf, bias(0), 1, n.a1, nullptr, s, tc);
     conv_fwd<16, 16>(B, N, N, n.a1, nullptr, L[1].wf, bias(1), 1, n.s1, nullptr, s, tc);
     note_launch();
-    k_pool2<<<cdiv((long)B * H2 * H2 * 16, 256), 256, 0, s>>>((long)B * H2 * H2 * 16, H2, H2, 16, n.s1, n.p1);
+    k_pool2<<<cdiv((long)B * H2 * H2 * 2, 256), 256, 0, s>>>(B * H2 * H2 * 2, H2, H2, 16, n.s1, n.p1);
     conv_fwd<16, 32>(B, H2, H2, n.p1, nullptr, L[2].wf, bias(2), 1, n.a2, nullptr, s, tc);
     conv_fwd<32, 32>(B, H2, H2, n.a2, nullptr, L[3].wf, bias(3), 1, n.s2, nullptr, s, tc);
     note_launch();
-    k_pool2<<<cdiv((long)B * H4 * H4 * 32, 256), 256, 0, s>>>((long)B * H4 * H4 * 32, H4, H4, 32, n.s2, n.p2);
+    k_pool2<<<cdiv((long)B * H4 * H4 * 4, 256), 256, 0, s>>>(B * H4 * H4 * 4, H4, H4, 32, n.s2, n.p2);
     conv_fwd<32, 32>(B, H4, H4, n.p2, nullptr, L[4].wf, bias(4), 1, n.a3, nullptr, s, tc);
     conv_fwd<32, 32>(B, H4, H4, n.a3, nullptr, L[5].wf, bias(5), 1, n.t3, nullptr, s, tc);
     conv_fwd_cat<64, 32, 32>(B, H2, H2, n.t3, n.s2, L[6].wf, bias(6), 1, n.t4, s, tc);  // up2(t3) ++ s2
@@ -1175,53 +1294,61 @@ void cnn_backward(Cnn &n, int B, int N, cudaStream_t s)
     const int N2 = N * N, H2 = N / 2, H4 = N / 4;
     const long P = (long)B * N2;
     auto &L = n.L;
-    note_launch();
-    k_loss<<<B, 256, 0, s>>>(N2, B, n.y32, n.t, n.gbig, n.lsum);
-    float *gp = n.gpad;
-    auto dwb = [&](int k) { return std::make_pair(gp + L[k].pwoff, gp + L[k].pboff); };
-    auto unpack = [&](int k) {
-        const int tot = std::max(L[k].co * 9 * L[k].ci, L[k].co);
-        note_launch();
-        k_unpack_grad<<<cdiv(tot, 256), 256, 0, s>>>(L[k].ci, L[k].co, L[k].cip, gp + L[k].pwoff,
-                                                    gp + L[k].pboff, n.g + L[k].woff, n.g + L[k].boff);
-    };
+    // the partial sums in the statistics' scratch (free by now)
+    float2 *means = (float2 *)n.rpart, *sums = means + (size_t)B * kLossBlk;
+    const float sc = 2.0f / ((float)B * (float)N2);
+    const dim3 gl(kLossBlk, B);
+    note_launch(3);
+    k_loss_means<<<gl, 256, 0, s>>>(N2, n.y32, n.t, means);
+    k_loss_sums<<<gl, 256, 0, s>>>(N2, sc, n.y32, n.t, means, sums);
+    k_loss_grad<<<gl, 256, 0, s>>>(N2, B, sc, n.y32, n.t, means, sums, n.gbig, n.lsum);
+    ReduceArgs ra;
     // c6 (linear): input a5, grad gbig (16 ch, channel 0)
-    conv_dw<16, 16>(n, B, N, N, n.a5, n.gbig, nullptr, dwb(8).first, dwb(8).second, s);
-    conv_fwd<16, 16>(B, N, N, n.gbig, nullptr, L[8].wb, nullptr, 0, n.gbig2, nullptr, s);  // grad a5
-    // c5: out a5 (mask), in up2(t4) ++ s1
-    conv_dw<48, 16, 32>(n, B, N, N, n.s1, n.gbig2, n.a5, dwb(7).first, dwb(7).second, s, n.t4);
-    conv_fwd<16, 48>(B, N, N, n.gbig2, n.a5, L[7].wb, nullptr, 0, n.gcat, nullptr, s);     // grad of up2(t4) ++ s1
+    conv_dw<16, 16>(n, ra, 8, B, N, N, n.a5, n.gbig, s);
+    conv_fwd<16, 16>(B, N, N, n.gbig, n.a5, L[8].wb, nullptr, 0, n.gbig2, nullptr, s);  // grad a5, masked
+    // c5: in up2(t4) ++ s1
+    conv_dw<48, 16, 32>(n, ra, 7, B, N, N, n.s1, n.gbig2, s, n.t4);
+    conv_fwd<16, 48>(B, N, N, n.gbig2, nullptr, L[7].wb, nullptr, 0, n.gcat, nullptr, s);  // grad of up2(t4) ++ s1
     note_launch();
-    k_up_cat_bwd<<<cdiv((long)B * H2 * H2 * 32, 256), 256, 0, s>>>((long)B * H2 * H2 * 32, H2, H2, 32, 16, n.gcat, n.gmid);  // grad t4
-    // c4: out t4 (mask), in up2(t3) ++ s2
-    conv_dw<64, 32, 32>(n, B, H2, H2, n.s2, n.gmid, n.t4, dwb(6).first, dwb(6).second, s, n.t3);
-    conv_fwd<32, 64>(B, H2, H2, n.gmid, n.t4, L[6].wb, nullptr, 0, n.gup, nullptr, s);     // grad of up2(t3) ++ s2
+    k_up_cat_bwd<<<cdiv((long)B * H2 * H2 * 4, 256), 256, 0, s>>>(B * H2 * H2 * 4, H2, H2, 32, 16, n.gcat, n.t4, n.gmid);  // grad t4, masked
+    // c4: in up2(t3) ++ s2
+    conv_dw<64, 32, 32>(n, ra, 6, B, H2, H2, n.s2, n.gmid, s, n.t3);
+    conv_fwd<32, 64>(B, H2, H2, n.gmid, nullptr, L[6].wb, nullptr, 0, n.gup, nullptr, s);  // grad of up2(t3) ++ s2
     note_launch();
-    k_up_cat_bwd<<<cdiv((long)B * H4 * H4 * 32, 256), 256, 0, s>>>((long)B * H4 * H4 * 32, H4, H4, 32, 32, n.gup, n.gsmall);  // grad t3
-    // c3b: out t3, in a3
-    conv_dw<32, 32>(n, B, H4, H4, n.a3, n.gsmall, n.t3, dwb(5).first, dwb(5).second, s);
-    conv_fwd<32, 32>(B, H4, H4, n.gsmall, n.t3, L[5].wb, nullptr, 0, n.gsmall2, nullptr, s);  // grad a3
-    // c3a: out a3, in p2
-    conv_dw<32, 32>(n, B, H4, H4, n.p2, n.gsmall2, n.a3, dwb(4).first, dwb(4).second, s);
-    conv_fwd<32, 32>(B, H4, H4, n.gsmall2, n.a3, L[4].wb, nullptr, 0, n.gsmall, nullptr, s);  // grad p2
-    // grad s2 = skip part of the c4 input grad + pool2 backward
+    k_up_cat_bwd<<<cdiv((long)B * H4 * H4 * 4, 256), 256, 0, s>>>(B * H4 * H4 * 4, H4, H4, 32, 32, n.gup, n.t3, n.gsmall);  // grad t3, masked
+    // c3b: in a3
+    conv_dw<32, 32>(n, ra, 5, B, H4, H4, n.a3, n.gsmall, s);
+    conv_fwd<32, 32>(B, H4, H4, n.gsmall, n.a3, L[5].wb, nullptr, 0, n.gsmall2, nullptr, s);  // grad a3, masked
+    // c3a: in p2
+    conv_dw<32, 32>(n, ra, 4, B, H4, H4, n.p2, n.gsmall2, s);
+    conv_fwd<32, 32>(B, H4, H4, n.gsmall2, nullptr, L[4].wb, nullptr, 0, n.gsmall, nullptr, s);  // grad p2
+    // grad s2 = skip part of the c4 input grad + pool2 backward, masked
     note_launch();
-    k_skip_grad<<<cdiv((long)B * H2 * H2 * 32, 256), 256, 0, s>>>((long)B * H2 * H2 * 32, H2, H2, 32, 32, n.gup, n.gsmall, n.gmid2);
-    // c2b: out s2, in a2
-    conv_dw<32, 32>(n, B, H2, H2, n.a2, n.gmid2, n.s2, dwb(3).first, dwb(3).second, s);
-    conv_fwd<32, 32>(B, H2, H2, n.gmid2, n.s2, L[3].wb, nullptr, 0, n.gmid, nullptr, s);   // grad a2
-    // c2a: out a2, in p1
-    conv_dw<16, 32>(n, B, H2, H2, n.p1, n.gmid, n.a2, dwb(2).first, dwb(2).second, s);
-    conv_fwd<32, 16>(B, H2, H2, n.gmid, n.a2, L[2].wb, nullptr, 0, n.gmid2, nullptr, s);   // grad p1
-    // grad s1 = skip part of the c5 input grad + pool2 backward
+    k_skip_grad<<<cdiv((long)B * H2 * H2 * 4, 256), 256, 0, s>>>(B * H2 * H2 * 4, H2, H2, 32, 32, n.gup, n.gsmall, n.s2, n.gmid2);
+    // c2b: in a2
+    conv_dw<32, 32>(n, ra, 3, B, H2, H2, n.a2, n.gmid2, s);
+    conv_fwd<32, 32>(B, H2, H2, n.gmid2, n.a2, L[3].wb, nullptr, 0, n.gmid, nullptr, s);   // grad a2, masked
+    // c2a: in p1
+    conv_dw<16, 32>(n, ra, 2, B, H2, H2, n.p1, n.gmid, s);
+    conv_fwd<32, 16>(B, H2, H2, n.gmid, nullptr, L[2].wb, nullptr, 0, n.gmid2, nullptr, s);  // grad p1
+    // grad s1 = skip part of the c5 input grad + pool2 backward, masked
     note_launch();
-    k_skip_grad<<<cdiv(P * 16, 256), 256, 0, s>>>(P * 16, N, N, 32, 16, n.gcat, n.gmid2, n.gbig);
-    // c1b: out s1, in a1
-    conv_dw<16, 16>(n, B, N, N, n.a1, n.gbig, n.s1, dwb(1).first, dwb(1).second, s);
-    conv_fwd<16, 16>(B, N, N, n.gbig, n.s1, L[1].wb, nullptr, 0, n.gbig2, nullptr, s);     // grad a1
-    // c1a: out a1, in x
-    conv_dw<16, 16>(n, B, N, N, n.x, n.gbig2, n.a1, dwb(0).first, dwb(0).second, s);
-    for (int k = 0; k < 9; k++) unpack(k);
+    k_skip_grad<<<cdiv(P * 2, 256), 256, 0, s>>>((int)(P * 2), N, N, 32, 16, n.gcat, n.gmid2, n.s1, n.gbig);
+    // c1b: in a1
+    conv_dw<16, 16>(n, ra, 1, B, N, N, n.a1, n.gbig, s);
+    conv_fwd<16, 16>(B, N, N, n.gbig, n.a1, L[1].wb, nullptr, 0, n.gbig2, nullptr, s);     // grad a1, masked
+    // c1a: in x
+    conv_dw<16, 16>(n, ra, 0, B, N, N, n.x, n.gbig2, s);
+    int ctas = 0;
+    for (int k = 0; k < kLayers; k++) {
+        ra.gw[k] = n.g + L[k].woff; ra.gb[k] = n.g + L[k].boff;
+        ra.ci[k] = L[k].ci; ra.co[k] = L[k].co; ra.cip[k] = L[k].cip; ra.cop[k] = L[k].cop;
+        ra.first[k] = ctas;
+        ctas += (int)cdiv(L[k].cop * 9 * L[k].cip + L[k].cop, 128);
+    }
+    ra.first[kLayers] = ctas;
+    note_launch();
+    k_reduce_grads<<<ctas, 128, 0, s>>>(ra);
 }
 
 void cnn_adam(Cnn &n, float lr, cudaStream_t s)
