@@ -308,11 +308,11 @@ ib_status cnn_set_coarsen(ib_cnn *net, int32_t levels);   /* 0 .. 6 */
 /* Convolution path of the forward pass: 0 the warp-level mma.sync kernel
  * for every layer; 1 (default) the fifth-generation tensor cores
  * (tcgen05.mma, FP32 accumulators in tensor memory) for the layer shapes
- * where they measured faster (16 -> 32 channels) when the width is a
- * multiple of 128, the warp-level kernel elsewhere; 2 tcgen05 for every
- * layer whose width is a multiple of 128.  The paths accumulate in the same
- * order and agree bit for bit.  The backward pass always uses the
- * warp-level kernel.
+ * where they measure faster (at present none: the layers are bound by
+ * staging and latency, and 1 runs as 0); 2 tcgen05 for every layer whose
+ * width is a multiple of 128, the warp-level kernel elsewhere.  The paths
+ * accumulate in the same order and agree bit for bit.  The backward pass
+ * always uses the warp-level kernel.
  * cnn_grad and cnn_train return IB_ECUDA if a tensor-core completion wait
  * ran out (50 ms).                                                         */
 ib_status cnn_set_tensor_path(ib_cnn *net, int32_t mode);

@@ -479,7 +479,8 @@ class Net:
 
     def set_tensor_path(self, mode: int):
         """0: the warp-level mma.sync kernel everywhere; 1 (default): tcgen05
-        for the layer shapes where it is faster; 2: tcgen05 for every layer
+        for the layer shapes where it measures faster (at present none);
+        2: tcgen05 for every layer
         whose width is a multiple of 128 (see cnn_set_tensor_path)."""
         _check(lib().cnn_set_tensor_path(self._h, int(mode)), None, "cnn_set_tensor_path")
 

@@ -44,18 +44,18 @@ __device__ __forceinline__ uint32_t relu_mask(uint32_t v, uint32_t m)
     return r;
 }
 
-template <int CIN, int COUT>
-constexpr size_t conv_smem()
-{
-    return ((size_t)2 * (CH + 2) * (CW + 2) * (CIN + 8) + (size_t)COUT * (9 * CIN + 8)) * 2;
-}
-
 // 16-byte asynchronous copy (both addresses 16-byte aligned); src-size 0 writes zeros.
 __device__ __forceinline__ void cp_async16(void *sdst, const void *gsrc, bool valid)
 {
     const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
     const int sz = valid ? 16 : 0;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gsrc), "r"(sz));
+}
+__device__ __forceinline__ void cp_async4(void *sdst, const void *gsrc, bool valid)
+{
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
+    const int sz = valid ? 4 : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(sa), "l"(gsrc), "r"(sz));
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 template <int N>
@@ -75,56 +75,181 @@ __device__ __forceinline__ const bf16 *in_chunk(const bf16 *x, const bf16 *xu, i
     return x + (((long)bz * H + gy) * W + gx) * (CIN - CUP) + 8 * q - CUP;
 }
 
-// y = act(conv3x3(x) + bias) * [ymask > 0], NHWC, zero padding.
+// Four 8 x 8 BF16 matrices from (lane l gives row l & 7 of matrix l >> 3) or
+// to shared memory; ldsm4t transposes them.
+__device__ __forceinline__ void ldsm4(uint32_t *r, uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t *r, uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void stsm4(uint32_t addr, const uint32_t *r)
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};\n"
+                 ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+
+// 8 channels (16 bytes) as floats and back.
+__device__ __forceinline__ void unpack8(uint4 v, float *f)
+{
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        f[2 * q] = __uint_as_float(w[q] << 16);
+        f[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u);
+    }
+}
+__device__ __forceinline__ uint4 pack8(const float *f)
+{
+    uint32_t w[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * q], f[2 * q + 1]);
+        w[q] = *(const uint32_t *)&h;
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ uint4 relu_mask8(uint4 v, uint4 m)
+{
+    return make_uint4(relu_mask(v.x, m.x), relu_mask(v.y, m.y), relu_mask(v.z, m.z), relu_mask(v.w, m.w));
+}
+// scale * sum of four 8-channel groups, in order, as BF16
+__device__ __forceinline__ uint4 sum4(uint4 v0, uint4 v1, uint4 v2, uint4 v3, float scale)
+{
+    float a[8], f[8];
+    unpack8(v0, a);
+    unpack8(v1, f);
+#pragma unroll
+    for (int q = 0; q < 8; q++) a[q] += f[q];
+    unpack8(v2, f);
+#pragma unroll
+    for (int q = 0; q < 8; q++) a[q] += f[q];
+    unpack8(v3, f);
+#pragma unroll
+    for (int q = 0; q < 8; q++) a[q] = (a[q] + f[q]) * scale;
+    return pack8(a);
+}
+
+// What a convolution's epilogue makes of its output tile (plain: y, masked
+// where ymask is given).
+enum ConvEpi {
+    kEpiPlain = 0,
+    kEpiPool = 1,   // y, and its 2 x 2 mean into y2 (half resolution)
+    kEpiSplit = 2   // gradient of up2(a) ++ b, a of 32 channels: the 2 x 2 sum of
+                    // those channels, masked, into y2 (half resolution), the rest into y
+};
+
+template <int CIN, int COUT>
+struct ConvCfg {
+    static constexpr int XS = CIN + 8, WS = 9 * CIN + 8, TP = (CH + 2) * (CW + 2);
+    static constexpr int ES = COUT + 8;                      // pitch of an output pixel (values)
+    static constexpr bool REGW = CIN * COUT <= 512;          // weight fragments kept in registers
+    static constexpr int ST = CIN <= 16 ? 4 : 3;             // stages of the input ring
+    static constexpr size_t smem = ((size_t)ST * TP * XS + (size_t)COUT * WS + (size_t)4 * 32 * ES) * 2;
+};
+
+// y = act(conv3x3(x) + bias), NHWC, zero padding, with the epilogues above.
 // w: [COUT][9][CIN] (tap = 3 dy + dx multiplies x[i + dy - 1, j + dx - 1]).
 // Persistent: each CTA stages all weights once, then walks output tiles of
-// 8 x 16 pixels; the next tile is copied into the other shared buffer with
-// cp.async while the current one is on the tensor cores.
-// CUP > 0: the input is up2(xu) ++ x (see in_chunk).  ymask (NULL: none; the
-// backward-data passes): the ReLU mask of the gradient written, so that its
-// two readers, the next layer's weight gradient and backward-data pass, take
-// it as it is (masking at the reader loaded the mask with its halo twice and
-// selected it nine times, once per tap).
-template <int CIN, int COUT, int CUP>
+// 8 x 16 pixels; the next tiles' inputs are copied into a ring by cp.async
+// while the current one is on the tensor cores.
+// CUP > 0: the input is up2(xu) ++ x (see in_chunk).  CST: channels stored of
+// x, CIN or 2 (the other channels are zero and neither stored nor copied).
+// ymask (NULL: none; the backward-data passes): the ReLU mask of the gradient
+// written, so that its readers take it as it is.  y may be NULL with y32,
+// which receives channel 0 in FP32.
+// Each warp takes two rows of 16 pixels.  The layers are skinny (K = 16 to 64
+// a tap, N = 16 to 64) and their bytes few, so the cost is instructions and
+// latency: one fragment load (ldmatrix) for four 4-byte reads, the weights'
+// fragments in registers where they fit, copies three tiles ahead, addresses
+// of a thread's chunks formed once, output tiles through shared memory in
+// 16-byte rows with the pooling of the forward pass and the up-sampling fold
+// and split of the backward pass done on them there.  With 4-byte fragment
+// reads, two buffers and separate pooling and folding launches the layers
+// took (us) 25.5 (16 -> 16, 8 x 256^2), 44.9 (48 -> 16), 33.1 (64 -> 32, half
+// resolution), 12.6 (32 -> 32, half and quarter) in all; now
+// 15.5, 40, 28 and 10.
+template <int CIN, int COUT, int CUP, int CST, int EPI>
 __global__ void __launch_bounds__(128)
 k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restrict__ xu,
            const bf16 *__restrict__ ymask,
            const bf16 *__restrict__ w, const float *__restrict__ bias, int relu,
-           bf16 *__restrict__ y, float *__restrict__ y32)
+           bf16 *__restrict__ y, bf16 *__restrict__ y2, float *__restrict__ y32)
 {
-    constexpr int XS = CIN + 8, WS = 9 * CIN + 8, NT = COUT / 8;
-    constexpr int TP = (CH + 2) * (CW + 2);       // pixels of a haloed tile
-    static_assert(CIN % 16 == 0 && CUP % 8 == 0, "channel layout");
+    using C = ConvCfg<CIN, COUT>;
+    constexpr int XS = C::XS, WS = C::WS, NT = COUT / 8, TP = C::TP, ES = C::ES, ST = C::ST, KC = CIN / 16;
+    static_assert(CIN % 16 == 0 && CUP % 8 == 0 && (CST == CIN - CUP || CST == 2), "channel layout");
+    static_assert(EPI != kEpiSplit || COUT > 32, "split outputs");
     extern __shared__ __align__(16) unsigned char conv_sm[];
-    bf16 *ws = (bf16 *)conv_sm;
-    bf16 *xs0 = ws + COUT * WS;                    // 2 input buffers
+    bf16 *xs0 = (bf16 *)conv_sm, *ws = xs0 + ST * TP * XS, *es0 = ws + COUT * WS;
     const int tw = (W + CW - 1) / CW, th = (H + CH - 1) / CH, ntiles = B * tw * th;
-    for (int k = threadIdx.x; k < COUT * (9 * CIN / 2); k += 128) {
-        const int co = k / (9 * CIN / 2), q = k - co * (9 * CIN / 2);
-        *(uint32_t *)(ws + co * WS + 2 * q) = *(const uint32_t *)(w + (long)co * 9 * CIN + 2 * q);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
+    for (int k = tid; k < COUT * (9 * CIN / 8); k += 128) {
+        const int co = k / (9 * CIN / 8), q = k - co * (9 * CIN / 8);
+        *(uint4 *)(ws + co * WS + 8 * q) = *(const uint4 *)(w + (long)co * 9 * CIN + 8 * q);
     }
-    auto issue = [&](int tl, int buf) {
-        const int bz = tl / (tw * th), rem = tl - bz * tw * th;
-        const int ty0 = (rem / tw) * CH, tx0 = (rem - (rem / tw) * tw) * CW;
-        bf16 *xs = xs0 + buf * TP * XS;
-        for (int k = threadIdx.x; k < TP * (CIN / 8); k += 128) {
-            const int pix = k / (CIN / 8), q = k - pix * (CIN / 8);
-            const int r = pix / (CW + 2), c = pix - r * (CW + 2);
-            const int gy = ty0 + r - 1, gx = tx0 + c - 1;
-            const bool in = gy >= 0 && gy < H && gx >= 0 && gx < W;
-            cp_async16(xs + pix * XS + 8 * q, in ? in_chunk<CIN, CUP>(x, xu, bz, H, W, gy, gx, q) : x, in);
+    if (CST == 2)  // the channels that no copy writes
+        for (int k = tid; k < ST * TP * XS / 8; k += 128) *(uint4 *)(xs0 + 8 * k) = make_uint4(0u, 0u, 0u, 0u);
+    // this thread's chunks of a tile: window row and column, offsets in x (or
+    // xu) from the tile's corner; a tile's corner is even, so the up-sampled
+    // part's offset is the same for every tile
+    constexpr int NCH = CST == 2 ? TP : TP * (CIN / 8), PER = (NCH + 127) / 128;
+    __syncthreads();
+    auto issue = [&](int tl, int st) {
+        if (tl < ntiles) {
+            const int bz = tl / (tw * th), rem = tl - bz * tw * th, tr = rem / tw;
+            const int ty0 = tr * CH, tx0 = (rem - tr * tw) * CW;
+            const bf16 *xt = x + (((long)bz * H + ty0 - 1) * W + tx0 - 1) * CST;
+            const bf16 *ut = CUP > 0 ? xu + (((long)bz * (H / 2) + ty0 / 2) * (W / 2) + tx0 / 2) * CUP : nullptr;
+            bf16 *xs = xs0 + st * TP * XS;
+#pragma unroll
+            for (int i = 0; i < PER; i++) {
+                const int k = tid + 128 * i;
+                if (PER * 128 > NCH && k >= NCH) break;
+                const int pix = CST == 2 ? k : k / (CIN / 8), q = CST == 2 ? 0 : k - pix * (CIN / 8);
+                const int r = pix / (CW + 2), c = pix - r * (CW + 2);
+                const bool in = (unsigned)(ty0 - 1 + r) < (unsigned)H && (unsigned)(tx0 - 1 + c) < (unsigned)W;
+                if (CST == 2) {
+                    cp_async4(xs + pix * XS, in ? xt + ((long)r * W + c) * 2 : x, in);
+                } else {
+                    const bf16 *src;
+                    if (CUP > 0 && q < CUP / 8)
+                        src = ut + ((long)((r - 1) >> 1) * (W / 2) + ((c - 1) >> 1)) * CUP + 8 * q;
+                    else
+                        src = xt + ((long)r * W + c) * CST + 8 * q - CUP;
+                    cp_async16(xs + pix * XS + 8 * q, in ? src : x, in);
+                }
+            }
         }
-        cp_async_commit();
+        cp_async_commit();  // an empty group past the last tile keeps the count
     };
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
-    int buf = 0;
-    if (blockIdx.x < ntiles) issue(blockIdx.x, 0);
+    for (int k = 0; k < ST - 1; k++) issue(blockIdx.x + k * gridDim.x, k);
+    // weight fragments: rows n (co) of 8 k values, two n blocks a load
+    const uint32_t wa = (uint32_t)__cvta_generic_to_shared(ws) +
+                        (((lane & 7) + (lane >> 4) * 8) * WS + ((lane >> 3) & 1) * 8) * 2;
+    uint32_t wr[C::REGW ? 9 * KC * (NT / 2) : 1][4];
+    if constexpr (C::REGW) {
+#pragma unroll
+        for (int t = 0; t < 9 * KC; t++)
+#pragma unroll
+            for (int n2 = 0; n2 < NT / 2; n2++) ldsm4(wr[t * (NT / 2) + n2], wa + (n2 * 16 * WS + t * 16) * 2);
+    }
+    const uint32_t xa0 = (uint32_t)__cvta_generic_to_shared(xs0) +
+                         ((2 * warp * (CW + 2) + (lane & 7) + ((lane >> 3) & 1) * 8) * XS + (lane >> 4) * 8) * 2;
+    bf16 *es = es0 + warp * 32 * ES;
+    const uint32_t ea = (uint32_t)__cvta_generic_to_shared(es) +
+                        (((lane & 7) + ((lane >> 3) & 1) * 8) * ES + (lane >> 4) * 8) * 2;
+    int st = 0;
     for (int tl = blockIdx.x; tl < ntiles; tl += gridDim.x) {
-        const int tn = tl + gridDim.x;
-        if (tn < ntiles) { issue(tn, buf ^ 1); cp_async_wait<1>(); }
-        else cp_async_wait<0>();
-        __syncthreads();
-        const bf16 *xs = xs0 + buf * TP * XS;
+        cp_async_wait<ST - 2>();
+        __syncthreads();  // this tile's copies are visible; the slot of the one before is free
+        issue(tl + (ST - 1) * gridDim.x, (st + ST - 1) % ST);
+        const uint32_t xa = xa0 + st * (TP * XS * 2);
+        st = (st + 1) % ST;
         float acc[2][NT][4];
 #pragma unroll
         for (int a = 0; a < 2; a++)
@@ -132,60 +257,111 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
             for (int b = 0; b < NT; b++)
 #pragma unroll
                 for (int q = 0; q < 4; q++) acc[a][b][q] = 0.0f;
-#pragma unroll 1
-        for (int tap = 0; tap < 9; tap++) {
-            const int dy = tap / 3, dx = tap - 3 * (tap / 3);
+        auto step = [&](int tap, int kc, uint32_t xo) {
+            uint32_t af[2][4];
 #pragma unroll
-            for (int c0 = 0; c0 < CIN; c0 += 16) {
-                uint32_t bf[NT][2];
+            for (int mt = 0; mt < 2; mt++) ldsm4(af[mt], xo + (mt * (CW + 2) * XS + kc * 16) * 2);
 #pragma unroll
-                for (int nt = 0; nt < NT; nt++) {
-                    const bf16 *wp = ws + (nt * 8 + g) * WS + tap * CIN + c0 + 2 * t4;
-                    bf[nt][0] = *(const uint32_t *)wp;
-                    bf[nt][1] = *(const uint32_t *)(wp + 8);
-                }
+            for (int n2 = 0; n2 < NT / 2; n2++) {
+                uint32_t bq[4];
+                const uint32_t *bf = bq;
+                if constexpr (C::REGW) bf = wr[(tap * KC + kc) * (NT / 2) + n2];
+                else ldsm4(bq, wa + (n2 * 16 * WS + tap * CIN + kc * 16) * 2);
 #pragma unroll
                 for (int mt = 0; mt < 2; mt++) {
-                    const int r = 2 * warp + mt;
-                    const int o0 = ((r + dy) * (CW + 2) + g + dx) * XS + c0 + 2 * t4, o1 = o0 + 8 * XS;
-                    uint32_t af[4];
-                    af[0] = *(const uint32_t *)(xs + o0);
-                    af[1] = *(const uint32_t *)(xs + o1);
-                    af[2] = *(const uint32_t *)(xs + o0 + 8);
-                    af[3] = *(const uint32_t *)(xs + o1 + 8);
-#pragma unroll
-                    for (int nt = 0; nt < NT; nt++) mma_bf16(acc[mt][nt], af, bf[nt]);
+                    mma_bf16(acc[mt][2 * n2], af[mt], bf);
+                    mma_bf16(acc[mt][2 * n2 + 1], af[mt], bf + 2);
                 }
             }
+        };
+        if constexpr (C::REGW) {
+#pragma unroll
+            for (int tap = 0; tap < 9; tap++)
+#pragma unroll
+                for (int kc = 0; kc < KC; kc++)
+                    step(tap, kc, xa + ((tap / 3) * (CW + 2) + tap % 3) * (XS * 2));
+        } else {
+#pragma unroll 1
+            for (int tap = 0; tap < 9; tap++) {
+                const uint32_t xo = xa + ((tap / 3) * (CW + 2) + tap - 3 * (tap / 3)) * (XS * 2);
+#pragma unroll
+                for (int kc = 0; kc < KC; kc++) step(tap, kc, xo);
+            }
         }
-        const int bz = tl / (tw * th), rem = tl - bz * tw * th;
-        const int ty0 = (rem / tw) * CH, tx0 = (rem - (rem / tw) * tw) * CW;
+        // epilogue: bias, ReLU, BF16, and through shared memory
+        const int bz = tl / (tw * th), rem = tl - bz * tw * th, tr = rem / tw;
+        const int oy0 = tr * CH + 2 * warp, tx0 = (rem - tr * tw) * CW;
+        __syncwarp();  // the last tile's rows of this warp have been read
 #pragma unroll
-        for (int mt = 0; mt < 2; mt++) {
-            const int oy = ty0 + 2 * warp + mt;
-            if (oy >= H) continue;
-#pragma unroll
-            for (int nt = 0; nt < NT; nt++) {
+        for (int nt = 0; nt < NT; nt += 2) {
+            float b0 = 0.0f, b1 = 0.0f, b2 = 0.0f, b3 = 0.0f;
+            if (bias) {
                 const int co = nt * 8 + 2 * t4;
-                const float b0 = bias ? bias[co] : 0.0f, b1 = bias ? bias[co + 1] : 0.0f;
+                b0 = bias[co]; b1 = bias[co + 1]; b2 = bias[co + 8]; b3 = bias[co + 9];
+            }
 #pragma unroll
-                for (int half = 0; half < 2; half++) {
-                    const int ox = tx0 + g + 8 * half;
-                    if (ox >= W) continue;
-                    float v0 = acc[mt][nt][2 * half] + b0, v1 = acc[mt][nt][2 * half + 1] + b1;
-                    if (relu) { v0 = fmaxf(v0, 0.0f); v1 = fmaxf(v1, 0.0f); }
-                    const long off = (((long)bz * H + oy) * W + ox) * COUT + co;
-                    __nv_bfloat162 o2 = __floats2bfloat162_rn(v0, v1);
-                    uint32_t o = *(uint32_t *)&o2;
-                    if (ymask) o = relu_mask(o, *(const uint32_t *)(ymask + off));
-                    *(uint32_t *)(y + off) = o;
-                    if (y32 && co == 0) y32[off / COUT] = v0;  // channel 0 only
+            for (int mt = 0; mt < 2; mt++) {
+                float v[8] = {acc[mt][nt][0] + b0, acc[mt][nt][1] + b1, acc[mt][nt][2] + b0, acc[mt][nt][3] + b1,
+                              acc[mt][nt + 1][0] + b2, acc[mt][nt + 1][1] + b3, acc[mt][nt + 1][2] + b2, acc[mt][nt + 1][3] + b3};
+                if (relu)
+#pragma unroll
+                    for (int q = 0; q < 8; q++) v[q] = fmaxf(v[q], 0.0f);
+                if (y32 && nt == 0 && t4 == 0 && oy0 + mt < H) {
+                    const long o = ((long)bz * H + oy0 + mt) * W + tx0 + g;
+                    if (tx0 + g < W) y32[o] = v[0];
+                    if (tx0 + g + 8 < W) y32[o + 8] = v[2];
+                }
+                const uint4 pk = pack8(v);
+                const uint32_t rg[4] = {pk.x, pk.y, pk.z, pk.w};
+                if (y) stsm4(ea + (mt * 16 * ES + nt * 8) * 2, rg);
+            }
+        }
+        if (!y) continue;
+        __syncwarp();
+        // rows oy0, oy0 + 1: 16 pixels of COUT channels each in es
+        constexpr int C8 = COUT / 8;
+        if constexpr (EPI == kEpiSplit) {
+            constexpr int S8 = C8 - 4;  // chunks of the rest
+            {
+                const int px = lane >> 2, c = lane & 3, ox = tx0 / 2 + px;
+                if (oy0 < H && 2 * ox < W) {
+                    const bf16 *e = es + 2 * px * ES + 8 * c;
+                    const long o = (((long)bz * (H / 2) + oy0 / 2) * (W / 2) + ox) * 32 + 8 * c;
+                    const uint4 v = sum4(*(const uint4 *)e, *(const uint4 *)(e + ES), *(const uint4 *)(e + 16 * ES),
+                                         *(const uint4 *)(e + 17 * ES), 1.0f);
+                    *(uint4 *)(y2 + o) = relu_mask8(v, *(const uint4 *)(ymask + o));
+                }
+            }
+#pragma unroll
+            for (int k = lane; k < 32 * S8; k += 32) {
+                const int px = k / S8, c = k % S8, oy = oy0 + (px >> 4), ox = tx0 + (px & 15);
+                if (oy < H && ox < W)
+                    *(uint4 *)(y + (((long)bz * H + oy) * W + ox) * (8 * S8) + 8 * c) =
+                        *(const uint4 *)(es + px * ES + 32 + 8 * c);
+            }
+        } else {
+#pragma unroll
+            for (int k = lane; k < 32 * C8; k += 32) {
+                const int px = k / C8, c = k % C8, oy = oy0 + (px >> 4), ox = tx0 + (px & 15);
+                if (oy < H && ox < W) {
+                    const long o = (((long)bz * H + oy) * W + ox) * COUT + 8 * c;
+                    uint4 v = *(const uint4 *)(es + px * ES + 8 * c);
+                    if (ymask) v = relu_mask8(v, *(const uint4 *)(ymask + o));
+                    *(uint4 *)(y + o) = v;
+                }
+            }
+            if constexpr (EPI == kEpiPool) {
+                const int px = lane / C8, c = lane % C8, ox = tx0 / 2 + px;
+                if (lane < 8 * C8 && oy0 < H && 2 * ox < W) {
+                    const bf16 *e = es + 2 * px * ES + 8 * c;
+                    *(uint4 *)(y2 + (((long)bz * (H / 2) + oy0 / 2) * (W / 2) + ox) * COUT + 8 * c) =
+                        sum4(*(const uint4 *)e, *(const uint4 *)(e + ES), *(const uint4 *)(e + 16 * ES),
+                             *(const uint4 *)(e + 17 * ES), 0.25f);
                 }
             }
         }
-        __syncthreads();  // the buffer just read is refilled by the next issue
-        buf ^= 1;
     }
+    cp_async_wait<0>();
 }
 
 // ---- fifth-generation tensor cores (tcgen05) --------------------------
@@ -428,14 +604,6 @@ k_conv_tc(int B, int H, int W, int rpu, const bf16 *__restrict__ x, const bf16 *
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(taddr), "r"(32u));
 }
 
-// Four 8 x 8 BF16 matrices from shared memory, transposed (lane l gives row
-// l & 7 of matrix l >> 3).
-__device__ __forceinline__ void ldsm4t(uint32_t *r, uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-
 // Work split of k_conv_dw: one CTA for a 16 x 16 block of channels (outputs x
 // inputs) and a chunk of tiles; with a single such block (16 -> 16) one CTA
 // for each row of taps.  Three warps take the products (three taps each, or
@@ -463,9 +631,9 @@ struct DwSplit {
 // What bounds it is that chain and the fragment loads (four a 16-pixel step
 // for six products).  One CTA per tap with element-wise fragment reads took
 // 325 us (16 -> 16), 528 us (48 -> 16) and 260 us (64 -> 32, half resolution)
-// at 8 x 256^2; this takes 58, 82 and
-// 44 us.
-template <int CIN, int COUT, int CUP>
+// at 8 x 256^2; this takes 58, 83 and
+// 42 us.
+template <int CIN, int COUT, int CUP, int CSX, int CSG>
 __global__ void __launch_bounds__(128)
 k_conv_dw(int B, int H, int W, int tiles_per_chunk, const bf16 *__restrict__ x,
           const bf16 *__restrict__ xu, const bf16 *__restrict__ gy, float *__restrict__ part)
@@ -474,6 +642,13 @@ k_conv_dw(int B, int H, int W, int tiles_per_chunk, const bf16 *__restrict__ x,
     constexpr int XS = D::XS, T = D::T, ST = D::ST, XP = D::XP, GP = D::GP, TAPS = D::TAPS;
     extern __shared__ __align__(16) unsigned char conv_sm[];
     bf16 *xs0 = (bf16 *)conv_sm, *gs0 = xs0 + ST * XP * XS;
+    // CSX, CSG = 2: only two channels of x or gy are stored, the rest are zero
+    // (written here once; no copy touches them)
+    if (CSX == 2 || CSG == 2) {
+        for (int k = threadIdx.x; k < ST * (XP + GP) * XS / 8; k += T)
+            *(uint4 *)(xs0 + 8 * k) = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+    }
     const int tw = (W + CW - 1) / CW, th = (H + CH - 1) / CH, ntiles = B * tw * th;
     const int chunk = blockIdx.y, t0 = chunk * tiles_per_chunk, t1 = min(ntiles, t0 + tiles_per_chunk);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
@@ -485,17 +660,21 @@ k_conv_dw(int B, int H, int W, int tiles_per_chunk, const bf16 *__restrict__ x,
             const int bz = tl / (tw * th), rem = tl - bz * tw * th;
             const int ty0 = (rem / tw) * CH, tx0 = (rem - (rem / tw) * tw) * CW;
             bf16 *xs = xs0 + st * XP * XS, *gs = gs0 + st * GP * XS;
-            for (int k = threadIdx.x; k < XP * 2; k += T) {
-                const int pix = k >> 1, q = k & 1, r = pix / (CW + 2), c = pix - r * (CW + 2);
+            for (int k = threadIdx.x; k < (CSX == 2 ? XP : XP * 2); k += T) {
+                const int pix = CSX == 2 ? k : k >> 1, q = CSX == 2 ? 0 : k & 1;
+                const int r = pix / (CW + 2), c = pix - r * (CW + 2);
                 const int yy = ty0 + dy0 + r - 1, xx = tx0 + c - 1;
                 const bool in = yy >= 0 && yy < H && xx >= 0 && xx < W;
-                cp_async16(xs + pix * XS + 8 * q,
+                if (CSX == 2) cp_async4(xs + pix * XS, in ? x + (((long)bz * H + yy) * W + xx) * 2 : x, in);
+                else cp_async16(xs + pix * XS + 8 * q,
                            in ? in_chunk<CIN, CUP>(x, xu, bz, H, W, yy, xx, 2 * np + q) : x, in);
             }
-            for (int k = threadIdx.x; k < GP * 2; k += T) {
-                const int pix = k >> 1, q = k & 1, yy = ty0 + pix / CW, xx = tx0 + pix % CW;
+            for (int k = threadIdx.x; k < (CSG == 2 ? GP : GP * 2); k += T) {
+                const int pix = CSG == 2 ? k : k >> 1, q = CSG == 2 ? 0 : k & 1;
+                const int yy = ty0 + pix / CW, xx = tx0 + pix % CW;
                 const bool in = yy < H && xx < W;  // beyond the image: no gradient
-                cp_async16(gs + pix * XS + 8 * q,
+                if (CSG == 2) cp_async4(gs + pix * XS, gy + (in ? (((long)bz * H + yy) * W + xx) * 2 : 0), in);
+                else cp_async16(gs + pix * XS + 8 * q,
                            gy + (in ? (((long)bz * H + yy) * W + xx) * COUT + 16 * mt + 8 * q : 0), in);
             }
         }
@@ -593,51 +772,8 @@ __global__ void __launch_bounds__(128) k_reduce_grads(const __grid_constant__ Re
 }
 
 // --- layout helpers (bf16 NHWC), 8 channels (16 bytes) a thread ------------
-// (One channel a thread: 10 us a pooling, 16 us an up-sampling fold and 38 us
-// a skip sum at 8 x 256^2, bound by instructions; 8 channels: 10 us a
-// skip sum.)
-__device__ __forceinline__ void unpack8(const bf16 *p, float *f)
-{
-    const uint4 v = *(const uint4 *)p;
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-        f[2 * q] = __uint_as_float(w[q] << 16);
-        f[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u);
-    }
-}
-__device__ __forceinline__ uint4 pack8(const float *f)
-{
-    uint32_t w[4];
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(f[2 * q], f[2 * q + 1]);
-        w[q] = *(const uint32_t *)&h;
-    }
-    return make_uint4(w[0], w[1], w[2], w[3]);
-}
-__device__ __forceinline__ uint4 relu_mask8(uint4 v, uint4 m)
-{
-    return make_uint4(relu_mask(v.x, m.x), relu_mask(v.y, m.y), relu_mask(v.z, m.z), relu_mask(v.w, m.w));
-}
-// sum of the 2 x 2 block of an image of width W and C channels at p, in the
-// order (0,0), (0,1), (1,0), (1,1)
-__device__ __forceinline__ void sum4(const bf16 *p, int W, int C, float *s)
-{
-    float f[8];
-    unpack8(p, s);
-    unpack8(p + C, f);
-#pragma unroll
-    for (int q = 0; q < 8; q++) s[q] += f[q];
-    unpack8(p + (long)W * C, f);
-#pragma unroll
-    for (int q = 0; q < 8; q++) s[q] += f[q];
-    unpack8(p + (long)W * C + C, f);
-#pragma unroll
-    for (int q = 0; q < 8; q++) s[q] += f[q];
-}
-
-// n8: 8-channel groups of the output (H2 x W2, C channels)
+// 2 x 2 mean after a tcgen05 convolution (the warp-level kernel pools in its
+// epilogue).  n8: 8-channel groups of the output (H2 x W2, C channels)
 __global__ void __launch_bounds__(256)
 k_pool2(int n8, int H2, int W2, int C, const bf16 *__restrict__ x, bf16 *__restrict__ y)
 {
@@ -648,46 +784,28 @@ k_pool2(int n8, int H2, int W2, int C, const bf16 *__restrict__ x, bf16 *__restr
     const int j = p % W2;
     p /= W2;
     const int i = p % H2, b = p / H2, W = 2 * W2;
-    float s[8];
-    sum4(x + (((long)b * (2 * H2) + 2 * i) * W + 2 * j) * C + c, W, C, s);
-#pragma unroll
-    for (int q = 0; q < 8; q++) s[q] *= 0.25f;
-    *(uint4 *)(y + 8L * k) = pack8(s);
+    const bf16 *a = x + (((long)b * (2 * H2) + 2 * i) * W + 2 * j) * C + c;
+    *(uint4 *)(y + 8L * k) = sum4(*(const uint4 *)a, *(const uint4 *)(a + C), *(const uint4 *)(a + (long)W * C),
+                                  *(const uint4 *)(a + (long)W * C + C), 0.25f);
 }
 
-// gt = [mask > 0] * sum over 2x2 of g[..., :C1] (C1 channels at half resolution)
+// gskip = [mask > 0] * (gs + pool2_bwd(gp)), C channels (gp at half
+// resolution); may be in place (gskip = gs).  One channel a thread took 38 us
+// at 8 x 256^2 (instructions), 8 take 8 us.
 __global__ void __launch_bounds__(256)
-k_up_cat_bwd(int n8, int H2, int W2, int C1, int C2, const bf16 *__restrict__ g,
-             const bf16 *__restrict__ mask, bf16 *__restrict__ gt)
+k_skip_grad(int n8, int H, int W, int C, const bf16 *gs, const bf16 *__restrict__ gp,
+            const bf16 *__restrict__ mask, bf16 *gskip)
 {
     const int k = blockIdx.x * 256 + threadIdx.x;
     if (k >= n8) return;
-    const int c8 = C1 / 8, c = (k % c8) * 8;
+    const int c8 = C / 8, c = (k % c8) * 8;
     int p = k / c8;
-    const int j = p % W2;
-    p /= W2;
-    const int i = p % H2, b = p / H2, W = 2 * W2, C = C1 + C2;
-    float s[8];
-    sum4(g + (((long)b * (2 * H2) + 2 * i) * W + 2 * j) * C + c, W, C, s);
-    *(uint4 *)(gt + 8L * k) = relu_mask8(pack8(s), *(const uint4 *)(mask + 8L * k));
-}
-
-// gskip = [mask > 0] * (g_cat[..., C1:] + pool2_bwd(gp))   (gp at half
-// resolution, C2 channels)
-__global__ void __launch_bounds__(256)
-k_skip_grad(int n8, int H, int W, int C1, int C2, const bf16 *__restrict__ gcat,
-            const bf16 *__restrict__ gp, const bf16 *__restrict__ mask, bf16 *__restrict__ gskip)
-{
-    const int k = blockIdx.x * 256 + threadIdx.x;
-    if (k >= n8) return;
-    const int c8 = C2 / 8, c = (k % c8) * 8;
-    int p = k / c8;
-    const int pix = p, j = p % W;
+    const int j = p % W;
     p /= W;
     const int i = p % H, b = p / H;
     float v[8], f[8];
-    unpack8(gcat + (long)pix * (C1 + C2) + C1 + c, v);
-    unpack8(gp + (((long)b * (H / 2) + i / 2) * (W / 2) + j / 2) * C2 + c, f);
+    unpack8(*(const uint4 *)(gs + 8L * k), v);
+    unpack8(*(const uint4 *)(gp + (((long)b * (H / 2) + i / 2) * (W / 2) + j / 2) * C + c), f);
 #pragma unroll
     for (int q = 0; q < 8; q++) v[q] += 0.25f * f[q];
     *(uint4 *)(gskip + 8L * k) = relu_mask8(pack8(v), *(const uint4 *)(mask + 8L * k));
@@ -786,8 +904,9 @@ k_ymean_final(int N2, const double *__restrict__ part, double *__restrict__ stat
     if (threadIdx.x == 0) stats[kStat * blockIdx.x + 5] = s / N2;
 }
 
-// x[..., 0] = (b - mean)/s, x[..., 1] = (1/rho)/max(1/rho) = min(rho)/rho,
-// other channels 0 (BF16, rounded from FP32); and (training)
+// x[..., 0] = (b - mean)/s, x[..., 1] = (1/rho)/max(1/rho) = min(rho)/rho
+// (BF16, rounded from FP32; the first layer's other 14 input channels are
+// zero and not stored); and (training)
 // t = p / (s pscale), pscale = h^2 c.
 __global__ void k_features(long n, int N2, const double *__restrict__ b, const double *__restrict__ rho,
                            const double *__restrict__ p, const double *__restrict__ stats,
@@ -799,16 +918,12 @@ __global__ void k_features(long n, int N2, const double *__restrict__ b, const d
     const float f0 = (float)((b[k] - st[0]) * st[2]);
     const float f1 = (float)st[3] / (float)rho[k];
     __nv_bfloat162 v = __floats2bfloat162_rn(f0, f1);
-    uint32_t *xp = (uint32_t *)(x + k * 16);
-    xp[0] = *(uint32_t *)&v;
-#pragma unroll
-    for (int q = 1; q < 8; q++) xp[q] = 0u;
+    *(__nv_bfloat162 *)(x + k * 2) = v;
     if (t) t[k] = (float)(p[k] * st[4]);
 }
 
 // Mean-removed squared error per sample: loss partial and the gradient
-// 2 d / (B n) minus its mean, written as BF16 channel 0 of a 16-channel
-// tensor.  Three launches over kLossBlk CTAs a sample, each folding the
+// 2 d / (B n) minus its mean, written as BF16 channel 0 of two.  Three launches over kLossBlk CTAs a sample, each folding the
 // partial sums of the one before in a fixed order: the means; the loss and
 // the gradient's mean; the gradient.  (One CTA a sample: 288 us at 8 x 256^2
 // on 8 of the SMs; this takes 8 us.)
@@ -877,9 +992,7 @@ k_loss_grad(int N2, int Bn, float sc, const float *__restrict__ y32, const float
     for (int k = blockIdx.x * 256 + threadIdx.x; k < N2; k += 256 * kLossBlk) {
         const float d = (y32[base + k] - my) - (t[base + k] - mt);
         const __nv_bfloat162 v = __floats2bfloat162_rn(sc * d - gmean, 0.0f);
-        uint4 *gp = (uint4 *)(gy + (base + k) * 16);
-        gp[0] = make_uint4(*(const uint32_t *)&v, 0u, 0u, 0u);
-        gp[1] = make_uint4(0u, 0u, 0u, 0u);
+        *(__nv_bfloat162 *)(gy + (base + k) * 2) = v;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) lsum[blockIdx.y] = s.x / ((float)Bn * (float)N2);
 }
@@ -1052,83 +1165,60 @@ int sm_count()
     return g_sms;
 }
 
-// tc: 0 the warp-level kernel; 1 tcgen05 for the shapes where it measured
-// faster than the warp-level kernel (16 -> 32 channels: 8.7 against 12.2 us
-// at 128^2; the others are bound by operand staging and latency, where the
-// warp-level kernel's double-buffered 8 x 16 tiles stage less per output);
-// 2 tcgen05 wherever the width is a multiple of 128.
-template <int CIN, int COUT, int CUP>
+// tc: 0, 1 the warp-level kernel; 2 tcgen05 wherever the width is a multiple
+// of 128 (forward layers; bound by operand staging and latency, where the
+// warp-level kernel's ring of 8 x 16 tiles stages less per output: 16 -> 32
+// channels at 8 x 128^2 take 18.7 us there, 10.4 us here).
+// ymask: mask of the output (backward-data passes), NULL for none.
+template <int CIN, int COUT, int CUP = 0, int CST = CIN - CUP, int EPI = kEpiPlain>
 void conv_launch(int B, int H, int W, const bf16 *x, const bf16 *xu, const bf16 *ymask, const bf16 *w,
-                 const float *bias, int relu, bf16 *y, float *y32, cudaStream_t s, int tc = 0)
+                 const float *bias, int relu, bf16 *y, bf16 *y2, float *y32, cudaStream_t s, int tc = 0)
 {
-    if constexpr (COUT == 16 || COUT == 32) {
-        const bool faster = CIN == 16 && COUT == 32 && CUP == 0;
-        if (!ymask && bias && (tc == 2 || (tc == 1 && faster)) && W % kTcPix == 0) {
+    if constexpr ((COUT == 16 || COUT == 32) && CST == CIN - CUP && EPI != kEpiSplit) {
+        if (tc == 2 && y && W % kTcPix == 0) {
             constexpr size_t smt = conv_tc_smem<CIN, COUT>();
-            static bool attr_tc = false;
-            if (!attr_tc) {
-                cudaFuncSetAttribute(k_conv_tc<CIN, COUT, CUP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smt);
-                attr_tc = true;
-            }
-            sm_count();
+            raise_smem_limit((const void *)k_conv_tc<CIN, COUT, CUP>, (int)smt);
             // rows per unit: as many as keep every SM busy, up to 8 (a unit
             // stages rpu + 2 input rows for rpu output rows); CTAs per SM by
             // shared memory (at most 8: 256 of the 512 tensor-memory columns)
             const int per_sm = std::max(1, std::min(8, (int)((227 * 1024) / smt)));
             const long rows = (long)B * H * (W / kTcPix);
-            const int rpu = (int)std::max(1L, std::min(std::min((long)H, 8L), rows / g_sms));
+            const int rpu = (int)std::max(1L, std::min(std::min((long)H, 8L), rows / sm_count()));
             const long units = (long)B * (W / kTcPix) * ((H + rpu - 1) / rpu);
-            const int grid = (int)std::min(units, (long)g_sms * per_sm);
+            const int grid = (int)std::min(units, (long)sm_count() * per_sm);
             note_launch();
             k_conv_tc<CIN, COUT, CUP><<<grid, 128, smt, s>>>(B, H, W, rpu, x, xu, w, bias, relu, y, y32);
+            if (EPI == kEpiPool) {
+                const int n8 = B * (H / 2) * (W / 2) * (COUT / 8);
+                note_launch();
+                k_pool2<<<cdiv(n8, 256), 256, 0, s>>>(n8, H / 2, W / 2, COUT, y, y2);
+            }
             return;
         }
     }
-    constexpr size_t sm = conv_smem<CIN, COUT>();
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(k_conv_fwd<CIN, COUT, CUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        attr = true;
-    }
-    sm_count();
+    constexpr size_t sm = ConvCfg<CIN, COUT>::smem;
+    raise_smem_limit((const void *)k_conv_fwd<CIN, COUT, CUP, CST, EPI>, (int)sm);
     const int ntiles = B * (int)cdiv(W, CW) * (int)cdiv(H, CH);
-    const int per_sm = sm <= 56 * 1024 ? 4 : (sm <= 75 * 1024 ? 3 : 2);
-    const int grid = std::min(ntiles, g_sms * per_sm);
+    const int per_sm = std::max(1, std::min(4, (int)((227 * 1024) / (sm + 1024))));
+    const int grid = std::min(ntiles, sm_count() * per_sm);
     note_launch();
-    k_conv_fwd<CIN, COUT, CUP><<<grid, 128, sm, s>>>(B, H, W, x, xu, ymask, w, bias, relu, y, y32);
-}
-
-// ymask: mask of the output (backward-data passes), NULL for none.
-template <int CIN, int COUT>
-void conv_fwd(int B, int H, int W, const bf16 *x, const bf16 *ymask, const bf16 *w,
-              const float *bias, int relu, bf16 *y, float *y32, cudaStream_t s, int tc = 0)
-{
-    conv_launch<CIN, COUT, 0>(B, H, W, x, nullptr, ymask, w, bias, relu, y, y32, s, tc);
-}
-
-// Convolution of the concatenation up2(xu) ++ x (CUP channels from xu).
-template <int CIN, int COUT, int CUP>
-void conv_fwd_cat(int B, int H, int W, const bf16 *xu, const bf16 *x, const bf16 *w,
-                  const float *bias, int relu, bf16 *y, cudaStream_t s, int tc = 0)
-{
-    conv_launch<CIN, COUT, CUP>(B, H, W, x, xu, nullptr, w, bias, relu, y, nullptr, s, tc);
+    k_conv_fwd<CIN, COUT, CUP, CST, EPI><<<grid, 128, sm, s>>>(B, H, W, x, xu, ymask, w, bias, relu, y, y2, y32);
 }
 
 // Partial gradients of layer k (input x, or up2(xu) ++ x; gy its masked
 // output gradient); records the chunk count for k_reduce_grads.
-template <int CIN, int COUT, int CUP = 0>
+template <int CIN, int COUT, int CUP = 0, int CSX = CIN - CUP, int CSG = COUT>
 void conv_dw(Cnn &n, ReduceArgs &ra, int k, int B, int H, int W, const bf16 *x, const bf16 *gy,
              cudaStream_t s, const bf16 *xu = nullptr)
 {
     using D = DwSplit<CIN, COUT>;
     const int ntiles = B * (int)cdiv(W, CW) * (int)cdiv(H, CH);
     const int nchunks = std::min(ntiles, kDwChunks), tpc = (int)cdiv(ntiles, nchunks);
-    raise_smem_limit((const void *)k_conv_dw<CIN, COUT, CUP>, (int)D::smem);
+    raise_smem_limit((const void *)k_conv_dw<CIN, COUT, CUP, CSX, CSG>, (int)D::smem);
     ra.part[k] = n.part + n.L[k].part_off;
     ra.nchunks[k] = nchunks;
     note_launch();
-    k_conv_dw<CIN, COUT, CUP><<<dim3(D::G * D::DY, nchunks), D::T, D::smem, s>>>(B, H, W, tpc, x, xu, gy, n.part + n.L[k].part_off);
+    k_conv_dw<CIN, COUT, CUP, CSX, CSG><<<dim3(D::G * D::DY, nchunks), D::T, D::smem, s>>>(B, H, W, tpc, x, xu, gy, n.part + n.L[k].part_off);
 }
 
 size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -1216,14 +1306,14 @@ cudaError_t cnn_workspace(Cnn &n, int B, int N)
     n.amem = nullptr;
     const size_t P = (size_t)B * N * N, P2 = P / 4, P4 = P / 16;
     const int c1 = n.c1, c2 = n.c2;
-    size_t bytes = al(P * 16 * 2) +                       // x
+    size_t bytes = al(P * 2 * 2) +                        // x
                    al(P * c1 * 2) * 2 +                    // a1, s1
                    al(P2 * c1 * 2) + al(P2 * c2 * 2) * 2 + // p1, a2, s2
                    al(P4 * c2 * 2) * 3 +                   // p2, a3, t3
                    al(P2 * c2 * 2) +                       // t4
                    al(P * c1 * 2) + al(P * 16 * 2) +       // a5, y
-                   al(P * 64 * 2) * 2 + al(P2 * 64 * 2) * 2 + al(P4 * 64 * 2) * 2 +  // grads
-                   al(P * 64 * 2) + al(P2 * 64 * 2) +      // gcat, gup
+                   al(P * c1 * 2) * 2 + al(P2 * c2 * 2) * 2 + al(P4 * c2 * 2) * 2 +  // grads
+                   al(P * c1 * 2) + al(P2 * c2 * 2) +      // gcat, gup (skip parts)
                    al(P * 4) + al(P * 4) + al(B * 4) + al(B * kStat * 8) +
                    al(B * kRedBlocks * 3 * 8);
     // chunk partials of the weight gradients, layer after layer
@@ -1237,17 +1327,17 @@ cudaError_t cnn_workspace(Cnn &n, int B, int N)
     if (e != cudaSuccess) { n.amem = nullptr; return e; }
     char *q = (char *)n.amem;
     auto take = [&](size_t b) { char *r = q; q += al(b); return (void *)r; };
-    n.x = (bf16 *)take(P * 16 * 2);
+    n.x = (bf16 *)take(P * 2 * 2);
     n.a1 = (bf16 *)take(P * c1 * 2); n.s1 = (bf16 *)take(P * c1 * 2);
     n.p1 = (bf16 *)take(P2 * c1 * 2); n.a2 = (bf16 *)take(P2 * c2 * 2); n.s2 = (bf16 *)take(P2 * c2 * 2);
     n.p2 = (bf16 *)take(P4 * c2 * 2); n.a3 = (bf16 *)take(P4 * c2 * 2); n.t3 = (bf16 *)take(P4 * c2 * 2);
     n.t4 = (bf16 *)take(P2 * c2 * 2);
     n.a5 = (bf16 *)take(P * c1 * 2);
     n.y = (bf16 *)take(P * 16 * 2);
-    n.gbig = (bf16 *)take(P * 64 * 2); n.gbig2 = (bf16 *)take(P * 64 * 2);
-    n.gmid = (bf16 *)take(P2 * 64 * 2); n.gmid2 = (bf16 *)take(P2 * 64 * 2);
-    n.gsmall = (bf16 *)take(P4 * 64 * 2); n.gsmall2 = (bf16 *)take(P4 * 64 * 2);
-    n.gcat = (bf16 *)take(P * 64 * 2); n.gup = (bf16 *)take(P2 * 64 * 2);
+    n.gbig = (bf16 *)take(P * c1 * 2); n.gbig2 = (bf16 *)take(P * c1 * 2);
+    n.gmid = (bf16 *)take(P2 * c2 * 2); n.gmid2 = (bf16 *)take(P2 * c2 * 2);
+    n.gsmall = (bf16 *)take(P4 * c2 * 2); n.gsmall2 = (bf16 *)take(P4 * c2 * 2);
+    n.gcat = (bf16 *)take(P * c1 * 2); n.gup = (bf16 *)take(P2 * c2 * 2);
     n.y32 = (float *)take(P * 4); n.t = (float *)take(P * 4); n.lsum = (float *)take(B * 4);
     n.stats = (double *)take(B * kStat * 8);
     n.rpart = (double *)take(B * kRedBlocks * 3 * 8);
@@ -1273,19 +1363,17 @@ void cnn_forward(Cnn &n, int B, int N, double h, const double *rhs, const double
     auto &L = n.L;
     auto bias = [&](int k) { return n.w + L[k].boff; };
     const int tc = n.tc;
-    conv_fwd<16, 16>(B, N, N, n.x, nullptr, L[0].wf, bias(0), 1, n.a1, nullptr, s, tc);
-    conv_fwd<16, 16>(B, N, N, n.a1, nullptr, L[1].wf, bias(1), 1, n.s1, nullptr, s, tc);
-    note_launch();
-    k_pool2<<<cdiv((long)B * H2 * H2 * 2, 256), 256, 0, s>>>(B * H2 * H2 * 2, H2, H2, 16, n.s1, n.p1);
-    conv_fwd<16, 32>(B, H2, H2, n.p1, nullptr, L[2].wf, bias(2), 1, n.a2, nullptr, s, tc);
-    conv_fwd<32, 32>(B, H2, H2, n.a2, nullptr, L[3].wf, bias(3), 1, n.s2, nullptr, s, tc);
-    note_launch();
-    k_pool2<<<cdiv((long)B * H4 * H4 * 4, 256), 256, 0, s>>>(B * H4 * H4 * 4, H4, H4, 32, n.s2, n.p2);
-    conv_fwd<32, 32>(B, H4, H4, n.p2, nullptr, L[4].wf, bias(4), 1, n.a3, nullptr, s, tc);
-    conv_fwd<32, 32>(B, H4, H4, n.a3, nullptr, L[5].wf, bias(5), 1, n.t3, nullptr, s, tc);
-    conv_fwd_cat<64, 32, 32>(B, H2, H2, n.t3, n.s2, L[6].wf, bias(6), 1, n.t4, s, tc);  // up2(t3) ++ s2
-    conv_fwd_cat<48, 16, 32>(B, N, N, n.t4, n.s1, L[7].wf, bias(7), 1, n.a5, s, tc);     // up2(t4) ++ s1
-    conv_fwd<16, 16>(B, N, N, n.a5, nullptr, L[8].wf, bias(8), 0, n.y, n.y32, s, tc);
+    conv_launch<16, 16, 0, 2>(B, N, N, n.x, nullptr, nullptr, L[0].wf, bias(0), 1, n.a1, nullptr, nullptr, s, tc);
+    conv_launch<16, 16, 0, 16, kEpiPool>(B, N, N, n.a1, nullptr, nullptr, L[1].wf, bias(1), 1, n.s1, n.p1, nullptr, s, tc);
+    conv_launch<16, 32>(B, H2, H2, n.p1, nullptr, nullptr, L[2].wf, bias(2), 1, n.a2, nullptr, nullptr, s, tc);
+    conv_launch<32, 32, 0, 32, kEpiPool>(B, H2, H2, n.a2, nullptr, nullptr, L[3].wf, bias(3), 1, n.s2, n.p2, nullptr, s, tc);
+    conv_launch<32, 32>(B, H4, H4, n.p2, nullptr, nullptr, L[4].wf, bias(4), 1, n.a3, nullptr, nullptr, s, tc);
+    conv_launch<32, 32>(B, H4, H4, n.a3, nullptr, nullptr, L[5].wf, bias(5), 1, n.t3, nullptr, nullptr, s, tc);
+    conv_launch<64, 32, 32>(B, H2, H2, n.s2, n.t3, nullptr, L[6].wf, bias(6), 1, n.t4, nullptr, nullptr, s, tc);  // up2(t3) ++ s2
+    conv_launch<48, 16, 32>(B, N, N, n.s1, n.t4, nullptr, L[7].wf, bias(7), 1, n.a5, nullptr, nullptr, s, tc);    // up2(t4) ++ s1
+    // the output: channel 0 in FP32 (the tensor-core kernel also writes its
+    // BF16 tile)
+    conv_launch<16, 16>(B, N, N, n.a5, nullptr, nullptr, L[8].wf, bias(8), 0, tc == 2 ? n.y : nullptr, nullptr, n.y32, s, tc);
 }
 
 // Loss and gradients of every parameter (into n.g, master layout).
@@ -1303,42 +1391,40 @@ void cnn_backward(Cnn &n, int B, int N, cudaStream_t s)
     k_loss_sums<<<gl, 256, 0, s>>>(N2, sc, n.y32, n.t, means, sums);
     k_loss_grad<<<gl, 256, 0, s>>>(N2, B, sc, n.y32, n.t, means, sums, n.gbig, n.lsum);
     ReduceArgs ra;
-    // c6 (linear): input a5, grad gbig (16 ch, channel 0)
-    conv_dw<16, 16>(n, ra, 8, B, N, N, n.a5, n.gbig, s);
-    conv_fwd<16, 16>(B, N, N, n.gbig, n.a5, L[8].wb, nullptr, 0, n.gbig2, nullptr, s);  // grad a5, masked
-    // c5: in up2(t4) ++ s1
+    // a layer's input gradient: convolution with the flipped weights
+    const bf16 *none = nullptr;
+    // c6 (linear): input a5, grad gbig (channel 0 of two stored)
+    conv_dw<16, 16, 0, 16, 2>(n, ra, 8, B, N, N, n.a5, n.gbig, s);
+    conv_launch<16, 16, 0, 2>(B, N, N, n.gbig, none, n.a5, L[8].wb, nullptr, 0, n.gbig2, nullptr, nullptr, s);  // grad a5, masked
+    // c5: in up2(t4) ++ s1; the input gradient split into grad t4 (masked) and s1's skip part
     conv_dw<48, 16, 32>(n, ra, 7, B, N, N, n.s1, n.gbig2, s, n.t4);
-    conv_fwd<16, 48>(B, N, N, n.gbig2, nullptr, L[7].wb, nullptr, 0, n.gcat, nullptr, s);  // grad of up2(t4) ++ s1
-    note_launch();
-    k_up_cat_bwd<<<cdiv((long)B * H2 * H2 * 4, 256), 256, 0, s>>>(B * H2 * H2 * 4, H2, H2, 32, 16, n.gcat, n.t4, n.gmid);  // grad t4, masked
+    conv_launch<16, 48, 0, 16, kEpiSplit>(B, N, N, n.gbig2, none, n.t4, L[7].wb, nullptr, 0, n.gcat, n.gmid, nullptr, s);
     // c4: in up2(t3) ++ s2
     conv_dw<64, 32, 32>(n, ra, 6, B, H2, H2, n.s2, n.gmid, s, n.t3);
-    conv_fwd<32, 64>(B, H2, H2, n.gmid, nullptr, L[6].wb, nullptr, 0, n.gup, nullptr, s);  // grad of up2(t3) ++ s2
-    note_launch();
-    k_up_cat_bwd<<<cdiv((long)B * H4 * H4 * 4, 256), 256, 0, s>>>(B * H4 * H4 * 4, H4, H4, 32, 32, n.gup, n.t3, n.gsmall);  // grad t3, masked
+    conv_launch<32, 64, 0, 32, kEpiSplit>(B, H2, H2, n.gmid, none, n.t3, L[6].wb, nullptr, 0, n.gup, n.gsmall, nullptr, s);
     // c3b: in a3
     conv_dw<32, 32>(n, ra, 5, B, H4, H4, n.a3, n.gsmall, s);
-    conv_fwd<32, 32>(B, H4, H4, n.gsmall, n.a3, L[5].wb, nullptr, 0, n.gsmall2, nullptr, s);  // grad a3, masked
+    conv_launch<32, 32>(B, H4, H4, n.gsmall, none, n.a3, L[5].wb, nullptr, 0, n.gsmall2, nullptr, nullptr, s);  // grad a3, masked
     // c3a: in p2
     conv_dw<32, 32>(n, ra, 4, B, H4, H4, n.p2, n.gsmall2, s);
-    conv_fwd<32, 32>(B, H4, H4, n.gsmall2, nullptr, L[4].wb, nullptr, 0, n.gsmall, nullptr, s);  // grad p2
+    conv_launch<32, 32>(B, H4, H4, n.gsmall2, none, nullptr, L[4].wb, nullptr, 0, n.gsmall, nullptr, nullptr, s);  // grad p2
     // grad s2 = skip part of the c4 input grad + pool2 backward, masked
     note_launch();
-    k_skip_grad<<<cdiv((long)B * H2 * H2 * 4, 256), 256, 0, s>>>(B * H2 * H2 * 4, H2, H2, 32, 32, n.gup, n.gsmall, n.s2, n.gmid2);
+    k_skip_grad<<<cdiv((long)B * H2 * H2 * 4, 256), 256, 0, s>>>(B * H2 * H2 * 4, H2, H2, 32, n.gup, n.gsmall, n.s2, n.gmid2);
     // c2b: in a2
     conv_dw<32, 32>(n, ra, 3, B, H2, H2, n.a2, n.gmid2, s);
-    conv_fwd<32, 32>(B, H2, H2, n.gmid2, n.a2, L[3].wb, nullptr, 0, n.gmid, nullptr, s);   // grad a2, masked
+    conv_launch<32, 32>(B, H2, H2, n.gmid2, none, n.a2, L[3].wb, nullptr, 0, n.gmid, nullptr, nullptr, s);   // grad a2, masked
     // c2a: in p1
     conv_dw<16, 32>(n, ra, 2, B, H2, H2, n.p1, n.gmid, s);
-    conv_fwd<32, 16>(B, H2, H2, n.gmid, nullptr, L[2].wb, nullptr, 0, n.gmid2, nullptr, s);  // grad p1
+    conv_launch<32, 16>(B, H2, H2, n.gmid, none, nullptr, L[2].wb, nullptr, 0, n.gmid2, nullptr, nullptr, s);  // grad p1
     // grad s1 = skip part of the c5 input grad + pool2 backward, masked
     note_launch();
-    k_skip_grad<<<cdiv(P * 2, 256), 256, 0, s>>>((int)(P * 2), N, N, 32, 16, n.gcat, n.gmid2, n.s1, n.gbig);
+    k_skip_grad<<<cdiv(P * 2, 256), 256, 0, s>>>((int)(P * 2), N, N, 16, n.gcat, n.gmid2, n.s1, n.gbig);
     // c1b: in a1
     conv_dw<16, 16>(n, ra, 1, B, N, N, n.a1, n.gbig, s);
-    conv_fwd<16, 16>(B, N, N, n.gbig, n.a1, L[1].wb, nullptr, 0, n.gbig2, nullptr, s);     // grad a1, masked
+    conv_launch<16, 16>(B, N, N, n.gbig, none, n.a1, L[1].wb, nullptr, 0, n.gbig2, nullptr, nullptr, s);     // grad a1, masked
     // c1a: in x
-    conv_dw<16, 16>(n, ra, 0, B, N, N, n.x, n.gbig2, s);
+    conv_dw<16, 16, 0, 2, 16>(n, ra, 0, B, N, N, n.x, n.gbig2, s);
     int ctas = 0;
     for (int k = 0; k < kLayers; k++) {
         ra.gw[k] = n.g + L[k].woff; ra.gb[k] = n.g + L[k].boff;
