@@ -1139,19 +1139,18 @@ __global__ void __launch_bounds__(1024) k_level_coeffs_small(LevelCoeffArgs a)
 // row c is scaled by 1 / A'_cc and eliminated from every other row, the
 // eliminated column becoming the inverse's (n^3 multiply-adds, all on one
 // SM's FP64 pipe: the size of the coarsest level decides its cost).  One
-// CTA; A' lives in shared memory when n^2 + n doubles fit in 96 KB, else in
-// the scratch `Ag`.
+// CTA, A' in shared memory: for at most kCoarseOneCta cells.
+constexpr int kCoarseOneCta = 64;  // larger coarsest levels: k_coarse_step
 __global__ void __launch_bounds__(1024)
 k_coarse_inv(int nx, int ny, double h, const double *__restrict__ bx,
-             const double *__restrict__ by, double *__restrict__ Ag, double *__restrict__ AinvT,
-             int in_smem)
+             const double *__restrict__ by, double *__restrict__ AinvT)
 {
     extern __shared__ __align__(16) double cinv_sm[];
-    __shared__ double colc[kMaxCoarsest];
+    __shared__ double colc[kCoarseOneCta];
     __shared__ double invp;
     const int n = nx * ny;
     const double hh = h * h;
-    double *A = in_smem ? cinv_sm : Ag;
+    double *A = cinv_sm;
     for (int k = threadIdx.x; k < n * n; k += blockDim.x) A[k] = 0.0;
     __syncthreads();
     for (int c = threadIdx.x; c < n; c += blockDim.x) {
@@ -1194,6 +1193,96 @@ k_coarse_inv(int nx, int ny, double h, const double *__restrict__ bx,
     }
 }
 
+// The same inverse for a larger coarsest level (grid sides with an odd
+// factor: 960 x 640 ends at 15 x 10), by block Gauss-Jordan elimination over
+// the whole device: k_coarse_mat forms A', then one launch per 16 columns
+// (k_coarse_step) reads one n x n buffer and writes the other.  In step K,
+// with D the diagonal block's inverse: row K becomes D A_KJ, column K
+// becomes -A_IK D, the rest A_IJ - A_IK (D A_KJ), the block itself D.  One
+// block per 16 x 16 tile; each inverts the diagonal block for itself (3 us of
+// latency, cheaper than a launch of its own).  One CTA does n^3 FP64
+// multiply-adds on one SM's FP64 pipe: 1988 us for 150 cells, here 152 us.
+constexpr int kCB = 16;
+__global__ void __launch_bounds__(256)
+k_coarse_mat(int nx, int ny, double ihh, const double *__restrict__ bx,
+             const double *__restrict__ by, double *__restrict__ A)
+{
+    const int n = nx * ny, k = blockIdx.x * 256 + threadIdx.x;
+    if (k >= n * n) return;
+    const int r = k / n, c = k - r * n;
+    // row r of the 5-point operator: faces of cell r
+    auto diag = [&](int q) {
+        const int i = q % nx, j = q / nx;
+        const long kx = (long)j * (nx + 1) + i;
+        double d = 0.0;
+        if (i + 1 < nx) d -= bx[kx + 1];
+        if (i > 0) d -= bx[kx];
+        if (j + 1 < ny) d -= by[q + nx];
+        if (j > 0) d -= by[q];
+        return d * ihh;
+    };
+    const int i = r % nx, j = r / nx;
+    const long kx = (long)j * (nx + 1) + i;
+    double v = 0.0;
+    if (c == r) v = diag(r);
+    else if (c == r + 1 && i + 1 < nx) v = bx[kx + 1] * ihh;
+    else if (c == r - 1 && i > 0) v = bx[kx] * ihh;
+    else if (c == r + nx) v = by[r + nx] * ihh;  // j + 1 < ny, since c < n
+    else if (c == r - nx) v = by[r] * ihh;       // j > 0, since c >= 0
+    A[k] = v + diag(0);
+}
+
+__global__ void __launch_bounds__(kCB * kCB)
+k_coarse_step(int n, int K, const double *__restrict__ A, double *__restrict__ out, int transpose)
+{
+    __shared__ double D[kCB][kCB + 1], P[kCB][kCB + 1], Q[kCB][kCB + 1];
+    const int r = threadIdx.x / kCB, c = threadIdx.x % kCB;
+    const int I = blockIdx.y, J = blockIdx.x, k0 = K * kCB;
+    // tiles beyond the matrix's edge read the identity (diagonal) or zero
+    auto at = [&](int gr, int gc) { return gr < n && gc < n ? A[(long)gr * n + gc] : (gr == gc ? 1.0 : 0.0); };
+    double d = at(k0 + r, k0 + c);
+    P[r][c] = at(I * kCB + r, k0 + c);   // A_IK
+    Q[r][c] = at(k0 + r, J * kCB + c);   // A_KJ
+    const double a = at(I * kCB + r, J * kCB + c);
+    D[r][c] = d;
+    for (int p = 0; p < kCB; p++) {
+        __syncthreads();
+        // every thread its own entry: row p scaled by the pivot's reciprocal,
+        // eliminated from the others
+        const double ip = recip_any(D[p][p]);
+        const double dp = D[p][c], f = D[r][p];
+        __syncthreads();
+        if (r == p) d = c == p ? ip : dp * ip;
+        else d = c == p ? -f * ip : fma(-f, dp * ip, d);
+        D[r][c] = d;
+    }
+    __syncthreads();
+    double v;
+    if (I == K && J == K) {
+        v = d;
+    } else if (J == K) {  // -A_IK D
+        v = 0.0;
+#pragma unroll
+        for (int q = 0; q < kCB; q++) v = fma(-P[r][q], D[q][c], v);
+    } else {
+        double t = 0.0;     // (D A_KJ)_rc
+#pragma unroll
+        for (int q = 0; q < kCB; q++) t = fma(D[r][q], Q[q][c], t);
+        if (I == K) {
+            v = t;
+        } else {
+            __syncthreads();
+            Q[r][c] = t;
+            __syncthreads();
+            v = a;
+#pragma unroll
+            for (int q = 0; q < kCB; q++) v = fma(-P[r][q], Q[q][c], v);
+        }
+    }
+    const int gr = I * kCB + r, gc = J * kCB + c;
+    if (gr < n && gc < n) out[transpose ? (long)gc * n + gr : (long)gr * n + gc] = v;
+}
+
 // ------------------------------------------------------------ tail kernel
 constexpr int kMaxLv = 16;
 template <typename T>
@@ -1225,6 +1314,7 @@ struct TailArgs {
 // solve reads it from global memory.
 constexpr int kTailPad = 16;
 constexpr size_t kTailInvMax = 64 * 1024;
+constexpr int kTailWarpSolve = 64;  // coarsest cells that one warp solves
 __host__ __device__ inline size_t tail_level_elems(int nx, int ny, bool coarsest)
 {
     const size_t n = (size_t)nx * ny;
@@ -1513,12 +1603,15 @@ __device__ __forceinline__ void tail_up(const TailArgs<T> &g, T *sm, int l0, int
 // there, and the level-lt iterate is copied back.  Levels of at least 512
 // cells use the whole block, those of at least 128 cells warps 0-3, the rest
 // and the coarsest solve warp 0.
-template <typename T>
+// BIG: a coarsest level of more than kTailWarpSolve cells, solved by the
+// whole block (an instantiation of its own: the code of this branch costs the
+// small levels 6 us a launch in one kernel).
+template <typename T, bool BIG>
 __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<T> g)
 {
     using P2 = typename Pair<T>::V;
     extern __shared__ __align__(16) unsigned char tail_sm[];
-    __shared__ double xs[kMaxCoarsest];
+    __shared__ double xs[BIG ? kMaxCoarsest : kTailWarpSolve], parts[BIG ? 1024 : 1];
     T *sm = reinterpret_cast<T *>(tail_sm);
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int L = g.nl, lc = L - 1, nco = g.nx[lc] * g.ny[lc];
@@ -1591,7 +1684,40 @@ __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<
     int lw = lb;    // first level of warp 0
     while (lw < lc && g.nx[lw] * g.ny[lw] >= 128) lw++;
     tail_down<T, 1024>(g, sm, g.lt, lb, tid);
-    if (tid < 128) {
+    if constexpr (BIG) {
+        // a larger coarsest level: the same product by the whole block, each
+        // warp 32 rows by a slice of the columns, the slices folded in order
+        // (one warp reads the inverse of 150 cells from L2 column by column:
+        // 30 of the tail's 54 us)
+        if (tid < 128) {
+            tail_down<T, 128>(g, sm, lb, lw, tid);
+            if (tid < 32) tail_down<T, 32>(g, sm, lw, lc, tid);
+        }
+        __syncthreads();
+        T *ecs = sm + g.off[lc];
+        for (int k = tid; k < nco; k += nthr) xs[k] = (double)ecs[nco + k];
+        __syncthreads();
+        const int chunks = (nco + 31) / 32, slices = 32 / chunks;
+        const int w = tid >> 5, k = (w % chunks) * 32 + (tid & 31), sl = w / chunks;
+        double acc = 0.0;
+        if (sl < slices && k < nco) {
+            const int q0 = nco * sl / slices, q1 = nco * (sl + 1) / slices;
+#pragma unroll 8
+            for (int q = q0; q < q1; q++) acc += ainv[q * nco + k] * xs[q];
+        }
+        parts[tid] = acc;
+        __syncthreads();
+        if (sl == 0 && k < nco) {
+            for (int q = 1; q < slices; q++) acc += parts[tid + q * chunks * 32];
+            ecs[k] = (T)acc;
+        }
+        __syncthreads();
+        if (tid < 128) {
+            if (tid < 32) tail_up<T, 32>(g, sm, lw, lc, tid);
+            gsync<128>();
+            tail_up<T, 128>(g, sm, lb, lw, tid);
+        }
+    } else if (tid < 128) {
         tail_down<T, 128>(g, sm, lb, lw, tid);
         if (tid < 32) {
             tail_down<T, 32>(g, sm, lw, lc, tid);
@@ -1937,7 +2063,8 @@ bool vcycle(MG &mg, int nu1, int nu2, cudaStream_t s, double *add64 = nullptr)
     ta.nu2 = nu2;
     note_launch();
     const size_t smem = tail_prepare(ta);
-    launch_pdl(k_tail<T>, 1, 1024, smem, s, ta);
+    const bool big = ta.nx[L - 1] * ta.ny[L - 1] > kTailWarpSolve;
+    launch_pdl(big ? k_tail<T, true> : k_tail<T, false>, 1, 1024, smem, s, ta);
     for (int l = lt - 1; l >= 0; l--) {
         Level &v = mg.lv[l];
         LevelT<T> &a = lvT(l);
@@ -2278,7 +2405,7 @@ long mg_bench_op(MG &mg, int op, int level, cudaStream_t s)
         ta.nu2 = 2;
         note_launch();
         const size_t smem = tail_prepare(ta);
-        launch_pdl(k_tail<float>, 1, 1024, smem, s, ta);
+        launch_pdl(nc > kTailWarpSolve ? k_tail<float, true> : k_tail<float, false>, 1, 1024, smem, s, ta);
         return (long)mg.lv[lt].nx * mg.lv[lt].ny;
     }
     case 7:
@@ -2360,17 +2487,32 @@ void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool w
         for (int l = mg.tail; l < L; l++) e += tail_level_elems(mg.lv[l].nx, mg.lv[l].ny, l == L - 1);
         for (int l = mg.tail_f; l < L; l++) ef += tail_level_elems(mg.lv[l].nx, mg.lv[l].ny, l == L - 1);
         const size_t inv = tail_inv_bytes(mg.lv[L - 1].nx * mg.lv[L - 1].ny);
-        raise_smem_limit((const void *)k_tail<double>, (int)(((e * 8 + 7) & ~(size_t)7) + inv));
-        raise_smem_limit((const void *)k_tail<float>, (int)(((ef * 4 + 7) & ~(size_t)7) + inv));
+        const int sd = (int)(((e * 8 + 7) & ~(size_t)7) + inv), sf = (int)(((ef * 4 + 7) & ~(size_t)7) + inv);
+        const bool big = mg.lv[L - 1].nx * mg.lv[L - 1].ny > kTailWarpSolve;
+        raise_smem_limit(big ? (const void *)k_tail<double, true> : (const void *)k_tail<double, false>, sd);
+        raise_smem_limit(big ? (const void *)k_tail<float, true> : (const void *)k_tail<float, false>, sf);
     }
     Level &vc = mg.lv[L - 1];
+    const int nc = vc.nx * vc.ny;
+    const size_t nc2 = (size_t)nc * nc;
+    if (nc > kCoarseOneCta) {
+        // the buffers (A' and its transposed inverse) alternate; the last
+        // step writes the inverse's place
+        const int steps = (int)cdiv(nc, kCB);
+        double *src = mg.lu + (steps % 2 ? 0 : nc2), *dst = mg.lu + (steps % 2 ? nc2 : 0);
+        note_launch(1 + steps);
+        k_coarse_mat<<<cdiv((long)nc2, 256), 256, 0, s>>>(vc.nx, vc.ny, 1.0 / (vc.h * vc.h), vc.d.bx,
+                                                         vc.d.by, src);
+        for (int K = 0; K < steps; K++) {
+            k_coarse_step<<<dim3(steps, steps), kCB * kCB, 0, s>>>(nc, K, src, dst, K == steps - 1);
+            std::swap(src, dst);
+        }
+        return;
+    }
     note_launch();
-    const size_t nc2 = (size_t)vc.nx * vc.ny * vc.nx * vc.ny;
     const size_t cbytes = nc2 * sizeof(double);
-    const int in_smem = cbytes <= 96 * 1024;
-    if (in_smem) raise_smem_limit((const void *)k_coarse_inv, (int)cbytes);
-    k_coarse_inv<<<1, 1024, in_smem ? cbytes : 0, s>>>(vc.nx, vc.ny, vc.h, vc.d.bx, vc.d.by, mg.lu,
-                                                       mg.lu + nc2, in_smem);
+    raise_smem_limit((const void *)k_coarse_inv, (int)cbytes);
+    k_coarse_inv<<<1, 1024, cbytes, s>>>(vc.nx, vc.ny, vc.h, vc.d.bx, vc.d.by, mg.lu + nc2);
 }
 
 // Host-driven solve: one launch per kernel and a host read of the residual
