@@ -1360,11 +1360,13 @@ __device__ __forceinline__ void stage_array(T *d, const T *src, int n, int tid, 
     int done = 0;
     if ((((uintptr_t)d | (uintptr_t)src) & 15) == 0) {
         const int nv = n / V;
+#pragma unroll 1
         for (int k = tid; k < nv; k += nthr)
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n"
                          ::"r"((unsigned)__cvta_generic_to_shared(d + V * k)), "l"(src + V * k));
         done = nv * V;
     }
+#pragma unroll 1
     for (int k = done + tid; k < n; k += nthr) cp_async_elem(d + k, src + k);
 }
 
@@ -1382,15 +1384,21 @@ __device__ __forceinline__ TailLv<T> tail_lv(const TailArgs<T> &g, T *sm, int l)
     return {b, b + s, b + 2 * s, b + 3 * s, b + 4 * s};
 }
 
-// Work of one level by a group of NT threads (thread index t): the whole
-// block (NT = 1024), warps 0-3 (128, named barrier 1) or warp 0 (32), chosen
-// by the level's size so that barriers are not wider than the work.
-template <int NT>
-__device__ __forceinline__ void gsync()
+// A level is worked on by the first NT threads of the block, NT chosen by
+// its size (tail_threads) so that barriers are not wider than the work; NT is
+// a run-time value and the levels are one loop, since instantiating the
+// phases per group size and direction made 86 KB of code (now 35 KB), part of
+// which a single CTA has to fetch anew in every launch.
+__device__ __forceinline__ int tail_threads(int cells)
 {
-    if constexpr (NT == 1024) __syncthreads();
-    else if constexpr (NT == 128) asm volatile("bar.sync 1, 128;\n" ::: "memory");
-    else __syncwarp();
+    // a phase has cells / 4 pairs of slots
+    return cells >= 2048 ? 1024 : (cells >= 1024 ? 512 : (cells >= 512 ? 256 : (cells >= 256 ? 128 : (cells >= 128 ? 64 : 32))));
+}
+__device__ __forceinline__ void gsync(int NT)
+{
+    // a named barrier of its own for each width
+    if (NT == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;\n" ::"r"(NT == 1024 ? 0 : NT >> 6), "r"(NT) : "memory");
 }
 
 // Walk of the slots q = t, t + NT, ... of a w-wide grid as (row, column)
@@ -1422,15 +1430,16 @@ template <> struct Pair<double> { using V = double2; };
 // shared-memory loads.  In row j the cells of colour c are i = 2m + o,
 // o = (j + c) & 1; their west / east neighbours are the other colour's slots
 // m - 1 + o and m + o of the same row.
-template <typename T, int NT>
-__device__ __forceinline__ void tail_phase2(const TailArgs<T> &g, const TailLv<T> &v, int l, int c, int t)
+template <typename T>
+__device__ __forceinline__ void tail_phase2(const TailArgs<T> &g, const TailLv<T> &v, int l, int c, int t,
+                                            int NT, Walk w)
 {
     using P2 = typename Pair<T>::V;
     const int nx = g.nx[l], ny = g.ny[l], hx = nx / 2, bl = hx * ny + kTailPad, hp = hx / 2;
     const int oc = c * bl, ob = bl - oc;
     const T h2 = g.h2[l];
     auto ld2 = [](const T *a, int k) { return *reinterpret_cast<const P2 *>(a + k); };
-    Walk w(t, NT, hp);
+#pragma unroll 1
     for (int q = t; q < hp * ny; q += NT, w.next()) {
         const int j = w.a, m = 2 * w.b, o = (j + c) & 1, k = j * hx + m;
         const P2 eo = ld2(v.e, ob + k), xo = ld2(v.cx, ob + k);
@@ -1464,22 +1473,27 @@ __device__ __forceinline__ void tail_phase2(const TailArgs<T> &g, const TailLv<T
     }
 }
 
-template <typename T, int NT>
-__device__ __forceinline__ void tail_smooth(const TailArgs<T> &g, T *sm, int l, int nsw, int first, int t)
+template <typename T>
+__device__ __forceinline__ void tail_smooth(const TailArgs<T> &g, T *sm, int l, int nsw, int first, int t, int NT)
 {
     const int nx = g.nx[l], ny = g.ny[l], hx = nx / 2, nh = hx * ny, bl = nh + kTailPad;
     const TailLv<T> v = tail_lv(g, sm, l);
     const T h2 = g.h2[l];
     if ((nx & 3) == 0) {
+        const Walk w(t, NT, hx / 2);
+#pragma unroll 1
         for (int ph = first; ph < 2 * nsw; ph++) {
-            tail_phase2<T, NT>(g, v, l, ph & 1, t);
-            gsync<NT>();
+            tail_phase2<T>(g, v, l, ph & 1, t, NT, w);
+            gsync(NT);
         }
         return;
     }
+    const Walk w0(t, NT, hx);
+#pragma unroll 1
     for (int ph = first; ph < 2 * nsw; ph++) {
         const int c = ph & 1, oc = c * bl, ob = bl - oc;
-        Walk w(t, NT, hx);
+        Walk w = w0;
+#pragma unroll 1
         for (int q = t; q < nh; q += NT, w.next()) {
             const int j = w.a, m = w.b, o = (j + c) & 1, i = 2 * m + o, k = j * hx + m;
             const T pE = (i + 1 < nx) ? v.e[ob + k + o] : T(0);
@@ -1494,7 +1508,7 @@ __device__ __forceinline__ void tail_smooth(const TailArgs<T> &g, T *sm, int l, 
             s = fma(bS, pS, s);
             v.e[oc + k] = (s - h2 * v.r[oc + k]) * v.iv[oc + k];
         }
-        gsync<NT>();
+        gsync(NT);
     }
 }
 
@@ -1503,8 +1517,8 @@ __device__ __forceinline__ void tail_smooth(const TailArgs<T> &g, T *sm, int l, 
 // correction starts at zero; with fold, the red cells of a split coarse level
 // get the result of the first red sweep from that zero start,
 // (0 - h_c^2 r_c) / diag_c, so its smoothing starts with the black phase.
-template <typename T, int NT>
-__device__ __forceinline__ void tail_restrict(const TailArgs<T> &g, T *sm, int l, int fold, int t)
+template <typename T>
+__device__ __forceinline__ void tail_restrict(const TailArgs<T> &g, T *sm, int l, int fold, int t, int NT)
 {
     const int nx = g.nx[l], ny = g.ny[l], hx = nx / 2, bl = hx * ny + kTailPad;
     const int nxc = nx / 2, nyc = ny / 2, nc = nxc * nyc;
@@ -1531,6 +1545,7 @@ __device__ __forceinline__ void tail_restrict(const TailArgs<T> &g, T *sm, int l
         return v.r[oc + k] - s * ih2;
     };
     Walk w(t, NT, nxc);
+#pragma unroll 1
     for (int k = t; k < nc; k += NT, w.next()) {
         const int J = w.a, I = w.b, i = 2 * I, j = 2 * J;
         T acc = res(i, j);
@@ -1547,14 +1562,14 @@ __device__ __forceinline__ void tail_restrict(const TailArgs<T> &g, T *sm, int l
             ec[kc] = (fold && cc == 0) ? (T(0) - h2c * rv) * ivc[kc] : T(0);
         }
     }
-    gsync<NT>();
+    gsync(NT);
 }
 
 // e_l += P e_{l+1} (bilinear, weights 9/16, 3/16, 3/16, 1/16).  With
 // black_only, the red cells are left out: the red phase that follows
 // overwrites them without reading them.
-template <typename T, int NT>
-__device__ __forceinline__ void tail_prolong(const TailArgs<T> &g, T *sm, int l, int black_only, int t)
+template <typename T>
+__device__ __forceinline__ void tail_prolong(const TailArgs<T> &g, T *sm, int l, int black_only, int t, int NT)
 {
     const int nx = g.nx[l], ny = g.ny[l], hx = nx / 2, nh = hx * ny, bl = nh + kTailPad;
     const int nxc = nx / 2, nyc = ny / 2, hxc = nxc / 2, blc = nxc * nyc / 2 + kTailPad;
@@ -1564,8 +1579,11 @@ __device__ __forceinline__ void tail_prolong(const TailArgs<T> &g, T *sm, int l,
     auto at = [&](int I, int J) {
         return cnat ? ec[J * nxc + I] : ec[((I + J) & 1) * blc + J * hxc + (I >> 1)];
     };
+    const Walk w0(t, NT, hx);
+#pragma unroll 1
     for (int c = black_only ? 1 : 0; c < 2; c++) {
-        Walk w(t, NT, hx);
+        Walk w = w0;
+#pragma unroll 1
         for (int q = t; q < nh; q += NT, w.next()) {
             const int j = w.a, m = w.b, i = 2 * m + ((j + c) & 1);
             const int I = m, J = j >> 1;
@@ -1575,37 +1593,19 @@ __device__ __forceinline__ void tail_prolong(const TailArgs<T> &g, T *sm, int l,
             ef[c * bl + j * hx + m] += (T(9) * c00 + T(3) * c10 + T(3) * c01 + c11) * T(0.0625);
         }
     }
-    gsync<NT>();
-}
-
-template <typename T, int NT>
-__device__ __forceinline__ void tail_down(const TailArgs<T> &g, T *sm, int l0, int l1, int t)
-{
-    for (int l = l0; l < l1; l++) {
-        tail_smooth<T, NT>(g, sm, l, g.nu1, (l > g.lt && g.nu1 > 0) ? 1 : 0, t);
-        tail_restrict<T, NT>(g, sm, l, g.nu1 > 0, t);
-    }
-}
-
-template <typename T, int NT>
-__device__ __forceinline__ void tail_up(const TailArgs<T> &g, T *sm, int l0, int l1, int t)
-{
-    for (int l = l1 - 1; l >= l0; l--) {
-        tail_prolong<T, NT>(g, sm, l, g.nu2 > 0, t);
-        tail_smooth<T, NT>(g, sm, l, g.nu2, 0, t);
-    }
+    gsync(NT);
 }
 
 // The lower V-cycle (levels lt..L-1) in one CTA: the coefficients, the
 // level-lt iterate and right-hand side and the coarsest inverse are loaded
 // into shared memory (into the colour-split layout: pairs of row neighbours
 // are loaded together and stored to their two colours), the cycle runs
-// there, and the level-lt iterate is copied back.  Levels of at least 512
-// cells use the whole block, those of at least 128 cells warps 0-3, the rest
-// and the coarsest solve warp 0.
-// BIG: a coarsest level of more than kTailWarpSolve cells, solved by the
-// whole block (an instantiation of its own: the code of this branch costs the
-// small levels 6 us a launch in one kernel).
+// there, and the level-lt iterate is copied back.  The cycle is one loop over
+// its 2 (L - 1 - lt) level visits, down then up, with the coarsest solve
+// between: by warp 0, or (BIG, more than kTailWarpSolve coarsest cells) by the
+// whole block, each warp 32 rows of the inverse by a slice of its columns, the
+// slices folded in order (one warp reading the inverse of 150 cells from L2
+// column by column took 30 of the tail's 54 us).
 template <typename T, bool BIG>
 __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<T> g)
 {
@@ -1627,7 +1627,9 @@ __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<
     // its stores
     constexpr int kStage = sizeof(T) == 4 ? 4 : 2;
     int npairs = 0;
+#pragma unroll 1
     for (int l = g.lt; l < lc; l++) npairs += g.nx[l] * g.ny[l] / 2;
+#pragma unroll 1
     for (int base = 0; base < npairs; base += kStage * nthr) {
         P2 d[kStage], yn[kStage];
         T x0[kStage], x1[kStage];
@@ -1637,6 +1639,7 @@ __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<
             int q = base + u * nthr + tid, l = g.lt;
             lv[u] = -1;
             if (q >= npairs) continue;
+#pragma unroll 1
             while (q >= g.nx[l] * g.ny[l] / 2) { q -= g.nx[l] * g.ny[l] / 2; l++; }
             // cells (i, j), (i + 1, j): colours c and 1 - c, slot m of both
             const int nx = g.nx[l], hx = nx / 2, bl = nx * g.ny[l] / 2 + kTailPad;
@@ -1668,6 +1671,7 @@ __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<
         const int nx = g.nx[g.lt], hx = nx / 2, n = nx * g.ny[g.lt], bl = n / 2 + kTailPad;
         const TailLv<T> v = tail_lv(g, sm, g.lt);
         Walk w(tid, nthr, hx);
+#pragma unroll 2
         for (int q = tid; q < n / 2; q += nthr, w.next()) {
             const int j = w.a, m = w.b, k = j * nx + 2 * m, c = j & 1;
             const P2 ev = *reinterpret_cast<const P2 *>(g.e[g.lt] + k);
@@ -1679,74 +1683,75 @@ __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<
     }
     asm volatile("cp.async.wait_all;\n" ::);
     __syncthreads();
-    int lb = g.lt;  // first level of warps 0-3
-    while (lb < lc && g.nx[lb] * g.ny[lb] >= 512) lb++;
-    int lw = lb;    // first level of warp 0
-    while (lw < lc && g.nx[lw] * g.ny[lw] >= 128) lw++;
-    tail_down<T, 1024>(g, sm, g.lt, lb, tid);
-    if constexpr (BIG) {
-        // a larger coarsest level: the same product by the whole block, each
-        // warp 32 rows by a slice of the columns, the slices folded in order
-        // (one warp reads the inverse of 150 cells from L2 column by column:
-        // 30 of the tail's 54 us)
-        if (tid < 128) {
-            tail_down<T, 128>(g, sm, lb, lw, tid);
-            if (tid < 32) tail_down<T, 32>(g, sm, lw, lc, tid);
-        }
-        __syncthreads();
-        T *ecs = sm + g.off[lc];
-        for (int k = tid; k < nco; k += nthr) xs[k] = (double)ecs[nco + k];
-        __syncthreads();
-        const int chunks = (nco + 31) / 32, slices = 32 / chunks;
-        const int w = tid >> 5, k = (w % chunks) * 32 + (tid & 31), sl = w / chunks;
-        double acc = 0.0;
-        if (sl < slices && k < nco) {
-            const int q0 = nco * sl / slices, q1 = nco * (sl + 1) / slices;
-#pragma unroll 8
-            for (int q = q0; q < q1; q++) acc += ainv[q * nco + k] * xs[q];
-        }
-        parts[tid] = acc;
-        __syncthreads();
-        if (sl == 0 && k < nco) {
-            for (int q = 1; q < slices; q++) acc += parts[tid + q * chunks * 32];
-            ecs[k] = (T)acc;
-        }
-        __syncthreads();
-        if (tid < 128) {
-            if (tid < 32) tail_up<T, 32>(g, sm, lw, lc, tid);
-            gsync<128>();
-            tail_up<T, 128>(g, sm, lb, lw, tid);
-        }
-    } else if (tid < 128) {
-        tail_down<T, 128>(g, sm, lb, lw, tid);
-        if (tid < 32) {
-            tail_down<T, 32>(g, sm, lw, lc, tid);
-            // coarsest: x = A'^{-1} r, one row of the inverse per lane
+    const int nlv = lc - g.lt;
+    int ntp = 32;  // threads of the previous visit on the way up
+#pragma unroll 1
+    for (int v = 0; v <= 2 * nlv; v++) {
+        if (v == nlv) {
+            // coarsest: x = A'^{-1} r
             T *ecs = sm + g.off[lc];
-            const T *rcs = ecs + nco;
-            for (int k = tid; k < nco; k += 32) xs[k] = (double)rcs[k];
-            __syncwarp();
-            for (int k = tid; k < nco; k += 32) {
+            if constexpr (BIG) {
+                __syncthreads();
+                for (int k = tid; k < nco; k += nthr) xs[k] = (double)ecs[nco + k];
+                __syncthreads();
+                const int chunks = (nco + 31) / 32, slices = 32 / chunks;
+                const int w = tid >> 5, k = (w % chunks) * 32 + (tid & 31), sl = w / chunks;
                 double acc = 0.0;
-                for (int q = 0; q < nco; q++) acc += ainv[q * nco + k] * xs[q];
-                ecs[k] = (T)acc;
+                if (sl < slices && k < nco) {
+                    const int q0 = nco * sl / slices, q1 = nco * (sl + 1) / slices;
+#pragma unroll 8
+                    for (int q = q0; q < q1; q++) acc += ainv[q * nco + k] * xs[q];
+                }
+                parts[tid] = acc;
+                __syncthreads();
+                if (sl == 0 && k < nco) {
+                    for (int q = 1; q < slices; q++) acc += parts[tid + q * chunks * 32];
+                    ecs[k] = (T)acc;
+                }
+                __syncthreads();
+            } else if (tid < 32) {
+                // one row of the inverse per lane
+#pragma unroll 1
+                for (int k = tid; k < nco; k += 32) xs[k] = (double)ecs[nco + k];
+                __syncwarp();
+#pragma unroll 1
+                for (int k = tid; k < nco; k += 32) {
+                    double acc = 0.0;
+#pragma unroll 8
+                    for (int q = 0; q < nco; q++) acc += ainv[q * nco + k] * xs[q];
+                    ecs[k] = (T)acc;
+                }
+                __syncwarp();
             }
-            __syncwarp();
-            tail_up<T, 32>(g, sm, lw, lc, tid);
+            continue;
         }
-        gsync<128>();
-        tail_up<T, 128>(g, sm, lb, lw, tid);
+        const bool down = v < nlv;
+        const int l = down ? g.lt + v : g.lt + 2 * nlv - v;
+        const int NT = tail_threads(g.nx[l] * g.ny[l]);
+        if (tid >= NT) { ntp = NT; continue; }
+        if (!down) {
+            if (NT != ntp) gsync(NT);  // the smaller group's work is done
+            ntp = NT;
+            tail_prolong<T>(g, sm, l, g.nu2 > 0, tid, NT);
+        }
+        // the first red sweep after a restriction is folded into it
+        tail_smooth<T>(g, sm, l, down ? g.nu1 : g.nu2, down && v > 0 && g.nu1 > 0 ? 1 : 0, tid, NT);
+        if (down) {
+            tail_restrict<T>(g, sm, l, g.nu1 > 0, tid, NT);
+            ntp = 32;
+        }
     }
     __syncthreads();
-    tail_up<T, 1024>(g, sm, g.lt, lb, tid);
     const int nx0 = g.nx[g.lt], n0 = nx0 * g.ny[g.lt];
     T *eo = g.e[g.lt];
     if (g.lt == lc) {
+#pragma unroll 1
         for (int k = tid; k < n0; k += nthr) eo[k] = sm[g.off[lc] + k];
     } else {
         const int hx = nx0 / 2, bl = n0 / 2 + kTailPad;
         const T *es = sm + g.off[g.lt];
         Walk w(tid, nthr, hx);
+#pragma unroll 1
         for (int q = tid; q < n0 / 2; q += nthr, w.next()) {
             const int j = w.a, m = w.b, c = j & 1;
             P2 o;
@@ -1758,44 +1763,47 @@ __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<
 }
 
 // --------------------------------------------------------------- reductions
-// Deterministic sum: each block folds a fixed strided slice in a fixed order
-// and a fixed tree; the last block to finish folds the block partials.
-// Returns true in the one thread that wrote the total.
-template <typename F>
-__device__ bool block_fold_and_finish(double v, double *part, unsigned *count,
-                                      double *out)
+// Deterministic sum: each block folds its share in a fixed order (a shuffle
+// tree per warp, the warps in order); the last block to finish folds the
+// block partials the same way.  Returns true in the one thread that wrote the
+// total.  (A shared-memory tree over 256 threads costs eight barriers, twice:
+// 2 us of the 11 us of a reduction over 64^2 cells.)
+__device__ __forceinline__ double warp_sum(double v)
 {
-    __shared__ double sh[kRedT];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ bool block_fold_and_finish(double v, double *part, unsigned *count, double *out)
+{
+    __shared__ double sh[kRedT / 32];
     __shared__ bool last;
-    sh[threadIdx.x] = v;
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
-    for (int o = kRedT / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
     if (threadIdx.x == 0) {
-        part[blockIdx.x] = sh[0];
+        double s = sh[0];
+#pragma unroll
+        for (int w = 1; w < kRedT / 32; w++) s += sh[w];
+        part[blockIdx.x] = s;
         __threadfence();
-        unsigned t = atomicAdd(count, 1u);
-        last = (t == gridDim.x - 1);
+        last = atomicAdd(count, 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return false;
     __threadfence();
     double s = 0.0;
     for (int k = threadIdx.x; k < (int)gridDim.x; k += kRedT) s += ((volatile double *)part)[k];
-    sh[threadIdx.x] = s;
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
     __syncthreads();
-    for (int o = kRedT / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        *out = sh[0];
-        *count = 0u;
-        return true;
-    }
-    return false;
+    if (threadIdx.x != 0) return false;
+    s = sh[0];
+#pragma unroll
+    for (int w = 1; w < kRedT / 32; w++) s += sh[w];
+    *out = s;
+    *count = 0u;
+    return true;
 }
 
 // Convergence test of the device-side solve loop (one thread, after the
@@ -1813,15 +1821,13 @@ __device__ void solve_check(SolveCtl *ctl, const double *res, cudaGraphCondition
     cudaGraphSetConditional(hnd, go);
 }
 
-struct NoOp {};
-
 __global__ void __launch_bounds__(kRedT)
 k_sum(long n, const double *__restrict__ a, double *part, unsigned *count, double *out)
 {
     double s = 0.0;
     for (long k = (long)blockIdx.x * kRedT + threadIdx.x; k < n; k += (long)gridDim.x * kRedT)
         s += a[k];
-    block_fold_and_finish<NoOp>(s, part, count, out);
+    block_fold_and_finish(s, part, count, out);
 }
 
 // r0 = b - sum/n; accumulates sum r0^2.  With bt, also the right-hand side
@@ -1843,7 +1849,7 @@ k_sub_mean(long n, const double *__restrict__ b, const double *__restrict__ sum,
         if (bt) bt[k] = v * h2 * invd[k];
         s += v * v;
     }
-    block_fold_and_finish<NoOp>(s, part, count, out);
+    block_fold_and_finish(s, part, count, out);
 }
 
 __global__ void k_apply_mean(long n, double *__restrict__ p, const double *__restrict__ sum,
@@ -1874,7 +1880,7 @@ k_resnorm(int nx, int ny, double ih2, const double *__restrict__ bx,
     const long per = (n + gridDim.x - 1) / gridDim.x;
     const long ke = min(n, (long)blockIdx.x * per + per);
     long k = (long)blockIdx.x * per + threadIdx.x;
-    int j = (int)(k / nx), i = (int)(k - (long)j * nx);
+    int j = (int)k / nx, i = (int)k - j * nx;  // at most 2^28 cells
     double s = 0.0;
     for (; k < ke; k += kRedT) {
         const double r = b0[k] - flux_sum(nx, ny, i, j, bx, by, p) * ih2;
@@ -1882,7 +1888,7 @@ k_resnorm(int nx, int ny, double ih2, const double *__restrict__ bx,
         if (rf) { rf[k] = d2f_rn(r); ef[k] = 0.0f; }
         for (i += kRedT; i >= nx; i -= nx) j++;
     }
-    if (block_fold_and_finish<NoOp>(s, part, count, res + 2) && check)
+    if (block_fold_and_finish(s, part, count, res + 2) && check)
         solve_check(ctl, res, hnd, check == 1, inc);
 }
 
@@ -2283,6 +2289,11 @@ static int resident_red_blocks()
     return nb;
 }
 
+// Blocks of a reduction over n cells: one wave, but none without a cell a
+// thread (1216 blocks on 64^2 cells left 3 threads a block with work and
+// 1216 partials to fold: 11 us).
+static int red_grid(const MG &mg, long n) { return std::min(mg.red_blocks, (int)cdiv(n, kRedT)); }
+
 size_t mg_layout(MG &mg, int nx, int ny, double h, char *base)
 {
     int nxs[16], nys[16], L = 0;
@@ -2427,7 +2438,7 @@ long mg_bench_op(MG &mg, int op, int level, cudaStream_t s)
     case 6: {
         Level &v0 = mg.lv[0];
         note_launch();
-        launch_pdl(k_resnorm, mg.red_blocks, kRedT, 0, s, v0.nx, v0.ny, 1.0 / (v0.h * v0.h), v0.d.bx,
+        launch_pdl(k_resnorm, red_grid(mg, (long)v0.nx * v0.ny), kRedT, 0, s, v0.nx, v0.ny, 1.0 / (v0.h * v0.h), v0.d.bx,
                    v0.d.by, (const double *)v0.d.r, (const double *)v0.d.e, v0.f.r, v0.f.e,
                    mg.red + 8, mg.red_count, mg.red, (SolveCtl *)nullptr,
                    (cudaGraphConditionalHandle)0, 0, 0);
@@ -2529,7 +2540,7 @@ ib_status mg_run_direct(MG &mg, const double *rhs, double *p, int precision, dou
     if (precision == 0) ensure_fp64_w(mg, s);
     Level &v0 = mg.lv[0];
     const long n = (long)v0.nx * v0.ny;
-    const int RB = mg.red_blocks;
+    const int RB = red_grid(mg, n);
     double *part = mg.red + 8;
     double *res = mg.red;  // res[0] sum b, res[1] |b0|^2, res[2] |r|^2, res[3] sum p
     double *e0 = v0.d.e, *b0 = v0.d.r;
@@ -2610,7 +2621,7 @@ static cudaError_t build_solve_graph(MG &mg, SolveGraph &sg)
 {
     Level &v0 = mg.lv[0];
     const long n = (long)v0.nx * v0.ny;
-    const int RB = mg.red_blocks;
+    const int RB = red_grid(mg, n);
     double *part = mg.red + 8, *res = mg.red;
     double *e0 = v0.d.e, *b0 = v0.d.r;
     const double ih2 = 1.0 / (v0.h * v0.h);
