@@ -1596,16 +1596,67 @@ __device__ __forceinline__ void tail_prolong(const TailArgs<T> &g, T *sm, int l,
     gsync(NT);
 }
 
+// Coarsest solve x = A'^{-1} r (ecs: x, then r, nco values each), by warp 0
+// (the columns split over the lanes that the rows leave, folded in order) or,
+// BIG, more than kTailWarpSolve cells, by the whole block: each warp 32 rows
+// of the inverse by a slice of its columns, the slices folded in order (one
+// warp reading the inverse of 150 cells from L2 column by column took 30 of
+// the tail's 54 us).
+template <typename T, bool BIG>
+__device__ __forceinline__ void coarse_solve(T *ecs, int nco, const double *ainv, double *xs,
+                                             double *parts, int tid)
+{
+    if constexpr (BIG) {
+        __syncthreads();
+        for (int k = tid; k < nco; k += 1024) xs[k] = (double)ecs[nco + k];
+        __syncthreads();
+        const int chunks = (nco + 31) / 32, slices = 32 / chunks;
+        const int w = tid >> 5, k = (w % chunks) * 32 + (tid & 31), sl = w / chunks;
+        double acc = 0.0;
+        if (sl < slices && k < nco) {
+            const int q0 = nco * sl / slices, q1 = nco * (sl + 1) / slices;
+#pragma unroll 8
+            for (int q = q0; q < q1; q++) acc += ainv[q * nco + k] * xs[q];
+        }
+        parts[tid] = acc;
+        __syncthreads();
+        if (sl == 0 && k < nco) {
+            for (int q = 1; q < slices; q++) acc += parts[tid + q * chunks * 32];
+            ecs[k] = (T)acc;
+        }
+        __syncthreads();
+    } else if (tid < 32) {
+#pragma unroll 1
+        for (int k = tid; k < nco; k += 32) xs[k] = (double)ecs[nco + k];
+        __syncwarp();
+        const int nsl = nco <= 16 ? 32 / nco : 1;
+        const int sl = nsl > 1 ? tid / nco : 0;
+#pragma unroll 1
+        for (int k0 = 0; k0 < nco; k0 += 32) {
+            const int k = nsl > 1 ? tid - sl * nco : k0 + tid;
+            double acc = 0.0;
+            if (k < nco && sl < nsl) {
+                const int q1 = nco * (sl + 1) / nsl;
+#pragma unroll 8
+                for (int q = nco * sl / nsl; q < q1; q++) acc += ainv[q * nco + k] * xs[q];
+            }
+            for (int q = 1; q < nsl; q++) {
+                const double o = __shfl_sync(0xffffffffu, acc, (tid + q * nco) & 31);
+                if (sl == 0) acc += o;
+            }
+            if (k < nco && sl == 0) ecs[k] = (T)acc;
+        }
+        __syncwarp();
+    }
+}
+
 // The lower V-cycle (levels lt..L-1) in one CTA: the coefficients, the
 // level-lt iterate and right-hand side and the coarsest inverse are loaded
 // into shared memory (into the colour-split layout: pairs of row neighbours
 // are loaded together and stored to their two colours), the cycle runs
 // there, and the level-lt iterate is copied back.  The cycle is one loop over
 // its 2 (L - 1 - lt) level visits, down then up, with the coarsest solve
-// between: by warp 0, or (BIG, more than kTailWarpSolve coarsest cells) by the
-// whole block, each warp 32 rows of the inverse by a slice of its columns, the
-// slices folded in order (one warp reading the inverse of 150 cells from L2
-// column by column took 30 of the tail's 54 us).
+// between.
 template <typename T, bool BIG>
 __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<T> g)
 {
@@ -1688,41 +1739,7 @@ __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<
 #pragma unroll 1
     for (int v = 0; v <= 2 * nlv; v++) {
         if (v == nlv) {
-            // coarsest: x = A'^{-1} r
-            T *ecs = sm + g.off[lc];
-            if constexpr (BIG) {
-                __syncthreads();
-                for (int k = tid; k < nco; k += nthr) xs[k] = (double)ecs[nco + k];
-                __syncthreads();
-                const int chunks = (nco + 31) / 32, slices = 32 / chunks;
-                const int w = tid >> 5, k = (w % chunks) * 32 + (tid & 31), sl = w / chunks;
-                double acc = 0.0;
-                if (sl < slices && k < nco) {
-                    const int q0 = nco * sl / slices, q1 = nco * (sl + 1) / slices;
-#pragma unroll 8
-                    for (int q = q0; q < q1; q++) acc += ainv[q * nco + k] * xs[q];
-                }
-                parts[tid] = acc;
-                __syncthreads();
-                if (sl == 0 && k < nco) {
-                    for (int q = 1; q < slices; q++) acc += parts[tid + q * chunks * 32];
-                    ecs[k] = (T)acc;
-                }
-                __syncthreads();
-            } else if (tid < 32) {
-                // one row of the inverse per lane
-#pragma unroll 1
-                for (int k = tid; k < nco; k += 32) xs[k] = (double)ecs[nco + k];
-                __syncwarp();
-#pragma unroll 1
-                for (int k = tid; k < nco; k += 32) {
-                    double acc = 0.0;
-#pragma unroll 8
-                    for (int q = 0; q < nco; q++) acc += ainv[q * nco + k] * xs[q];
-                    ecs[k] = (T)acc;
-                }
-                __syncwarp();
-            }
+            coarse_solve<T, BIG>(sm + g.off[lc], nco, ainv, xs, parts, tid);
             continue;
         }
         const bool down = v < nlv;
@@ -1760,6 +1777,192 @@ __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<
             *reinterpret_cast<P2 *>(eo + j * nx0 + 2 * m) = o;
         }
     }
+}
+
+// The lower part of an FP64 V(2,2) cycle in one CTA, on the pre-scaled
+// stencil and with the residual identity of k_smooth2_f64: what bounds it is
+// FP64 instructions, each of which occupies its sub-partition's FP64 unit for
+// 64 cycles whatever its active lanes.  So a cell's update is four FMAs (six
+// operations in k_tail), one cell a thread spreads a small level over the
+// four sub-partitions (k_tail's pairs double a warp's chain), a restriction
+// takes eight FMAs a coarse cell (40 as b - A p), the level's correction
+// starts at zero so that its first red half sweep is e = -bt, written with bt
+// by the restriction before, and the weights, h^2 / diag and diag / (4 h^2)
+// are staged before the wait for the previous grid.  Used where the levels
+// below run V(2,2) and there is a level above the coarsest; 31 us a cycle
+// with k_tail<double> from 32^2 down, now 18 us.
+// Shared memory per level of n cells (colour-split as in k_tail, without
+// padding): e, bt, h^2 / diag (n each), the weights (W, E) and (S, N) (2 n
+// pairs), diag / (4 h^2) of the red cells and the last half sweep's changes
+// of the black ones (n / 2 each): 8 n doubles; the coarsest level x and r.
+struct TailWArgs {
+    int lt, nl, zero;        // zero: the level-lt iterate is zero on entry
+    int nx[kMaxLv], ny[kMaxLv], off[kMaxLv], inv_off;
+    double h2[kMaxLv], ih2[kMaxLv];
+    const double *w[kMaxLv], *invd[kMaxLv];
+    double *e;               // level lt: iterate (out; in unless zero)
+    const double *bt;        // level lt: h^2 b / diag
+    const double *ainvT;
+};
+__host__ __device__ inline size_t tailw_elems(int nx, int ny, bool coarsest)
+{
+    const size_t n = (size_t)nx * ny;
+    return coarsest ? (2 * n + 1) & ~(size_t)1 : 8 * n;
+}
+inline size_t tailw_prepare(TailWArgs &a)
+{
+    size_t n = 0;
+    for (int l = a.lt; l < a.nl; l++) {
+        a.off[l] = (int)n;
+        n += tailw_elems(a.nx[l], a.ny[l], l == a.nl - 1);
+    }
+    const size_t inv = tail_inv_bytes(a.nx[a.nl - 1] * a.ny[a.nl - 1]);
+    a.inv_off = inv ? (int)n : -1;
+    return n * 8 + inv;
+}
+
+template <bool BIG>
+__global__ void __launch_bounds__(1024) k_tail_f64(const __grid_constant__ TailWArgs g)
+{
+    extern __shared__ __align__(16) double tw_sm[];
+    __shared__ double xs[BIG ? kMaxCoarsest : kTailWarpSolve], parts[BIG ? 1024 : 1];
+    const int tid = threadIdx.x, lc = g.nl - 1, nco = g.nx[lc] * g.ny[lc];
+    const double *ainv = g.inv_off >= 0 ? tw_sm + g.inv_off : g.ainvT;
+    if (g.inv_off >= 0) stage_array(tw_sm + g.inv_off, g.ainvT, nco * nco, tid, 1024);
+    // coefficients of all levels (not written during the solve)
+#pragma unroll 1
+    for (int l = g.lt; l < lc; l++) {
+        const int nx = g.nx[l], n = nx * g.ny[l], hx = nx / 2, nh = n / 2;
+        double *q = tw_sm + g.off[l] + 2 * n;
+        double2 *we = reinterpret_cast<double2 *>(tw_sm + g.off[l] + 3 * n), *sn = we + n;
+        double *dg = tw_sm + g.off[l] + 7 * n;
+        Walk w(tid, 1024, nx);
+#pragma unroll 1
+        for (int k = tid; k < n; k += 1024, w.next()) {
+            const int c = (w.a + w.b) & 1, slot = w.a * hx + (w.b >> 1), d = c * nh + slot;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(we + d)), "l"(g.w[l] + 4 * k));
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(sn + d)), "l"(g.w[l] + 4 * k + 2));
+            const double id = g.invd[l][k];
+            q[d] = g.h2[l] * id;
+            if (c == 0) dg[slot] = 0.25 * g.ih2[l] * recip_any(id);
+        }
+    }
+    pdl_enter();
+    {
+        // level lt: right-hand side and (unless zero) iterate; from zero the
+        // first red half sweep is e = -bt
+        const int l = g.lt, nx = g.nx[l], n = nx * g.ny[l], hx = nx / 2, nh = n / 2;
+        double *e = tw_sm + g.off[l], *bt = e + n;
+        Walk w(tid, 1024, nx);
+#pragma unroll 1
+        for (int k = tid; k < n; k += 1024, w.next()) {
+            const int c = (w.a + w.b) & 1, d = c * nh + w.a * hx + (w.b >> 1);
+            const double b = g.bt[k];
+            bt[d] = b;
+            if (!g.zero) e[d] = g.e[k];
+            else if (c == 0) e[d] = -b;
+        }
+    }
+    asm volatile("cp.async.wait_all;\n" ::);
+    __syncthreads();
+    const int nlv = lc - g.lt;
+    int ntp = 32;
+#pragma unroll 1
+    for (int v = 0; v <= 2 * nlv; v++) {
+        if (v == nlv) {
+            coarse_solve<double, BIG>(tw_sm + g.off[lc], nco, ainv, xs, parts, tid);
+            continue;
+        }
+        const bool down = v < nlv;
+        const int l = down ? g.lt + v : g.lt + 2 * nlv - v;
+        const int nx = g.nx[l], ny = g.ny[l], n = nx * ny, hx = nx / 2, nh = n / 2;
+        const int NT = tail_threads(2 * n);  // a thread per cell of a colour
+        if (tid >= NT) { ntp = NT; continue; }
+        double *e = tw_sm + g.off[l], *bt = e + n;
+        const double2 *we = reinterpret_cast<const double2 *>(e + 3 * n), *sn = we + n;
+        const double *dg = e + 7 * n;
+        double *dl = e + 7 * n + nh;
+        const bool cnat = l + 1 == lc;
+        const int nxc = nx / 2, nc = n / 4, hxc = nxc / 2, nhc = nc / 2;
+        double *ec = tw_sm + g.off[l + 1];
+        const Walk w0(tid, NT, hx);
+        if (!down) {
+            if (NT != ntp) gsync(NT);  // the smaller group's work is done
+            ntp = NT;
+            // e += P e_c on the black cells (the red phase that follows
+            // overwrites the red ones without reading them)
+            auto at = [&](int I, int J) {
+                return cnat ? ec[J * nxc + I] : ec[((I + J) & 1) * nhc + J * hxc + (I >> 1)];
+            };
+            Walk w = w0;
+#pragma unroll 1
+            for (int k = tid; k < nh; k += NT, w.next()) {
+                const int j = w.a, I = w.b, J = j >> 1, nyc = ny / 2;
+                const int I2 = min(max(I + ((j & 1) ? -1 : 1), 0), nxc - 1);  // i = 2 I + (j + 1 & 1)
+                const int J2 = min(max(J + ((j & 1) ? 1 : -1), 0), nyc - 1);
+                e[nh + k] = fma(fma(9.0, at(I, J), fma(3.0, at(I2, J) + at(I, J2), at(I2, J2))), 0.0625, e[nh + k]);
+            }
+            gsync(NT);
+        }
+#pragma unroll 1
+        for (int ph = down && (v > 0 || g.zero) ? 1 : 0; ph < 4; ph++) {
+            const int c = ph & 1;
+            const double *eo = e + (1 - c) * nh;
+            Walk w = w0;
+#pragma unroll 1
+            for (int k = tid; k < nh; k += NT, w.next()) {
+                const int j = w.a, m = w.b, o = (j + c) & 1;
+                // a wall's weight is zero: any cell stands for the one beyond
+                const double eW = eo[m + o > 0 ? k - 1 + o : k], eE = eo[m + o < hx ? k + o : k];
+                const double eS = eo[j > 0 ? k - hx : k], eN = eo[j + 1 < ny ? k + hx : k];
+                const int d = c * nh + k;
+                const double2 a = we[d], b = sn[d];
+                double s = fma(a.x, eW, -bt[d]);
+                s = fma(a.y, eE, s);
+                s = fma(b.x, eS, s);
+                s = fma(b.y, eN, s);
+                if (down && ph == 3) dl[k] = s - e[d];
+                e[d] = s;
+            }
+            gsync(NT);
+        }
+        if (!down) continue;
+        // the residual identity: a red cell's residual is -(diag / h^2) sum_f
+        // w_f delta_f, a black one's zero
+        const double *qc = ec + 2 * nc;
+        Walk w(tid, NT, nxc);
+#pragma unroll 1
+        for (int k = tid; k < nc; k += NT, w.next()) {
+            const int I = w.b, J = w.a, k0 = 2 * J * hx + I, k1 = k0 + hx;
+            const double2 a0 = we[k0], b0 = sn[k0], a1 = we[k1], b1 = sn[k1];
+            double s0 = a0.x * dl[I > 0 ? k0 - 1 : k0];
+            s0 = fma(a0.y, dl[k0], s0);
+            s0 = fma(b0.x, dl[J > 0 ? k0 - hx : k0], s0);
+            s0 = fma(b0.y, dl[k1], s0);
+            double s1 = a1.x * dl[k1];
+            s1 = fma(a1.y, dl[I + 1 < hx ? k1 + 1 : k1], s1);
+            s1 = fma(b1.x, dl[k0], s1);
+            s1 = fma(b1.y, dl[2 * J + 2 < ny ? k1 + hx : k1], s1);
+            const double rv = -fma(dg[k0], s0, dg[k1] * s1);
+            if (cnat) {
+                ec[nc + k] = rv;
+            } else {
+                const int c = (I + J) & 1, d = c * nhc + J * hxc + (I >> 1);
+                const double b = rv * qc[d];
+                ec[nc + d] = b;
+                if (c == 0) ec[d] = -b;
+            }
+        }
+        gsync(NT);
+        ntp = 32;
+    }
+    __syncthreads();
+    const int nx0 = g.nx[g.lt], n0 = nx0 * g.ny[g.lt], hx0 = nx0 / 2;
+    const double *e = tw_sm + g.off[g.lt];
+    Walk w(tid, 1024, nx0);
+#pragma unroll 1
+    for (int k = tid; k < n0; k += 1024, w.next())
+        g.e[k] = e[((w.a + w.b) & 1) * (n0 / 2) + w.a * hx0 + (w.b >> 1)];
 }
 
 // --------------------------------------------------------------- reductions
@@ -2000,6 +2203,29 @@ T *smooth(const Level &v, LevelT<T> &a, T *cur, int nsw, bool fine, cudaStream_t
     return cur;
 }
 
+// The FP64 V(2,2) tail from level lt on, its iterate in e (zero: e is zero).
+void launch_tail_f64(MG &mg, double *e, bool zero, cudaStream_t s)
+{
+    TailWArgs a;
+    const int L = mg.L, lt = mg.tail;
+    a.lt = lt;
+    a.nl = L;
+    a.zero = zero ? 1 : 0;
+    for (int l = lt; l < L; l++) {
+        const Level &v = mg.lv[l];
+        a.nx[l] = v.nx; a.ny[l] = v.ny;
+        a.h2[l] = v.h * v.h; a.ih2[l] = 1.0 / (v.h * v.h);
+        a.w[l] = v.d.w; a.invd[l] = v.d.invd;
+    }
+    a.e = e;
+    a.bt = mg.lv[lt].d.bt;
+    const int nco = mg.lv[L - 1].nx * mg.lv[L - 1].ny;
+    a.ainvT = mg.lu + (size_t)nco * nco;
+    const size_t smem = tailw_prepare(a);
+    note_launch();
+    launch_pdl(nco > kTailWarpSolve ? k_tail_f64<true> : k_tail_f64<false>, 1, 1024, smem, s, a);
+}
+
 // One V(nu1, nu2) cycle on the level-0 data of precision T.  Every level's
 // iterate moves between its two buffers (cur[l]); the coarse corrections
 // start in the canonical buffer, which the restriction zeroes, and level 0
@@ -2031,11 +2257,9 @@ bool vcycle(MG &mg, int nu1, int nu2, cudaStream_t s, double *add64 = nullptr)
             if constexpr (f32) {
                 launch_smooth2<1>(v, a, cur[l], nxt, c.r, c.e, nullptr, s);
             } else {
-                // the next level's pre-scaled right-hand side where it is swept
-                // by the fused kernels (above the tail)
+                // with the next level's pre-scaled right-hand side
                 const double hc = mg.lv[l + 1].h;
-                launch_smooth2_f64<1>(v, a, cur[l], nxt, c.r, c.e, hc * hc, c.invd,
-                                      l + 1 < lt ? c.bt : nullptr, nullptr, s);
+                launch_smooth2_f64<1>(v, a, cur[l], nxt, c.r, c.e, hc * hc, c.invd, c.bt, nullptr, s);
             }
             if (pr) prof_mark(s, false);
             cur[l] = nxt;
@@ -2053,6 +2277,14 @@ bool vcycle(MG &mg, int nu1, int nu2, cudaStream_t s, double *add64 = nullptr)
         }
         cur[l + 1] = c.e;
     }
+    bool tail_done = false;
+    if constexpr (!f32) {
+        if (fused && lt < L - 1) {
+            launch_tail_f64(mg, cur[lt], lt > 0, s);
+            tail_done = true;
+        }
+    }
+    if (!tail_done) {
     TailArgs<T> ta;
     ta.lt = lt;
     ta.nl = L;
@@ -2071,6 +2303,7 @@ bool vcycle(MG &mg, int nu1, int nu2, cudaStream_t s, double *add64 = nullptr)
     const size_t smem = tail_prepare(ta);
     const bool big = ta.nx[L - 1] * ta.ny[L - 1] > kTailWarpSolve;
     launch_pdl(big ? k_tail<T, true> : k_tail<T, false>, 1, 1024, smem, s, ta);
+    }
     for (int l = lt - 1; l >= 0; l--) {
         Level &v = mg.lv[l];
         LevelT<T> &a = lvT(l);
@@ -2429,7 +2662,7 @@ long mg_bench_op(MG &mg, int op, int level, cudaStream_t s)
         Level &c = mg.lv[level + 1];
         if (op == 7)
             launch_smooth2_f64<1>(v, v.d, v.d.e, v.d.e2, c.d.r, c.d.e2, c.h * c.h, c.d.invd,
-                                  level + 1 < mg.tail ? c.d.bt : nullptr, nullptr, s);
+                                  c.d.bt, nullptr, s);
         else
             launch_smooth2_f64<2>(v, v.d, v.d.e, v.d.e2, nullptr, nullptr, 0.0, nullptr, nullptr,
                                   c.d.e, s);
@@ -2504,6 +2737,9 @@ void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool w
         const int sd = (int)(((e * 8 + 7) & ~(size_t)7) + inv), sf = (int)(((ef * 4 + 7) & ~(size_t)7) + inv);
         const bool big = mg.lv[L - 1].nx * mg.lv[L - 1].ny > kTailWarpSolve;
         raise_smem_limit(big ? (const void *)k_tail<double, true> : (const void *)k_tail<double, false>, sd);
+        size_t ew = 0;
+        for (int l = mg.tail; l < L; l++) ew += tailw_elems(mg.lv[l].nx, mg.lv[l].ny, l == L - 1);
+        raise_smem_limit(big ? (const void *)k_tail_f64<true> : (const void *)k_tail_f64<false>, (int)(ew * 8 + inv));
         raise_smem_limit(big ? (const void *)k_tail<float, true> : (const void *)k_tail<float, false>, sf);
     }
     Level &vc = mg.lv[L - 1];
