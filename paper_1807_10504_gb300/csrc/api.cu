@@ -44,7 +44,10 @@ struct ib_ctx {
     double *uw = nullptr, *vw = nullptr, *Hw = nullptr, *Fxw = nullptr, *Fyw = nullptr,
            *bxa = nullptr, *bya = nullptr, *fr = nullptr;
     double *frame = nullptr;   // non-inertial frame record (kFrSlots doubles)
-    double *ue = nullptr, *ve = nullptr, *mh = nullptr;  // Crank-Nicolson: u_e and mu / 2
+    double *ue = nullptr, *ve = nullptr;  // Crank-Nicolson: the other pair of iterate buffers
+    double *cnw = nullptr, *cnr = nullptr;  // its weights and right-hand sides (cnmem)
+    void *cnmem = nullptr;
+    double *mh = nullptr;      // the indicator function
     double *pprev = nullptr;   // the previous step's pressure (warm start 3)
     bool have_pprev = false;
     // indicator function (Eq. (ind_psn)): unit coefficients, the solution
@@ -396,12 +399,11 @@ ib_status step_pre(ib_ctx *c, double dt, bool reloc, bool mass, int warm)
     launch_coeffs(g.nx, g.ny, g.rho_g, g.rho_l, g.mu_g, g.mu_l, prop, c->rho, c->mu, c->bx, c->by,
                   c->s);
     // explicit viscous term, or Crank-Nicolson: the explicit predictor with
-    // half the viscosity, then the implicit half
-    const double *mup = c->mu;
-    if (g.viscous) {
-        launch_scale((long)g.nx * g.ny, 0.5, c->mu, c->mh, c->s);
-        mup = c->mh;
-    }
+    // half the viscosity into the pair of buffers from which the implicit
+    // half's launches end in us, vs
+    const double visc = g.viscous ? 0.5 : 1.0;
+    const bool odd = g.viscous && cn_launches(g.cn_sweeps) % 2;
+    double *pu = odd ? c->ue : c->us, *pv = odd ? c->ve : c->vs;
     // on two side streams, overlapping the predictor: the hierarchy of the
     // pressure coefficients (the r-weighted operator r_face beta in
     // axisymmetric form), and (with the indicator) the face force; neither
@@ -417,17 +419,16 @@ ib_status step_pre(ib_ctx *c, double dt, bool reloc, bool mass, int warm)
         cudaEventRecord(c->ev_join3, c->s3);
     }
     if (g.axisym)
-        launch_predictor_axi(g.nx, g.ny, g.h, dt, c->rho, mup, c->u, c->v, c->au, c->av, c->have_prev,
-                             0.0, g.gy, g.frame ? c->frame : nullptr, c->bx, c->by, c->us, c->vs,
-                             c->au, c->av, c->s);
+        launch_predictor_axi(g.nx, g.ny, g.h, dt, c->rho, c->mu, c->u, c->v, c->au, c->av, c->have_prev,
+                             0.0, g.gy, g.frame ? c->frame : nullptr, c->bx, c->by, pu, pv,
+                             c->au, c->av, c->s, visc);
     else
-        launch_predictor(g.nx, g.ny, g.h, dt, c->rho, mup, c->u, c->v, c->au, c->av, c->have_prev,
-                         g.gx, g.gy, c->bx, c->by, c->us, c->vs, c->au, c->av, c->s);
+        launch_predictor(g.nx, g.ny, g.h, dt, c->rho, c->mu, c->u, c->v, c->au, c->av, c->have_prev,
+                         g.gx, g.gy, c->bx, c->by, pu, pv, c->au, c->av, c->s, visc);
     if (g.viscous) {
-        cudaMemcpyAsync(c->ue, c->us, (size_t)(g.nx + 1) * g.ny * 8, cudaMemcpyDeviceToDevice, c->s);
-        cudaMemcpyAsync(c->ve, c->vs, (size_t)g.nx * (g.ny + 1) * 8, cudaMemcpyDeviceToDevice, c->s);
-        launch_cn_solve(g.nx, g.ny, g.h, dt, c->rho, c->mu, g.axisym, g.frame ? c->frame : nullptr,
-                        g.cn_sweeps, c->ue, c->ve, c->us, c->vs, c->s);
+        launch_cn_solve_tab(g.nx, g.ny, g.h, dt, c->rho, c->mu, g.axisym, g.frame ? c->frame : nullptr,
+                            g.cn_sweeps, c->cnw, c->cnr, pu, pv, odd ? c->us : c->ue,
+                            odd ? c->vs : c->ve, c->s);
     }
     c->mg_ready = true;
     cudaStreamWaitEvent(c->s, c->ev_join, 0);   // the hierarchy is complete
@@ -527,6 +528,7 @@ void ib_destroy(ib_ctx *c)
     if (c->amem) cudaFree(c->amem);
     if (c->dmem) cudaFree(c->dmem);
     if (c->imem) cudaFree(c->imem);
+    if (c->cnmem) cudaFree(c->cnmem);
     for (auto &q : c->sgraphs)
         if (q.exec) cudaGraphExecDestroy(q.exec);
     if (c->cap) cudaStreamDestroy(c->cap);
@@ -619,6 +621,15 @@ ib_status ib_init(ib_ctx **out, const ib_config *cfg, const double *X, const dou
     if (e == cudaSuccess && g.frame) {
         launch_axi_frame(c->mk, 1.0, g.c1, g.c2, 1, c->frame, c->s);
         e = cudaStreamSynchronize(c->s);
+    }
+    if (e == cudaSuccess && g.viscous) {
+        e = cudaMalloc(&c->cnmem, al((fx + fy) * 32) + al((fx + fy) * 8));
+        if (e == cudaSuccess) {
+            c->cnw = (double *)c->cnmem;
+            c->cnr = (double *)((char *)c->cnmem + al((fx + fy) * 32));
+        } else {
+            c->cnmem = nullptr;
+        }
     }
     if (e == cudaSuccess && g.indicator) {
         const size_t ib = al(fx * 8) + al(fy * 8) + al(nc * 8) + al(8) + al((size_t)M * 8);

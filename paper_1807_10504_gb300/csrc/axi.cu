@@ -35,7 +35,8 @@ constexpr int kT = 256;
 // on the z boundary faces, the outer wall's reflected ghost is 2 wb - v.
 constexpr int PX = 32, PY = 8;
 __global__ void __launch_bounds__(PX * PY)
-k_predictor_axi(int nx, int ny, double h, double dt, const double *__restrict__ rho,
+k_predictor_axi(int nx, int ny, double h, double dt, double visc, double ivisc,
+                const double *__restrict__ rho,
                 const double *__restrict__ mu, const double *__restrict__ u,
                 const double *__restrict__ v, const double *__restrict__ aup,
                 const double *__restrict__ avp, int have_prev, double gx, double gy,
@@ -127,7 +128,7 @@ k_predictor_axi(int nx, int ny, double h, double dt, const double *__restrict__ 
     const int tx = threadIdx.x, ty = threadIdx.y, i = i0 + tx, j = j0 + ty;
     if (i >= nx || j >= ny) return;
     const int R = ty + 1, C = tx + 1;
-    const double h2 = h * h;
+    const double h2 = h * h * ivisc;  // the factor visc on mu, a power of two
     // radial face (i, j) at r = i h, control volume [r_(i-1), r_i]
     {
         const long k = (long)j * nxf + i;
@@ -137,7 +138,7 @@ k_predictor_axi(int nx, int ny, double h, double dt, const double *__restrict__ 
             const double r0 = i * h;
             const double uc = su[R][C];
             const double adv = ((fx[ty][tx + 1] - fx[ty][tx]) + (gxn[ty + 1][tx] - gxn[ty][tx])) / (r0 * h);
-            const double muf = 0.5 * (sm[R][C - 1] + sm[R][C]);
+            const double muf = (0.5 * visc) * (sm[R][C - 1] + sm[R][C]);
             const double vis = (vx[ty][tx + 1] - vx[ty][tx] + wxn[ty + 1][tx] - wxn[ty][tx]) / (r0 * h2) -
                                muf * uc / (r0 * r0);
             // 1 / rho_face: the plain face coefficient beta when given
@@ -374,11 +375,11 @@ void launch_predictor_axi(int nx, int ny, double h, double dt, const double *rho
                           const double *au_prev, const double *av_prev, int have_prev,
                           double gx, double gy, const double *frame, const double *bx,
                           const double *by, double *us, double *vs, double *au, double *av,
-                          cudaStream_t s)
+                          cudaStream_t s, double visc)
 {
     dim3 g(cdiv(nx, PX), cdiv(ny, PY)), b(PX, PY);
     note_launch();
-    k_predictor_axi<<<g, b, 0, s>>>(nx, ny, h, dt, rho, mu, u, v, au_prev, av_prev, have_prev, gx,
+    k_predictor_axi<<<g, b, 0, s>>>(nx, ny, h, dt, visc, 1.0 / visc, rho, mu, u, v, au_prev, av_prev, have_prev, gx,
                                     gy, frame, bx, by, us, vs, au, av);
 }
 

@@ -6,6 +6,8 @@
 //
 // All kernels are single-pass, one thread per cell or face, coalesced along
 // x; they are HBM-bound and small next to the multigrid solve.
+#include <utility>
+
 #include "ib_internal.cuh"
 
 namespace ibk {
@@ -297,6 +299,130 @@ __global__ void k_cn_sweep(int nx, int ny, double h, double dt, const double *__
     vs[k] = (ve[k] + tau * nb) / (1.0 + tau * (cs + ex));
 }
 
+// The same solve with its coefficients formed once (k_cn_coeffs) and two
+// sweeps a launch (k_cn_smooth).  k_cn_sweep forms every coefficient of a
+// face, with two divisions, in each of its 2 nsweeps half sweeps: ~60 FP64
+// operations where the update itself needs four, and FP64 arithmetic is what
+// bounds it on this part (20 sweeps at 512^2: 40 launches, 2.53 ms).
+//
+// k_cn_coeffs: per face the update u <- r + W u_W + E u_E + S u_S + N u_N of
+// k_cn_sweep, u = (u_e + tau nb) / (1 + tau (cs + ex)), as four weights and a
+// right-hand side (w[2k], w[2k + 1], r[k]; x-faces then y-faces).  Boundary
+// faces get zero weights and their own value.
+__global__ void k_cn_coeffs(int nx, int ny, double h, double dt, const double *__restrict__ rho,
+                            const double *__restrict__ mu, int axisym,
+                            const double *__restrict__ frame, const double *__restrict__ ue,
+                            const double *__restrict__ ve, double2 *__restrict__ w,
+                            double *__restrict__ r)
+{
+    const long nxf = nx + 1, nu = nxf * ny;
+    const long f = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    auto M = [&](int i, int j) { return mu[(long)j * nx + i]; };
+    if (f < nu) {
+        const int j = (int)(f / nxf), i = (int)(f - (long)j * nxf);
+        if (i == 0 || i == nx) {
+            w[2 * f] = make_double2(0.0, 0.0); w[2 * f + 1] = make_double2(0.0, 0.0);
+            r[f] = ue[f];
+            return;
+        }
+        const double r0 = axisym ? i * h : 1.0, rE = axisym ? (i + 0.5) * h : 1.0,
+                     rW = axisym ? (i - 0.5) * h : 1.0;
+        const double s = axisym ? recip_any(r0 * h * h) : recip_any(h * h);
+        const double m0 = M(i - 1, j), m1 = M(i, j), m = m0 + m1;
+        const double muN = (j + 1 < ny) ? 0.25 * (m + (M(i - 1, j + 1) + M(i, j + 1))) : 0.5 * m;
+        const double muS = (j > 0) ? 0.25 * ((M(i - 1, j - 1) + M(i, j - 1)) + m) : 0.5 * m;
+        const double cE = rE * m1 * s, cW = rW * m0 * s, cN = r0 * muN * s, cS = r0 * muS * s;
+        const bool n = j + 1 < ny, b = j > 0;
+        // a wall's reflected ghost: twice its weight on the diagonal
+        double d = (cE + cW) + (n ? cN : 2.0 * cN) + (b ? cS : 2.0 * cS);
+        if (axisym) d += 0.5 * m * recip_any(r0 * r0);
+        const double tau = dt * recip_any(rho[(long)j * nx + i - 1] + rho[(long)j * nx + i]);
+        const double g = recip_any(1.0 + tau * d), tg = tau * g;
+        w[2 * f] = make_double2(cW * tg, cE * tg);
+        w[2 * f + 1] = make_double2(b ? cS * tg : 0.0, n ? cN * tg : 0.0);
+        r[f] = ue[f] * g;
+        return;
+    }
+    const long k = f - nu;
+    if (k >= (long)nx * (ny + 1)) return;
+    const int j = (int)(k / nx), i = (int)(k - (long)j * nx);
+    if (j == 0 || j == ny) {
+        w[2 * f] = make_double2(0.0, 0.0); w[2 * f + 1] = make_double2(0.0, 0.0);
+        r[f] = ve[k];
+        return;
+    }
+    const double r0 = axisym ? (i + 0.5) * h : 1.0, rE = axisym ? (i + 1) * h : 1.0,
+                 rW = axisym ? i * h : 1.0;
+    const double s = axisym ? recip_any(r0 * h * h) : recip_any(h * h);
+    const double m0 = M(i, j - 1), m1 = M(i, j), m = m0 + m1;
+    const double muE = (i + 1 < nx) ? 0.25 * (m + (M(i + 1, j - 1) + M(i + 1, j))) : 0.5 * m;
+    const double muW = (i > 0) ? 0.25 * ((M(i - 1, j - 1) + M(i - 1, j)) + m) : 0.5 * m;
+    const double cN = r0 * m1 * s, cS = r0 * m0 * s, cE = rE * muE * s, cW = rW * muW * s;
+    const bool e = i + 1 < nx, b = i > 0;
+    double d = (cN + cS) + (e ? cE : 2.0 * cE);
+    if (b) d += cW;
+    else if (!axisym) d += 2.0 * cW;
+    const double tau = dt * recip_any(rho[(long)(j - 1) * nx + i] + rho[(long)j * nx + i]);
+    const double g = recip_any(1.0 + tau * d), tg = tau * g;
+    w[2 * f] = make_double2(b ? cW * tg : 0.0, e ? cE * tg : 0.0);
+    w[2 * f + 1] = make_double2(cS * tg, cN * tg);
+    double v = ve[k] * g;
+    if (!e && frame) v += 2.0 * cE * tg * frame[kFrWb];  // the outer wall moves with the frame
+    r[f] = v;
+}
+
+// NS red-black sweeps of both components in one launch, out of place: a block
+// stages a DW x DH tile of one component with a halo of 2 NS faces, runs the
+// 2 NS colour phases in shared memory on shrinking rings (so the tile equals
+// NS global sweeps of k_cn_sweep up to rounding), reading the weights from L2
+// (40 B a face), and stores the tile.  Blocks below nbu take x-faces, the
+// rest y-faces.  Bound by the FP64 pipe (four operations an update, 1.15
+// times that with the halo at 64 x 32 and NS = 2).
+template <int NS, int DW, int DH>
+__global__ void __launch_bounds__(256)
+k_cn_smooth(int nx, int ny, int nbu, const double2 *__restrict__ w, const double *__restrict__ r,
+            const double *__restrict__ uin, const double *__restrict__ vin,
+            double *__restrict__ uout, double *__restrict__ vout)
+{
+    constexpr int HA = 2 * NS, PW = DW + 2 * HA, PH = DH + 2 * HA;
+    __shared__ double ps[PH][PW];
+    const bool isv = (int)blockIdx.x >= nbu;
+    const int bk = (int)blockIdx.x - (isv ? nbu : 0);
+    const int W = isv ? nx : nx + 1, Hh = isv ? ny + 1 : ny;
+    const int tw = (W + DW - 1) / DW;
+    const int gi0 = (bk % tw) * DW - HA, gj0 = (bk / tw) * DH - HA;
+    const double *in = isv ? vin : uin;
+    double *out = isv ? vout : uout;
+    const long off = isv ? (long)(nx + 1) * ny : 0;
+    for (int k = threadIdx.x; k < PH * PW; k += 256) {
+        const int a = k / PW, c = k - a * PW, gi = gi0 + c, gj = gj0 + a;
+        ps[a][c] = (gi >= 0 && gi < W && gj >= 0 && gj < Hh) ? in[(long)gj * W + gi] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int ph = 0; ph < 2 * NS; ph++) {
+        const int q = HA - 1 - ph, color = ph & 1;
+        const int hw = (DW + 2 * q) / 2, hq = DH + 2 * q;
+        for (int k = threadIdx.x; k < hq * hw; k += 256) {
+            const int rr = k / hw, cc = k - rr * hw;
+            const int a = HA - q + rr, gj = gj0 + a;
+            const int c = HA - q + 2 * cc + ((gi0 + HA - q + gj + color) & 1), gi = gi0 + c;
+            if (gi < 0 || gi >= W || gj < 0 || gj >= Hh) continue;
+            const long f = off + (long)gj * W + gi;
+            const double2 we = w[2 * f], sn = w[2 * f + 1];
+            double s = fma(we.x, ps[a][c - 1], r[f]);
+            s = fma(we.y, ps[a][c + 1], s);
+            s = fma(sn.x, ps[a - 1][c], s);
+            ps[a][c] = fma(sn.y, ps[a + 1][c], s);
+        }
+        __syncthreads();
+    }
+    for (int k = threadIdx.x; k < DH * DW; k += 256) {
+        const int a = HA + k / DW, c = HA + k % DW, gi = gi0 + c, gj = gj0 + a;
+        if (gi < W && gj < Hh) out[(long)gj * W + gi] = ps[a][c];
+    }
+}
+
 // Indicator function of Section 2.2 Eq. (ind_psn), div grad I = div G:
 // the right-hand side div G of the face field G (the spread delta vector),
 // r_i times the axisymmetric divergence in that form; unit coefficients with
@@ -365,12 +491,6 @@ __global__ void k_fill(long n, double a, double *__restrict__ y)
     if (k < n) y[k] = a;
 }
 
-__global__ void k_scale(long n, double a, const double *__restrict__ x, double *__restrict__ y)
-{
-    const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) y[k] = a * x[k];
-}
-
 }  // namespace
 
 void launch_cn_solve(int nx, int ny, double h, double dt, const double *rho, const double *mu,
@@ -384,6 +504,39 @@ void launch_cn_solve(int nx, int ny, double h, double dt, const double *rho, con
             k_cn_sweep<<<cdiv(nf, kT), kT, 0, s>>>(nx, ny, h, dt, rho, mu, axisym, frame, c, ue, ve,
                                                    us, vs);
         }
+}
+
+int cn_launches(int nsweeps) { return (nsweeps + 1) / 2; }
+
+// Tiles of 64 x 32 faces once they fill the device four times over, 32 x 16
+// below (a small grid's weights come from L2 with too few blocks in flight
+// otherwise).
+void launch_cn_solve_tab(int nx, int ny, double h, double dt, const double *rho, const double *mu,
+                         int axisym, const double *frame, int nsweeps, double *w, double *r,
+                         double *ua, double *va, double *ub, double *vb, cudaStream_t s)
+{
+    const long nf = (long)(nx + 1) * ny + (long)nx * (ny + 1);
+    note_launch();
+    k_cn_coeffs<<<cdiv(nf, 128), 128, 0, s>>>(nx, ny, h, dt, rho, mu, axisym, frame, ua, va,
+                                              (double2 *)w, r);
+    auto go = [&](auto kern, int dw, int dh) {
+        const int nbu = (int)(cdiv(nx + 1, dw) * cdiv(ny, dh)), nbv = (int)(cdiv(nx, dw) * cdiv(ny + 1, dh));
+        note_launch();
+        kern<<<nbu + nbv, 256, 0, s>>>(nx, ny, nbu, (const double2 *)w, (const double *)r, (const double *)ua,
+                                       (const double *)va, ub, vb);
+        std::swap(ua, ub);
+        std::swap(va, vb);
+    };
+    const bool big = nf >= 4L * 152 * 64 * 32;
+    int k = 0;
+    for (; k + 2 <= nsweeps; k += 2) {
+        if (big) go(k_cn_smooth<2, 64, 32>, 64, 32);
+        else go(k_cn_smooth<2, 32, 16>, 32, 16);
+    }
+    if (k < nsweeps) {
+        if (big) go(k_cn_smooth<1, 64, 32>, 64, 32);
+        else go(k_cn_smooth<1, 32, 16>, 32, 16);
+    }
 }
 
 void launch_div_faces(int nx, int ny, double h, int axisym, const double *Gx, const double *Gy,
@@ -419,12 +572,6 @@ void launch_fill(long n, double a, double *y, cudaStream_t s)
 {
     note_launch();
     k_fill<<<cdiv(n, kT), kT, 0, s>>>(n, a, y);
-}
-
-void launch_scale(long n, double a, const double *x, double *y, cudaStream_t s)
-{
-    note_launch();
-    k_scale<<<cdiv(n, kT), kT, 0, s>>>(n, a, x, y);
 }
 
 void launch_coeffs(int nx, int ny, double rho_g, double rho_l, double mu_g,
@@ -465,11 +612,11 @@ void launch_predictor(int nx, int ny, double h, double dt, const double *rho,
                       const double *au_prev, const double *av_prev,
                       int have_prev, double gx, double gy, const double *bx,
                       const double *by, double *us, double *vs, double *au, double *av,
-                      cudaStream_t s)
+                      cudaStream_t s, double visc)
 {
     dim3 g(cdiv(nx, PX), cdiv(ny, PY)), b(PX, PY);
     note_launch();
-    k_predictor<<<g, b, 0, s>>>(nx, ny, 1.0 / h, 1.0 / (h * h), dt, rho, mu, u, v, au_prev,
+    k_predictor<<<g, b, 0, s>>>(nx, ny, 1.0 / h, visc / (h * h), dt, rho, mu, u, v, au_prev,
                                 av_prev, have_prev, gx, gy, bx, by, us, vs, au, av);
 }
 

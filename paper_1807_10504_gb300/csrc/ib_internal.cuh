@@ -155,7 +155,7 @@ void launch_predictor(int nx, int ny, double h, double dt, const double *rho,
                       const double *au_prev, const double *av_prev,
                       int have_prev, double gx, double gy, const double *bx,
                       const double *by, double *us, double *vs, double *au, double *av,
-                      cudaStream_t s);
+                      cudaStream_t s, double visc = 1.0);  // visc: factor on mu, a power of two
 
 // Crank-Nicolson viscous solve: nsweeps red-black sweeps of
 // u* - dt / (2 rho_f) D(u*) = u_e on both components; (us, vs) hold the
@@ -163,7 +163,14 @@ void launch_predictor(int nx, int ny, double h, double dt, const double *rho,
 void launch_cn_solve(int nx, int ny, double h, double dt, const double *rho, const double *mu,
                      int axisym, const double *frame, int nsweeps, const double *ue,
                      const double *ve, double *us, double *vs, cudaStream_t s);
-void launch_scale(long n, double a, const double *x, double *y, cudaStream_t s);
+// The same with scratch for the coefficients (w: 4 doubles and r: 1 double per
+// face, x-faces then y-faces) and a second pair of iterate buffers: u_e is in
+// (ua, va) on entry; the sweeps alternate between the pairs, so u* ends in
+// (ua, va) when cn_launches is even and in (ub, vb) when it is odd.
+int cn_launches(int nsweeps);
+void launch_cn_solve_tab(int nx, int ny, double h, double dt, const double *rho, const double *mu,
+                         int axisym, const double *frame, int nsweeps, double *w, double *r,
+                         double *ua, double *va, double *ub, double *vb, cudaStream_t s);
 void launch_fill(long n, double a, double *y, cudaStream_t s);
 void launch_extrapolate(long n, double *p, double *q, cudaStream_t s);
 // Indicator function (Section 2.2 Eq. (ind_psn)): right-hand side div G, the
@@ -185,7 +192,7 @@ void launch_predictor_axi(int nx, int ny, double h, double dt, const double *rho
                           const double *au_prev, const double *av_prev, int have_prev,
                           double gx, double gy, const double *frame, const double *bx,
                           const double *by, double *us, double *vs, double *au, double *av,
-                          cudaStream_t s);
+                          cudaStream_t s, double visc = 1.0);
 void launch_axi_zbc(int nx, int ny, const double *frame, double *v, cudaStream_t s);
 void launch_rhs_axi(int nx, int ny, double h, double dt, const double *us, const double *vs,
                     const double *Fx, const double *Fy, const double *bx, const double *by,
