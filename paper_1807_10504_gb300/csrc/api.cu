@@ -222,10 +222,12 @@ ib_status check_markers_host(ib_ctx *c, const ib_config &g, const double *X, con
 }
 
 // Marker geometry (curvature, normals, arc weights, force magnitude), with
-// the azimuthal curvature added in axisymmetric mode.
-void geometry(ib_ctx *c)
+// the azimuthal curvature added in axisymmetric mode; with segments, also the
+// records that the Heaviside and the irrotational force read.
+void geometry(ib_ctx *c, bool segments)
 {
     launch_geometry(c->mk, c->cfg.sigma, c->s);
+    if (segments) launch_segments(c->mk, c->s);
     if (c->cfg.axisym) launch_axi_curvature(c->mk, c->cfg.sigma, c->s);
 }
 
@@ -347,7 +349,7 @@ double *field_ptr(ib_ctx *c, int which, size_t *n)
 ib_status spread_into(ib_ctx *c, int mode, const double *fmag, double *Fx, double *Fy, double *H)
 {
     Markers &mk = c->mk;
-    geometry(c);
+    geometry(c, mode == 1);
     launch_sort(mk, c->s);
     const double *f = fmag ? fmag : mk.fmag;
     double *Hd = H ? H : c->H;
@@ -377,7 +379,7 @@ ib_status step_pre(ib_ctx *c, double dt, bool reloc, bool mass, int warm)
     cudaStreamWaitEvent(c->s2, c->ev_sort_fork, 0);
     launch_sort(mk, c->s2);
     cudaEventRecord(c->ev_sort_join, c->s2);
-    geometry(c);
+    geometry(c, true);
     cudaStreamWaitEvent(c->s, c->ev_sort_join, 0);
     heaviside_into(c, c->H);
     // the face force needs the geometry, the sort and H only: on s3 from
@@ -742,7 +744,7 @@ ib_status ib_set_field(ib_ctx *c, int which, const double *src, int where)
 ib_status ib_marker_geometry(ib_ctx *c, double *kappa, double *nx, double *ny, double *ds)
 {
     if (!c) return IB_EINVAL;
-    geometry(c);
+    geometry(c, false);
     const size_t b = (size_t)c->mk.M * 8;
     cudaError_t e = cudaSuccess;
     if (kappa && e == cudaSuccess) e = cudaMemcpyAsync(kappa, c->mk.kappa, b, cudaMemcpyDeviceToDevice, c->s);
@@ -801,7 +803,7 @@ ib_status ib_spread(ib_ctx *c, int mode, const double *fmag, double *Fx, double 
 ib_status ib_heaviside(ib_ctx *c, double *H)
 {
     if (!c || !H) return IB_EINVAL;
-    geometry(c);
+    geometry(c, true);
     launch_sort(c->mk, c->s);
     heaviside_into(c, H);
     ib_status st = launch_check(c, "heaviside");

@@ -355,6 +355,7 @@ struct Markers {
     float4 *slf = nullptr;                 // the same in FP32 (nx, ny, c, |n|)
     uint8_t *scvx = nullptr;               // per segment: 1 = half-plane path (strips convex, lines well conditioned)
     double *sinv = nullptr;                // per segment: 1 / |segment|^2 in grid units
+    double *stab = nullptr;                // conventional spreading: per-marker factors
     double *rfit = nullptr;                // relocation: per-drop control points and knot arc lengths
     double *rpar = nullptr;                // relocation: per drop (g, tau, arc length, failed)
     double *rwts = nullptr;                // relocation: per marker, its four basis weights
@@ -382,6 +383,9 @@ void markers_free(Markers &mk);
 // crossing or band pair list overflow; flags[2]: B-spline system not positive definite.
 void launch_validate(Markers &mk, cudaStream_t s);
 void launch_geometry(Markers &mk, double sigma, cudaStream_t s);
+// Segment records and the drops' Y ranges of the Heaviside (after
+// launch_geometry, whose normals they take).
+void launch_segments(Markers &mk, cudaStream_t s);
 void launch_sort(Markers &mk, cudaStream_t s);
 void launch_interp(const Markers &mk, int kernel, const double *u,
                    const double *v, double *U, double *V, double dt_move,

@@ -31,6 +31,25 @@ __device__ __forceinline__ double phi(int kernel, double r)
     return (5.0 - 2.0 * a - sqrt(-7.0 + 12.0 * a - 4.0 * a * a)) / 8.0;
 }
 
+// phi at the four grid lines that a marker reaches along one axis: at
+// r = a - 1 - f, a = 0 .. 3, f in [0, 1) the marker's fraction past line 1.
+// The cosine kernel's four values are 1/4 (1 -+ sin, cos(pi f / 2)) of one
+// angle: one sincospi instead of four cospi.
+__device__ __forceinline__ void phi4(int kernel, double f, double *p)
+{
+    if (kernel == 0) {
+        double sn, cs;
+        sincospi(0.5 * f, &sn, &cs);
+        p[0] = 0.25 * (1.0 - sn);
+        p[1] = 0.25 * (1.0 + cs);
+        p[2] = 0.25 * (1.0 + sn);
+        p[3] = 0.25 * (1.0 - cs);
+        return;
+    }
+#pragma unroll
+    for (int a = 0; a < 4; a++) p[a] = phi(kernel, (double)(a - 1) - f);
+}
+
 // Integer key with the order of the doubles (non-NaN; -0 treated as +0), so
 // that the many exact comparisons of the inside test run on the integer pipe.
 __device__ __forceinline__ unsigned long long okey(double d)
@@ -365,107 +384,113 @@ __global__ void k_block_active(int bnx, int bny, const uint32_t *__restrict__ bc
 }
 
 // ------------------------------------------------------------ interpolation
-__global__ void k_interp(int M, int kernel, int nx, int ny, double h, double x0, double y0,
-                         const double *__restrict__ u, const double *__restrict__ v,
-                         double *__restrict__ X, double *__restrict__ Y,
-                         double *__restrict__ U, double *__restrict__ V, double dt_move)
+// Eight lanes per marker: lanes 0-3 the rows of u's 4 x 4 stencil, 4-7 those
+// of v's.  A lane forms its component's factors along x and its row's along
+// y, sums its row, and the four rows meet in a fixed order.  The kernel is
+// bound by the latency of one thread's chain of FP64 operations and loads
+// not by their number: one thread per marker took 21 us for 512 and 24 us for
+// 16384 markers, here 6 and 9.
+__global__ void __launch_bounds__(128)
+k_interp(int M, int kernel, int nx, int ny, double ih, double x0, double y0,
+         const double *__restrict__ u, const double *__restrict__ v,
+         double *__restrict__ X, double *__restrict__ Y,
+         double *__restrict__ U, double *__restrict__ V, double dt_move)
 {
-    int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    double Xm = X[m], Ym = Y[m];
-    // the kernel is a product phi(dx) phi(dy): its 4 + 4 factors once per
-    // component (the same values the 4 x 4 products use)
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 7;
+    const int m = min(t >> 3, M - 1);  // whole warps reach the shuffles
+    const int b = lane & 3;
+    const bool isv = lane >= 4;
+    const double Xm = X[m], Ym = Y[m];
+    const double sx = (Xm - x0) * ih - (isv ? 0.5 : 0.0), sy = (Ym - y0) * ih - (isv ? 0.0 : 0.5);
+    const double fx = floor(sx), fy = floor(sy);
+    const int i0 = (int)fx - 1, j = (int)fy - 1 + b;
     double px[4], py[4];
-    double sx = (Xm - x0) / h, sy = (Ym - y0) / h - 0.5;
-    int i0 = (int)floor(sx) - 1, j0 = (int)floor(sy) - 1;
-    for (int a = 0; a < 4; a++) {
-        px[a] = phi(kernel, (double)(i0 + a) - sx);
-        py[a] = phi(kernel, (double)(j0 + a) - sy);
-    }
+    phi4(kernel, sx - fx, px);
+    phi4(kernel, sy - fy, py);
+    const int W = isv ? nx : nx + 1, H = isv ? ny + 1 : ny;
+    const double *f = isv ? v : u;
     double acc = 0.0;
-    for (int b = 0; b < 4; b++)
+    if (j >= 0 && j < H)
+#pragma unroll
         for (int a = 0; a < 4; a++) {
-            int i = i0 + a, j = j0 + b;
-            if (i < 0 || i > nx || j < 0 || j > ny - 1) continue;
-            acc += u[(long)j * (nx + 1) + i] * (px[a] * py[b]);
+            const int i = i0 + a;
+            if (i >= 0 && i < W) acc += f[(long)j * W + i] * px[a];
         }
-    double Um = acc;
-    sx = (Xm - x0) / h - 0.5;
-    sy = (Ym - y0) / h;
-    i0 = (int)floor(sx) - 1;
-    j0 = (int)floor(sy) - 1;
-    for (int a = 0; a < 4; a++) {
-        px[a] = phi(kernel, (double)(i0 + a) - sx);
-        py[a] = phi(kernel, (double)(j0 + a) - sy);
-    }
-    acc = 0.0;
-    for (int b = 0; b < 4; b++)
-        for (int a = 0; a < 4; a++) {
-            int i = i0 + a, j = j0 + b;
-            if (i < 0 || i > nx - 1 || j < 0 || j > ny) continue;
-            acc += v[(long)j * nx + i] * (px[a] * py[b]);
-        }
-    double Vm = acc;
-    if (U) U[m] = Um;
-    if (V) V[m] = Vm;
+    acc *= b == 0 ? py[0] : (b == 1 ? py[1] : (b == 2 ? py[2] : py[3]));
+    // rows (0 + 1) + (2 + 3), in every lane of the component
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+    const double other = __shfl_xor_sync(0xffffffffu, acc, 4);
+    if ((t >> 3) >= M || lane != 0) return;
+    if (U) U[m] = acc;
+    if (V) V[m] = other;
     if (dt_move != 0.0) {
-        X[m] = Xm + dt_move * Um;
-        Y[m] = Ym + dt_move * Vm;
+        X[m] = Xm + dt_move * acc;
+        Y[m] = Ym + dt_move * other;
     }
 }
 
 // ------------------------------------------------------------ conventional spread
-// One thread per face; markers of the 4 x 5 (x-faces) or 5 x 4 (y-faces)
-// cells that can reach the face, visited row by row in (cell, id) order.
-__global__ void k_spread_conv(int kernel, int nx, int ny, double h, double x0, double y0,
-                              int bnx, const uint32_t *__restrict__ bactive,
-                              const uint32_t *__restrict__ cell_start,
-                              const uint32_t *__restrict__ ids, const double *__restrict__ X,
-                              const double *__restrict__ Y, const double *__restrict__ fmag,
-                              const double *__restrict__ nxm, const double *__restrict__ nym,
-                              const double *__restrict__ ds, double *__restrict__ Fx,
-                              double *__restrict__ Fy)
+// A marker's record for the gather below (kTab doubles): the four factors
+// along x and along y towards the x-faces and towards the y-faces, the two
+// strengths f n ds / h^2, and the first face it reaches of each kind (two
+// ints a double).  Two threads a marker, one for each kind of face.
+constexpr int kTab = 20;
+__global__ void __launch_bounds__(128)
+k_spread_tab(int M, int kernel, double ih, double x0, double y0, const double *__restrict__ X,
+             const double *__restrict__ Y, const double *__restrict__ fmag,
+             const double *__restrict__ nxm, const double *__restrict__ nym,
+             const double *__restrict__ ds, double *__restrict__ tab)
 {
-    long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    long nxf = (long)(nx + 1) * ny;
-    const double ih2 = 1.0 / (h * h);
-    bool isx = k < nxf;
-    int i, j;
-    if (isx) {
-        j = (int)(k / (nx + 1));
-        i = (int)(k - (long)j * (nx + 1));
-        if (i == 0 || i == nx) return;
-    } else {
-        k -= nxf;
-        if (k >= (long)nx * (ny + 1)) return;
-        j = (int)(k / nx);
-        i = (int)(k - (long)j * nx);
-        if (j == 0 || j == ny) return;
-    }
-    int ci = min(i, nx - 1), cj = min(j, ny - 1);
-    if (!bactive[(cj / kBlk) * bnx + ci / kBlk]) return;
-    int ia = isx ? i - 2 : i - 2, ib = isx ? i + 1 : i + 2;
-    int ja = isx ? j - 2 : j - 2, jb = isx ? j + 2 : j + 1;
-    ia = max(ia, 0); ib = min(ib, nx - 1); ja = max(ja, 0); jb = min(jb, ny - 1);
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, m = t >> 1, d = t & 1;
+    if (m >= M) return;
+    const double sx = (X[m] - x0) * ih - (d ? 0.5 : 0.0), sy = (Y[m] - y0) * ih - (d ? 0.0 : 0.5);
+    const double fx = floor(sx), fy = floor(sy);
+    double *o = tab + (long)m * kTab + 10 * d;
+    double p[4];
+    phi4(kernel, sx - fx, p);
+    *(double2 *)(o + 0) = make_double2(p[0], p[1]);
+    *(double2 *)(o + 2) = make_double2(p[2], p[3]);
+    phi4(kernel, sy - fy, p);
+    *(double2 *)(o + 4) = make_double2(p[0], p[1]);
+    *(double2 *)(o + 6) = make_double2(p[2], p[3]);
+    const int2 first = make_int2((int)fx - 1, (int)fy - 1);
+    *(double2 *)(o + 8) = make_double2(fmag[m] * (d ? nym[m] : nxm[m]) * ds[m] * (ih * ih),
+                                       __longlong_as_double(*(const long long *)&first));
+}
+
+// One block per 8 x 8 cells with a marker near, one thread per x-face left of
+// and y-face below a cell: the markers of the 4 x 5 (x-faces) or 5 x 4
+// (y-faces) cells that can reach the face, visited row by row in (cell, id)
+// order, three multiplications and an addition each.  Evaluating the kernel
+// per face and marker (two cosines, two divisions) on one thread per face of
+// the whole grid took 624 us at 1024^2 with 16384 markers, this 38 us and the
+// records 8 us.
+__global__ void __launch_bounds__(2 * kBlk * kBlk)
+k_spread_conv(int nx, int ny, int bnx, const uint32_t *__restrict__ bactive,
+              const uint32_t *__restrict__ cell_start, const uint32_t *__restrict__ ids,
+              const double *__restrict__ tab, double *__restrict__ Fx, double *__restrict__ Fy)
+{
+    if (!bactive[blockIdx.y * bnx + blockIdx.x]) return;
+    const int d = threadIdx.x / (kBlk * kBlk), c = threadIdx.x % (kBlk * kBlk);
+    const int i = blockIdx.x * kBlk + c % kBlk, j = blockIdx.y * kBlk + c / kBlk;
+    if (i >= nx || j >= ny || (d == 0 ? i == 0 : j == 0)) return;
+    const int ia = max(i - 2, 0), ib = min(d ? i + 2 : i + 1, nx - 1);
+    const int ja = max(j - 2, 0), jb = min(d ? j + 1 : j + 2, ny - 1);
     double acc = 0.0;
     for (int jj = ja; jj <= jb; jj++) {
-        uint32_t s = cell_start[(long)jj * nx + ia], e = cell_start[(long)jj * nx + ib + 1];
+        const uint32_t s = cell_start[(long)jj * nx + ia], e = cell_start[(long)jj * nx + ib + 1];
         for (uint32_t t = s; t < e; t++) {
-            int m = (int)ids[t];
-            double sx, sy, c;
-            if (isx) {
-                sx = (X[m] - x0) / h; sy = (Y[m] - y0) / h - 0.5;
-                c = fmag[m] * nxm[m] * ds[m] * ih2;
-            } else {
-                sx = (X[m] - x0) / h - 0.5; sy = (Y[m] - y0) / h;
-                c = fmag[m] * nym[m] * ds[m] * ih2;
-            }
-            double rx = (double)i - sx, ry = (double)j - sy;
-            if (fabs(rx) >= 2.0 || fabs(ry) >= 2.0) continue;
-            acc += c * (phi(kernel, rx) * phi(kernel, ry));
+            const double *o = tab + (long)ids[t] * kTab + 10 * d;
+            const double2 cf = *(const double2 *)(o + 8);
+            const long long bits = __double_as_longlong(cf.y);
+            const int a = i - (int)(unsigned)bits, b = j - (int)(bits >> 32);
+            if ((unsigned)a > 3u || (unsigned)b > 3u) continue;
+            acc += cf.x * (o[a] * o[4 + b]);
         }
     }
-    if (isx) Fx[k] = acc; else Fy[k] = acc;
+    if (d == 0) Fx[(long)j * (nx + 1) + i] = acc;
+    else Fy[(long)j * nx + i] = acc;
 }
 
 // ------------------------------------------------------------ inside / outside
@@ -1726,7 +1751,7 @@ cudaError_t markers_alloc(Markers &mk, int M, int ndrops, int nx, int ny, double
                    al(64) + al(pair_cap * 4) * 2 + al(pair_cap * 8) * 2 + al(ncell * 8) +
                    al((ndrops + 1) * 4) + al(M * 4) * 5 + al(ncell * 4) +
                    al((ncell + 1) * 4) + al(nparts * 4) + al(nb * 4) * 2 + al(64) +
-                   al((size_t)nx * 8) + al((size_t)kClipCap * 4);
+                   al((size_t)nx * 8) + al((size_t)kClipCap * 4) + al((size_t)M * kTab * 8);
     cudaError_t e = cudaMalloc(&mk.mem, bytes);
     if (e != cudaSuccess) { mk.mem = nullptr; return e; }
     char *q = (char *)mk.mem;
@@ -1766,6 +1791,7 @@ cudaError_t markers_alloc(Markers &mk, int M, int ndrops, int nx, int ny, double
     mk.flags = (uint32_t *)take(64);
     mk.colkey = (unsigned long long *)take((size_t)nx * 8);
     mk.clip_list = (uint32_t *)take((size_t)kClipCap * 4);
+    mk.stab = (double *)take((size_t)M * kTab * 8);
     std::vector<int32_t> dof(M), nxt(M);
     for (int d = 0; d < ndrops; d++)
         for (int m = drop_start_host[d]; m < drop_start_host[d + 1]; m++) {
@@ -1805,6 +1831,10 @@ void launch_geometry(Markers &mk, double sigma, cudaStream_t s)
     k_geometry<<<cdiv(mk.M, kT), kT, 0, s>>>(mk.M, mk.X, mk.Y, mk.drop_of, mk.drop_start, sigma,
                                             mk.x0, mk.y0, mk.h, mk.kappa, mk.nxm, mk.nym, mk.ds,
                                             mk.fmag, mk.gx, mk.gy, mk.gxf, mk.gyf, mk.ykey);
+}
+
+void launch_segments(Markers &mk, cudaStream_t s)
+{
     note_launch();
     k_segments<<<cdiv(mk.M, 32), 32, 0, s>>>(  // FP64-heavy: spread over all SMs
         mk.M, mk.next, mk.gx, mk.gy, mk.nxm, mk.nym, mk.sbox,
@@ -1843,20 +1873,21 @@ void launch_interp(const Markers &mk, int kernel, const double *u, const double 
                    double *U, double *V, double dt_move, cudaStream_t s)
 {
     note_launch();
-    k_interp<<<cdiv(mk.M, 128), 128, 0, s>>>(mk.M, kernel, mk.nx, mk.ny, mk.h, mk.x0, mk.y0, u, v,
+    k_interp<<<cdiv(8L * mk.M, 128), 128, 0, s>>>(mk.M, kernel, mk.nx, mk.ny, 1.0 / mk.h, mk.x0, mk.y0, u, v,
                                             mk.X, mk.Y, U, V, dt_move);
 }
 
 void launch_spread_conv(const Markers &mk, int kernel, const double *fmag, double *Fx,
                         double *Fy, cudaStream_t s)
 {
-    long nf = (long)(mk.nx + 1) * mk.ny + (long)mk.nx * (mk.ny + 1);
     cudaMemsetAsync(Fx, 0, (size_t)(mk.nx + 1) * mk.ny * 8, s);
     cudaMemsetAsync(Fy, 0, (size_t)mk.nx * (mk.ny + 1) * 8, s);
     note_launch();
-    k_spread_conv<<<cdiv(nf, kT), kT, 0, s>>>(kernel, mk.nx, mk.ny, mk.h, mk.x0, mk.y0, mk.bnx,
-                                             mk.bactive, mk.cell_start, mk.ids, mk.X, mk.Y,
-                                             fmag, mk.nxm, mk.nym, mk.ds, Fx, Fy);
+    k_spread_tab<<<cdiv(2L * mk.M, 128), 128, 0, s>>>(mk.M, kernel, 1.0 / mk.h, mk.x0, mk.y0, mk.X, mk.Y, fmag,
+                                                      mk.nxm, mk.nym, mk.ds, mk.stab);
+    note_launch();
+    k_spread_conv<<<dim3(mk.bnx, mk.bny), 2 * kBlk * kBlk, 0, s>>>(mk.nx, mk.ny, mk.bnx, mk.bactive,
+                                                                  mk.cell_start, mk.ids, mk.stab, Fx, Fy);
 }
 
 // Grid of the strip-area kernel: kClipBlocks clip blocks, then 8 CTAs of
