@@ -45,15 +45,13 @@ __device__ __forceinline__ uint32_t relu_mask(uint32_t v, uint32_t m)
 }
 
 // 16-byte asynchronous copy (both addresses 16-byte aligned); src-size 0 writes zeros.
-__device__ __forceinline__ void cp_async16(void *sdst, const void *gsrc, bool valid)
+__device__ __forceinline__ void cp_async16(uint32_t sa, const void *gsrc, bool valid)
 {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
     const int sz = valid ? 16 : 0;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gsrc), "r"(sz));
 }
-__device__ __forceinline__ void cp_async4(void *sdst, const void *gsrc, bool valid)
+__device__ __forceinline__ void cp_async4(uint32_t sa, const void *gsrc, bool valid)
 {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
     const int sz = valid ? 4 : 0;
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(sa), "l"(gsrc), "r"(sz));
 }
@@ -134,6 +132,19 @@ __device__ __forceinline__ uint4 sum4(uint4 v0, uint4 v1, uint4 v2, uint4 v3, fl
     return pack8(a);
 }
 
+// A tile's image, row and column among tw x th tiles an image, advanced by a
+// fixed number of tiles without a division per step.
+struct TilePos {
+    int b, r, c;
+    __device__ TilePos(int tl, int tw, int th) { b = tl / (tw * th); const int m = tl - b * tw * th; r = m / tw; c = m - r * tw; }
+    __device__ void advance(const TilePos &d, int tw, int th)
+    {
+        c += d.c; r += d.r; b += d.b;
+        if (c >= tw) { c -= tw; r++; }
+        if (r >= th) { r -= th; b++; }
+    }
+};
+
 // What a convolution's epilogue makes of its output tile (plain: y, masked
 // where ymask is given).
 enum ConvEpi {
@@ -194,40 +205,55 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
     }
     if (CST == 2)  // the channels that no copy writes
         for (int k = tid; k < ST * TP * XS / 8; k += 128) *(uint4 *)(xs0 + 8 * k) = make_uint4(0u, 0u, 0u, 0u);
-    // this thread's chunks of a tile: window row and column, offsets in x (or
-    // xu) from the tile's corner; a tile's corner is even, so the up-sampled
-    // part's offset is the same for every tile
+    // this thread's chunks of a tile: window row and column, offset from the
+    // tile's corner in x (or xu; a tile's corner is even, so the up-sampled
+    // part's offset is the same for every tile)
     constexpr int NCH = CST == 2 ? TP : TP * (CIN / 8), PER = (NCH + 127) / 128;
+    int go[PER], rc[PER], so[PER];
+    unsigned up = 0;
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        const int k = tid + 128 * i, pix = CST == 2 ? k : k / (CIN / 8), q = CST == 2 ? 0 : k - pix * (CIN / 8);
+        const int r = pix / (CW + 2), c = pix - r * (CW + 2);
+        rc[i] = k < NCH ? r | c << 8 : -1;
+        so[i] = (pix * XS + 8 * q) * 2;
+        if (CST == 2) go[i] = (r * W + c) * 2;
+        else if (CUP > 0 && q < CUP / 8) {
+            go[i] = (((r - 1) >> 1) * (W / 2) + ((c - 1) >> 1)) * CUP + 8 * q;
+            up |= 1u << i;
+        } else go[i] = (r * W + c) * CST + 8 * q - CUP;
+    }
+    const TilePos stride(gridDim.x, tw, th);
+    TilePos pi(blockIdx.x, tw, th);  // the next tile to copy
+    int ti = blockIdx.x;
+    const uint32_t xsa = (uint32_t)__cvta_generic_to_shared(xs0);
     __syncthreads();
-    auto issue = [&](int tl, int st) {
-        if (tl < ntiles) {
-            const int bz = tl / (tw * th), rem = tl - bz * tw * th, tr = rem / tw;
-            const int ty0 = tr * CH, tx0 = (rem - tr * tw) * CW;
-            const bf16 *xt = x + (((long)bz * H + ty0 - 1) * W + tx0 - 1) * CST;
-            const bf16 *ut = CUP > 0 ? xu + (((long)bz * (H / 2) + ty0 / 2) * (W / 2) + tx0 / 2) * CUP : nullptr;
-            bf16 *xs = xs0 + st * TP * XS;
+    auto issue = [&](int st) {
+        if (ti < ntiles) {
+            const int ty0 = pi.r * CH, tx0 = pi.c * CW;
+            const bf16 *xt = x + (((long)pi.b * H + ty0 - 1) * W + tx0 - 1) * CST;
+            const bf16 *ut = CUP > 0 ? xu + (((long)pi.b * (H / 2) + ty0 / 2) * (W / 2) + tx0 / 2) * CUP : nullptr;
+            const uint32_t sb = xsa + st * (TP * XS * 2);
 #pragma unroll
             for (int i = 0; i < PER; i++) {
-                const int k = tid + 128 * i;
-                if (PER * 128 > NCH && k >= NCH) break;
-                const int pix = CST == 2 ? k : k / (CIN / 8), q = CST == 2 ? 0 : k - pix * (CIN / 8);
-                const int r = pix / (CW + 2), c = pix - r * (CW + 2);
-                const bool in = (unsigned)(ty0 - 1 + r) < (unsigned)H && (unsigned)(tx0 - 1 + c) < (unsigned)W;
-                if (CST == 2) {
-                    cp_async4(xs + pix * XS, in ? xt + ((long)r * W + c) * 2 : x, in);
-                } else {
-                    const bf16 *src;
-                    if (CUP > 0 && q < CUP / 8)
-                        src = ut + ((long)((r - 1) >> 1) * (W / 2) + ((c - 1) >> 1)) * CUP + 8 * q;
-                    else
-                        src = xt + ((long)r * W + c) * CST + 8 * q - CUP;
-                    cp_async16(xs + pix * XS + 8 * q, in ? src : x, in);
-                }
+                if (PER * 128 > NCH && i == PER - 1 && rc[i] < 0) break;
+                const bool in = (unsigned)(ty0 - 1 + (rc[i] & 255)) < (unsigned)H && (unsigned)(tx0 - 1 + (rc[i] >> 8)) < (unsigned)W;
+                const bf16 *src = (CUP > 0 && (up >> i & 1u) ? ut : xt) + go[i];
+                if (CST == 2) cp_async4(sb + so[i], in ? src : x, in);
+                else cp_async16(sb + so[i], in ? src : x, in);
             }
         }
+        ti += gridDim.x;
+        pi.advance(stride, tw, th);
         cp_async_commit();  // an empty group past the last tile keeps the count
     };
-    for (int k = 0; k < ST - 1; k++) issue(blockIdx.x + k * gridDim.x, k);
+    for (int k = 0; k < ST - 1; k++) issue(k);
+    float bv[2 * NT];  // this lane's biases
+#pragma unroll
+    for (int nt = 0; nt < NT; nt++) {
+        bv[2 * nt] = bias ? bias[nt * 8 + 2 * t4] : 0.0f;
+        bv[2 * nt + 1] = bias ? bias[nt * 8 + 2 * t4 + 1] : 0.0f;
+    }
     // weight fragments: rows n (co) of 8 k values, two n blocks a load
     const uint32_t wa = (uint32_t)__cvta_generic_to_shared(ws) +
                         (((lane & 7) + (lane >> 4) * 8) * WS + ((lane >> 3) & 1) * 8) * 2;
@@ -244,10 +270,11 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
     const uint32_t ea = (uint32_t)__cvta_generic_to_shared(es) +
                         (((lane & 7) + ((lane >> 3) & 1) * 8) * ES + (lane >> 4) * 8) * 2;
     int st = 0;
-    for (int tl = blockIdx.x; tl < ntiles; tl += gridDim.x) {
+    TilePos po(blockIdx.x, tw, th);
+    for (int tl = blockIdx.x; tl < ntiles; tl += gridDim.x, po.advance(stride, tw, th)) {
         cp_async_wait<ST - 2>();
         __syncthreads();  // this tile's copies are visible; the slot of the one before is free
-        issue(tl + (ST - 1) * gridDim.x, (st + ST - 1) % ST);
+        issue((st + ST - 1) % ST);
         const uint32_t xa = xa0 + st * (TP * XS * 2);
         st = (st + 1) % ST;
         float acc[2][NT][4];
@@ -289,16 +316,13 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
             }
         }
         // epilogue: bias, ReLU, BF16, and through shared memory
-        const int bz = tl / (tw * th), rem = tl - bz * tw * th, tr = rem / tw;
-        const int oy0 = tr * CH + 2 * warp, tx0 = (rem - tr * tw) * CW;
+        const int oy0 = po.r * CH + 2 * warp, tx0 = po.c * CW;
+        const long o0 = ((long)po.b * H + oy0) * W + tx0;                        // first pixel of the warp's rows
+        const long h0 = ((long)po.b * (H / 2) + oy0 / 2) * (W / 2) + tx0 / 2;    // the same at half resolution
         __syncwarp();  // the last tile's rows of this warp have been read
 #pragma unroll
         for (int nt = 0; nt < NT; nt += 2) {
-            float b0 = 0.0f, b1 = 0.0f, b2 = 0.0f, b3 = 0.0f;
-            if (bias) {
-                const int co = nt * 8 + 2 * t4;
-                b0 = bias[co]; b1 = bias[co + 1]; b2 = bias[co + 8]; b3 = bias[co + 9];
-            }
+            const float b0 = bv[2 * nt], b1 = bv[2 * nt + 1], b2 = bv[2 * nt + 2], b3 = bv[2 * nt + 3];
 #pragma unroll
             for (int mt = 0; mt < 2; mt++) {
                 float v[8] = {acc[mt][nt][0] + b0, acc[mt][nt][1] + b1, acc[mt][nt][2] + b0, acc[mt][nt][3] + b1,
@@ -307,9 +331,9 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
 #pragma unroll
                     for (int q = 0; q < 8; q++) v[q] = fmaxf(v[q], 0.0f);
                 if (y32 && nt == 0 && t4 == 0 && oy0 + mt < H) {
-                    const long o = ((long)bz * H + oy0 + mt) * W + tx0 + g;
-                    if (tx0 + g < W) y32[o] = v[0];
-                    if (tx0 + g + 8 < W) y32[o + 8] = v[2];
+                    float *o = y32 + o0 + mt * W + g;
+                    if (tx0 + g < W) o[0] = v[0];
+                    if (tx0 + g + 8 < W) o[8] = v[2];
                 }
                 const uint4 pk = pack8(v);
                 const uint32_t rg[4] = {pk.x, pk.y, pk.z, pk.w};
@@ -326,7 +350,7 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
                 const int px = lane >> 2, c = lane & 3, ox = tx0 / 2 + px;
                 if (oy0 < H && 2 * ox < W) {
                     const bf16 *e = es + 2 * px * ES + 8 * c;
-                    const long o = (((long)bz * (H / 2) + oy0 / 2) * (W / 2) + ox) * 32 + 8 * c;
+                    const long o = (h0 + px) * 32 + 8 * c;
                     const uint4 v = sum4(*(const uint4 *)e, *(const uint4 *)(e + ES), *(const uint4 *)(e + 16 * ES),
                                          *(const uint4 *)(e + 17 * ES), 1.0f);
                     *(uint4 *)(y2 + o) = relu_mask8(v, *(const uint4 *)(ymask + o));
@@ -336,7 +360,7 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
             for (int k = lane; k < 32 * S8; k += 32) {
                 const int px = k / S8, c = k % S8, oy = oy0 + (px >> 4), ox = tx0 + (px & 15);
                 if (oy < H && ox < W)
-                    *(uint4 *)(y + (((long)bz * H + oy) * W + ox) * (8 * S8) + 8 * c) =
+                    *(uint4 *)(y + o0 * (8 * S8) + ((px >> 4) * W + (px & 15)) * (8 * S8) + 8 * c) =
                         *(const uint4 *)(es + px * ES + 32 + 8 * c);
             }
         } else {
@@ -344,7 +368,7 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
             for (int k = lane; k < 32 * C8; k += 32) {
                 const int px = k / C8, c = k % C8, oy = oy0 + (px >> 4), ox = tx0 + (px & 15);
                 if (oy < H && ox < W) {
-                    const long o = (((long)bz * H + oy) * W + ox) * COUT + 8 * c;
+                    const long o = o0 * COUT + ((px >> 4) * W + (px & 15)) * COUT + 8 * c;
                     uint4 v = *(const uint4 *)(es + px * ES + 8 * c);
                     if (ymask) v = relu_mask8(v, *(const uint4 *)(ymask + o));
                     *(uint4 *)(y + o) = v;
@@ -354,7 +378,7 @@ k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restri
                 const int px = lane / C8, c = lane % C8, ox = tx0 / 2 + px;
                 if (lane < 8 * C8 && oy0 < H && 2 * ox < W) {
                     const bf16 *e = es + 2 * px * ES + 8 * c;
-                    *(uint4 *)(y2 + (((long)bz * (H / 2) + oy0 / 2) * (W / 2) + ox) * COUT + 8 * c) =
+                    *(uint4 *)(y2 + (h0 + px) * COUT + 8 * c) =
                         sum4(*(const uint4 *)e, *(const uint4 *)(e + ES), *(const uint4 *)(e + 16 * ES),
                              *(const uint4 *)(e + 17 * ES), 0.25f);
                 }
@@ -655,29 +679,56 @@ k_conv_dw(int B, int H, int W, int tiles_per_chunk, const bf16 *__restrict__ x,
     const int grp = blockIdx.x / D::DY, dy0 = D::DY == 3 ? blockIdx.x % 3 : 0;
     const int mt = grp / D::NP, np = grp % D::NP;
     const bool bias = np == 0 && (D::DY == 1 || dy0 == 0);
-    auto issue = [&](int tl, int st) {
-        if (tl < t1) {
-            const int bz = tl / (tw * th), rem = tl - bz * tw * th;
-            const int ty0 = (rem / tw) * CH, tx0 = (rem - (rem / tw) * tw) * CW;
-            bf16 *xs = xs0 + st * XP * XS, *gs = gs0 + st * GP * XS;
-            for (int k = threadIdx.x; k < (CSX == 2 ? XP : XP * 2); k += T) {
-                const int pix = CSX == 2 ? k : k >> 1, q = CSX == 2 ? 0 : k & 1;
-                const int r = pix / (CW + 2), c = pix - r * (CW + 2);
-                const int yy = ty0 + dy0 + r - 1, xx = tx0 + c - 1;
-                const bool in = yy >= 0 && yy < H && xx >= 0 && xx < W;
-                if (CSX == 2) cp_async4(xs + pix * XS, in ? x + (((long)bz * H + yy) * W + xx) * 2 : x, in);
-                else cp_async16(xs + pix * XS + 8 * q,
-                           in ? in_chunk<CIN, CUP>(x, xu, bz, H, W, yy, xx, 2 * np + q) : x, in);
+    // this thread's chunks of a tile: pixel (tid / 2 + 64 i), half (tid & 1)
+    // of the 16 channels, or pixel tid + 128 i of two stored channels; their
+    // offsets from the tile's corner, formed once
+    constexpr int XN = CSX == 2 ? 1 : 2, GN = CSG == 2 ? 1 : 2;   // chunks a pixel
+    constexpr int XI = (XP * XN + T - 1) / T, GI = (GP * GN) / T;
+    const bool up = CUP > 0 && np < CUP / 16;                     // the CTA's channels come from xu
+    int xo[XI], xrc[XI], go[GI];
+#pragma unroll
+    for (int i = 0; i < XI; i++) {
+        const int pix = (threadIdx.x + T * i) / XN, q = (threadIdx.x + T * i) % XN;
+        const int r = pix / (CW + 2), c = pix - r * (CW + 2);
+        xrc[i] = pix < XP ? r | c << 8 : -1;
+        if (CSX == 2) xo[i] = (r * W + c) * 2;
+        else if (up) xo[i] = (((r - 1) >> 1) * (W / 2) + ((c - 1) >> 1)) * CUP + 16 * np + 8 * q;
+        else xo[i] = (r * W + c) * (CIN - CUP) + 16 * np + 8 * q - CUP;
+    }
+#pragma unroll
+    for (int i = 0; i < GI; i++) {
+        const int pix = (threadIdx.x + T * i) / GN, q = (threadIdx.x + T * i) % GN;
+        go[i] = ((pix / CW) * W + pix % CW) * CSG + (CSG == 2 ? 0 : 16 * mt + 8 * q);
+    }
+    const uint32_t xsa = (uint32_t)__cvta_generic_to_shared(xs0), gsa = (uint32_t)__cvta_generic_to_shared(gs0);
+    TilePos pi(t0, tw, th);
+    const TilePos one(1, tw, th);
+    int ti = t0;
+    auto issue = [&](int st) {
+        if (ti < t1) {
+            const int ty0 = pi.r * CH, tx0 = pi.c * CW, ys = ty0 + dy0 - 1;
+            const bf16 *xt = up ? xu + (((long)pi.b * (H / 2) + ty0 / 2) * (W / 2) + tx0 / 2) * CUP
+                                : x + (((long)pi.b * H + ys) * W + tx0 - 1) * (CSX == 2 ? 2 : CIN - CUP);
+            const bf16 *gt = gy + (((long)pi.b * H + ty0) * W + tx0) * CSG;
+            const uint32_t xd = xsa + st * (XP * XS * 2) + (threadIdx.x / XN * XS + threadIdx.x % XN * 8) * 2;
+            const uint32_t gd = gsa + st * (GP * XS * 2) + (threadIdx.x / GN * XS + threadIdx.x % GN * 8) * 2;
+#pragma unroll
+            for (int i = 0; i < XI; i++) {
+                if (XI * T > XP * XN && i == XI - 1 && xrc[i] < 0) break;
+                const bool in = (unsigned)(ys + (xrc[i] & 255)) < (unsigned)H && (unsigned)(tx0 - 1 + (xrc[i] >> 8)) < (unsigned)W;
+                if (CSX == 2) cp_async4(xd + i * (T / XN) * XS * 2, in ? xt + xo[i] : x, in);
+                else cp_async16(xd + i * (T / XN) * XS * 2, in ? xt + xo[i] : x, in);
             }
-            for (int k = threadIdx.x; k < (CSG == 2 ? GP : GP * 2); k += T) {
-                const int pix = CSG == 2 ? k : k >> 1, q = CSG == 2 ? 0 : k & 1;
-                const int yy = ty0 + pix / CW, xx = tx0 + pix % CW;
-                const bool in = yy < H && xx < W;  // beyond the image: no gradient
-                if (CSG == 2) cp_async4(gs + pix * XS, gy + (in ? (((long)bz * H + yy) * W + xx) * 2 : 0), in);
-                else cp_async16(gs + pix * XS + 8 * q,
-                           gy + (in ? (((long)bz * H + yy) * W + xx) * COUT + 16 * mt + 8 * q : 0), in);
+#pragma unroll
+            for (int i = 0; i < GI; i++) {
+                const int pix = (threadIdx.x + T * i) / GN;
+                const bool in = ty0 + pix / CW < H && tx0 + pix % CW < W;  // beyond the image: no gradient
+                if (CSG == 2) cp_async4(gd + i * (T / GN) * XS * 2, in ? gt + go[i] : gy, in);
+                else cp_async16(gd + i * (T / GN) * XS * 2, in ? gt + go[i] : gy, in);
             }
         }
+        ti++;
+        pi.advance(one, tw, th);
         cp_async_commit();  // an empty group past the chunk's end keeps the count
     };
     float acc[TAPS][2][4], accb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -692,12 +743,12 @@ k_conv_dw(int B, int H, int W, int tiles_per_chunk, const bf16 *__restrict__ x,
                          ((shift + (lane & 7) + ((lane >> 3) & 1) * 8) * XS + (lane >> 4) * 8) * 2;
     const uint32_t ga0 = (uint32_t)__cvta_generic_to_shared(gs0) +
                          (((lane & 7) + (lane >> 4) * 8) * XS + ((lane >> 3) & 1) * 8) * 2;
-    for (int k = 0; k < ST - 1; k++) issue(t0 + k, k);
+    for (int k = 0; k < ST - 1; k++) issue(k);
     int st = 0;
     for (int tl = t0; tl < t1; tl++) {
         cp_async_wait<ST - 2>();
         __syncthreads();  // this tile's copies are visible; the slot of the one before is free
-        issue(tl + ST - 1, (st + ST - 1) % ST);
+        issue((st + ST - 1) % ST);
         if (warp < 3) {
             const uint32_t xa = xa0 + st * (XP * XS * 2), ga = ga0 + st * (GP * XS * 2);
 #pragma unroll 4
@@ -1199,7 +1250,7 @@ void conv_launch(int B, int H, int W, const bf16 *x, const bf16 *xu, const bf16 
     constexpr size_t sm = ConvCfg<CIN, COUT>::smem;
     raise_smem_limit((const void *)k_conv_fwd<CIN, COUT, CUP, CST, EPI>, (int)sm);
     const int ntiles = B * (int)cdiv(W, CW) * (int)cdiv(H, CH);
-    const int per_sm = std::max(1, std::min(4, (int)((227 * 1024) / (sm + 1024))));
+    const int per_sm = std::max(1, std::min(5, (int)((227 * 1024) / (sm + 1024))));
     const int grid = std::min(ntiles, sm_count() * per_sm);
     note_launch();
     k_conv_fwd<CIN, COUT, CUP, CST, EPI><<<grid, 128, sm, s>>>(B, H, W, x, xu, ymask, w, bias, relu, y, y2, y32);
