@@ -209,8 +209,9 @@ template <typename T>
 struct LevelT {
     T *e = nullptr, *r = nullptr, *bx = nullptr, *by = nullptr, *invd = nullptr;
     T *e2 = nullptr;  // second iterate buffer: sweeps read one and write the other
-    // FP64 levels only: the pre-scaled stencil of the sweep, 4 weights per
-    // cell (W, E, S, N) = beta_f / diag, and the right-hand side h^2 b / diag
+    // the pre-scaled stencil of the sweep, 4 weights per cell (W, E, S, N) =
+    // beta_f / diag (FP32: the tail's levels only), and, FP64, the right-hand
+    // side h^2 b / diag
     T *w = nullptr, *bt = nullptr;
     // FP32 levels only: the x-face coefficients again, rows at a pitch of
     // (nx + 1) rounded up to 4 values (zero padded), for tensor copies, whose

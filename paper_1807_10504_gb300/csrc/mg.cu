@@ -837,8 +837,13 @@ __device__ __forceinline__ T flux_sum(int nx, int ny, int i, int j, const T *bx,
 // while staging, then the sweeps (halo 4).
 // The FP64 pipe bounds these kernels on this part (its instruction rate, not
 // HBM), so the design counts FP64 instructions: fused sweeps, the residual
-// identity, prolongation in FMAs; tiles of 32 x 16 spread the small levels
-// over more SMs.
+// identity, prolongation in FMAs; tiles of 32 x 16 spread the levels below
+// 2^20 cells over the SMs.  With those a block is few warps and every phase
+// would wait for its weights from L2, so a thread keeps its (at most two)
+// cells' weights and right-hand sides of the next phase in registers, loaded
+// while the current one runs, the first phase's weights before the wait for
+// the previous grid (PF).
+constexpr int kTwoBlocks = 60 * 1024;  // with the static tile, two blocks fill an SM's shared memory
 template <int MODE, int DW, int DH>
 __global__ void __launch_bounds__(256)
 k_smooth2_f64(int nx, int ny, double ih2, const double2 *__restrict__ w,
@@ -854,7 +859,45 @@ k_smooth2_f64(int nx, int ny, double ih2, const double2 *__restrict__ w,
     __shared__ double ps[PH][PW];
     const int gi0 = blockIdx.x * DW - HA, gj0 = blockIdx.y * DH - HA;
     const int nxc = nx / 2, nyc = ny / 2;
+    // ring q = HA - 1 - ph of phase ph: local rows [HA - q, HA + DH + q),
+    // columns [HA - q, HA + DW + q); cell n = threadIdx.x + NT i of its colour:
+    // window row and column, false beyond the ring or the walls
+    auto cell = [&](int ph, int i, int &r, int &c) {
+        const int q = HA - 1 - ph, hw = (DW + 2 * q) / 2, hq = DH + 2 * q, k = threadIdx.x + NT * i;
+        const int rr = k / hw, cc = k - rr * hw;
+        r = HA - q + rr;
+        c = HA - q + 2 * cc + ((gi0 + HA - q + gj0 + r + ph) & 1);
+        const int gi = gi0 + c, gj = gj0 + r;
+        return rr < hq && gi >= 0 && gi < nx && gj >= 0 && gj < ny;
+    };
+    constexpr int NPC = ((DW + 2 * HA - 2) * (DH + 2 * HA - 2) / 2 + NT - 1) / NT;  // cells a thread, first phase
+    constexpr bool PF = NPC <= 2;
+    double2 we_[2][PF ? NPC : 1], sn_[2][PF ? NPC : 1];
+    double bt_[2][PF ? NPC : 1];
+    int at_[2][PF ? NPC : 1];  // r * PW + c, or -1
+    auto fetch_w = [&](int ph) {
+#pragma unroll
+        for (int i = 0; i < (PF ? NPC : 0); i++) {
+            int r, c;
+            const bool in = cell(ph, i, r, c);
+            at_[ph & 1][i] = in ? r * PW + c : -1;
+            if (in) {
+                const long kc = (long)(gj0 + r) * nx + gi0 + c;
+                we_[ph & 1][i] = w[2 * kc];
+                sn_[ph & 1][i] = w[2 * kc + 1];
+            }
+        }
+    };
+    auto fetch_b = [&](int ph) {
+#pragma unroll
+        for (int i = 0; i < (PF ? NPC : 0); i++) {
+            const int o = at_[ph & 1][i], r = o / PW, c = o - r * PW;
+            if (o >= 0) bt_[ph & 1][i] = bt[(long)(gj0 + r) * nx + gi0 + c];
+        }
+    };
+    if (PF) fetch_w(0);
     pdl_enter();
+    if (PF) fetch_b(0);
     for (int k = threadIdx.x; k < PH * PW; k += NT) {
         const int r = k / PW, c = k - r * PW, gi = gi0 + c, gj = gj0 + r;
         double v = 0.0;
@@ -873,30 +916,36 @@ k_smooth2_f64(int nx, int ny, double ih2, const double2 *__restrict__ w,
         ps[r][c] = v;
     }
     __syncthreads();
-    // ring q: local rows [HA - q, HA + DH + q), columns [HA - q, HA + DW + q)
+    auto relax = [&](int ph, int r, int c, double2 we, double2 sn, double b) {
+        double sm = fma(we.x, ps[r][c - 1], -b);
+        sm = fma(we.y, ps[r][c + 1], sm);
+        sm = fma(sn.x, ps[r - 1][c], sm);
+        sm = fma(sn.y, ps[r + 1][c], sm);
+        if (MODE == 1 && ph == 3) {
+            // last black half-sweep: tile cells go out now, every black
+            // cell of the ring keeps its change for the residual
+            if (r >= HA && r < HA + DH && c >= HA && c < HA + DW) p[(long)(gj0 + r) * nx + gi0 + c] = sm;
+            ps[r][c] = sm - ps[r][c];
+        } else {
+            ps[r][c] = sm;
+        }
+    };
 #pragma unroll
     for (int ph = 0; ph < 4; ph++) {
-        const int q = HA - 1 - ph, color = ph & 1;
-        const int wq = DW + 2 * q, hq = DH + 2 * q, hw = wq / 2;
-        for (int k = threadIdx.x; k < hq * hw; k += NT) {
-            const int rr = k / hw, cc = k - rr * hw;
-            const int r = HA - q + rr, gj = gj0 + r;
-            const int c = HA - q + 2 * cc + ((gi0 + HA - q + gj + color) & 1);
-            const int gi = gi0 + c;
-            if (gi < 0 || gi >= nx || gj < 0 || gj >= ny) continue;
-            const long kc = (long)gj * nx + gi;
-            const double2 we = w[2 * kc], sn = w[2 * kc + 1];
-            double sm = fma(we.x, ps[r][c - 1], -bt[kc]);
-            sm = fma(we.y, ps[r][c + 1], sm);
-            sm = fma(sn.x, ps[r - 1][c], sm);
-            sm = fma(sn.y, ps[r + 1][c], sm);
-            if (MODE == 1 && ph == 3) {
-                // last black half-sweep: tile cells go out now, every black
-                // cell of the ring keeps its change for the residual
-                if (r >= HA && r < HA + DH && c >= HA && c < HA + DW) p[kc] = sm;
-                ps[r][c] = sm - ps[r][c];
-            } else {
-                ps[r][c] = sm;
+        if constexpr (PF) {
+            if (ph < 3) { fetch_w(ph + 1); fetch_b(ph + 1); }
+#pragma unroll
+            for (int i = 0; i < NPC; i++) {
+                const int o = at_[ph & 1][i], r = o / PW, c = o - r * PW;
+                if (o >= 0) relax(ph, r, c, we_[ph & 1][i], sn_[ph & 1][i], bt_[ph & 1][i]);
+            }
+        } else {
+            const int q = HA - 1 - ph, n = (DW + 2 * q) / 2 * (DH + 2 * q);
+            for (int i = 0; threadIdx.x + NT * i < n; i++) {
+                int r, c;
+                if (!cell(ph, i, r, c)) continue;
+                const long kc = (long)(gj0 + r) * nx + gi0 + c;
+                relax(ph, r, c, w[2 * kc], w[2 * kc + 1], bt[kc]);
             }
         }
         __syncthreads();
@@ -1030,7 +1079,7 @@ __device__ __forceinline__ void level_coeffs_cell(int nx, int ny, int level0, in
                                                   float *__restrict__ bxf, float *__restrict__ byf,
                                                   float *__restrict__ bxp,
                                                   double *__restrict__ invd, float *__restrict__ invdf,
-                                                  double *__restrict__ w4)
+                                                  double *__restrict__ w4, float4 *__restrict__ w4f)
 {
     const int fnx = 2 * nx;  // finer level width (unused at level 0)
     auto xface = [&](int I, int J) -> double {   // coefficient of x-face (I, J)
@@ -1062,9 +1111,13 @@ __device__ __forceinline__ void level_coeffs_cell(int nx, int ny, int level0, in
     const double id = d > 0.0 ? recip_nr(d) : 0.0;
     invd[kc] = id;
     invdf[kc] = d2f_rn(id);
-    if (w4) {
-        reinterpret_cast<double2 *>(w4)[2 * kc] = make_double2(w * id, e * id);
-        reinterpret_cast<double2 *>(w4)[2 * kc + 1] = make_double2(s * id, n * id);
+    if (w4 || w4f) {
+        const double ww = w * id, we = e * id, ws = s * id, wn = n * id;
+        if (w4) {
+            reinterpret_cast<double2 *>(w4)[2 * kc] = make_double2(ww, we);
+            reinterpret_cast<double2 *>(w4)[2 * kc + 1] = make_double2(ws, wn);
+        }
+        if (w4f) w4f[kc] = make_float4(d2f_rn(ww), d2f_rn(we), d2f_rn(ws), d2f_rn(wn));
     }
 }
 
@@ -1100,11 +1153,11 @@ __global__ void k_level_coeffs(int nx, int ny, int level0, const double *__restr
                                double *__restrict__ by, float *__restrict__ bxf,
                                float *__restrict__ byf, float *__restrict__ bxp,
                                double *__restrict__ invd, float *__restrict__ invdf,
-                               double *__restrict__ w4)
+                               double *__restrict__ w4, float4 *__restrict__ w4f)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
     if (i >= nx) return;
-    level_coeffs_cell(nx, ny, level0, i, j, fbx, fby, bx, by, bxf, byf, bxp, invd, invdf, w4);
+    level_coeffs_cell(nx, ny, level0, i, j, fbx, fby, bx, by, bxf, byf, bxp, invd, invdf, w4, w4f);
 }
 
 // The small levels (from `first` on) in one CTA, level after level; a level
@@ -1114,7 +1167,7 @@ struct LevelCoeffArgs {
     int first, nl;
     int nx[16], ny[16];
     double *bx[16], *by[16], *invd[16], *w4[16];
-    float *bxf[16], *byf[16], *bxp[16], *invdf[16];
+    float *bxf[16], *byf[16], *bxp[16], *invdf[16], *wf[16];
 };
 
 __global__ void __launch_bounds__(1024) k_level_coeffs_small(LevelCoeffArgs a)
@@ -1124,7 +1177,7 @@ __global__ void __launch_bounds__(1024) k_level_coeffs_small(LevelCoeffArgs a)
         for (int k = threadIdx.x; k < nx * ny; k += blockDim.x) {
             const int j = k / nx, i = k - j * nx;
             level_coeffs_cell(nx, ny, l == 0, i, j, a.bx[l - 1], a.by[l - 1], a.bx[l], a.by[l], a.bxf[l],
-                              a.byf[l], a.bxp[l], a.invd[l], a.invdf[l], a.w4[l]);
+                              a.byf[l], a.bxp[l], a.invd[l], a.invdf[l], a.w4[l], (float4 *)a.wf[l]);
         }
         __syncthreads();
     }
@@ -1779,72 +1832,105 @@ __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<
     }
 }
 
-// The lower part of an FP64 V(2,2) cycle in one CTA, on the pre-scaled
-// stencil and with the residual identity of k_smooth2_f64: what bounds it is
-// FP64 instructions, each of which occupies its sub-partition's FP64 unit for
-// 64 cycles whatever its active lanes.  So a cell's update is four FMAs (six
-// operations in k_tail), one cell a thread spreads a small level over the
-// four sub-partitions (k_tail's pairs double a warp's chain), a restriction
-// takes eight FMAs a coarse cell (40 as b - A p), the level's correction
-// starts at zero so that its first red half sweep is e = -bt, written with bt
-// by the restriction before, and the weights, h^2 / diag and diag / (4 h^2)
-// are staged before the wait for the previous grid.  Used where the levels
-// below run V(2,2) and there is a level above the coarsest; 31 us a cycle
-// with k_tail<double> from 32^2 down, now 18 us.
+// The lower part of a V(2,2) cycle in one CTA, on the pre-scaled stencil and
+// with the residual identity of k_smooth2_f64: a cell's update is four FMAs
+// from one vector of weights, a restriction eight FMAs a coarse cell (40 as
+// b - A p), the level's correction starts at zero so that its first red half
+// sweep is e = -bt, written with bt by the restriction before, and the
+// weights, h^2 / diag and diag / (4 h^2) are staged before the wait for the
+// previous grid.  Used where the cycle is V(2,2) and there is a level above
+// the coarsest.
+// FP64: what bounds it is FP64 instructions, each of which occupies its
+// sub-partition for 64 cycles whatever its active lanes: one cell a thread
+// spreads a small level over the four sub-partitions (k_tail's pairs double a
+// warp's chain).  From 32^2 down 31 us a cycle with k_tail<double>, now 18.
+// FP32: latency (a phase of a small level is one chain of address, loads,
+// FMAs and barrier, 600 cycles in k_tail with its parameter reads in every
+// phase) and issue on the largest level.  From 64^2 down 24.6 us a cycle with
+// k_tail<float>, now 22.5.
 // Shared memory per level of n cells (colour-split as in k_tail, without
-// padding): e, bt, h^2 / diag (n each), the weights (W, E) and (S, N) (2 n
-// pairs), diag / (4 h^2) of the red cells and the last half sweep's changes
-// of the black ones (n / 2 each): 8 n doubles; the coarsest level x and r.
+// padding): e, bt, h^2 / diag (n each), the weights (W, E, S, N; 4 n), diag /
+// (4 h^2) of the red cells and the last half sweep's changes of the black
+// ones (n / 2 each): 8 n values; the coarsest level x and r.
+template <typename T>
 struct TailWArgs {
     int lt, nl, zero;        // zero: the level-lt iterate is zero on entry
     int nx[kMaxLv], ny[kMaxLv], off[kMaxLv], inv_off;
-    double h2[kMaxLv], ih2[kMaxLv];
-    const double *w[kMaxLv], *invd[kMaxLv];
-    double *e;               // level lt: iterate (out; in unless zero)
-    const double *bt;        // level lt: h^2 b / diag
+    T h2[kMaxLv], ih2[kMaxLv];
+    const T *w[kMaxLv], *invd[kMaxLv];
+    T *e;                    // level lt: iterate (out; in unless zero)
+    const T *b;              // level lt: h^2 b / diag (FP64), b (FP32)
     const double *ainvT;
 };
 __host__ __device__ inline size_t tailw_elems(int nx, int ny, bool coarsest)
 {
     const size_t n = (size_t)nx * ny;
-    return coarsest ? (2 * n + 1) & ~(size_t)1 : 8 * n;
+    return coarsest ? (2 * n + 3) & ~(size_t)3 : 8 * n;
 }
-inline size_t tailw_prepare(TailWArgs &a)
+template <typename T>
+size_t tailw_bytes(const MG &mg, int lt)
 {
     size_t n = 0;
-    for (int l = a.lt; l < a.nl; l++) {
-        a.off[l] = (int)n;
-        n += tailw_elems(a.nx[l], a.ny[l], l == a.nl - 1);
-    }
-    const size_t inv = tail_inv_bytes(a.nx[a.nl - 1] * a.ny[a.nl - 1]);
-    a.inv_off = inv ? (int)n : -1;
-    return n * 8 + inv;
+    for (int l = lt; l < mg.L; l++) n += tailw_elems(mg.lv[l].nx, mg.lv[l].ny, l == mg.L - 1);
+    return n * sizeof(T) + tail_inv_bytes(mg.lv[mg.L - 1].nx * mg.lv[mg.L - 1].ny);
 }
 
-template <bool BIG>
-__global__ void __launch_bounds__(1024) k_tail_f64(const __grid_constant__ TailWArgs g)
+// Four weights of a cell as one (FP32) or two (FP64) shared-memory vectors.
+template <typename T> struct Weights;
+template <> struct Weights<float> {
+    static __device__ __forceinline__ void stage(float *d, int n, int k, const float *src)
+    {
+        (void)n;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(d + 4 * k)), "l"(src));
+    }
+    static __device__ __forceinline__ float4 load(const float *d, int n, int k)
+    {
+        (void)n;
+        return *reinterpret_cast<const float4 *>(d + 4 * k);
+    }
+};
+struct D4 { double x, y, z, w; };
+template <> struct Weights<double> {
+    static __device__ __forceinline__ void stage(double *d, int n, int k, const double *src)
+    {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(d + 2 * k)), "l"(src));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(d + 2 * (n + k))), "l"(src + 2));
+    }
+    static __device__ __forceinline__ D4 load(const double *d, int n, int k)
+    {
+        const double2 a = *reinterpret_cast<const double2 *>(d + 2 * k);
+        const double2 b = *reinterpret_cast<const double2 *>(d + 2 * (n + k));
+        return {a.x, a.y, b.x, b.y};
+    }
+};
+__device__ __forceinline__ double recip_of(double x) { return recip_any(x); }
+__device__ __forceinline__ float recip_of(float x) { return x != 0.0f ? __frcp_rn(x) : 0.0f; }
+
+template <typename T, bool BIG>
+__global__ void __launch_bounds__(1024) k_tail_w(const __grid_constant__ TailWArgs<T> g)
 {
-    extern __shared__ __align__(16) double tw_sm[];
+    extern __shared__ __align__(16) unsigned char tail_sm[];
     __shared__ double xs[BIG ? kMaxCoarsest : kTailWarpSolve], parts[BIG ? 1024 : 1];
+    T *sm = reinterpret_cast<T *>(tail_sm);
     const int tid = threadIdx.x, lc = g.nl - 1, nco = g.nx[lc] * g.ny[lc];
-    const double *ainv = g.inv_off >= 0 ? tw_sm + g.inv_off : g.ainvT;
-    if (g.inv_off >= 0) stage_array(tw_sm + g.inv_off, g.ainvT, nco * nco, tid, 1024);
+    const double *ainv = g.inv_off >= 0 ? reinterpret_cast<const double *>(tail_sm + g.inv_off) : g.ainvT;
+    if (g.inv_off >= 0)
+        stage_array(reinterpret_cast<double *>(tail_sm + g.inv_off), g.ainvT, nco * nco, tid, 1024);
     // coefficients of all levels (not written during the solve)
 #pragma unroll 1
     for (int l = g.lt; l < lc; l++) {
         const int nx = g.nx[l], n = nx * g.ny[l], hx = nx / 2, nh = n / 2;
-        double *q = tw_sm + g.off[l] + 2 * n;
-        double2 *we = reinterpret_cast<double2 *>(tw_sm + g.off[l] + 3 * n), *sn = we + n;
-        double *dg = tw_sm + g.off[l] + 7 * n;
+        T *q = sm + g.off[l] + 2 * n, *wt = q + n, *dg = wt + 4 * n;
+        const T h2 = g.h2[l], iq = T(0.25) * g.ih2[l];
+        const T *wg = g.w[l], *ig = g.invd[l];
         Walk w(tid, 1024, nx);
-#pragma unroll 1
+#pragma unroll 2
         for (int k = tid; k < n; k += 1024, w.next()) {
             const int c = (w.a + w.b) & 1, slot = w.a * hx + (w.b >> 1), d = c * nh + slot;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(we + d)), "l"(g.w[l] + 4 * k));
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(sn + d)), "l"(g.w[l] + 4 * k + 2));
-            const double id = g.invd[l][k];
-            q[d] = g.h2[l] * id;
-            if (c == 0) dg[slot] = 0.25 * g.ih2[l] * recip_any(id);
+            Weights<T>::stage(wt, n, d, wg + 4 * k);
+            const T id = ig[k];
+            q[d] = h2 * id;
+            if (c == 0) dg[slot] = iq * recip_of(id);
         }
     }
     pdl_enter();
@@ -1852,12 +1938,13 @@ __global__ void __launch_bounds__(1024) k_tail_f64(const __grid_constant__ TailW
         // level lt: right-hand side and (unless zero) iterate; from zero the
         // first red half sweep is e = -bt
         const int l = g.lt, nx = g.nx[l], n = nx * g.ny[l], hx = nx / 2, nh = n / 2;
-        double *e = tw_sm + g.off[l], *bt = e + n;
+        T *e = sm + g.off[l], *bt = e + n;
+        const T *q = bt + n;  // this thread's own entries
         Walk w(tid, 1024, nx);
-#pragma unroll 1
+#pragma unroll 4
         for (int k = tid; k < n; k += 1024, w.next()) {
             const int c = (w.a + w.b) & 1, d = c * nh + w.a * hx + (w.b >> 1);
-            const double b = g.bt[k];
+            const T b = sizeof(T) == 8 ? g.b[k] : g.b[k] * q[d];
             bt[d] = b;
             if (!g.zero) e[d] = g.e[k];
             else if (c == 0) e[d] = -b;
@@ -1870,7 +1957,7 @@ __global__ void __launch_bounds__(1024) k_tail_f64(const __grid_constant__ TailW
 #pragma unroll 1
     for (int v = 0; v <= 2 * nlv; v++) {
         if (v == nlv) {
-            coarse_solve<double, BIG>(tw_sm + g.off[lc], nco, ainv, xs, parts, tid);
+            coarse_solve<T, BIG>(sm + g.off[lc], nco, ainv, xs, parts, tid);
             continue;
         }
         const bool down = v < nlv;
@@ -1878,13 +1965,12 @@ __global__ void __launch_bounds__(1024) k_tail_f64(const __grid_constant__ TailW
         const int nx = g.nx[l], ny = g.ny[l], n = nx * ny, hx = nx / 2, nh = n / 2;
         const int NT = tail_threads(2 * n);  // a thread per cell of a colour
         if (tid >= NT) { ntp = NT; continue; }
-        double *e = tw_sm + g.off[l], *bt = e + n;
-        const double2 *we = reinterpret_cast<const double2 *>(e + 3 * n), *sn = we + n;
-        const double *dg = e + 7 * n;
-        double *dl = e + 7 * n + nh;
+        T *e = sm + g.off[l], *bt = e + n;
+        const T *wt = e + 3 * n, *dg = e + 7 * n;
+        T *dl = e + 7 * n + nh;
         const bool cnat = l + 1 == lc;
         const int nxc = nx / 2, nc = n / 4, hxc = nxc / 2, nhc = nc / 2;
-        double *ec = tw_sm + g.off[l + 1];
+        T *ec = sm + g.off[l + 1];
         const Walk w0(tid, NT, hx);
         if (!down) {
             if (NT != ntp) gsync(NT);  // the smaller group's work is done
@@ -1900,55 +1986,57 @@ __global__ void __launch_bounds__(1024) k_tail_f64(const __grid_constant__ TailW
                 const int j = w.a, I = w.b, J = j >> 1, nyc = ny / 2;
                 const int I2 = min(max(I + ((j & 1) ? -1 : 1), 0), nxc - 1);  // i = 2 I + (j + 1 & 1)
                 const int J2 = min(max(J + ((j & 1) ? 1 : -1), 0), nyc - 1);
-                e[nh + k] = fma(fma(9.0, at(I, J), fma(3.0, at(I2, J) + at(I, J2), at(I2, J2))), 0.0625, e[nh + k]);
+                e[nh + k] = fma(fma(T(9), at(I, J), fma(T(3), at(I2, J) + at(I, J2), at(I2, J2))), T(0.0625), e[nh + k]);
             }
             gsync(NT);
         }
 #pragma unroll 1
         for (int ph = down && (v > 0 || g.zero) ? 1 : 0; ph < 4; ph++) {
             const int c = ph & 1;
-            const double *eo = e + (1 - c) * nh;
+            const T *eo = e + (1 - c) * nh;
+            T *em = e + c * nh;
             Walk w = w0;
 #pragma unroll 1
             for (int k = tid; k < nh; k += NT, w.next()) {
                 const int j = w.a, m = w.b, o = (j + c) & 1;
                 // a wall's weight is zero: any cell stands for the one beyond
-                const double eW = eo[m + o > 0 ? k - 1 + o : k], eE = eo[m + o < hx ? k + o : k];
-                const double eS = eo[j > 0 ? k - hx : k], eN = eo[j + 1 < ny ? k + hx : k];
-                const int d = c * nh + k;
-                const double2 a = we[d], b = sn[d];
-                double s = fma(a.x, eW, -bt[d]);
+                const T eW = eo[m + o > 0 ? k - 1 + o : k], eE = eo[m + o < hx ? k + o : k];
+                const T eS = eo[j > 0 ? k - hx : k], eN = eo[j + 1 < ny ? k + hx : k];
+                const auto a = Weights<T>::load(wt, n, c * nh + k);
+                T s = fma(a.x, eW, -bt[c * nh + k]);
                 s = fma(a.y, eE, s);
-                s = fma(b.x, eS, s);
-                s = fma(b.y, eN, s);
-                if (down && ph == 3) dl[k] = s - e[d];
-                e[d] = s;
+                s = fma(a.z, eS, s);
+                s = fma(a.w, eN, s);
+                if (down && ph == 3) dl[k] = s - em[k];
+                em[k] = s;
             }
             gsync(NT);
         }
         if (!down) continue;
         // the residual identity: a red cell's residual is -(diag / h^2) sum_f
         // w_f delta_f, a black one's zero
-        const double *qc = ec + 2 * nc;
+        const T *qc = ec + 2 * nc;
         Walk w(tid, NT, nxc);
 #pragma unroll 1
         for (int k = tid; k < nc; k += NT, w.next()) {
             const int I = w.b, J = w.a, k0 = 2 * J * hx + I, k1 = k0 + hx;
-            const double2 a0 = we[k0], b0 = sn[k0], a1 = we[k1], b1 = sn[k1];
-            double s0 = a0.x * dl[I > 0 ? k0 - 1 : k0];
-            s0 = fma(a0.y, dl[k0], s0);
-            s0 = fma(b0.x, dl[J > 0 ? k0 - hx : k0], s0);
-            s0 = fma(b0.y, dl[k1], s0);
-            double s1 = a1.x * dl[k1];
+            const auto a0 = Weights<T>::load(wt, n, k0);
+            const auto a1 = Weights<T>::load(wt, n, k1);
+            const T d0 = dl[k0], d1 = dl[k1];
+            T s0 = a0.x * dl[I > 0 ? k0 - 1 : k0];
+            s0 = fma(a0.y, d0, s0);
+            s0 = fma(a0.z, dl[J > 0 ? k0 - hx : k0], s0);
+            s0 = fma(a0.w, d1, s0);
+            T s1 = a1.x * d1;
             s1 = fma(a1.y, dl[I + 1 < hx ? k1 + 1 : k1], s1);
-            s1 = fma(b1.x, dl[k0], s1);
-            s1 = fma(b1.y, dl[2 * J + 2 < ny ? k1 + hx : k1], s1);
-            const double rv = -fma(dg[k0], s0, dg[k1] * s1);
+            s1 = fma(a1.z, d0, s1);
+            s1 = fma(a1.w, dl[2 * J + 2 < ny ? k1 + hx : k1], s1);
+            const T rv = -fma(dg[k0], s0, dg[k1] * s1);
             if (cnat) {
                 ec[nc + k] = rv;
             } else {
                 const int c = (I + J) & 1, d = c * nhc + J * hxc + (I >> 1);
-                const double b = rv * qc[d];
+                const T b = rv * qc[d];
                 ec[nc + d] = b;
                 if (c == 0) ec[d] = -b;
             }
@@ -1958,9 +2046,9 @@ __global__ void __launch_bounds__(1024) k_tail_f64(const __grid_constant__ TailW
     }
     __syncthreads();
     const int nx0 = g.nx[g.lt], n0 = nx0 * g.ny[g.lt], hx0 = nx0 / 2;
-    const double *e = tw_sm + g.off[g.lt];
+    const T *e = sm + g.off[g.lt];
     Walk w(tid, 1024, nx0);
-#pragma unroll 1
+#pragma unroll 2
     for (int k = tid; k < n0; k += 1024, w.next())
         g.e[k] = e[((w.a + w.b) & 1) * (n0 / 2) + w.a * hx0 + (w.b >> 1)];
 }
@@ -2145,8 +2233,14 @@ void launch_smooth2(const Level &v, const LevelT<float> &a, const float *pin, fl
 }
 
 // One fused FP64 smoother launch of MODE on level v (pin -> p): 64 x 32 tiles
-// from 512^2 cells up, 32 x 16 below (more tiles, so more SMs share the FP64
-// work of a small level).
+// from 2^20 cells up, 32 x 16 below, where more tiles share the FP64 work
+// more evenly (512^2 as 128 tiles of 64 x 32, several of them on one SM while
+// others had none: 22 and 44 us in the cycle; as 512 of 32 x 16 and with
+// their weights prefetched SM64_TIMES).  Up to four waves of 64 x 32 tiles
+// leave room (dynamic shared memory) for two blocks an SM only, so that the
+// scheduler hands the rest to the SMs that finish first instead of placing
+// all at once (1024^2: FP64 cycle 246 -> 222 us; 2048^2, with 13 tiles an SM,
+// would lose a tenth).
 template <int MODE>
 void launch_smooth2_f64(const Level &v, const LevelT<double> &a, const double *pin, double *p,
                         double *rc, double *ecz, double h2c, const double *invdc, double *btc,
@@ -2154,9 +2248,10 @@ void launch_smooth2_f64(const Level &v, const LevelT<double> &a, const double *p
 {
     const double ih2 = 1.0 / (v.h * v.h);
     note_launch();
-    if ((long)v.nx * v.ny >= (1L << 18)) {
+    if ((long)v.nx * v.ny >= (1L << 20)) {
         dim3 g(cdiv(v.nx, 64), cdiv(v.ny, 32));
-        launch_pdl(k_smooth2_f64<MODE, 64, 32>, g, 256, 0, s, v.nx, v.ny, ih2, (const double2 *)a.w,
+        const int pad = g.x * g.y <= 4 * 152 ? kTwoBlocks : 0;
+        launch_pdl(k_smooth2_f64<MODE, 64, 32>, g, 256, pad, s, v.nx, v.ny, ih2, (const double2 *)a.w,
                    (const double *)a.bt, (const double *)a.bx, (const double *)a.by, pin, p, rc,
                    ecz, h2c, invdc, btc, ecp);
     } else {
@@ -2203,27 +2298,34 @@ T *smooth(const Level &v, LevelT<T> &a, T *cur, int nsw, bool fine, cudaStream_t
     return cur;
 }
 
-// The FP64 V(2,2) tail from level lt on, its iterate in e (zero: e is zero).
-void launch_tail_f64(MG &mg, double *e, bool zero, cudaStream_t s)
+// The V(2,2) tail from level lt on, its iterate in e (zero: e is zero).
+template <typename T>
+void launch_tail_w(MG &mg, T *e, bool zero, cudaStream_t s)
 {
-    TailWArgs a;
-    const int L = mg.L, lt = mg.tail;
+    TailWArgs<T> a;
+    const int L = mg.L, lt = sizeof(T) == 8 ? mg.tail : mg.tail_f;
+    auto lvT = [&](int l) -> const LevelT<T> & {
+        if constexpr (sizeof(T) == 8) return mg.lv[l].d; else return mg.lv[l].f;
+    };
     a.lt = lt;
     a.nl = L;
     a.zero = zero ? 1 : 0;
+    size_t off = 0;
     for (int l = lt; l < L; l++) {
         const Level &v = mg.lv[l];
         a.nx[l] = v.nx; a.ny[l] = v.ny;
-        a.h2[l] = v.h * v.h; a.ih2[l] = 1.0 / (v.h * v.h);
-        a.w[l] = v.d.w; a.invd[l] = v.d.invd;
+        a.h2[l] = (T)(v.h * v.h); a.ih2[l] = (T)(1.0 / (v.h * v.h));
+        a.w[l] = lvT(l).w; a.invd[l] = lvT(l).invd;
+        a.off[l] = (int)off;
+        off += tailw_elems(v.nx, v.ny, l == L - 1);
     }
     a.e = e;
-    a.bt = mg.lv[lt].d.bt;
+    a.b = sizeof(T) == 8 ? lvT(lt).bt : lvT(lt).r;
     const int nco = mg.lv[L - 1].nx * mg.lv[L - 1].ny;
     a.ainvT = mg.lu + (size_t)nco * nco;
-    const size_t smem = tailw_prepare(a);
+    a.inv_off = tail_inv_bytes(nco) ? (int)(off * sizeof(T)) : -1;
     note_launch();
-    launch_pdl(nco > kTailWarpSolve ? k_tail_f64<true> : k_tail_f64<false>, 1, 1024, smem, s, a);
+    launch_pdl(nco > kTailWarpSolve ? k_tail_w<T, true> : k_tail_w<T, false>, 1, 1024, tailw_bytes<T>(mg, lt), s, a);
 }
 
 // One V(nu1, nu2) cycle on the level-0 data of precision T.  Every level's
@@ -2277,14 +2379,9 @@ bool vcycle(MG &mg, int nu1, int nu2, cudaStream_t s, double *add64 = nullptr)
         }
         cur[l + 1] = c.e;
     }
-    bool tail_done = false;
-    if constexpr (!f32) {
-        if (fused && lt < L - 1) {
-            launch_tail_f64(mg, cur[lt], lt > 0, s);
-            tail_done = true;
-        }
-    }
-    if (!tail_done) {
+    if (fused && lt < L - 1) {
+        launch_tail_w<T>(mg, cur[lt], lt > 0, s);
+    } else {
     TailArgs<T> ta;
     ta.lt = lt;
     ta.nl = L;
@@ -2557,6 +2654,7 @@ size_t mg_layout(MG &mg, int nx, int ny, double h, char *base)
         v.f.r = (float *)take(n * 4); v.f.invd = (float *)take(n * 4);
         v.f.bx = (float *)take(fx * 4); v.f.by = (float *)take(fy * 4);
         v.f.bxp = (float *)take((size_t)xface_pitch(v.nx) * v.ny * 4);
+        v.f.w = n <= (size_t)kTailCellsF32 ? (float *)take(n * 16) : nullptr;
     }
     mg.lu = (double *)take((size_t)nc * nc * 8 * 2);  // A' and its transposed inverse
     mg.piv = (int *)take((size_t)nc * 4);
@@ -2635,26 +2733,10 @@ long mg_bench_op(MG &mg, int op, int level, cudaStream_t s)
         launch_smooth2<2>(v, v.f, v.f.e, v.f.e2, nullptr, nullptr, mg.lv[level + 1].f.e, s,
                           level == 0 ? v.d.e : nullptr);
         return cells;
-    case 5: {
-        const int lt = mg.tail_f, L = mg.L;
-        TailArgs<float> ta;
-        ta.lt = lt;
-        ta.nl = L;
-        for (int l = lt; l < L; l++) {
-            Level &w = mg.lv[l];
-            ta.nx[l] = w.nx; ta.ny[l] = w.ny;
-            ta.h2[l] = (float)(w.h * w.h); ta.ih2[l] = (float)(1.0 / (w.h * w.h));
-            ta.e[l] = w.f.e2; ta.r[l] = w.f.r; ta.bx[l] = w.f.bx; ta.by[l] = w.f.by; ta.invd[l] = w.f.invd;
-        }
-        const long nc = (long)mg.lv[L - 1].nx * mg.lv[L - 1].ny;
-        ta.ainvT = mg.lu + nc * nc;
-        ta.nu1 = 2;
-        ta.nu2 = 2;
-        note_launch();
-        const size_t smem = tail_prepare(ta);
-        launch_pdl(nc > kTailWarpSolve ? k_tail<float, true> : k_tail<float, false>, 1, 1024, smem, s, ta);
-        return (long)mg.lv[lt].nx * mg.lv[lt].ny;
-    }
+    case 5:
+        if (mg.tail_f >= mg.L - 1) return -1;
+        launch_tail_w<float>(mg, mg.lv[mg.tail_f].f.e2, mg.tail_f > 0, s);
+        return (long)mg.lv[mg.tail_f].nx * mg.lv[mg.tail_f].ny;
     case 7:
     case 8: {  // the fused FP64 smoothers (7: sweeps + restriction, 8: prolongation + sweeps)
         if (level >= mg.tail) return -1;
@@ -2712,7 +2794,8 @@ void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool w
         dim3 g(cdiv(v.nx, 128), v.ny);
         note_launch();
         k_level_coeffs<<<g, 128, 0, s>>>(v.nx, v.ny, l == 0, fbx, fby, v.d.bx, v.d.by, v.f.bx, v.f.by,
-                                         v.f.bxp, v.d.invd, v.f.invd, with_w ? v.d.w : nullptr);
+                                         v.f.bxp, v.d.invd, v.f.invd, with_w ? v.d.w : nullptr,
+                                         (float4 *)v.f.w);
     }
     if (lsmall < L) {
         LevelCoeffArgs a;
@@ -2722,7 +2805,7 @@ void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool w
             Level &v = mg.lv[l];
             a.nx[l] = v.nx; a.ny[l] = v.ny;
             a.bx[l] = v.d.bx; a.by[l] = v.d.by; a.invd[l] = v.d.invd; a.w4[l] = with_w ? v.d.w : nullptr;
-            a.bxf[l] = v.f.bx; a.byf[l] = v.f.by; a.bxp[l] = v.f.bxp; a.invdf[l] = v.f.invd;
+            a.bxf[l] = v.f.bx; a.byf[l] = v.f.by; a.bxp[l] = v.f.bxp; a.invdf[l] = v.f.invd; a.wf[l] = v.f.w;
         }
         note_launch();
         k_level_coeffs_small<<<1, 1024, 0, s>>>(a);
@@ -2734,12 +2817,15 @@ void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool w
         for (int l = mg.tail; l < L; l++) e += tail_level_elems(mg.lv[l].nx, mg.lv[l].ny, l == L - 1);
         for (int l = mg.tail_f; l < L; l++) ef += tail_level_elems(mg.lv[l].nx, mg.lv[l].ny, l == L - 1);
         const size_t inv = tail_inv_bytes(mg.lv[L - 1].nx * mg.lv[L - 1].ny);
+        raise_smem_limit((const void *)k_smooth2_f64<1, 64, 32>, kTwoBlocks);
+        raise_smem_limit((const void *)k_smooth2_f64<2, 64, 32>, kTwoBlocks);
         const int sd = (int)(((e * 8 + 7) & ~(size_t)7) + inv), sf = (int)(((ef * 4 + 7) & ~(size_t)7) + inv);
         const bool big = mg.lv[L - 1].nx * mg.lv[L - 1].ny > kTailWarpSolve;
         raise_smem_limit(big ? (const void *)k_tail<double, true> : (const void *)k_tail<double, false>, sd);
-        size_t ew = 0;
-        for (int l = mg.tail; l < L; l++) ew += tailw_elems(mg.lv[l].nx, mg.lv[l].ny, l == L - 1);
-        raise_smem_limit(big ? (const void *)k_tail_f64<true> : (const void *)k_tail_f64<false>, (int)(ew * 8 + inv));
+        raise_smem_limit(big ? (const void *)k_tail_w<double, true> : (const void *)k_tail_w<double, false>,
+                         (int)tailw_bytes<double>(mg, mg.tail));
+        raise_smem_limit(big ? (const void *)k_tail_w<float, true> : (const void *)k_tail_w<float, false>,
+                         (int)tailw_bytes<float>(mg, mg.tail_f));
         raise_smem_limit(big ? (const void *)k_tail<float, true> : (const void *)k_tail<float, false>, sf);
     }
     Level &vc = mg.lv[L - 1];
