@@ -450,21 +450,31 @@ __global__ void k_unit_beta(int nx, int ny, double h, int axisym, double *__rest
 }
 
 // I = clamp(sol - mean over the cells along the walls (the axis column is not
-// a wall), 0, 1); the mean in a fixed order (bottom row, top row, then the
-// right column and, planar, the left column, each in index order) by one
-// thread into *ref, then the shift by a grid of threads.
-__global__ void k_wall_mean(int nx, int ny, int axisym, const double *__restrict__ sol,
-                            double *__restrict__ ref)
+// a wall), 0, 1): the mean by one block into *ref (each thread a strided
+// share of the bottom row, top row, right column and, planar, left column,
+// then a fixed tree; one thread alone took 53 us at 256^2, a chain of 1020
+// additions), then the shift by a grid of threads.
+__global__ void __launch_bounds__(kT)
+k_wall_mean(int nx, int ny, int axisym, const double *__restrict__ sol, double *__restrict__ ref)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    __shared__ double sh[kT / 32];
+    const int side = ny > 2 ? ny - 2 : 0, n = 2 * nx + side * (axisym ? 1 : 2);
     double s = 0.0;
-    long cnt = 0;
-    for (int i = 0; i < nx; i++) { s += sol[i]; cnt++; }
-    for (int i = 0; i < nx; i++) { s += sol[(long)(ny - 1) * nx + i]; cnt++; }
-    for (int j = 1; j < ny - 1; j++) { s += sol[(long)j * nx + nx - 1]; cnt++; }
-    if (!axisym)
-        for (int j = 1; j < ny - 1; j++) { s += sol[(long)j * nx]; cnt++; }
-    *ref = s / (double)cnt;
+    for (int k = threadIdx.x; k < n; k += kT) {
+        long c;
+        if (k < nx) c = k;
+        else if (k < 2 * nx) c = (long)(ny - 1) * nx + k - nx;
+        else if (k < 2 * nx + side) c = (long)(k - 2 * nx + 1) * nx + nx - 1;
+        else c = (long)(k - 2 * nx - side + 1) * nx;
+        s += sol[c];
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int w = 1; w < kT / 32; w++) s += sh[w];
+    *ref = s / (double)n;
 }
 
 __global__ void k_shift_clip(long n, const double *__restrict__ sol, const double *__restrict__ ref,
@@ -556,7 +566,7 @@ void launch_indicator_finish(int nx, int ny, int axisym, const double *sol, doub
                              cudaStream_t s)
 {
     note_launch();
-    k_wall_mean<<<1, 32, 0, s>>>(nx, ny, axisym, sol, ref);
+    k_wall_mean<<<1, kT, 0, s>>>(nx, ny, axisym, sol, ref);
     const long n = (long)nx * ny;
     note_launch();
     k_shift_clip<<<cdiv(n, kT), kT, 0, s>>>(n, sol, ref, I);

@@ -1170,7 +1170,7 @@ struct LevelCoeffArgs {
     float *bxf[16], *byf[16], *bxp[16], *invdf[16], *wf[16];
 };
 
-__global__ void __launch_bounds__(1024) k_level_coeffs_small(LevelCoeffArgs a)
+__global__ void __launch_bounds__(256) k_level_coeffs_small(LevelCoeffArgs a)
 {
     for (int l = a.first; l < a.nl; l++) {
         const int nx = a.nx[l], ny = a.ny[l];
@@ -1192,57 +1192,72 @@ __global__ void __launch_bounds__(1024) k_level_coeffs_small(LevelCoeffArgs a)
 // row c is scaled by 1 / A'_cc and eliminated from every other row, the
 // eliminated column becoming the inverse's (n^3 multiply-adds, all on one
 // SM's FP64 pipe: the size of the coarsest level decides its cost).  One
-// CTA, A' in shared memory: for at most kCoarseOneCta cells.
+// CTA, for at most kCoarseOneCta cells; A' lies in two shared-memory buffers,
+// a column step reading one and writing the other behind one barrier, and the
+// thread that forms the next pivot also forms its reciprocal (recip_any: a
+// division is a chain of ~1.5 k cycles on this part).  With four barriers and
+// a division a column 16 cells took 15.7 us, now CI_TIMES.
 constexpr int kCoarseOneCta = 64;  // larger coarsest levels: k_coarse_step
+
+// Entry (r, c) of A on a grid of nx x ny cells, and its diagonal (r, r).
+__device__ __forceinline__ double coarse_diag(int nx, int ny, double ihh, const double *bx, const double *by, int q)
+{
+    const int i = q % nx, j = q / nx;
+    const long kx = (long)j * (nx + 1) + i;
+    double d = 0.0;
+    if (i + 1 < nx) d -= bx[kx + 1];
+    if (i > 0) d -= bx[kx];
+    if (j + 1 < ny) d -= by[q + nx];
+    if (j > 0) d -= by[q];
+    return d * ihh;
+}
+__device__ __forceinline__ double coarse_entry(int nx, int ny, double ihh, const double *bx, const double *by,
+                                               int r, int c)
+{
+    const int i = r % nx, j = r / nx;
+    const long kx = (long)j * (nx + 1) + i;
+    if (c == r) return coarse_diag(nx, ny, ihh, bx, by, r);
+    if (c == r + 1 && i + 1 < nx) return bx[kx + 1] * ihh;
+    if (c == r - 1 && i > 0) return bx[kx] * ihh;
+    if (c == r + nx) return by[r + nx] * ihh;  // j + 1 < ny, since c < n
+    if (c == r - nx) return by[r] * ihh;       // j > 0, since c >= 0
+    return 0.0;
+}
+
 __global__ void __launch_bounds__(1024)
-k_coarse_inv(int nx, int ny, double h, const double *__restrict__ bx,
+k_coarse_inv(int nx, int ny, double ihh, const double *__restrict__ bx,
              const double *__restrict__ by, double *__restrict__ AinvT)
 {
     extern __shared__ __align__(16) double cinv_sm[];
-    __shared__ double colc[kCoarseOneCta];
-    __shared__ double invp;
-    const int n = nx * ny;
-    const double hh = h * h;
-    double *A = cinv_sm;
-    for (int k = threadIdx.x; k < n * n; k += blockDim.x) A[k] = 0.0;
+    __shared__ double s0, ip_s[2];
+    const int n = nx * ny, nn = n * n, T = blockDim.x;
+    if (threadIdx.x == 0) s0 = coarse_diag(nx, ny, ihh, bx, by, 0);
     __syncthreads();
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        int i = c % nx, j = c / nx;
-        long kx = (long)j * (nx + 1) + i, kc = c;
-        double d = 0.0;
-        if (i + 1 < nx) { d += bx[kx + 1] * (0.0 - 1.0); A[(c + 1) * n + c] = bx[kx + 1] * (1.0 - 0.0) / hh; }
-        if (i > 0) { d -= bx[kx] * (1.0 - 0.0); A[(c - 1) * n + c] = -bx[kx] * (0.0 - 1.0) / hh; }
-        if (j + 1 < ny) { d += by[kc + nx] * (0.0 - 1.0); A[(c + nx) * n + c] = by[kc + nx] * (1.0 - 0.0) / hh; }
-        if (j > 0) { d -= by[kc] * (1.0 - 0.0); A[(c - nx) * n + c] = -by[kc] * (0.0 - 1.0) / hh; }
-        A[c * n + c] = d / hh;
+    for (int k = threadIdx.x; k < nn; k += T) {
+        const int r = k / n;
+        const double v = coarse_entry(nx, ny, ihh, bx, by, r, k - r * n) + s0;
+        cinv_sm[k] = v;
+        if (k == 0) ip_s[0] = recip_any(v);
     }
-    __syncthreads();
-    __shared__ double s0;
-    if (threadIdx.x == 0) s0 = A[0];
-    __syncthreads();
-    for (int k = threadIdx.x; k < n * n; k += blockDim.x) A[k] += s0;
-    __syncthreads();
     for (int c = 0; c < n; c++) {
-        if (threadIdx.x == 0) invp = 1.0 / A[c * n + c];
         __syncthreads();
-        const double ip = invp;
-        for (int r = threadIdx.x; r < n; r += blockDim.x) colc[r] = A[r * n + c];
-        __syncthreads();
-        // row c scaled (its pivot entry becomes 1 / pivot)
-        for (int k = threadIdx.x; k < n; k += blockDim.x) A[c * n + k] = (k == c) ? ip : A[c * n + k] * ip;
-        __syncthreads();
-        // every other row: subtract its column-c multiple of row c; the
-        // eliminated entry becomes -A'_rc / pivot
-        for (int k = threadIdx.x; k < n * n; k += blockDim.x) {
+        const double *src = cinv_sm + (c & 1) * nn;
+        double *dst = cinv_sm + ((c + 1) & 1) * nn;
+        const double ip = ip_s[c & 1];
+        // row c scaled (its pivot entry becomes 1 / pivot); every other row
+        // minus its column-c multiple of that, its column-c entry -A'_rc / pivot
+        for (int k = threadIdx.x; k < nn; k += T) {
             const int r = k / n, q = k - r * n;
-            if (r == c) continue;
-            A[k] = (q == c) ? -colc[r] * ip : A[k] - colc[r] * A[c * n + q];
+            const double f = src[r * n + c], dp = (q == c ? 1.0 : src[c * n + q]) * ip;
+            const double v = r == c ? dp : fma(-f, dp, q == c ? 0.0 : src[k]);
+            dst[k] = v;
+            if (k == (c + 1) * (n + 1)) ip_s[(c + 1) & 1] = recip_any(v);
         }
-        __syncthreads();
     }
-    for (int k = threadIdx.x; k < n * n; k += blockDim.x) {
+    __syncthreads();
+    for (int k = threadIdx.x; k < nn; k += T) {
         const int r = k / n, q = k - r * n;
-        AinvT[q * n + r] = A[k];
+        AinvT[q * n + r] = cinv_sm[(n & 1) * nn + k];
     }
 }
 
@@ -1263,26 +1278,7 @@ k_coarse_mat(int nx, int ny, double ihh, const double *__restrict__ bx,
     const int n = nx * ny, k = blockIdx.x * 256 + threadIdx.x;
     if (k >= n * n) return;
     const int r = k / n, c = k - r * n;
-    // row r of the 5-point operator: faces of cell r
-    auto diag = [&](int q) {
-        const int i = q % nx, j = q / nx;
-        const long kx = (long)j * (nx + 1) + i;
-        double d = 0.0;
-        if (i + 1 < nx) d -= bx[kx + 1];
-        if (i > 0) d -= bx[kx];
-        if (j + 1 < ny) d -= by[q + nx];
-        if (j > 0) d -= by[q];
-        return d * ihh;
-    };
-    const int i = r % nx, j = r / nx;
-    const long kx = (long)j * (nx + 1) + i;
-    double v = 0.0;
-    if (c == r) v = diag(r);
-    else if (c == r + 1 && i + 1 < nx) v = bx[kx + 1] * ihh;
-    else if (c == r - 1 && i > 0) v = bx[kx] * ihh;
-    else if (c == r + nx) v = by[r + nx] * ihh;  // j + 1 < ny, since c < n
-    else if (c == r - nx) v = by[r] * ihh;       // j > 0, since c >= 0
-    A[k] = v + diag(0);
+    A[k] = coarse_entry(nx, ny, ihh, bx, by, r, c) + coarse_diag(nx, ny, ihh, bx, by, 0);
 }
 
 __global__ void __launch_bounds__(kCB * kCB)
@@ -2236,7 +2232,7 @@ void launch_smooth2(const Level &v, const LevelT<float> &a, const float *pin, fl
 // from 2^20 cells up, 32 x 16 below, where more tiles share the FP64 work
 // more evenly (512^2 as 128 tiles of 64 x 32, several of them on one SM while
 // others had none: 22 and 44 us in the cycle; as 512 of 32 x 16 and with
-// their weights prefetched SM64_TIMES).  Up to four waves of 64 x 32 tiles
+// their weights prefetched a 512^2 V-cycle went from 139 to 105 us).  Up to four waves of 64 x 32 tiles
 // leave room (dynamic shared memory) for two blocks an SM only, so that the
 // scheduler hands the rest to the SMs that finish first instead of placing
 // all at once (1024^2: FP64 cycle 246 -> 222 us; 2048^2, with 13 tiles an SM,
@@ -2784,10 +2780,11 @@ void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool w
 {
     const int L = mg.L;
     mg.fp64_w = with_w;
-    // levels above 1024 cells one launch each (their FP64 work spread over
-    // the SMs), the rest in one CTA
+    // levels above 256 cells one launch each (their FP64 work spread over the
+    // SMs: 1024 cells in one CTA take 8 of its 15 us, as a launch 3), the rest
+    // in one CTA
     int lsmall = 1;
-    while (lsmall < L && (long)mg.lv[lsmall].nx * mg.lv[lsmall].ny > 1024) lsmall++;
+    while (lsmall < L && (long)mg.lv[lsmall].nx * mg.lv[lsmall].ny > 256) lsmall++;
     for (int l = 0; l < lsmall; l++) {
         Level &v = mg.lv[l];
         const double *fbx = l == 0 ? bx : mg.lv[l - 1].d.bx, *fby = l == 0 ? by : mg.lv[l - 1].d.by;
@@ -2808,7 +2805,7 @@ void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool w
             a.bxf[l] = v.f.bx; a.byf[l] = v.f.by; a.bxp[l] = v.f.bxp; a.invdf[l] = v.f.invd; a.wf[l] = v.f.w;
         }
         note_launch();
-        k_level_coeffs_small<<<1, 1024, 0, s>>>(a);
+        k_level_coeffs_small<<<1, 256, 0, s>>>(a);
     }
     {
         // shared memory of the single-CTA tail (set here, outside any capture)
@@ -2846,9 +2843,10 @@ void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool w
         return;
     }
     note_launch();
-    const size_t cbytes = nc2 * sizeof(double);
+    const size_t cbytes = 2 * nc2 * sizeof(double);
     raise_smem_limit((const void *)k_coarse_inv, (int)cbytes);
-    k_coarse_inv<<<1, 1024, cbytes, s>>>(vc.nx, vc.ny, vc.h, vc.d.bx, vc.d.by, mg.lu + nc2);
+    const int threads = std::min(1024, (int)cdiv((long)nc2, 32) * 32);
+    k_coarse_inv<<<1, threads, cbytes, s>>>(vc.nx, vc.ny, 1.0 / (vc.h * vc.h), vc.d.bx, vc.d.by, mg.lu + nc2);
 }
 
 // Host-driven solve: one launch per kernel and a host read of the residual
