@@ -11,8 +11,13 @@
 
 namespace ibk {
 
-constexpr int kTailCells = 1024;     // levels with at most this many cells run in one CTA (FP64)
-constexpr int kTailCellsF32 = 4096;  // the same for the FP32 cycle (its levels fit shared memory)
+// Levels with at most this many cells run in one CTA, in the FP64 and in the
+// FP32 cycle.  FP64 with 256: 40.1 -> 43.1 us a cycle at 64^2, 63.5 -> 69.0 at
+// 256 x 192.  FP32: with 4096 a cycle took 78.9 us at 1024^2, 52.7 at 512^2,
+// 25.9 at 64^2 (a level of 64^2 costs one CTA 11 us, its two launches 7.5),
+// with 1024 it takes 76.4, 49.9 and 22.9, with 256 78.7, 52.6 and 24.5.
+constexpr int kTailCells = 1024;
+constexpr int kTailCellsF32 = 1024;
 constexpr int kMaxCoarsest = 1024;   // dense LU limit of the coarsest level
 constexpr int kBlk = 8;              // marker-activity block edge (cells)
 constexpr int kSearch = 7;           // marker search radius (cells) around a cell or face

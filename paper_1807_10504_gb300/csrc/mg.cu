@@ -21,9 +21,9 @@
 //  * kernels of the cycle use programmatic dependent launch: the next grid is
 //    scheduled while the previous one drains and waits (griddepcontrol) for
 //    its results.
-//  * levels with <= 1024 cells (FP64) / <= 4096 cells (FP32) run as one
-//    single-CTA kernel (the whole lower V-cycle and the coarsest solve) with
-//    its data in shared memory, since launches dominate there.
+//  * levels with <= 1024 cells run as one single-CTA kernel (the whole lower
+//    V-cycle and the coarsest solve) with its data in shared memory, since
+//    launches dominate there.
 //  * norms are deterministic two-stage reductions (fixed per-thread order,
 //    fixed tree, last-block fold) with no floating-point atomics.
 //  * the FP32 instantiations of the same kernels form the inner cycle of the
