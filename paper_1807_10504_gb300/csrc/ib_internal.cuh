@@ -348,7 +348,7 @@ struct Markers {
     double h = 0, x0 = 0, y0 = 0;
     double *X = nullptr, *Y = nullptr, *kappa = nullptr, *nxm = nullptr,
            *nym = nullptr, *ds = nullptr, *fmag = nullptr, *U = nullptr,
-           *V = nullptr, *Xn = nullptr, *Yn = nullptr;
+           *V = nullptr;
     double *gx = nullptr, *gy = nullptr;   // marker positions in grid units
     float *gxf = nullptr, *gyf = nullptr;  // the same rounded to FP32 (screening only)
     float4 *sbox = nullptr;                // slab box of segment (m, next m), grid units

@@ -1256,46 +1256,21 @@ k_spread_irrot(int nx, int ny, double ih, int bnx, const uint32_t *__restrict__ 
 
 // ------------------------------------------------------------ B-spline
 // Section 4: relocation along a periodic cubic B-spline fitted to each drop
-// by least squares.  Same steps as the definition: chord-length parameters,
-// g = round(L / 1.5h) spans (4 <= g <= n), normal equations accumulated in
-// ascending marker order, Cholesky in the matrix's envelope (band of 3 plus
-// the last three rows, which is where the cyclic wrap fills in), arc length
-// by 8-point Gauss-Legendre per span, 12 Newton steps per new marker.  Two
-// kernels: the fit (one CTA per drop) and the placement of the new markers
-// (one thread per marker over the whole grid).
-// The basis follows the same arithmetic as a serial program: the span of a
-// parameter is floor(s / tau) and the weights come from the Cox-de Boor
-// recursion on knots t_k = k tau, so that relocated markers agree with it to
-// rounding of the same operations.
+// by least squares: chord-length parameters, g = round(L / 1.5h) spans
+// (4 <= g <= n), normal equations accumulated in ascending marker order and
+// solved by block elimination, arc length by 8-point Gauss-Legendre per span,
+// at most 12 Newton steps per new marker.  Two kernels: the fit (one CTA per
+// drop) and the placement of the new markers over the whole grid.
+//
+// The knots t_k = k tau are uniform, so on span q (u = s / tau - q in [0, 1])
+// the four cubic B-splines that do not vanish, of control points q-3 .. q,
+// are (1-u)^3/6, (3u^3 - 6u^2 + 4)/6, (-3u^3 + 3u^2 + 3u + 1)/6, u^3/6.
 __device__ __forceinline__ int bspl_span(double s, double tau, int g)
 {
     int q = (int)floor(s / tau);
     if (q > g - 1) q = g - 1;
     if (q < 0) q = 0;
     return q;
-}
-
-__device__ void bspl_basis(double s, double tau, int g, int *idx, double *w, double *dw)
-{
-    const int q = bspl_span(s, tau, g);
-    double N[4][4];
-    N[0][0] = 1.0;
-    for (int d = 1; d <= 3; d++)
-        for (int r = 0; r <= d; r++) {
-            int k = q - d + r;
-            double tk = k * tau, tkd = (k + d) * tau, tk1 = (k + 1) * tau, tkd1 = (k + d + 1) * tau;
-            double left = (r >= 1) ? (s - tk) / (tkd - tk) * N[d - 1][r - 1] : 0.0;
-            double right = (r <= d - 1) ? (tkd1 - s) / (tkd1 - tk1) * N[d - 1][r] : 0.0;
-            N[d][r] = left + right;
-        }
-    for (int r = 0; r <= 3; r++) {
-        int k = q - 3 + r;
-        idx[r] = ((k % g) + g) % g;
-        w[r] = N[3][r];
-        double a = (r >= 1) ? N[2][r - 1] : 0.0;
-        double b = (r <= 2) ? N[2][r] : 0.0;
-        dw[r] = 3.0 / (3.0 * tau) * a - 3.0 / (3.0 * tau) * b;
-    }
 }
 
 __constant__ double cGLX[8] = {-0.9602898564975363, -0.7966664774136267,
@@ -1307,231 +1282,293 @@ __constant__ double cGLW[8] = {0.1012285362903763, 0.2223810344533745,
                                0.3626837833783620, 0.3137066458778873,
                                0.2223810344533745, 0.1012285362903763};
 
-// The same basis in closed form.  The knots t_k = k tau are uniform, so on
-// span q (u = s / tau - q in [0, 1]) the four cubic B-splines that do not
-// vanish, of control points q-3 .. q, are the uniform ones:
-// (1-u)^3/6, (3u^3 - 6u^2 + 4)/6, (-3u^3 + 3u^2 + 3u + 1)/6, u^3/6, and their
-// derivatives in s are these polynomials' derivatives over tau.  The
-// recursion above gives the same functions with about eight times the FP64
-// operations (a dozen divisions); the Newton placement evaluates the speed
-// ~100 times per marker, so it uses this form (the values agree to
-// rounding).  The span is floor(s / tau) clamped to [0, g-1], found from
-// s (1/tau): at a knot either neighbouring span gives the same value and
-// first derivative (the curve is C^2).
-struct SpanU {
-    int i0, i1, i2, i3;  // control points q-3 .. q (cyclic)
-    double u;
+// The curve on span q: its control points q-3 .. q (cyclic) and its
+// derivative in u, a quadratic d0 + u (d1 + u d2) per coordinate, so that a
+// speed costs six FP64 operations before its square root.
+struct SpanCurve {
+    double x[4], y[4], dx[3], dy[3];
 };
-__device__ __forceinline__ SpanU bspl_span_u(double s, double itau, int g)
+__device__ __forceinline__ SpanCurve span_curve(const double *cx, const double *cy, int g, int q)
 {
-    const double x = s * itau;
-    int q = (int)floor(x);
-    q = q > g - 1 ? g - 1 : (q < 0 ? 0 : q);
-    SpanU r;
-    r.u = x - (double)q;
-    const int k = q - 3;  // >= -3, and q <= g - 1
-    r.i0 = k < 0 ? k + g : k;
-    r.i1 = k + 1 < 0 ? k + 1 + g : k + 1;
-    r.i2 = k + 2 < 0 ? k + 2 + g : k + 2;
-    r.i3 = q;
-    return r;
-}
-
-__device__ double bspl_speed(double s, double tau, int g, const double *cx, const double *cy)
-{
-    const double itau = 1.0 / tau;
-    const SpanU p = bspl_span_u(s, itau, g);
-    const double u = p.u, v = 1.0 - u;
-    // twice the derivatives in u: -(1-u)^2, 3u^2 - 4u, -3u^2 + 2u + 1, u^2
-    const double d0 = -v * v, d1 = u * (3.0 * u - 4.0), d2 = fma(u, 2.0 - 3.0 * u, 1.0), d3 = u * u;
-    const double dx = d0 * cx[p.i0] + d1 * cx[p.i1] + d2 * cx[p.i2] + d3 * cx[p.i3];
-    const double dy = d0 * cy[p.i0] + d1 * cy[p.i1] + d2 * cy[p.i2] + d3 * cy[p.i3];
-    return 0.5 * itau * sqrt(dx * dx + dy * dy);
-}
-
-// The curve's point at s (closed form, as bspl_speed).
-__device__ void bspl_point(double s, double tau, int g, const double *cx, const double *cy,
-                           double &px, double &py)
-{
-    const SpanU p = bspl_span_u(s, 1.0 / tau, g);
-    const double u = p.u, v = 1.0 - u, u2 = u * u, u3 = u2 * u;
-    const double b0 = v * v * v, b1 = fma(3.0, u3, fma(-6.0, u2, 4.0));
-    const double b2 = fma(-3.0, u3, fma(3.0, u2, fma(3.0, u, 1.0))), b3 = u3;
-    const double s6 = 1.0 / 6.0;
-    px = s6 * (b0 * cx[p.i0] + b1 * cx[p.i1] + b2 * cx[p.i2] + b3 * cx[p.i3]);
-    py = s6 * (b0 * cy[p.i0] + b1 * cy[p.i1] + b2 * cy[p.i2] + b3 * cy[p.i3]);
-}
-
-__device__ double gl_len(double a, double b, double tau, int g, const double *cx, const double *cy)
-{
-    double mid = 0.5 * (a + b), half = 0.5 * (b - a), s = 0.0;
-    for (int k = 0; k < 8; k++) s += cGLW[k] * bspl_speed(mid + half * cGLX[k], tau, g, cx, cy);
-    return s * half;
-}
-
-struct Env {
-    // L (lower Cholesky factor) in its envelope: band rows r in [3, g-3) keep
-    // columns r-3..r, the other rows are dense.
-    int g;
-    double *band, *dense;
-    __device__ bool is_band(int r) const { return r >= 3 && r < g - 3; }
-    __device__ int dense_row(int r) const { return r < 3 ? r : 3 + (r - (g - 3)); }
-    __device__ int first(int r) const { return is_band(r) ? r - 3 : 0; }
-    __device__ double get(int r, int c) const {
-        if (is_band(r)) return (c >= r - 3 && c <= r) ? band[r * 4 + (c - r + 3)] : 0.0;
-        return dense[(long)dense_row(r) * g + c];
+    SpanCurve c;
+    for (int r = 0; r < 4; r++) {
+        const int k = q - 3 + r, id = k < 0 ? k + g : k;  // q <= g - 1
+        c.x[r] = cx[id];
+        c.y[r] = cy[id];
     }
-    __device__ void set(int r, int c, double v) {
-        if (is_band(r)) band[r * 4 + (c - r + 3)] = v;
-        else dense[(long)dense_row(r) * g + c] = v;
-    }
-};
-
-// G[r][c] of the cyclic band matrix stored as Gc[i*4 + d] = G[i][(i+d) mod g].
-__device__ double gval(const double *Gc, int g, int r, int c)
+    c.dx[0] = 0.5 * (c.x[2] - c.x[0]);
+    c.dy[0] = 0.5 * (c.y[2] - c.y[0]);
+    c.dx[1] = (c.x[0] - c.x[1]) + (c.x[2] - c.x[1]);
+    c.dy[1] = (c.y[0] - c.y[1]) + (c.y[2] - c.y[1]);
+    c.dx[2] = 0.5 * fma(3.0, c.x[1] - c.x[2], c.x[3] - c.x[0]);
+    c.dy[2] = 0.5 * fma(3.0, c.y[1] - c.y[2], c.y[3] - c.y[0]);
+    return c;
+}
+__device__ __forceinline__ double speed2(const SpanCurve &c, double u)
 {
-    int d1 = ((c - r) % g + g) % g, d2 = ((r - c) % g + g) % g;
-    if (d1 <= 3) return Gc[r * 4 + d1];
-    if (d2 <= 3) return Gc[c * 4 + d2];
-    return 0.0;
+    const double vx = fma(u, fma(u, c.dx[2], c.dx[1]), c.dx[0]);
+    const double vy = fma(u, fma(u, c.dy[2], c.dy[1]), c.dy[0]);
+    return fma(vx, vx, vy * vy);
+}
+// 1 / sqrt(s): rsqrt_nr well inside the FP32 range (tested on the bit
+// pattern, which orders positive values), square root and division elsewhere.
+__device__ __forceinline__ double rsqrt_any(double s)
+{
+    const unsigned long long a = (unsigned long long)__double_as_longlong(s);
+    if (a > (unsigned long long)__double_as_longlong(1e-30) &&
+        a < (unsigned long long)__double_as_longlong(1e30))
+        return rsqrt_nr(s);
+    return 1.0 / sqrt(s);
+}
+__device__ __forceinline__ double sqrt_any(double s)
+{
+    const unsigned long long a = (unsigned long long)__double_as_longlong(s);
+    if (a > (unsigned long long)__double_as_longlong(1e-30) &&
+        a < (unsigned long long)__double_as_longlong(1e30))
+        return s * rsqrt_nr(s);
+    return sqrt(s);
 }
 
-// Cholesky factorisation in the envelope by warp 0 (lane t of 32), each
-// entry by the sums of a dense Cholesky in ascending order: per column c,
-// lane 0 takes the diagonal while lanes 1..6 take the envelope rows below it
-// (c+1..c+3 and the dense last three rows), whose sums need only earlier
-// columns; they are then scaled by the diagonal's reciprocal, which is kept
-// in rinv[c] for the substitutions.  The columns are a serial chain of FP64
-// latencies on this part (a division costs about 1.5 k cycles there), so
-// the reciprocal comes from rsqrt_nr (FP32 seed, two Newton steps), the
-// diagonal is s times it, and the entries multiply by it.  Returns -1 (in every lane) if not positive
-// definite.
-__device__ int env_factor(Env &L, const double *Gc, int g, int t, double *rinv)
+// out[k] = in[0] + ... + in[k-1], k = 0 .. n, of values >= 0, by the block's
+// kT threads; returns the total.  The sums run on 64-bit integers at a power
+// of two that keeps n times the largest value below 2^62: exact, so they do
+// not depend on the split and ascend with k, and off the FP64 pipe, where one
+// thread's running sum took 64 cycles a value.  A value that is not finite
+// makes every sum NaN.  scr: scratch of 12 8-byte words.
+__device__ double block_scan(int n, const double *in, double *out, void *scr)
 {
-    for (int c = 0; c < g; c++) {
-        // envelope row of lane t (t >= 1): the (t-1)-th of the ascending walk
-        int r = -1;
-        if (t >= 1 && t <= 6) {
-            int k = 0;
-            for (int q = c + 1; q < g; q = (q == c + 3 && q + 1 < g - 3) ? g - 3 : q + 1) {
-                if (L.is_band(q) && q - 3 > c) continue;
-                if (++k == t) { r = q; break; }
-            }
-        }
-        double acc = 0.0;
-        if (c >= g - 3 && c > 32) {
-            // the last columns: the diagonal and the (dense) rows below have
-            // sums over all earlier columns; the warp takes them in strided
-            // partial sums and a shuffle tree (the same total in every lane)
-            double pd = 0.0, p1 = 0.0, p2 = 0.0;
-            for (int k = t; k < c; k += 32) {
-                const double lc = L.get(c, k);
-                pd += lc * lc;
-                if (c + 1 < g) p1 += L.get(c + 1, k) * lc;
-                if (c + 2 < g) p2 += L.get(c + 2, k) * lc;
-            }
-            for (int o = 16; o; o >>= 1) {
-                pd += __shfl_xor_sync(0xffffffffu, pd, o);
-                p1 += __shfl_xor_sync(0xffffffffu, p1, o);
-                p2 += __shfl_xor_sync(0xffffffffu, p2, o);
-            }
-            // rows c + 1, c + 2 are the walk's first two: lanes 1 and 2
-            if (t == 0) acc = gval(Gc, g, c, c) - pd;
-            else if (r == c + 1) acc = gval(Gc, g, r, c) - p1;
-            else if (r == c + 2) acc = gval(Gc, g, r, c) - p2;
-        } else {
-            // lane 0 the diagonal (its row is c), lanes 1..6 the rows below:
-            // one code path, so the same FP64 warp instructions serve all
-            // (on this part they cost the same for one lane as for 32)
-            const int rr = t == 0 ? c : r;
-            if (rr >= 0) {
-                acc = gval(Gc, g, rr, c);
-                for (int k = max(L.first(rr), L.first(c)); k < c; k++) acc -= L.get(rr, k) * L.get(c, k);
-            }
-        }
-        const double s = __shfl_sync(0xffffffffu, acc, 0);
-        if (!(s > 0.0)) return -1;
-        // the diagonal d = sqrt(s) and its reciprocal from one reciprocal
-        // square root (a shorter chain than a square root and a reciprocal)
-        const bool fast = s > 1e-30 && s < 1e30;
-        const double rd = fast ? rsqrt_nr(s) : 1.0 / sqrt(s);
-        const double d = fast ? s * rd : sqrt(s);
-        if (t == 0) { L.set(c, c, d); rinv[c] = rd; }
-        else if (r >= 0) L.set(r, c, acc * rd);
-        __syncwarp();
+    long long *ts = (long long *)scr;
+    unsigned *hs = (unsigned *)(ts + kT / 32);
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const int per = (n + kT - 1) / kT, k0 = min(n, (int)threadIdx.x * per), k1 = min(n, k0 + per);
+    unsigned hi = 0;
+    for (int k = k0; k < k1; k++) hi = max(hi, (unsigned)__double2hiint(in[k]));
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) hs[wp] = hi;
+    __syncthreads();
+    for (int w = 0; w < kT / 32; w++) hi = max(hi, hs[w]);
+    // every value is below 2^(E - 1022), n below 2^nb
+    const int E = (int)(hi >> 20), nb = 32 - __clz(n);
+    const int f = max(1, min(2045, 2107 - E - nb));  // exponent field of the scale
+    const double sc = __longlong_as_double((long long)f << 52);
+    const double inv = E >= 2047 ? __longlong_as_double(0x7ff8000000000000LL)
+                                 : __longlong_as_double((long long)(2046 - f) << 52);
+    long long s = 0;
+    for (int k = k0; k < k1; k++) s += __double2ll_rn(in[k] * sc);
+    long long inc = s;
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
     }
-    return 0;
+    if (lane == 31) ts[wp] = inc;
+    __syncthreads();
+    long long base = 0, tot = 0;
+    for (int w = 0; w < kT / 32; w++) {
+        if (w == wp) base = tot;
+        tot += ts[w];
+    }
+    long long run = base + inc - s;
+    for (int k = k0; k < k1; k++) {
+        out[k] = (double)run * inv;
+        run += __double2ll_rn(in[k] * sc);
+    }
+    const double total = (double)tot * inv;
+    if (threadIdx.x == 0) out[n] = total;
+    __syncthreads();
+    return total;
 }
 
-// L L^T x = b for the two right-hand sides bx, by (in place) by warp 0
-// (lane t): every lane runs the serial substitution, lane 0 stores each
-// entry; the long sums of the dense last rows go to the whole warp (strided
-// partial sums and a shuffle tree); scaling by the diagonal's reciprocals
-// rinv (no division on the serial chain).
-__device__ void env_subst(const Env &L, int g, const double *rinv, double *bx, double *by, int t)
+// The normal equations' matrix is a cyclic band of half-width 3.  Its last w
+// rows (w = 3 .. 5, so that 3 m rows remain) are the border; the other rows
+// form a chain of m 3 x 3 blocks, each coupled to its two neighbours, whose
+// ends couple to the border.  A chain block holds, per row, the right-hand
+// sides x and y and its (at most five) border entries, seven columns that are
+// solved together; its diagonal block, symmetric, then its Cholesky factor
+// (diagonal as reciprocals); its coupling to the next chain block still
+// there; and, once eliminated, that to the one before.
+constexpr int kBR = 0, kBD = 21, kBU = 27, kBW = 36, kBlkLen = 45;
+constexpr int kBorder = 5;
+constexpr int kEndLen = 7 * kBorder;  // the border's rows: x, y, matrix
+
+// Solves the system by odd-even elimination of the chain (every second block
+// that is left goes at once, log2 m times), then the border's 5 x 5 rest,
+// then back: 3 log2 m short parallel steps in place of g serial columns and
+// 2 g serial rows, each a chain of FP64 latencies (64 cycles an instruction
+// on this part; 516 us of the fit for g about 130).  A block elimination in the
+// order of a symmetric permutation is a Cholesky factorisation of the
+// permuted matrix, as stable as the row by row one.  S: the border's rows, scr: scratch of 30
+// values.  Sets *bad if a pivot is not positive.
+__device__ void ring_solve(double *blk, int m, int g, double *S, double *scr, double *cx, double *cy,
+                           int *bad)
 {
-    // Even lanes take the x right-hand side, odd lanes the y one, so that
-    // one warp instruction advances both: on this part an FP64 warp
-    // instruction occupies the FP64 unit as long for one lane as for 32, and
-    // the passes are chains of them.  Each lane keeps its side's latest
-    // three entries (and, backwards, the dense last rows') in registers;
-    // lanes 0 and 1 store them for the long sums and the other pass, after
-    // one warp barrier a row (every lane has read the row's right-hand side).
-    double *b = (t & 1) ? by : bx;
-    double x1 = 0.0, x2 = 0.0, x3 = 0.0;  // rows r-1, r-2, r-3
-    for (int r = 0; r < g; r++) {
-        double s = b[r];
-        const int k0 = L.first(r);
-        if (r - k0 > 3) {
-            // a dense last row: all earlier entries, from shared memory
-            __syncwarp();
-            if (r - k0 > 32) {
-                double ps = 0.0, pu = 0.0;
-                for (int k = k0 + t; k < r; k += 32) { const double l = L.get(r, k); ps += l * bx[k]; pu += l * by[k]; }
-                for (int o = 16; o; o >>= 1) {
-                    ps += __shfl_xor_sync(0xffffffffu, ps, o);
-                    pu += __shfl_xor_sync(0xffffffffu, pu, o);
+    const int t = threadIdx.x;
+    // the border entries of the first and the last block, (row, entry)
+    double *C0 = scr, *C1 = scr + 3 * kBorder;
+    if (m > 0 && t < 2 * 3 * kBorder) {
+        const int e = t / (3 * kBorder), k = t % (3 * kBorder), r = k / kBorder, c = k % kBorder;
+        scr[t] = blk[kBlkLen * (e ? m - 1 : 0) + kBR + 7 * r + 2 + c];
+    }
+    __syncthreads();
+    int st = 1;
+    for (; st <= m; st <<= 1) {
+        // eliminated: odd multiples of st among positions 1 .. m; sixteen
+        // lanes a block, each with the factor of the block's own 3 x 3 and
+        // one of the 13 columns [to the left | to the right | right-hand sides]
+        const int ne = (m / st + 1) >> 1;
+        for (int e0 = 0; e0 < ne; e0 += kT / 16) {
+            const int e = e0 + (t >> 4), lane = t & 15, pos = (2 * e + 1) * st;
+            double *B = blk + kBlkLen * (pos - 1);
+            double *dst = nullptr;
+            int ds = 3;
+            double r0 = 0, l10 = 0, r1 = 0, l20 = 0, l21 = 0, r2 = 0, v0 = 0, v1 = 0, v2 = 0;
+            if (e < ne) {
+                const double *D = B + kBD;
+                const double d11 = D[2], d21 = D[4], d22 = D[5];
+                const double s0 = D[0];
+                l10 = D[1]; l20 = D[3];
+                r0 = rsqrt_any(s0);
+                l10 *= r0; l20 *= r0;
+                const double s1 = fma(-l10, l10, d11);
+                r1 = rsqrt_any(s1);
+                l21 = fma(-l20, l10, d21) * r1;
+                const double s2 = fma(-l21, l21, fma(-l20, l20, d22));
+                r2 = rsqrt_any(s2);
+                if (lane == 13 && !(s0 > 0.0 && s1 > 0.0 && s2 > 0.0)) *bad = 1;
+                const double *src = nullptr;
+                int ss = 3;
+                if (lane < 3) {
+                    if (pos > st) { src = B - kBlkLen * st + kBU + 3 * lane; ss = 1; dst = B + kBW + lane; }
+                } else if (lane < 6) {
+                    if (pos + st <= m) { dst = B + kBU + lane - 3; src = dst; }
+                } else if (lane < 13) {
+                    dst = B + kBR + lane - 6; src = dst; ss = ds = 7;
                 }
-                s -= (t & 1) ? pu : ps;
+                if (src) {
+                    v0 = src[0] * r0;
+                    v1 = fma(-l10, v0, src[ss]) * r1;
+                    v2 = fma(-l21, v1, fma(-l20, v0, src[2 * ss])) * r2;
+                }
+            }
+            __syncwarp();
+            if (dst) {
+                dst[0] = v0; dst[ds] = v1; dst[2 * ds] = v2;
+            } else if (lane == 13 && e < ne) {
+                double *D = B + kBD;
+                D[0] = r0; D[1] = l10; D[2] = r1; D[3] = l20; D[4] = l21; D[5] = r2;
+            }
+        }
+        __syncthreads();
+        // the blocks left over: their 36 entries less the products of the
+        // columns of the neighbours just eliminated, one entry a thread
+        const int ns = (m / st) >> 1;
+        for (int it = t; it < 36 * ns; it += kT) {
+            const int sv = it / 36, k = it - 36 * sv, pos = 2 * (sv + 1) * st;
+            double *B = blk + kBlkLen * (pos - 1);
+            const double *e1 = B - kBlkLen * st;
+            const double *e2 = pos + st <= m ? B + kBlkLen * st : nullptr;
+            int r, oc, ow, q = 3;  // row; the column in e1 and in e2, its stride
+            if (k < kBD) {
+                r = k / 7; oc = ow = kBR + k - 7 * r; q = 7;
+            } else if (k < kBU) {
+                const int d = k - kBD;
+                r = d >= 3 ? 2 : (d >= 1 ? 1 : 0);
+                oc = kBU + d - r * (r + 1) / 2; ow = oc - kBU + kBW;
             } else {
-                for (int k = k0; k < r; k++) s -= L.get(r, k) * b[k];
+                if (pos + 2 * st > m) continue;
+                r = (k - kBU) / 3; ow = kBU + (k - kBU) - 3 * r; oc = -1;
             }
+            double v = oc < 0 ? 0.0 : B[k];
+            if (oc >= 0)
+                for (int i = 0; i < 3; i++) v = fma(-e1[kBU + 3 * i + r], e1[oc + q * i], v);
+            if (e2)
+                for (int i = 0; i < 3; i++) v = fma(-e2[kBW + 3 * i + r], e2[ow + q * i], v);
+            B[k] = v;
+        }
+        __syncthreads();
+    }
+    for (st >>= 1; st >= 1; st >>= 1) {
+        const int ne = (m / st + 1) >> 1;
+        for (int it = t; it < 8 * ne; it += kT) {
+            const int e = it >> 3, c = it & 7, pos = (2 * e + 1) * st;
+            if (c == 7) continue;
+            double *B = blk + kBlkLen * (pos - 1), *R = B + kBR + c;
+            double y0 = R[0], y1 = R[7], y2 = R[14];
+            auto sub = [&](const double *W, const double *x) {
+                for (int i = 0; i < 3; i++) {
+                    const double xi = x[7 * i];
+                    y0 = fma(-W[i], xi, y0);
+                    y1 = fma(-W[3 + i], xi, y1);
+                    y2 = fma(-W[6 + i], xi, y2);
+                }
+            };
+            if (pos > st) sub(B + kBW, R - kBlkLen * st);
+            if (pos + st <= m) sub(B + kBU, R + kBlkLen * st);
+            const double *D = B + kBD;
+            y2 *= D[5];
+            y1 = fma(-D[4], y2, y1) * D[2];
+            y0 = fma(-D[3], y2, fma(-D[1], y1, y0)) * D[0];
+            R[0] = y0; R[7] = y1; R[14] = y2;
+        }
+        __syncthreads();
+    }
+    if (m > 0 && t < 7 * kBorder) {
+        const int r = t / 7, c = t % 7;
+        double v = S[t];
+        for (int i = 0; i < 3; i++) v = fma(-C0[kBorder * i + r], blk[kBR + 7 * i + c], v);
+        if (m > 1)
+            for (int i = 0; i < 3; i++)
+                v = fma(-C1[kBorder * i + r], blk[kBlkLen * (m - 1) + kBR + 7 * i + c], v);
+        S[t] = v;
+    }
+    __syncthreads();
+    double *x0 = scr;  // the border's solution, x then y
+    if (t < 2) {  // one lane a right-hand side, each with the factor
+        double L[kBorder][kBorder], b[kBorder];
+#pragma unroll
+        for (int c = 0; c < kBorder; c++) {
+#pragma unroll
+            for (int r = c; r < kBorder; r++) {
+                double v = S[7 * r + 2 + c];
+#pragma unroll
+                for (int k = 0; k < c; k++) v = fma(-L[r][k], L[c][k], v);
+                if (r == c) {
+                    if (!(v > 0.0)) *bad = 1;
+                    L[c][c] = rsqrt_any(v);
+                } else {
+                    L[r][c] = v * L[c][c];
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < kBorder; r++) {
+            double v = S[7 * r + t];
+#pragma unroll
+            for (int k = 0; k < r; k++) v = fma(-L[r][k], b[k], v);
+            b[r] = v * L[r][r];
+        }
+#pragma unroll
+        for (int r = kBorder - 1; r >= 0; r--) {
+            double v = b[r];
+#pragma unroll
+            for (int k = r + 1; k < kBorder; k++) v = fma(-L[k][r], b[k], v);
+            b[r] = v * L[r][r];
+            x0[kBorder * t + r] = b[r];
+        }
+    }
+    __syncthreads();
+    for (int it = t; it < 2 * g; it += kT) {
+        const int r = it >> 1, a = it & 1, br = r - 3 * m;
+        double v;
+        if (br >= 0) {
+            v = x0[kBorder * a + br];
         } else {
-            for (int k = k0; k < r; k++) {  // ascending k, the last (at most) three rows
-                const int back = r - k;
-                s -= L.get(r, k) * (back == 1 ? x1 : (back == 2 ? x2 : x3));
-            }
+            const double *R = blk + kBlkLen * (r / 3) + kBR + 7 * (r % 3);
+            v = R[a];
+            for (int k = 0; k < kBorder; k++) v = fma(-R[2 + k], x0[kBorder * a + k], v);
         }
-        s *= rinv[r];
-        __syncwarp();
-        if (t < 2) b[r] = s;
-        x3 = x2; x2 = x1; x1 = s;
+        (a ? cy : cx)[r] = v;
     }
-    __syncwarp();
-    double f1 = 0.0, f2 = 0.0, f3 = 0.0;  // rows r+1, r+2, r+3
-    double t0 = 0.0, t1 = 0.0, t2 = 0.0;  // rows g-3, g-2, g-1
-    for (int r = g - 1; r >= 0; r--) {
-        double s = b[r];
-        for (int k = r + 1; k < g; k = (k == r + 3 && k + 1 < g - 3) ? g - 3 : k + 1) {
-            if (L.is_band(k) && k - 3 > r) continue;
-            double xv;
-            if (k - r <= 3) {
-                const int back = k - r;
-                xv = back == 1 ? f1 : (back == 2 ? f2 : f3);
-            } else {  // k >= g - 3
-                const int q = k - (g - 3);
-                xv = q == 0 ? t0 : (q == 1 ? t1 : t2);
-            }
-            s -= L.get(k, r) * xv;
-        }
-        s *= rinv[r];
-        __syncwarp();
-        if (t < 2) b[r] = s;
-        f3 = f2; f2 = f1; f1 = s;
-        if (r == g - 1) t2 = s;
-        else if (r == g - 2) t1 = s;
-        else if (r == g - 3) t0 = s;
-    }
+    __syncthreads();
 }
 
 // Per-drop fit results: at offset 3 * s0 + d of fit (s0 the drop's first
@@ -1540,6 +1577,11 @@ __device__ void env_subst(const Env &L, int g, const double *rinv, double *bx, d
 // total arc length, failed).
 __device__ __forceinline__ long fit_base(int s0, int d) { return 3L * s0 + d; }
 
+// One CTA per drop; FP64 latency and one SM's FP64 pipe bound it, so that
+// every stage is spread over the block and written for few FP64
+// instructions.  (With the recursive basis, the sums and the factorisation by
+// one thread or warp the fit took 529 us and the placement 173 for 16 drops of
+// 256 markers; this form takes 0.6 ms off the 1.73 ms of such a step.)
 __global__ void __launch_bounds__(kT)
 k_reloc_fit(const double *__restrict__ X, const double *__restrict__ Y,
             const int32_t *__restrict__ drop_start, double h, int maxn,
@@ -1548,50 +1590,47 @@ k_reloc_fit(const double *__restrict__ X, const double *__restrict__ Y,
 {
     extern __shared__ double sm[];
     const int d = blockIdx.x, s0 = drop_start[d], n = drop_start[d + 1] - s0;
-    // shared layout: sp[n+1], qs[maxg+1] and span[maxn] (ints), Gc[4g],
-    // cx[g], cy[g], band[4g], dense[6g], cum[g+1]
-    const int maxg = maxn;
+    // shared layout: sp[n+1] (then scratch, then cum[g+1]), qs[n+1] and
+    // span[n] (ints, also the sums' scratch), cx[n], cy[n], the chain's blocks
+    // (15 a row, at most n - 3 rows) and behind them the border's rows
     double *sp = sm;
     int *qs = (int *)(sp + maxn + 1);
-    int *span = qs + (maxg + 1);
-    double *Gc = (double *)(qs + 2 * (maxg + 1));
-    double *cx = Gc + 4 * maxg, *cy = cx + maxg, *band = cy + maxg, *dense = band + 4 * maxg;
-    double *cum = dense + 6 * maxg;
-    __shared__ int g_s, bad;
-    __shared__ double tau_s;
-    // chord lengths in parallel (cx as scratch), their running sum in marker
-    // order by one thread
-    for (int m = threadIdx.x; m < n; m += kT) {
+    int *span = qs + (maxn + 1);
+    double *cx = (double *)(qs + 2 * (maxn + 1)), *cy = cx + maxn, *blk = cy + maxn;
+    double *S = blk + 15 * maxn - kEndLen;
+    __shared__ int bad;
+    if (threadIdx.x == 0) bad = 0;
+    for (int m = threadIdx.x; m < n; m += kT) {  // chord lengths
         const int a = s0 + m, b = s0 + (m + 1 == n ? 0 : m + 1);
         const double dx = X[b] - X[a], dy = Y[b] - Y[a];
         cx[m] = sqrt(dx * dx + dy * dy);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double L = 0.0;
-        for (int m = 0; m < n; m++) {
-            sp[m] = L;
-            L += cx[m];
-        }
-        int g = (int)floor(L / (1.5 * h) + 0.5);
-        if (g < 4) g = 4;
-        if (g > n) g = n;
-        g_s = g;
-        tau_s = L / g;
-        bad = 0;
-    }
-    __syncthreads();
-    const int g = g_s;
-    const double tau = tau_s;
+    const double Lc = block_scan(n, cx, sp, qs);
+    int g = (int)floor(Lc / (1.5 * h) + 0.5);
+    if (g < 4) g = 4;
+    if (g > n) g = n;
+    const double tau = Lc / g, itau = 1.0 / tau;
+    const int w = 3 + g % 3, nch = (g - w) / 3, gc = 3 * nch;
     // each marker's span and basis weights once (wts, 4 per marker); the
     // first marker of every span (parameters ascend with m): qs[k] is the
     // first marker of span >= k, n if none
     for (int m = threadIdx.x; m < n; m += kT) {
-        int idx[4];
-        double w[4], dw[4];
-        bspl_basis(sp[m], tau, g, idx, w, dw);
-        span[m] = bspl_span(sp[m], tau, g);
-        for (int r = 0; r < 4; r++) wts[4L * (s0 + m) + r] = w[r];
+        const double s = sp[m];
+        const int q = bspl_span(s, tau, g);
+        const double u = fma(-(double)q, tau, s) * itau, v = 1.0 - u, u2 = u * u;
+        const double s6 = 1.0 / 6.0;
+        double *o = wts + 4L * (s0 + m);
+        span[m] = q;
+        o[0] = s6 * (v * v * v);
+        o[1] = s6 * fma(u2, fma(3.0, u, -6.0), 4.0);
+        o[2] = s6 * fma(u, fma(u, fma(-3.0, u, 3.0), 3.0), 1.0);
+        o[3] = s6 * (u2 * u);
+    }
+    for (int k = threadIdx.x; k < kBlkLen * nch; k += kT) blk[k] = 0.0;
+    if (threadIdx.x < kEndLen) {
+        const int r = threadIdx.x / 7, c = threadIdx.x % 7;
+        S[threadIdx.x] = c == 2 + r && r >= w ? 1.0 : 0.0;
     }
     __syncthreads();
     for (int m = threadIdx.x; m < n; m += kT) {
@@ -1600,46 +1639,51 @@ k_reloc_fit(const double *__restrict__ X, const double *__restrict__ Y,
     }
     for (int k = span[n - 1] + 1 + threadIdx.x; k <= g; k += kT) qs[k] = n;
     __syncthreads();
-    // normal equations: entry (i, i+d) and rhs i, markers of spans i..i+3 in
-    // ascending marker order
+    // normal equations: entry (i, i+dd), dd = 0 .. 3, and right-hand side i
+    // (dd = 4), markers of spans i .. i+3 in ascending marker order; on span
+    // i + t row i has weight 3 - t
     for (int e = threadIdx.x; e < 5 * g; e += kT) {
-        int i = e / 5, dd = e % 5;  // dd 0..3: G[i][(i+dd)%g]; dd 4: rhs row i
-        int sp4[4];
-        for (int t = 0; t < 4; t++) sp4[t] = (i + t) % g;
-        for (int a = 1; a < 4; a++)
-            for (int b = a; b > 0 && sp4[b] < sp4[b - 1]; b--) { int tt = sp4[b]; sp4[b] = sp4[b - 1]; sp4[b - 1] = tt; }
-        int jcol = (i + (dd < 4 ? dd : 0)) % g;
+        const int i = e / 5, dd = e - 5 * i;
+        const int t0 = i + 3 >= g ? g - i : 0;
         double acc = 0.0, accy = 0.0;
-        for (int t = 0; t < 4; t++) {
-            if (t > 0 && sp4[t] == sp4[t - 1]) continue;
-            for (int m = qs[sp4[t]]; m < qs[sp4[t] + 1]; m++) {
-                const double *w = wts + 4L * (s0 + m);
-                int a = -1, b = -1;
-                for (int r = 0; r < 4; r++) {
-                    const int k = span[m] - 3 + r, id = ((k % g) + g) % g;
-                    if (id == i) a = r;
-                    if (id == jcol) b = r;
+        for (int k = 0; k < 4; k++) {
+            const int tt = (t0 + k) & 3, a = 3 - tt;
+            if (tt == g) continue;  // three spans: i + 3 is span i again
+            const int q = i + tt >= g ? i + tt - g : i + tt;
+            int b = a + dd;
+            if (b > 3) b -= g;  // fewer than seven spans: the band meets itself
+            const double *wm = wts + 4L * (s0 + qs[q]);
+            const int ke = qs[q + 1];
+            if (dd < 4) {
+                if (b >= 0)
+                    for (int m = qs[q]; m < ke; m++, wm += 4) acc += wm[a] * wm[b];
+            } else {
+                for (int m = qs[q]; m < ke; m++, wm += 4) {
+                    acc += wm[a] * X[s0 + m];
+                    accy += wm[a] * Y[s0 + m];
                 }
-                if (a < 0) continue;
-                if (dd < 4) { if (b >= 0) acc += w[a] * w[b]; }
-                else { acc += w[a] * X[s0 + m]; accy += w[a] * Y[s0 + m]; }
             }
         }
-        if (dd < 4) Gc[i * 4 + dd] = acc;
-        else { cx[i] = acc; cy[i] = accy; }
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        Env L{g, band, dense};
-        // cum holds the diagonal's reciprocals until the arc lengths below
-        const int f = env_factor(L, Gc, g, threadIdx.x, cum);  // the same in every lane
-        if (f != 0) {
-            if (threadIdx.x == 0) bad = 1;
+        if (dd == 4) {
+            double *r = i < gc ? blk + kBlkLen * (i / 3) + kBR + 7 * (i % 3) : S + 7 * (i - gc);
+            r[0] = acc; r[1] = accy;
+            continue;
+        }
+        const int j = i + dd >= g ? i + dd - g : i + dd;
+        const int lo = min(i, j), hi = max(i, j);
+        if (lo >= gc) {
+            S[7 * (lo - gc) + 2 + hi - gc] = acc;
+            S[7 * (hi - gc) + 2 + lo - gc] = acc;
         } else {
-            env_subst(L, g, cum, cx, cy, threadIdx.x);
+            const int bl = lo / 3, r = lo - 3 * bl;
+            double *B = blk + kBlkLen * bl;
+            if (hi >= gc) B[kBR + 7 * r + 2 + hi - gc] = acc;
+            else if (hi / 3 == bl) { const int c = hi - 3 * bl; B[kBD + c * (c + 1) / 2 + r] = acc; }
+            else B[kBU + 3 * r + hi - 3 * (bl + 1)] = acc;
         }
     }
     __syncthreads();
+    ring_solve(blk, nch, g, S, sp, cx, cy, &bad);
     double *out = fit + fit_base(s0, d);
     if (bad) {
         if (threadIdx.x == 0) {
@@ -1648,45 +1692,48 @@ k_reloc_fit(const double *__restrict__ X, const double *__restrict__ Y,
         }
         return;
     }
-    for (int q = threadIdx.x; q < g; q += kT) cum[q + 1] = gl_len(q * tau, (q + 1) * tau, tau, g, cx, cy);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        cum[0] = 0.0;
-        for (int q = 0; q < g; q++) cum[q + 1] = cum[q] + cum[q + 1];
-        par[4 * d] = (double)g; par[4 * d + 1] = tau; par[4 * d + 2] = cum[g]; par[4 * d + 3] = 0.0;
+    // arc length of every span (blk is free now), its running sum
+    for (int q = threadIdx.x; q < g; q += kT) {
+        const SpanCurve c = span_curve(cx, cy, g, q);
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < 8; k++)
+            s = fma(0.5 * cGLW[k], sqrt_any(speed2(c, fma(0.5, cGLX[k], 0.5))), s);
+        blk[q] = s;
     }
     __syncthreads();
+    const double len = block_scan(g, blk, sp, qs);
+    if (threadIdx.x == 0) {
+        par[4 * d] = (double)g; par[4 * d + 1] = tau; par[4 * d + 2] = len; par[4 * d + 3] = 0.0;
+    }
     for (int q = threadIdx.x; q < g; q += kT) { out[q] = cx[q]; out[n + q] = cy[q]; }
-    for (int q = threadIdx.x; q <= g; q += kT) out[2 * n + q] = cum[q];
+    for (int q = threadIdx.x; q <= g; q += kT) out[2 * n + q] = sp[q];
 }
 
 // New marker m of its drop at arc length L m / n along the fitted curve: the
-// span by bisection of the knot arc lengths, then 12 Newton steps on the
-// partial arc length, kept in the span.  With LN = 8 lanes per marker (few
-// markers: the FP64 latency of one thread's steps dominates), lane k
-// evaluates the k-th Gauss-Legendre term of the partial arc length and lane
-// 0 also the speed at s; every lane then sums the eight terms in order, so
-// all lanes carry the same s.  With LN = 1 (many markers: FP64 throughput
-// dominates) one thread does all.  A drop whose fit failed keeps its markers.
+// span by bisection of the knot arc lengths, then Newton steps on the partial
+// arc length in u, kept in the span; at most 12, ended when the iterate
+// repeats itself (all later steps would, so the result is that of 12).  LN
+// lanes share a marker's eight Gauss-Legendre terms: a step costs about
+// 104 / LN + 27 FP64 instructions, and up to four warps an SM the time is
+// that of one warp, so LN = 8 below 4096 markers, 4 up to 8192, 1 above
+// (with the curve evaluated from control points at every node and always 12
+// steps 4096 markers took 173 us, 16384 markers 193).  A drop whose fit failed
+// keeps its markers.
 constexpr int kPlaceT = 64;
 template <int LN>
 __global__ void __launch_bounds__(kPlaceT)
-k_reloc_place(int M, const double *__restrict__ X, const double *__restrict__ Y,
-              const int32_t *__restrict__ drop_of, const int32_t *__restrict__ drop_start,
+k_reloc_place(int M, const int32_t *__restrict__ drop_of, const int32_t *__restrict__ drop_start,
               const double *__restrict__ fit, const double *__restrict__ par,
-              double *__restrict__ Xo, double *__restrict__ Yo)
+              double *__restrict__ X, double *__restrict__ Y)
 {
-    const int lane = LN == 8 ? (threadIdx.x & 7) : 0, tid = blockIdx.x * kPlaceT + threadIdx.x;
-    const int j = LN == 8 ? tid >> 3 : tid;
-    const unsigned grp = 0xffu << (threadIdx.x & 24);  // the eight lanes of this marker
-    if (j >= M) return;  // whole groups leave together (groups of LN lanes)
+    const int lane = threadIdx.x & (LN - 1), j = (blockIdx.x * kPlaceT + threadIdx.x) / LN;
+    const unsigned grp = ((1u << LN) - 1u) << (threadIdx.x & 31 & ~(LN - 1));  // this marker's lanes
+    if (j >= M) return;  // whole groups leave together
     const int d = drop_of[j], s0 = drop_start[d], n = drop_start[d + 1] - s0, m = j - s0;
-    if (par[4 * d + 3] != 0.0) {
-        if (lane == 0) { Xo[j] = X[j]; Yo[j] = Y[j]; }
-        return;
-    }
+    if (par[4 * d + 3] != 0.0) return;
     const int g = (int)par[4 * d];
-    const double tau = par[4 * d + 1], Lp = par[4 * d + 2];
+    const double Lp = par[4 * d + 2];
     const double *cx = fit + fit_base(s0, d), *cy = cx + n, *cum = cx + 2 * n;
     const double target = Lp * (double)m / (double)n;
     int lo = 0, hi = g - 1;  // largest q <= g-1 with cum[q] <= target
@@ -1695,34 +1742,39 @@ k_reloc_place(int M, const double *__restrict__ X, const double *__restrict__ Y,
         if (cum[mid] <= target) lo = mid; else hi = mid - 1;
     }
     const int q = lo;
-    const double a = q * tau, b = (q + 1) * tau;
-    const double seg = cum[q + 1] - cum[q];
-    double s = a + tau * (target - cum[q]) / seg;
-    for (int it = 0; it < 12; it++) {
-        if constexpr (LN == 1) {
-            const double f = cum[q] + gl_len(a, s, tau, g, cx, cy) - target;
-            const double sp_ = bspl_speed(s, tau, g, cx, cy);
-            s -= f / sp_;
-            if (s < a) s = a;
-            if (s > b) s = b;
-            continue;
-        }
-        // cum[q] + gl_len(a, s) - target, the Gauss-Legendre sum as gl_len
-        const double mid = 0.5 * (a + s), half = 0.5 * (s - a);
-        const double term = cGLW[lane] * bspl_speed(mid + half * cGLX[lane], tau, g, cx, cy);
-        const double sp_ = lane == 0 ? bspl_speed(s, tau, g, cx, cy) : 0.0;
+    const SpanCurve c = span_curve(cx, cy, g, q);
+    const double c0 = cum[q] - target;
+    double node[8 / LN], wgt[8 / LN];
+#pragma unroll
+    for (int k = 0; k < 8 / LN; k++) {
+        node[k] = fma(0.5, cGLX[lane + LN * k], 0.5);
+        wgt[k] = 0.5 * cGLW[lane + LN * k];
+    }
+    double u = -c0 / (cum[q + 1] - cum[q]), prev = u;
+    for (int it = 1; it <= 12; it++) {
         double sum = 0.0;
-        for (int k = 0; k < 8; k++) sum += __shfl_sync(grp, term, k, 8);
-        const double f = cum[q] + sum * half - target;
-        s -= f / __shfl_sync(grp, sp_, 0, 8);
-        if (s < a) s = a;
-        if (s > b) s = b;
+#pragma unroll
+        for (int k = 0; k < 8 / LN; k++) sum = fma(wgt[k], sqrt_any(speed2(c, u * node[k])), sum);
+        for (int o = LN / 2; o; o >>= 1) sum += __shfl_xor_sync(grp, sum, o);
+        double un = fma(-fma(u, sum, c0), rsqrt_any(speed2(c, u)), u);
+        if (un < 0.0) un = 0.0;
+        if (un > 1.0) un = 1.0;
+        const long long bn = __double_as_longlong(un);
+        if (bn == __double_as_longlong(u)) break;
+        if (it > 1 && bn == __double_as_longlong(prev)) {  // a cycle of two
+            if (!((12 - it) & 1)) u = un;
+            break;
+        }
+        prev = u;
+        u = un;
     }
     if (lane != 0) return;
-    double px, py;
-    bspl_point(s, tau, g, cx, cy, px, py);
-    Xo[j] = px;
-    Yo[j] = py;
+    const double v = 1.0 - u, u2 = u * u, u3 = u2 * u;
+    const double b0 = v * v * v, b1 = fma(3.0, u3, fma(-6.0, u2, 4.0));
+    const double b2 = fma(-3.0, u3, fma(3.0, u2, fma(3.0, u, 1.0))), b3 = u3;
+    const double s6 = 1.0 / 6.0;
+    X[j] = s6 * (b0 * c.x[0] + b1 * c.x[1] + b2 * c.x[2] + b3 * c.x[3]);
+    Y[j] = s6 * (b0 * c.y[0] + b1 * c.y[1] + b2 * c.y[2] + b3 * c.y[3]);
 }
 
 }  // namespace
@@ -1746,7 +1798,7 @@ cudaError_t markers_alloc(Markers &mk, int M, int ndrops, int nx, int ny, double
     // per segment; 64 per segment covers segments up to ~9 cells long.
     const size_t pair_cap = (size_t)M * 64 + 4096;
     mk.pair_cap = (uint32_t)pair_cap;
-    size_t bytes = al(M * 8) * 13 + al(M * 4) * 2 + al(M * 16) + al(ndrops * 16) * 2 + al((3 * (size_t)M + ndrops) * 8) + al((size_t)ndrops * 32) + al((size_t)M * 32) +
+    size_t bytes = al(M * 8) * 11 + al(M * 4) * 2 + al(M * 16) + al(ndrops * 16) * 2 + al((3 * (size_t)M + ndrops) * 8) + al((size_t)ndrops * 32) + al((size_t)M * 32) +
                    al((size_t)M * 24 * 8) + al((size_t)M * kSegLine * 8) + al((size_t)M * 8 * 16) + al((size_t)M * 5 * 16) + al(M * 8) + al(M) + al(M * 8) +
                    al(64) + al(pair_cap * 4) * 2 + al(pair_cap * 8) * 2 + al(ncell * 8) +
                    al((ndrops + 1) * 4) + al(M * 4) * 5 + al(ncell * 4) +
@@ -1760,7 +1812,6 @@ cudaError_t markers_alloc(Markers &mk, int M, int ndrops, int nx, int ny, double
     mk.kappa = (double *)take(M * 8); mk.nxm = (double *)take(M * 8); mk.nym = (double *)take(M * 8);
     mk.ds = (double *)take(M * 8); mk.fmag = (double *)take(M * 8);
     mk.U = (double *)take(M * 8); mk.V = (double *)take(M * 8);
-    mk.Xn = (double *)take(M * 8); mk.Yn = (double *)take(M * 8);
     mk.gx = (double *)take(M * 8); mk.gy = (double *)take(M * 8);
     mk.gxf = (float *)take(M * 4); mk.gyf = (float *)take(M * 4);
     mk.sbox = (float4 *)take(M * 16);
@@ -1953,10 +2004,13 @@ void launch_spread_irrot(const Markers &mk, const double *fmag, const double *H,
                                        H, Fx, Fy, mk.flags);
 }
 
+// Shared memory of k_reloc_fit: 19 doubles a marker.  Its layout takes a drop
+// of at least 32 markers, so that the scratch in sp and qs fits.
+static int relocate_maxn(int maxn) { return std::max(maxn, 32); }
 size_t relocate_smem(int maxn)
 {
-    return (size_t)(maxn + 1) * 8 + (size_t)2 * (maxn + 1) * 4 + (size_t)4 * maxn * 8 +
-           (size_t)2 * maxn * 8 + (size_t)4 * maxn * 8 + (size_t)6 * maxn * 8 + (size_t)(maxn + 1) * 8 + 64;
+    const size_t n = (size_t)relocate_maxn(maxn);
+    return (19 * n + 11) * 8;
 }
 
 // ------------------------------------------------------------ measure correction
@@ -2105,19 +2159,16 @@ void launch_relocate(Markers &mk, cudaStream_t s)
     size_t sm = relocate_smem(mk.max_drop);
     raise_smem_limit((const void *)k_reloc_fit, (int)sm);
     note_launch();
-    k_reloc_fit<<<mk.ndrops, kT, sm, s>>>(mk.X, mk.Y, mk.drop_start, mk.h, mk.max_drop, mk.rfit,
+    k_reloc_fit<<<mk.ndrops, kT, sm, s>>>(mk.X, mk.Y, mk.drop_start, mk.h, relocate_maxn(mk.max_drop), mk.rfit,
                                           mk.rpar, mk.rwts, mk.flags);
     note_launch();
-    if (mk.M < 4096)
-        k_reloc_place<8><<<cdiv(8 * mk.M, kPlaceT), kPlaceT, 0, s>>>(mk.M, mk.X, mk.Y, mk.drop_of,
-                                                                     mk.drop_start, mk.rfit, mk.rpar,
-                                                                     mk.Xn, mk.Yn);
-    else
-        k_reloc_place<1><<<cdiv(mk.M, kPlaceT), kPlaceT, 0, s>>>(mk.M, mk.X, mk.Y, mk.drop_of,
-                                                                 mk.drop_start, mk.rfit, mk.rpar,
-                                                                 mk.Xn, mk.Yn);
-    cudaMemcpyAsync(mk.X, mk.Xn, (size_t)mk.M * 8, cudaMemcpyDeviceToDevice, s);
-    cudaMemcpyAsync(mk.Y, mk.Yn, (size_t)mk.M * 8, cudaMemcpyDeviceToDevice, s);
+    auto place = [&](auto kernel, int ln) {
+        kernel<<<cdiv((long)ln * mk.M, kPlaceT), kPlaceT, 0, s>>>(mk.M, mk.drop_of, mk.drop_start,
+                                                                  mk.rfit, mk.rpar, mk.X, mk.Y);
+    };
+    if (mk.M < 4096) place(k_reloc_place<8>, 8);
+    else if (mk.M < 8192) place(k_reloc_place<4>, 4);
+    else place(k_reloc_place<1>, 1);
 }
 
 }  // namespace ibk
