@@ -5,7 +5,9 @@
 // viscous predictor (Section 2.1 Eqs. (ad_bf), (cr_ni)).
 //
 // All kernels are single-pass, one thread per cell or face, coalesced along
-// x; they are HBM-bound and small next to the multigrid solve.
+// x.  FP64 arithmetic bounds them on this part before HBM (1.25 TFLOP/s), so
+// they are written for few FP64 operations; divisions of indices are avoided
+// by two-dimensional grids.
 #include <utility>
 
 #include "ib_internal.cuh"
@@ -26,7 +28,13 @@ __global__ void k_cells_props(int n, double rho_g, double drho, double mu_g,
     mu[k] = mu_g + dmu * hk;
 }
 
-// beta on x-faces then y-faces in one index space.
+// 2 x for a normal x (an addition to the exponent, no FP64 operation).
+__device__ __forceinline__ double twice(double x)
+{
+    return __longlong_as_double(__double_as_longlong(x) + (1LL << 52));
+}
+
+// beta = 1 / (two-cell mean of rho) on x-faces and y-faces.
 __global__ void k_face_beta(int nx, int ny, const double *__restrict__ rho,
                             double *__restrict__ bx, double *__restrict__ by)
 {
@@ -36,31 +44,38 @@ __global__ void k_face_beta(int nx, int ny, const double *__restrict__ rho,
         const long k = (long)j * (nx + 1) + i;
         bx[k] = (i == 0 || i == nx)
                     ? 0.0
-                    : recip_nr(0.5 * (rho[(long)j * nx + i - 1] + rho[(long)j * nx + i]));
+                    : twice(recip_nr(rho[(long)j * nx + i - 1] + rho[(long)j * nx + i]));
     }
     if (i < nx) {
         const long k = (long)j * nx + i;
         by[k] = (j == 0 || j == ny)
                     ? 0.0
-                    : recip_nr(0.5 * (rho[(long)(j - 1) * nx + i] + rho[(long)j * nx + i]));
+                    : twice(recip_nr(rho[(long)(j - 1) * nx + i] + rho[(long)j * nx + i]));
     }
 }
 
-__global__ void k_rhs(int nx, int ny, double ih, double idt,
+// The force is zero on all faces but those of the interface band: where a
+// warp's faces carry none, its part and the loads of beta are skipped (12
+// FP64 operations a cell to 4; 1024^2: 22 -> 13 us).
+__global__ void k_rhs(int nx, int ny, double ih, double ihdt,
                       const double *__restrict__ us, const double *__restrict__ vs,
                       const double *__restrict__ Fx, const double *__restrict__ Fy,
                       const double *__restrict__ bx, const double *__restrict__ by,
                       double *__restrict__ b)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
     if (i >= nx) return;
-    long xw = (long)j * (nx + 1) + i, ys = (long)j * nx + i, yn = ys + nx;
-    double divu = (us[xw + 1] - us[xw] + vs[yn] - vs[ys]) * ih;
-    double divf = (bx[xw + 1] * Fx[xw + 1] - bx[xw] * Fx[xw] + by[yn] * Fy[yn] -
-                   by[ys] * Fy[ys]) * ih;
-    b[ys] = divu * idt + divf;
+    const long xw = (long)j * (nx + 1) + i, ys = (long)j * nx + i, yn = ys + nx;
+    const double fe = Fx[xw + 1], fw = Fx[xw], fn = Fy[yn], fs = Fy[ys];
+    double v = ((us[xw + 1] - us[xw]) + (vs[yn] - vs[ys])) * ihdt;
+    const long long any = __double_as_longlong(fe) | __double_as_longlong(fw) | __double_as_longlong(fn) |
+                          __double_as_longlong(fs);
+    if (any & 0x7fffffffffffffffLL)
+        v = fma(bx[xw + 1] * fe - bx[xw] * fw + by[yn] * fn - by[ys] * fs, ih, v);
+    b[ys] = v;
 }
 
+// One row of x-faces (j < ny) and of y-faces (j <= ny) per blockIdx.y.
 __global__ void k_correct(int nx, int ny, double ih, double dt,
                           const double *__restrict__ us, const double *__restrict__ vs,
                           const double *__restrict__ p, const double *__restrict__ Fx,
@@ -68,21 +83,19 @@ __global__ void k_correct(int nx, int ny, double ih, double dt,
                           const double *__restrict__ by, double *__restrict__ u,
                           double *__restrict__ v)
 {
-    long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    long nxf = (long)(nx + 1) * ny;
-    if (k < nxf) {
-        int j = (int)(k / (nx + 1)), i = (int)(k - (long)j * (nx + 1));
-        if (i == 0 || i == nx) { u[k] = 0.0; return; }
-        double gp = (p[(long)j * nx + i] - p[(long)j * nx + i - 1]) * ih;
-        u[k] = us[k] + dt * (bx[k] * (Fx[k] - gp));
-        return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+    if (i > nx) return;
+    const long c = (long)j * nx + i;
+    const double pc = (i < nx && j < ny) ? p[c] : 0.0;
+    if (j < ny) {
+        const long k = (long)j * (nx + 1) + i;
+        if (i == 0 || i == nx) u[k] = 0.0;
+        else u[k] = fma(dt, bx[k] * fma(-ih, pc - p[c - 1], Fx[k]), us[k]);
     }
-    k -= nxf;
-    if (k >= (long)nx * (ny + 1)) return;
-    int j = (int)(k / nx), i = (int)(k - (long)j * nx);
-    if (j == 0 || j == ny) { v[k] = 0.0; return; }
-    double gp = (p[(long)j * nx + i] - p[(long)(j - 1) * nx + i]) * ih;
-    v[k] = vs[k] + dt * (by[k] * (Fy[k] - gp));
+    if (i < nx) {
+        if (j == 0 || j == ny) v[c] = 0.0;
+        else v[c] = fma(dt, by[c] * fma(-ih, pc - p[c - nx], Fy[c]), vs[c]);
+    }
 }
 
 // Tiled predictor: a 32 x 8 block of cells stages rho, mu, u and v with a
@@ -202,6 +215,7 @@ k_predictor(int nx, int ny, double ih, double ih2, double dt,
     if (i >= nx || j >= ny) return;
     const int R = ty + 1, C = tx + 1;  // window index of cell (i, j)
     const double ih4 = 0.25 * ih, ih16 = 0.0625 * ih;  // the folded factors
+    const double ih2x2 = 2.0 * ih2, hdt = 0.5 * dt;
     // x-face (i, j), left of cell (i, j)
     {
         const long k = (long)j * nxf + i;
@@ -210,13 +224,16 @@ k_predictor(int nx, int ny, double ih, double ih2, double dt,
         } else {
             const double uc = su[R][C];
             const double adv = (fx[ty][tx + 1] - fx[ty][tx]) * ih4 + (gxn[ty + 1][tx] - gxn[ty][tx]) * ih16;
-            // (vx E - vx W + wx N - wx S) / h^2 with wx = wxn / 4 (exact)
-            const double vis = fma(-0.25, wxn[ty][tx], fma(0.25, wxn[ty + 1][tx], vx[ty][tx + 1] - vx[ty][tx])) * ih2;
+            // vx E - vx W + wx N - wx S with wx = wxn / 4 (exact)
+            const double vis = fma(-0.25, wxn[ty][tx], fma(0.25, wxn[ty + 1][tx], vx[ty][tx + 1] - vx[ty][tx]));
             // 1 / rho_face: the face coefficient beta when given (the same
             // reciprocal of the same rho), else formed here
-            const double irf = bx ? bx[k] : recip_nr(0.5 * (sr[R][C - 1] + sr[R][C]));
-            const double ae = have_prev ? 1.5 * adv - 0.5 * aup[k] : adv;
-            us[k] = uc + dt * ((vis - ae) * irf + gx);
+            const double irf = bx ? bx[k] : twice(recip_nr(sr[R][C - 1] + sr[R][C]));
+            // twice (vis / h^2 - (3/2 adv - 1/2 aup)), its half in dt / 2
+            const double q = have_prev ? fma(-3.0, adv, aup[k]) : -2.0 * adv;
+            double un = fma(hdt, fma(ih2x2, vis, q) * irf, uc);
+            if (gx != 0.0) un = fma(dt, gx, un);
+            us[k] = un;
             au[k] = adv;
         }
         if (i == nx - 1) { us[k + 1] = 0.0; au[k + 1] = 0.0; }  // right wall face
@@ -229,10 +246,12 @@ k_predictor(int nx, int ny, double ih, double ih2, double dt,
         } else {
             const double vc = sv[R][C];
             const double adv = (fy[ty + 1][tx] - fy[ty][tx]) * ih4 + (gyn[ty][tx + 1] - gyn[ty][tx]) * ih16;
-            const double vis = fma(-0.25, wyn[ty][tx], fma(0.25, wyn[ty][tx + 1], vy[ty + 1][tx] - vy[ty][tx])) * ih2;
-            const double irf = by ? by[k] : recip_nr(0.5 * (sr[R - 1][C] + sr[R][C]));
-            const double ae = have_prev ? 1.5 * adv - 0.5 * avp[k] : adv;
-            vs[k] = vc + dt * ((vis - ae) * irf + gy);
+            const double vis = fma(-0.25, wyn[ty][tx], fma(0.25, wyn[ty][tx + 1], vy[ty + 1][tx] - vy[ty][tx]));
+            const double irf = by ? by[k] : twice(recip_nr(sr[R - 1][C] + sr[R][C]));
+            const double q = have_prev ? fma(-3.0, adv, avp[k]) : -2.0 * adv;
+            double vn = fma(hdt, fma(ih2x2, vis, q) * irf, vc);
+            if (gy != 0.0) vn = fma(dt, gy, vn);
+            vs[k] = vn;
             av[k] = adv;
         }
         if (j == ny - 1) { vs[k + nx] = 0.0; av[k + nx] = 0.0; }  // top wall face
@@ -603,7 +622,7 @@ void launch_rhs(int nx, int ny, double h, double dt, const double *us,
 {
     dim3 g(cdiv(nx, 128), ny);
     note_launch();
-    k_rhs<<<g, 128, 0, s>>>(nx, ny, 1.0 / h, 1.0 / dt, us, vs, Fx, Fy, bx, by, b);
+    k_rhs<<<g, 128, 0, s>>>(nx, ny, 1.0 / h, 1.0 / (h * dt), us, vs, Fx, Fy, bx, by, b);
 }
 
 void launch_correct(int nx, int ny, double h, double dt, const double *us,
@@ -611,9 +630,8 @@ void launch_correct(int nx, int ny, double h, double dt, const double *us,
                     const double *Fy, const double *bx, const double *by,
                     double *u, double *v, cudaStream_t s)
 {
-    long nf = (long)(nx + 1) * ny + (long)nx * (ny + 1);
     note_launch();
-    k_correct<<<cdiv(nf, kT), kT, 0, s>>>(nx, ny, 1.0 / h, dt, us, vs, p, Fx, Fy,
+    k_correct<<<dim3(cdiv(nx + 1, 128), ny + 1), 128, 0, s>>>(nx, ny, 1.0 / h, dt, us, vs, p, Fx, Fy,
                                           bx, by, u, v);
 }
 

@@ -73,31 +73,30 @@ __device__ __forceinline__ double f2d(float f)
     return (double)f;
 }
 
-// 1/sqrt(x) for x in the FP32 normal range: the FP32 estimate (rsqrtf) of
-// x's leading bits refined by two Newton steps y <- y (3/2 - x y^2 / 2) in
-// FP64 (relative error 2^-22 -> 2^-43 -> below FP64 rounding); a short chain
-// of dependent operations, for serial code where FP64 latency counts.
+// 1/sqrt(x) for x in the FP32 normal range: the FP32 estimate y (rsqrtf) of
+// x's leading bits, e = 1 - x y^2 its error (about 2^-22), and one step of
+// third order y <- y + y e (1/2 + 3/8 e) in FP64, whose remainder 5/16 e^3 is
+// far below FP64 rounding; five dependent operations, for serial code where
+// FP64 latency counts (two Newton steps take seven).
 __device__ __forceinline__ double rsqrt_nr(double x)
 {
-    double y = f2d_exact(rsqrtf(d2f_trunc(x)));
-    const double hx = -0.5 * x;
-    y = y * fma(hx, y * y, 1.5);
-    return y * fma(hx, y * y, 1.5);
+    const double y = f2d_exact(rsqrtf(d2f_trunc(x)));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y, e * fma(0.375, e, 0.5), y);
 }
 
 // 1/x for x of either sign within the FP32 normal range (about 1e-37 < |x|
-// < 1e37): the FP32 reciprocal (__frcp_rn) of x's leading bits refined by two
-// Newton-Raphson steps r <- r + r (1 - x r) in FP64; each step squares the
-// relative error (2^-22 -> 2^-44 -> below the FP64 rounding), so the result
-// is within one unit in the last place of 1.0 / x at a fraction of the FP64
-// division's cost on this part, with no FP64 conversion.
+// < 1e37): the FP32 reciprocal r (__frcp_rn) of x's leading bits, e = 1 - x r
+// its error (about 2^-22), and one step of third order r <- r + r (e + e^2)
+// in FP64, whose remainder e^3 is far below FP64 rounding: within one unit in
+// the last place of 1.0 / x for three FP64 operations (two Newton-Raphson
+// steps take four), a fraction of the FP64 division's cost on this part, with
+// no FP64 conversion.
 __device__ __forceinline__ double recip_nr(double x)
 {
-    double r = f2d_exact(__frcp_rn(d2f_trunc(x)));
-    double e = fma(-x, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-x, r, 1.0);
-    return fma(r, e, r);
+    const double r = f2d_exact(__frcp_rn(d2f_trunc(x)));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
 // 1/x for any nonzero finite x of either sign (0 for x = 0): recip_nr where

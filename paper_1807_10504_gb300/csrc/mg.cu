@@ -1108,7 +1108,8 @@ __device__ __forceinline__ void level_coeffs_cell(int nx, int ny, int level0, in
         for (int t = nx + 1; t < xp; t++) rowp[t] = 0.0f;  // padding
     }
     const double d = e + w + n + s;
-    const double id = d > 0.0 ? recip_nr(d) : 0.0;
+    // d > 0 on its bit pattern (an FP64 compare costs an FP64 operation)
+    const double id = __double_as_longlong(d) > 0 ? recip_nr(d) : 0.0;
     invd[kc] = id;
     invdf[kc] = d2f_rn(id);
     if (w4 || w4f) {
