@@ -116,14 +116,23 @@ __global__ void k_geometry(int M, const double *__restrict__ X, const double *__
     fmag[m] = sigma * k;
 }
 
-// Half-plane {x : n.x - c >= 0} on the left of the directed line P -> Q, with
-// n the unit left normal (a zero vector, which constrains nothing, if P = Q).
-__device__ __forceinline__ void left_of(double px, double py, double qx, double qy, double *l)
+// 1 / sqrt(s): rsqrt_nr well inside the FP32 range (tested on the bit
+// pattern, which orders positive values), square root and division elsewhere.
+__device__ __forceinline__ double rsqrt_any(double s)
 {
-    const double dx = qx - px, dy = qy - py, len = sqrt(dx * dx + dy * dy);
-    const double il = recip_any(len);
-    const double nx_ = -dy * il, ny_ = dx * il;
-    l[0] = nx_; l[1] = ny_; l[2] = nx_ * px + ny_ * py;
+    const unsigned long long a = (unsigned long long)__double_as_longlong(s);
+    if (a > (unsigned long long)__double_as_longlong(1e-30) &&
+        a < (unsigned long long)__double_as_longlong(1e30))
+        return rsqrt_nr(s);
+    return 1.0 / sqrt(s);
+}
+__device__ __forceinline__ double sqrt_any(double s)
+{
+    const unsigned long long a = (unsigned long long)__double_as_longlong(s);
+    if (a > (unsigned long long)__double_as_longlong(1e-30) &&
+        a < (unsigned long long)__double_as_longlong(1e30))
+        return s * rsqrt_nr(s);
+    return sqrt(s);
 }
 
 // Segment geometry of (m, next m): the strip corners at offsets -2.5 .. 2.5
@@ -131,33 +140,45 @@ __device__ __forceinline__ void left_of(double px, double py, double qx, double 
 // rounded outward to FP32 so that an FP32 test against a cell never rejects
 // a strip that touches it, the eight bounding half-planes and whether all
 // five strips are convex.
-
-__global__ void k_segments(int M, const int32_t *__restrict__ next, const double *__restrict__ gx,
-                           const double *__restrict__ gy, const double *__restrict__ nxm,
-                           const double *__restrict__ nym, float4 *__restrict__ sbox,
-                           double *__restrict__ sv, float4 *__restrict__ sb5,
-                           double *__restrict__ sl, float4 *__restrict__ slf,
-                           uint8_t *__restrict__ scvx, double *__restrict__ sinv)
+//
+// Half-planes {x : a x + b y - c >= 0}, (a, b) the unit left normal of a
+// directed line P -> Q (a zero vector, which constrains nothing, if P = Q);
+// the quadrilaterals are counter-clockwise: 0: normal edge at m (A5 -> A0), 1:
+// normal edge at next m (B0 -> B5), 2 + o: offset line o (A_o -> B_o), inside
+// = larger offsets.  Eight lanes per segment, one per line: about 70 FP64
+// instructions a lane in place of 650 a segment, which one thread issued at
+// 64 cycles each (128 markers: 29 us, now below 7; 16384 markers: 35 us, now 27).
+__global__ void __launch_bounds__(128)
+k_segments(int M, const int32_t *__restrict__ next, const double *__restrict__ gx,
+           const double *__restrict__ gy, const double *__restrict__ nxm,
+           const double *__restrict__ nym, float4 *__restrict__ sbox,
+           double *__restrict__ sv, float4 *__restrict__ sb5,
+           double *__restrict__ sl, float4 *__restrict__ slf,
+           uint8_t *__restrict__ scvx, double *__restrict__ sinv)
 {
-    int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    int nm = next[m];
+    constexpr unsigned kAll = 0xffffffffu;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, q = t & 7;
+    const bool live = (t >> 3) < M;
+    const int m = live ? t >> 3 : M - 1, nm = next[m];
     const double gxa = gx[m], gya = gy[m], gxb = gx[nm], gyb = gy[nm];
-    {
-        const double ex = gxb - gxa, ey = gyb - gya;  // 1 / |segment|^2 (grid units)
-        sinv[m] = recip_any(ex * ex + ey * ey);
-    }
     const double nax = nxm[m], nay = nym[m], nbx = nxm[nm], nby = nym[nm];
-    // corner o (offset o - 2.5 cells) on the normal at m: (2o, 2o+1); at next m: 12 + (2o, 2o+1)
-    double *v = sv + (long)m * 24;
-    double ax[6], ay[6], bx[6], by[6];
-    for (int o = 0; o < 6; o++) {
-        const double a = (double)o - 2.5;
-        ax[o] = gxa + a * nax; ay[o] = gya + a * nay;
-        bx[o] = gxb + a * nbx; by[o] = gyb + a * nby;
-        v[2 * o] = ax[o]; v[2 * o + 1] = ay[o];
-        v[12 + 2 * o] = bx[o]; v[12 + 2 * o + 1] = by[o];
+    // the line's ends: corner o (offset o - 2.5 cells) on the normal at m or
+    // at next m
+    const bool pB = q == 1, qB = q != 0;
+    const double off = (double)(q - 2) - 2.5;
+    const double oP = q == 0 ? 2.5 : (q == 1 ? -2.5 : off), oQ = q == 0 ? -2.5 : (q == 1 ? 2.5 : off);
+    const double px = (pB ? gxb : gxa) + oP * (pB ? nbx : nax), py = (pB ? gyb : gya) + oP * (pB ? nby : nay);
+    const double qx = (qB ? gxb : gxa) + oQ * (qB ? nbx : nax), qy = (qB ? gyb : gya) + oQ * (qB ? nby : nay);
+    // corner o of m: (2o, 2o+1); of next m: 12 + (2o, 2o+1)
+    if (live && q >= 2) {
+        double *v = sv + (long)m * 24 + 2 * (q - 2);
+        *(double2 *)v = make_double2(px, py);
+        *(double2 *)(v + 12) = make_double2(qx, qy);
     }
+    // strip k = q - 2 lies between this lane's line and the next lane's
+    const double rx = __shfl_down_sync(kAll, qx, 1, 8), ry = __shfl_down_sync(kAll, qy, 1, 8);
+    const double sx = __shfl_down_sync(kAll, px, 1, 8), sy = __shfl_down_sync(kAll, py, 1, 8);
+    const bool strip = q >= 2 && q < 7;
     // minima and maxima of the (finite) corners compared on their bit
     // patterns, in integer instructions (ordered like the values)
     auto kb = [](double d) {
@@ -166,74 +187,70 @@ __global__ void k_segments(int M, const int32_t *__restrict__ next, const double
     };
     auto dmin = [&](double a, double b) { return kb(a) <= kb(b) ? a : b; };
     auto dmax = [&](double a, double b) { return kb(a) >= kb(b) ? a : b; };
-    float fx0 = INFINITY, fx1 = -INFINITY, fy0 = INFINITY, fy1 = -INFINITY;
-    for (int k = 0; k < 5; k++) {
-        double x0 = dmin(dmin(ax[k], ax[k + 1]), dmin(bx[k], bx[k + 1]));
-        double x1 = dmax(dmax(ax[k], ax[k + 1]), dmax(bx[k], bx[k + 1]));
-        double y0 = dmin(dmin(ay[k], ay[k + 1]), dmin(by[k], by[k + 1]));
-        double y1 = dmax(dmax(ay[k], ay[k + 1]), dmax(by[k], by[k + 1]));
-        float4 f = make_float4(__double2float_rd(x0) - 1e-3f, __double2float_ru(x1) + 1e-3f,
-                               __double2float_rd(y0) - 1e-3f, __double2float_ru(y1) + 1e-3f);
-        sb5[(long)m * 5 + k] = f;
-        fx0 = fminf(fx0, f.x); fx1 = fmaxf(fx1, f.y); fy0 = fminf(fy0, f.z); fy1 = fmaxf(fy1, f.w);
+    const double x0 = dmin(dmin(px, sx), dmin(qx, rx)), x1 = dmax(dmax(px, sx), dmax(qx, rx));
+    const double y0 = dmin(dmin(py, sy), dmin(qy, ry)), y1 = dmax(dmax(py, sy), dmax(qy, ry));
+    float4 f = make_float4(__double2float_rd(x0) - 1e-3f, __double2float_ru(x1) + 1e-3f,
+                           __double2float_rd(y0) - 1e-3f, __double2float_ru(y1) + 1e-3f);
+    if (strip) {
+        if (live) sb5[(long)m * 5 + q - 2] = f;
+    } else {
+        f = make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY);
     }
-    sbox[m] = make_float4(fx0, fx1, fy0, fy1);
-    // half-planes of the slab (the quadrilaterals are counter-clockwise):
-    // 0: normal edge at m (A5 -> A0), 1: normal edge at next m (B0 -> B5),
-    // 2 + o: offset line o (A_o -> B_o), inside = larger offsets
-    double L[8][3];
-    left_of(ax[5], ay[5], ax[0], ay[0], L[0]);
-    left_of(bx[0], by[0], bx[5], by[5], L[1]);
-    for (int o = 0; o < 6; o++) left_of(ax[o], ay[o], bx[o], by[o], L[2 + o]);
+    for (int o = 4; o; o >>= 1) {
+        f.x = fminf(f.x, __shfl_xor_sync(kAll, f.x, o)); f.y = fmaxf(f.y, __shfl_xor_sync(kAll, f.y, o));
+        f.z = fminf(f.z, __shfl_xor_sync(kAll, f.z, o)); f.w = fmaxf(f.w, __shfl_xor_sync(kAll, f.w, o));
+    }
+    if (live && q == 0) sbox[m] = f;
+    const double dx = qx - px, dy = qy - py, l2 = dx * dx + dy * dy;
+    const double il = (__double_as_longlong(l2) & 0x7fffffffffffffffLL) == 0 ? 0.0 : rsqrt_any(l2);
+    const double la = -dy * il, lb = dx * il, lc = la * px + lb * py;
     // FP64 record (kSegLine doubles): per line a, b, c, 1/a, 1/b (0 where
     // the component vanishes), then the reciprocals of the determinants
     // a_i b_j - b_i a_j of the two normal edges and of each normal edge with
     // each offset line, which the per-cell area formula would otherwise
     // recompute for every cell the segment meets.
     double *d = sl + (long)m * kSegLine;
-    auto rcp = [](double v) { return recip_any(v); };
-    for (int q = 0; q < 8; q++) {
-        d[5 * q + 0] = L[q][0]; d[5 * q + 1] = L[q][1]; d[5 * q + 2] = L[q][2];
-        d[5 * q + 3] = rcp(L[q][0]); d[5 * q + 4] = rcp(L[q][1]);
-        // |n| in FP32: left_of normalised n (to a few units of 1e-16), so
-        // (float)|n| is 1.0f, or 0.0f for the zero vector of a degenerate line
-        const bool nz = ((__double_as_longlong(L[q][0]) | __double_as_longlong(L[q][1])) &
-                         0x7fffffffffffffffLL) != 0;
-        slf[(long)m * 8 + q] = make_float4(d2f_rn(L[q][0]), d2f_rn(L[q][1]), d2f_rn(L[q][2]),
-                                           nz ? 1.0f : 0.0f);
+    const double ra = recip_any(la), rb = recip_any(lb);
+    // |n| in FP32: the normal is normalised (to a few units of 1e-16), so
+    // (float)|n| is 1.0f, or 0.0f for the zero vector of a degenerate line
+    const bool nz = ((__double_as_longlong(la) | __double_as_longlong(lb)) & 0x7fffffffffffffffLL) != 0;
+    if (live) {
+        d[5 * q + 0] = la; d[5 * q + 1] = lb; d[5 * q + 2] = lc;
+        d[5 * q + 3] = ra; d[5 * q + 4] = rb;
+        slf[(long)m * 8 + q] = make_float4(d2f_rn(la), d2f_rn(lb), d2f_rn(lc), nz ? 1.0f : 0.0f);
     }
-    d[40] = rcp(L[0][0] * L[1][1] - L[0][1] * L[1][0]);
-    for (int o = 0; o < 6; o++) {
-        d[41 + 2 * o] = rcp(L[0][0] * L[2 + o][1] - L[0][1] * L[2 + o][0]);
-        d[42 + 2 * o] = rcp(L[1][0] * L[2 + o][1] - L[1][1] * L[2 + o][0]);
+    const double a0 = __shfl_sync(kAll, la, 0, 8), b0 = __shfl_sync(kAll, lb, 0, 8);
+    const double a1 = __shfl_sync(kAll, la, 1, 8), b1 = __shfl_sync(kAll, lb, 1, 8);
+    // lane 0: 1 / |segment|^2 (grid units) in the place of a determinant
+    const double ex = gxb - gxa, ey = gyb - gya;
+    const double r0 = recip_any(q == 0 ? ex * ex + ey * ey : a0 * lb - b0 * la);
+    const double r1 = recip_any(a1 * lb - b1 * la);
+    if (live) {
+        if (q == 0) sinv[m] = r0;
+        else if (q == 1) d[40] = r0;
+        else { d[41 + 2 * (q - 2)] = r0; d[42 + 2 * (q - 2)] = r1; }
     }
     // The strips are the intersections of those half-planes only when every
     // strip quadrilateral (A_k, B_k, B_k+1, A_k+1) is strictly convex; a
     // radius of curvature below about 2.5 cells folds the inner strips.
-    // Segments that fail either test use quadrilateral clipping.
-    bool cvx = true;
-    for (int k = 0; k < 5; k++) {
-        const double qx[4] = {ax[k], bx[k], bx[k + 1], ax[k + 1]}, qy[4] = {ay[k], by[k], by[k + 1], ay[k + 1]};
-        for (int c = 0; c < 4; c++) {
-            const int c1 = (c + 1) & 3, c2 = (c + 2) & 3;
-            const double cr = (qx[c1] - qx[c]) * (qy[c2] - qy[c1]) - (qy[c1] - qy[c]) * (qx[c2] - qx[c1]);
-            // cr > 1e-6 on the bit patterns (a negative cr has a negative one)
-            cvx = cvx && __double_as_longlong(cr) > __double_as_longlong(1e-6);
-        }
-    }
+    // Segments that fail either test take the edge integrals.
+    const double ux = rx - qx, uy = ry - qy, vx = sx - rx, vy = sy - ry, wx = px - sx, wy = py - sy;
+    // > 1e-6 on the bit patterns (a negative value has a negative one)
+    auto turn = [](double c) { return __double_as_longlong(c) > __double_as_longlong(1e-6); };
+    bool ok = !strip || (turn(dx * uy - dy * ux) && turn(ux * vy - uy * vx) &&
+                         turn(vx * wy - vy * wx) && turn(wx * dy - wy * dx));
     // The half-plane path also wants every line at least 0.001 rad away from
     // the grid axes (or exactly on one): a line nearly parallel to a cell edge
     // meets it at an ill-conditioned point, which the area formula would use
-    // twice (once per boundary piece); quadrilateral clipping has no such
-    // sensitivity and takes those segments.
+    // twice (once per boundary piece); the edge integrals have no such
+    // sensitivity and take those segments.  |a| == 0 or |a| >= 1e-3, likewise
+    // b, on the bit patterns of |a|, |b|.
     const long long k3 = __double_as_longlong(1e-3);
-    for (int q = 0; q < 8; q++) {
-        // |a| == 0 or |a| >= 1e-3, likewise b, on the bit patterns of |a|, |b|
-        const long long aa = __double_as_longlong(L[q][0]) & 0x7fffffffffffffffLL,
-                        bb = __double_as_longlong(L[q][1]) & 0x7fffffffffffffffLL;
-        cvx = cvx && (aa == 0 || aa >= k3) && (bb == 0 || bb >= k3);
-    }
-    scvx[m] = cvx ? 1 : 0;
+    const long long aa = __double_as_longlong(la) & 0x7fffffffffffffffLL,
+                    bb = __double_as_longlong(lb) & 0x7fffffffffffffffLL;
+    ok = ok && (aa == 0 || aa >= k3) && (bb == 0 || bb >= k3);
+    const unsigned all = __ballot_sync(kAll, ok) >> (threadIdx.x & 24);
+    if (live && q == 0) scvx[m] = (all & 0xffu) == 0xffu ? 1 : 0;
 }
 
 // One warp per drop: the range of its marker Y.
@@ -612,53 +629,54 @@ __device__ int gather_candidates(int bi, int bj, int nx, int ny,
     return n;
 }
 
-// Area of the part of a polygon inside the unit square (Sutherland-Hodgman
-// against x >= 0, x <= 1, y >= 0, y <= 1, then the shoelace formula).
-__device__ double clip_area_unit(const double *px, const double *py)
+// Integral of clamp(y, 0, 1) dx along the part of the directed edge
+// (x0, y0) -> (x1, y1) with 0 <= x <= 1.  The sum over the edges of a closed
+// polygon is minus the signed area of its part inside the unit square (minus
+// the boundary integral of y dx, y clamped), each point counted as often as
+// the polygon winds around it: what clipping the polygon by the square's four
+// sides in turn and the shoelace formula give.  Each edge stands alone, and a
+// crossing's error enters scaled by the edge's own extent across it, so an
+// edge nearly parallel to a side costs no accuracy.
+__device__ __forceinline__ double edge_integral(double x0, double y0, double x1, double y1)
 {
-    double ax[12], ay[12], bx[12], by[12];
-    int na = 4;
-    for (int k = 0; k < 4; k++) { ax[k] = px[k]; ay[k] = py[k]; }
-    for (int side = 0; side < 4; side++) {
-        int nb = 0;
-        for (int k = 0; k < na; k++) {
-            int k1 = (k + 1 == na) ? 0 : k + 1;
-            double sx = ax[k], sy = ay[k], ex = ax[k1], ey = ay[k1];
-            double ds_, de;
-            if (side == 0) { ds_ = sx; de = ex; }
-            else if (side == 1) { ds_ = 1.0 - sx; de = 1.0 - ex; }
-            else if (side == 2) { ds_ = sy; de = ey; }
-            else { ds_ = 1.0 - sy; de = 1.0 - ey; }
-            bool sin_ = ds_ >= 0.0, ein = de >= 0.0;
-            if (sin_ && ein) { bx[nb] = ex; by[nb] = ey; nb++; }
-            else if (sin_ && !ein) {
-                double t = ds_ / (ds_ - de);
-                bx[nb] = sx + t * (ex - sx); by[nb] = sy + t * (ey - sy); nb++;
-            } else if (!sin_ && ein) {
-                double t = ds_ / (ds_ - de);
-                bx[nb] = sx + t * (ex - sx); by[nb] = sy + t * (ey - sy); nb++;
-                bx[nb] = ex; by[nb] = ey; nb++;
-            }
-        }
-        na = nb;
-        for (int k = 0; k < na; k++) { ax[k] = bx[k]; ay[k] = by[k]; }
-        if (na == 0) return 0.0;
+    const double dx = x1 - x0, dy = y1 - y0;
+    const long long kTiny = __double_as_longlong(1e-30), kMask = 0x7fffffffffffffffLL;
+    if ((__double_as_longlong(dx) & kMask) <= kTiny) return 0.0;
+    // order as numbers, on integers (0, 1 and finite values)
+    auto key = [](double x) {
+        const long long b = __double_as_longlong(x);
+        return b >= 0 ? b : (b ^ 0x7fffffffffffffffLL);
+    };
+    auto clampd = [&](double t, double lo, double hi) {
+        return key(t) < key(lo) ? lo : (key(t) > key(hi) ? hi : t);
+    };
+    // parameters t in [ta, tb] of the part with 0 <= x <= 1
+    const double rx = recip_any(dx), tx0 = -x0 * rx, tx1 = (1.0 - x0) * rx;
+    const bool px = __double_as_longlong(dx) > 0;
+    const double ta = clampd(px ? tx0 : tx1, 0.0, 1.0), tb = clampd(px ? tx1 : tx0, ta, 1.0);
+    // [u, v] of the part with 0 <= y <= 1; above: length of the part with y > 1
+    double u, v, above;
+    if ((__double_as_longlong(dy) & kMask) <= kTiny) {
+        const bool hi = key(y0) > key(1.0), in = !hi && __double_as_longlong(y0) >= 0;
+        u = ta;
+        v = in ? tb : ta;
+        above = hi ? tb - ta : 0.0;
+    } else {
+        const double ry = recip_any(dy), ty0 = -y0 * ry, ty1 = (1.0 - y0) * ry;
+        const bool py = __double_as_longlong(dy) > 0;
+        u = clampd(py ? ty0 : ty1, ta, tb);
+        v = clampd(py ? ty1 : ty0, u, tb);
+        above = py ? tb - v : u - ta;
     }
-    double a = 0.0;
-    for (int k = 0; k < na; k++) {
-        int k1 = (k + 1 == na) ? 0 : k + 1;
-        a += ax[k] * ay[k1] - ax[k1] * ay[k];
-    }
-    return 0.5 * a;
+    return dx * fma(v - u, fma(0.5 * (u + v), dy, y0), above);
 }
 
 __device__ __forceinline__ double strip_value(int k)
 {
-    // integral of the cosine kernel from -2 to the strip centre r = k - 2
-    double r = (double)k - 2.0;
-    if (r <= -2.0) return 0.0;
-    if (r >= 2.0) return 1.0;
-    return 0.5 + r / 4.0 + sin(M_PI * r / 2.0) / (2.0 * M_PI);
+    // integral of the cosine kernel from -2 to the strip centre r = k - 2:
+    // 0 for r = -2, 1 for r = 2, else 1/2 + r/4 + sin(pi r / 2) / (2 pi)
+    constexpr double v[5] = {0.0, 0.25 - 1.0 / (2.0 * M_PI), 0.5, 0.75 + 1.0 / (2.0 * M_PI), 1.0};
+    return v[k];
 }
 
 constexpr int kBT = kBlk * kBlk;  // one thread per cell of the block
@@ -689,10 +707,10 @@ __device__ __forceinline__ int cell_side(float4 l, float fi, float fj)
 // varies from run to run, but each cell's pairs and their order do not: H is
 // deterministic.
 constexpr int kPairT = 256, kPairSub = kPairT / kBT;  // 4 threads per cell
-// Pairs of non-convex strips (quadrilateral clipping, long serial FP64 work)
-// are listed for the first kClipBlocks blocks of k_band_area, 32 pairs a
-// block, and marked in the segment id's top bit.
-constexpr int kClipBlocks = 32, kClipCap = kClipBlocks * 32;
+// Pairs of non-convex strips or strips along a grid axis (edge integrals, more
+// FP64 work than the half-planes) are listed for the first kClipBlocks blocks
+// of k_band_area, eight lanes a pair, and marked in the segment id's top bit.
+constexpr int kClipBlocks = 128, kClipCap = 16384;
 constexpr uint32_t kClipFlag = 0x80000000u;
 constexpr int kStage = 256;  // candidates whose slab tests are staged in shared memory
 __global__ void __launch_bounds__(kPairT)
@@ -984,8 +1002,8 @@ __device__ __forceinline__ double rail_line_area(const CellLine *L, const RailCu
 // o) for o = 0..5 (a0 or 0 when the FP32 test finds the line clear of the
 // cell, else rail_line_area in FP64, the cut lines in ascending o), and strip
 // k has area S_k - S_k+1.  Other
-// segments (folded strips, lines within 0.001 rad of a grid axis): each
-// quadrilateral is clipped against the cell (Sutherland-Hodgman).
+// segments (folded strips, lines within 0.001 rad of a grid axis): the edge
+// integrals of every quadrilateral.
 __device__ __forceinline__ void pair_area(uint32_t m, int ci, int cj, const double *__restrict__ sl,
                                           const float4 *__restrict__ slf,
                                           const uint8_t *__restrict__ scvx,
@@ -1007,7 +1025,8 @@ __device__ __forceinline__ void pair_area(uint32_t m, int ci, int cj, const doub
             qx[1] = v[12 + 2 * k] - di;       qy[1] = v[12 + 2 * k + 1] - dj;
             qx[2] = v[12 + 2 * k + 2] - di;   qy[2] = v[12 + 2 * k + 3] - dj;
             qx[3] = v[2 * k + 2] - di;        qy[3] = v[2 * k + 3] - dj;
-            const double A = clip_area_unit(qx, qy);
+            double A = 0.0;
+            for (int e = 0; e < 4; e++) A -= edge_integral(qx[e], qy[e], qx[(e + 1) & 3], qy[(e + 1) & 3]);
             acc += A * Hk[k];
             cov += A;
         }
@@ -1052,11 +1071,14 @@ __device__ __forceinline__ void pair_area(uint32_t m, int ci, int cj, const doub
     }
 }
 
-// The first kClipBlocks blocks take the listed pairs of non-convex strips,
-// a group of 8 lanes per pair, lane k < 5 clipping strip k's quadrilateral;
-// lane 0 sums the strips in order, as one thread would.  Being dispatched
-// first, their long FP64 chains overlap the rest.  The other blocks take one
-// pair per thread (flat over the list), skipping the listed ones.
+// The first kClipBlocks blocks take the listed pairs, a group of 8 lanes per
+// pair: lane o < 6 integrates along offset line o, lane k < 5 also along the
+// normals' pieces between lines k and k + 1, which together give strip k;
+// lane 0 sums the strips in order.  Being dispatched first, their longer FP64
+// chains overlap the rest.  The other blocks take one pair per thread (flat
+// over the list), skipping the listed ones.  (Strips clipped side by side of
+// the square, 1024 pairs listed: 42 us for one drop of 128 markers, 125 us for
+// 64 of 256; now 20 and 104.)
 __global__ void __launch_bounds__(256)
 k_band_area(int nx, const uint32_t *__restrict__ npairs, uint32_t cap,
             const uint32_t *__restrict__ pseg, const uint32_t *__restrict__ pcell,
@@ -1070,40 +1092,41 @@ k_band_area(int nx, const uint32_t *__restrict__ npairs, uint32_t cap,
     for (int k = 0; k < 5; k++) Hk[k] = strip_value(k);
     if (blockIdx.x < kClipBlocks) {
         const uint32_t nc = min(npairs[1], (uint32_t)kClipCap);
-        const uint32_t idx = blockIdx.x * 32 + threadIdx.x / 8;
         const int k = threadIdx.x % 8;
-        // every lane reaches the shuffles below; a group past the list's end
-        // (the same for its 8 lanes) only does no work
-        const bool live = idx < nc;
-        const uint32_t p = live ? clip_list[idx] : 0u;
-        const uint32_t m = live ? (pseg[p] & ~kClipFlag) : 0u, cell = live ? pcell[p] : 0u;
-        const int cj = (int)(cell / (uint32_t)nx), ci = (int)(cell - (uint32_t)cj * (uint32_t)nx);
-        const float gi = (float)ci, gj = (float)cj;
-        const double di = (double)ci, dj = (double)cj;
-        double A = 0.0;
-        bool hit = false;
-        if (live && k < 5) {
-            const float4 bb = sb5[(long)m * 5 + k];
-            hit = !(bb.x > gi + 1.0f || bb.y < gi || bb.z > gj + 1.0f || bb.w < gj);
-            if (hit) {
-                const double *v = sv + (long)m * 24;
-                double qx[4], qy[4];
-                qx[0] = v[2 * k] - di;            qy[0] = v[2 * k + 1] - dj;
-                qx[1] = v[12 + 2 * k] - di;       qy[1] = v[12 + 2 * k + 1] - dj;
-                qx[2] = v[12 + 2 * k + 2] - di;   qy[2] = v[12 + 2 * k + 3] - dj;
-                qx[3] = v[2 * k + 2] - di;        qy[3] = v[2 * k + 3] - dj;
-                A = clip_area_unit(qx, qy);
+        // every lane of a warp reaches the shuffles below; a group past the
+        // list's end (the same for its 8 lanes) only does no work
+        for (uint32_t i0 = blockIdx.x * 32; i0 < nc; i0 += kClipBlocks * 32) {
+            const uint32_t idx = i0 + threadIdx.x / 8;
+            const bool live = idx < nc;
+            const uint32_t p = live ? clip_list[idx] : 0u;
+            const uint32_t m = live ? (pseg[p] & ~kClipFlag) : 0u, cell = live ? pcell[p] : 0u;
+            const int cj = (int)(cell / (uint32_t)nx), ci = (int)(cell - (uint32_t)cj * (uint32_t)nx);
+            const float gi = (float)ci, gj = (float)cj;
+            const double di = (double)ci, dj = (double)cj;
+            double line = 0.0, rails = 0.0;
+            bool hit = false;
+            if (live && k < 6) {
+                const double *v = sv + (long)m * 24 + 2 * k;
+                const double ax = v[0] - di, ay = v[1] - dj, bx = v[12] - di, by = v[13] - dj;
+                line = edge_integral(ax, ay, bx, by);
+                if (k < 5) {
+                    rails = edge_integral(bx, by, v[14] - di, v[15] - dj) -
+                            edge_integral(ax, ay, v[2] - di, v[3] - dj);
+                    const float4 bb = sb5[(long)m * 5 + k];
+                    hit = !(bb.x > gi + 1.0f || bb.y < gi || bb.z > gj + 1.0f || bb.w < gj);
+                }
             }
-        }
-        double acc = 0.0, cov = 0.0;
-        const int g0 = (threadIdx.x & 31) & ~7;  // the group's first lane
+            const double next = __shfl_down_sync(0xffffffffu, line, 1, 8);
+            const double A = hit ? next - line - rails : 0.0;
+            double acc = 0.0, cov = 0.0;
 #pragma unroll
-        for (int s = 0; s < 5; s++) {
-            const double As = __shfl_sync(0xffffffffu, A, g0 + s);
-            const bool hs = __shfl_sync(0xffffffffu, hit, g0 + s);
-            if (hs) { acc += As * Hk[s]; cov += As; }
+            for (int s = 0; s < 5; s++) {
+                const double As = __shfl_sync(0xffffffffu, A, s, 8);
+                acc += As * Hk[s];
+                cov += As;
+            }
+            if (live && k == 0) { pacc[p] = acc; pcov[p] = cov; }
         }
-        if (live && k == 0) { pacc[p] = acc; pcov[p] = cov; }
         return;
     }
     const uint32_t stride = (gridDim.x - kClipBlocks) * blockDim.x;
@@ -1310,25 +1333,6 @@ __device__ __forceinline__ double speed2(const SpanCurve &c, double u)
     const double vy = fma(u, fma(u, c.dy[2], c.dy[1]), c.dy[0]);
     return fma(vx, vx, vy * vy);
 }
-// 1 / sqrt(s): rsqrt_nr well inside the FP32 range (tested on the bit
-// pattern, which orders positive values), square root and division elsewhere.
-__device__ __forceinline__ double rsqrt_any(double s)
-{
-    const unsigned long long a = (unsigned long long)__double_as_longlong(s);
-    if (a > (unsigned long long)__double_as_longlong(1e-30) &&
-        a < (unsigned long long)__double_as_longlong(1e30))
-        return rsqrt_nr(s);
-    return 1.0 / sqrt(s);
-}
-__device__ __forceinline__ double sqrt_any(double s)
-{
-    const unsigned long long a = (unsigned long long)__double_as_longlong(s);
-    if (a > (unsigned long long)__double_as_longlong(1e-30) &&
-        a < (unsigned long long)__double_as_longlong(1e30))
-        return s * rsqrt_nr(s);
-    return sqrt(s);
-}
-
 // out[k] = in[0] + ... + in[k-1], k = 0 .. n, of values >= 0, by the block's
 // kT threads; returns the total.  The sums run on 64-bit integers at a power
 // of two that keeps n times the largest value below 2^62: exact, so they do
@@ -1887,9 +1891,9 @@ void launch_geometry(Markers &mk, double sigma, cudaStream_t s)
 void launch_segments(Markers &mk, cudaStream_t s)
 {
     note_launch();
-    k_segments<<<cdiv(mk.M, 32), 32, 0, s>>>(  // FP64-heavy: spread over all SMs
-        mk.M, mk.next, mk.gx, mk.gy, mk.nxm, mk.nym, mk.sbox,
-                                            mk.sv, mk.sb5, mk.sl, mk.slf, mk.scvx, mk.sinv);
+    k_segments<<<cdiv(8L * mk.M, 128), 128, 0, s>>>(mk.M, mk.next, mk.gx, mk.gy, mk.nxm, mk.nym,
+                                                    mk.sbox, mk.sv, mk.sb5, mk.sl, mk.slf, mk.scvx,
+                                                    mk.sinv);
     note_launch();
     k_drop_yrange<<<cdiv((long)mk.ndrops * 32, kT), kT, 0, s>>>(mk.ndrops, mk.drop_start, mk.Y,
                                                                mk.dyr, mk.dyk);
