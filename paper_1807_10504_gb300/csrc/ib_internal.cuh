@@ -374,7 +374,7 @@ struct Markers {
     int32_t *drop_start = nullptr, *drop_of = nullptr, *next = nullptr;
     uint32_t *key = nullptr, *tmp_ids = nullptr, *ids = nullptr,
              *cell_count = nullptr, *cell_start = nullptr, *scan_part = nullptr,
-             *bcount = nullptr, *bactive = nullptr, *flags = nullptr;
+             *bcount = nullptr, *blist = nullptr, *nact = nullptr, *flags = nullptr;
     std::vector<int32_t> drop_start_h;
     int max_drop = 0;
     void *mem = nullptr;

@@ -385,19 +385,28 @@ __global__ void k_rerank(int M, const uint32_t *__restrict__ key,
     ids[s + r] = (uint32_t)m;
 }
 
+// list[0 .. *count): the active blocks, in no fixed order (each block's results
+// are its own); *count zero before.  The kernels over active blocks run a
+// resident grid over this list: with a CTA for every block of the grid the
+// empty ones alone cost 5 us a launch at 1024^2 and 20 at 2048^2.
 __global__ void k_block_active(int bnx, int bny, const uint32_t *__restrict__ bcount,
-                               uint32_t *__restrict__ active)
+                               uint32_t *__restrict__ list, uint32_t *__restrict__ count)
 {
     int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= bnx * bny) return;
-    int bi = b % bnx, bj = b / bnx;
     uint32_t any = 0;
-    for (int dj = -1; dj <= 1; dj++)
-        for (int di = -1; di <= 1; di++) {
-            int ii = bi + di, jj = bj + dj;
-            if (ii >= 0 && ii < bnx && jj >= 0 && jj < bny) any |= bcount[jj * bnx + ii];
-        }
-    active[b] = any ? 1u : 0u;
+    if (b < bnx * bny) {
+        int bi = b % bnx, bj = b / bnx;
+        for (int dj = -1; dj <= 1; dj++)
+            for (int di = -1; di <= 1; di++) {
+                int ii = bi + di, jj = bj + dj;
+                if (ii >= 0 && ii < bnx && jj >= 0 && jj < bny) any |= bcount[jj * bnx + ii];
+            }
+    }
+    const unsigned vote = __ballot_sync(0xffffffffu, any != 0), lane = threadIdx.x & 31;
+    uint32_t at = 0;
+    if (lane == 0 && vote) at = atomicAdd(count, (uint32_t)__popc(vote));
+    at = __shfl_sync(0xffffffffu, at, 0);
+    if (any) list[at + __popc(vote & ((1u << lane) - 1u))] = (uint32_t)b;
 }
 
 // ------------------------------------------------------------ interpolation
@@ -484,30 +493,33 @@ k_spread_tab(int M, int kernel, double ih, double x0, double y0, const double *_
 // the whole grid took 624 us at 1024^2 with 16384 markers, this 38 us and the
 // records 8 us.
 __global__ void __launch_bounds__(2 * kBlk * kBlk)
-k_spread_conv(int nx, int ny, int bnx, const uint32_t *__restrict__ bactive,
+k_spread_conv(int nx, int ny, int bnx, const uint32_t *__restrict__ blist,
+              const uint32_t *__restrict__ nact,
               const uint32_t *__restrict__ cell_start, const uint32_t *__restrict__ ids,
               const double *__restrict__ tab, double *__restrict__ Fx, double *__restrict__ Fy)
 {
-    if (!bactive[blockIdx.y * bnx + blockIdx.x]) return;
     const int d = threadIdx.x / (kBlk * kBlk), c = threadIdx.x % (kBlk * kBlk);
-    const int i = blockIdx.x * kBlk + c % kBlk, j = blockIdx.y * kBlk + c / kBlk;
-    if (i >= nx || j >= ny || (d == 0 ? i == 0 : j == 0)) return;
-    const int ia = max(i - 2, 0), ib = min(d ? i + 2 : i + 1, nx - 1);
-    const int ja = max(j - 2, 0), jb = min(d ? j + 1 : j + 2, ny - 1);
-    double acc = 0.0;
-    for (int jj = ja; jj <= jb; jj++) {
-        const uint32_t s = cell_start[(long)jj * nx + ia], e = cell_start[(long)jj * nx + ib + 1];
-        for (uint32_t t = s; t < e; t++) {
-            const double *o = tab + (long)ids[t] * kTab + 10 * d;
-            const double2 cf = *(const double2 *)(o + 8);
-            const long long bits = __double_as_longlong(cf.y);
-            const int a = i - (int)(unsigned)bits, b = j - (int)(bits >> 32);
-            if ((unsigned)a > 3u || (unsigned)b > 3u) continue;
-            acc += cf.x * (o[a] * o[4 + b]);
+    for (uint32_t ab = blockIdx.x; ab < *nact; ab += gridDim.x) {
+        const int bl = (int)blist[ab], bj = bl / bnx, bi = bl - bj * bnx;
+        const int i = bi * kBlk + c % kBlk, j = bj * kBlk + c / kBlk;
+        if (i >= nx || j >= ny || (d == 0 ? i == 0 : j == 0)) continue;
+        const int ia = max(i - 2, 0), ib = min(d ? i + 2 : i + 1, nx - 1);
+        const int ja = max(j - 2, 0), jb = min(d ? j + 1 : j + 2, ny - 1);
+        double acc = 0.0;
+        for (int jj = ja; jj <= jb; jj++) {
+            const uint32_t s = cell_start[(long)jj * nx + ia], e = cell_start[(long)jj * nx + ib + 1];
+            for (uint32_t t = s; t < e; t++) {
+                const double *o = tab + (long)ids[t] * kTab + 10 * d;
+                const double2 cf = *(const double2 *)(o + 8);
+                const long long bits = __double_as_longlong(cf.y);
+                const int a = i - (int)(unsigned)bits, b = j - (int)(bits >> 32);
+                if ((unsigned)a > 3u || (unsigned)b > 3u) continue;
+                acc += cf.x * (o[a] * o[4 + b]);
+            }
         }
+        if (d == 0) Fx[(long)j * (nx + 1) + i] = acc;
+        else Fy[(long)j * nx + i] = acc;
     }
-    if (d == 0) Fx[(long)j * (nx + 1) + i] = acc;
-    else Fy[(long)j * nx + i] = acc;
 }
 
 // ------------------------------------------------------------ inside / outside
@@ -714,8 +726,8 @@ constexpr int kClipBlocks = 128, kClipCap = 16384;
 constexpr uint32_t kClipFlag = 0x80000000u;
 constexpr int kStage = 256;  // candidates whose slab tests are staged in shared memory
 __global__ void __launch_bounds__(kPairT)
-k_band_pairs(int nx, int ny, int bnx, const uint32_t *__restrict__ bactive,
-             const uint32_t *__restrict__ cell_start, const uint32_t *__restrict__ ids,
+k_band_pairs(int nx, int ny, int bnx, const uint32_t *__restrict__ blist,
+             const uint32_t *__restrict__ nact, const uint32_t *__restrict__ cell_start, const uint32_t *__restrict__ ids,
              const float4 *__restrict__ slf, const uint8_t *__restrict__ scvx,
              const float4 *__restrict__ sbox, uint32_t cap, uint32_t *__restrict__ npairs,
              uint32_t *__restrict__ pseg, uint32_t *__restrict__ pcell, uint2 *__restrict__ crange,
@@ -727,106 +739,108 @@ k_band_pairs(int nx, int ny, int bnx, const uint32_t *__restrict__ bactive,
     __shared__ uint8_t s_cvx[kStage];
     __shared__ uint32_t cnt[kPairT], wsum[kPairT / 32 + 1];
     __shared__ uint32_t base;
-    const int bi = blockIdx.x, bj = blockIdx.y;
-    if (!bactive[bj * bnx + bi]) return;
-    const int n = gather_candidates(bi, bj, nx, ny, cell_start, ids, cand, tmp, flags);
-    const int ns = min(n, kStage);
-    for (int q = threadIdx.x; q < ns; q += kPairT) {
-        const uint32_t m = cand[q];
-        s_box[q] = sbox[m];
-        s_l[0][q] = slf[(long)m * 8 + 0];
-        s_l[1][q] = slf[(long)m * 8 + 1];
-        s_l[2][q] = slf[(long)m * 8 + 2];
-        s_l[3][q] = slf[(long)m * 8 + 7];
-        s_cvx[q] = scvx[m];
-    }
-    __syncthreads();
-    const int t = threadIdx.x, cl = t / kPairSub, sub = t - cl * kPairSub;
-    const int i = bi * kBlk + (cl % kBlk), j = bj * kBlk + (cl / kBlk);
-    const bool live = i < nx && j < ny;
-    const float fi = (float)i, fj = (float)j;
-    auto meets = [&](int q) {
-        const uint32_t m = cand[q];
-        const bool st = q < kStage;
-        const float4 b = st ? s_box[q] : sbox[m];
-        if (b.x > fi + 1.0f || b.y < fi || b.z > fj + 1.0f || b.w < fj) return false;
-        if (!(st ? s_cvx[q] : scvx[m])) return true;
-        const float4 *L = slf + (long)m * 8;
-        return cell_side(st ? s_l[0][q] : L[0], fi, fj) >= 0 &&
-               cell_side(st ? s_l[1][q] : L[1], fi, fj) >= 0 &&
-               cell_side(st ? s_l[2][q] : L[2], fi, fj) >= 0 &&
-               cell_side(st ? s_l[3][q] : L[7], fi, fj) <= 0;
-    };
-    // this thread's contiguous share of the (ascending) candidate list; its
-    // test results are kept as bits in tmp (free after the gathering: four
-    // words a thread, word w of thread t at tmp[w * kPairT + t]) for the
-    // second pass, when the block has at most 4 x 128 candidates
-    const int q0 = (n * sub) / kPairSub, q1 = (n * (sub + 1)) / kPairSub;
-    static_assert(kMaxCand >= 4 * kPairT, "four words of tmp per thread");
-    const bool keep = n <= kPairSub * 128;
-    uint32_t c = 0;
-    if (live) {
-        uint32_t word = 0;
-        for (int q = q0; q < q1; q++) {
-            const bool mt = meets(q);
-            c += mt ? 1u : 0u;
-            if (keep) {
-                const int b = q - q0;
-                word |= (mt ? 1u : 0u) << (b & 31);
-                if ((b & 31) == 31 || q + 1 == q1) { tmp[(b >> 5) * kPairT + t] = word; word = 0; }
+    for (uint32_t ab = blockIdx.x; ab < *nact; ab += gridDim.x) {
+        const int bl = (int)blist[ab], bj = bl / bnx, bi = bl - bj * bnx;
+        __syncthreads();  // the block before is done with the shared arrays
+        const int n = gather_candidates(bi, bj, nx, ny, cell_start, ids, cand, tmp, flags);
+        const int ns = min(n, kStage);
+        for (int q = threadIdx.x; q < ns; q += kPairT) {
+            const uint32_t m = cand[q];
+            s_box[q] = sbox[m];
+            s_l[0][q] = slf[(long)m * 8 + 0];
+            s_l[1][q] = slf[(long)m * 8 + 1];
+            s_l[2][q] = slf[(long)m * 8 + 2];
+            s_l[3][q] = slf[(long)m * 8 + 7];
+            s_cvx[q] = scvx[m];
+        }
+        __syncthreads();
+        const int t = threadIdx.x, cl = t / kPairSub, sub = t - cl * kPairSub;
+        const int i = bi * kBlk + (cl % kBlk), j = bj * kBlk + (cl / kBlk);
+        const bool live = i < nx && j < ny;
+        const float fi = (float)i, fj = (float)j;
+        auto meets = [&](int q) {
+            const uint32_t m = cand[q];
+            const bool st = q < kStage;
+            const float4 b = st ? s_box[q] : sbox[m];
+            if (b.x > fi + 1.0f || b.y < fi || b.z > fj + 1.0f || b.w < fj) return false;
+            if (!(st ? s_cvx[q] : scvx[m])) return true;
+            const float4 *L = slf + (long)m * 8;
+            return cell_side(st ? s_l[0][q] : L[0], fi, fj) >= 0 &&
+                   cell_side(st ? s_l[1][q] : L[1], fi, fj) >= 0 &&
+                   cell_side(st ? s_l[2][q] : L[2], fi, fj) >= 0 &&
+                   cell_side(st ? s_l[3][q] : L[7], fi, fj) <= 0;
+        };
+        // this thread's contiguous share of the (ascending) candidate list; its
+        // test results are kept as bits in tmp (free after the gathering: four
+        // words a thread, word w of thread t at tmp[w * kPairT + t]) for the
+        // second pass, when the block has at most 4 x 128 candidates
+        const int q0 = (n * sub) / kPairSub, q1 = (n * (sub + 1)) / kPairSub;
+        static_assert(kMaxCand >= 4 * kPairT, "four words of tmp per thread");
+        const bool keep = n <= kPairSub * 128;
+        uint32_t c = 0;
+        if (live) {
+            uint32_t word = 0;
+            for (int q = q0; q < q1; q++) {
+                const bool mt = meets(q);
+                c += mt ? 1u : 0u;
+                if (keep) {
+                    const int b = q - q0;
+                    word |= (mt ? 1u : 0u) << (b & 31);
+                    if ((b & 31) == 31 || q + 1 == q1) { tmp[(b >> 5) * kPairT + t] = word; word = 0; }
+                }
             }
         }
-    }
-    // exclusive scan over threads (cell-major, then share): warp scans, then
-    // the warp totals
-    const int lane = t & 31, warp = t >> 5;
-    uint32_t incl = c;
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    if (t == 0) {
-        uint32_t acc = 0;
-        for (int w = 0; w < kPairT / 32; w++) { const uint32_t v = wsum[w]; wsum[w] = acc; acc += v; }
-        wsum[kPairT / 32] = acc;
-        const uint32_t b0 = atomicAdd(npairs, acc);
-        if (b0 > cap || acc > cap - b0) {
-            atomicOr(&flags[1], 1u);
-            base = 0xffffffffu;
-        } else {
-            base = b0;
+        // exclusive scan over threads (cell-major, then share): warp scans, then
+        // the warp totals
+        const int lane = t & 31, warp = t >> 5;
+        uint32_t incl = c;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
         }
-    }
-    __syncthreads();
-    const uint32_t excl = wsum[warp] + incl - c;
-    cnt[t] = excl;
-    __syncthreads();
-    if (!live) return;
-    const long cidx = (long)j * nx + i;
-    if (base == 0xffffffffu) {
-        if (sub == 0) crange[cidx] = make_uint2(0u, 0u);
-        return;
-    }
-    if (sub == 0) {
-        const uint32_t end = (cl + 1 < kBT) ? cnt[t + kPairSub] : wsum[kPairT / 32];
-        crange[cidx] = make_uint2(base + excl, end - excl);
-    }
-    uint32_t o = base + excl;
-    for (int q = q0; q < q1; q++)
-        if (keep ? ((tmp[((q - q0) >> 5) * kPairT + t] >> ((q - q0) & 31)) & 1u) : meets(q)) {
-            uint32_t seg = cand[q];
-            // a pair of a non-convex strip goes to the clip list of
-            // k_band_area (while it has room), marked in the id's top bit
-            if (!(q < kStage ? s_cvx[q] : scvx[seg])) {
-                const uint32_t at = atomicAdd(npairs + 1, 1u);
-                if (at < kClipCap) { clip_list[at] = o; seg |= kClipFlag; }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        if (t == 0) {
+            uint32_t acc = 0;
+            for (int w = 0; w < kPairT / 32; w++) { const uint32_t v = wsum[w]; wsum[w] = acc; acc += v; }
+            wsum[kPairT / 32] = acc;
+            const uint32_t b0 = atomicAdd(npairs, acc);
+            if (b0 > cap || acc > cap - b0) {
+                atomicOr(&flags[1], 1u);
+                base = 0xffffffffu;
+            } else {
+                base = b0;
             }
-            pseg[o] = seg;
-            pcell[o] = (uint32_t)cidx;
-            o++;
         }
+        __syncthreads();
+        const uint32_t excl = wsum[warp] + incl - c;
+        cnt[t] = excl;
+        __syncthreads();
+        if (!live) continue;
+        const long cidx = (long)j * nx + i;
+        if (base == 0xffffffffu) {
+            if (sub == 0) crange[cidx] = make_uint2(0u, 0u);
+            continue;
+        }
+        if (sub == 0) {
+            const uint32_t end = (cl + 1 < kBT) ? cnt[t + kPairSub] : wsum[kPairT / 32];
+            crange[cidx] = make_uint2(base + excl, end - excl);
+        }
+        uint32_t o = base + excl;
+        for (int q = q0; q < q1; q++)
+            if (keep ? ((tmp[((q - q0) >> 5) * kPairT + t] >> ((q - q0) & 31)) & 1u) : meets(q)) {
+                uint32_t seg = cand[q];
+                // a pair of a non-convex strip goes to the clip list of
+                // k_band_area (while it has room), marked in the id's top bit
+                if (!(q < kStage ? s_cvx[q] : scvx[seg])) {
+                    const uint32_t at = atomicAdd(npairs + 1, 1u);
+                    if (at < kClipCap) { clip_list[at] = o; seg |= kClipFlag; }
+                }
+                pseg[o] = seg;
+                pcell[o] = (uint32_t)cidx;
+                o++;
+            }
+    }
 }
 
 // A bounding line of a strip in the cell's local frame (the cell is the unit
@@ -1143,21 +1157,22 @@ k_band_area(int nx, const uint32_t *__restrict__ npairs, uint32_t cap,
 }
 
 __global__ void __launch_bounds__(kBT)
-k_band_sum(int nx, int ny, int bnx, const uint32_t *__restrict__ bactive,
-           const uint2 *__restrict__ crange, const double *__restrict__ pacc,
-           const double *__restrict__ pcov, double *__restrict__ H)
+k_band_sum(int nx, int ny, int bnx, const uint32_t *__restrict__ blist,
+           const uint32_t *__restrict__ nact, const uint2 *__restrict__ crange,
+           const double *__restrict__ pacc, const double *__restrict__ pcov, double *__restrict__ H)
 {
-    const int bi = blockIdx.x, bj = blockIdx.y;
-    if (!bactive[bj * bnx + bi]) return;
-    const int i = bi * kBlk + (threadIdx.x % kBlk), j = bj * kBlk + (threadIdx.x / kBlk);
-    if (i >= nx || j >= ny) return;
-    const long cidx = (long)j * nx + i;
-    const uint2 r = crange[cidx];
-    double acc = 0.0, cov = 0.0;
-    for (uint32_t p = r.x; p < r.x + r.y; p++) { acc += pacc[p]; cov += pcov[p]; }
-    double unc = 1.0 - cov;
-    if (unc < 0.0) unc = 0.0;
-    H[cidx] = acc + unc * H[cidx];
+    for (uint32_t ab = blockIdx.x; ab < *nact; ab += gridDim.x) {
+        const int bl = (int)blist[ab], bj = bl / bnx, bi = bl - bj * bnx;
+        const int i = bi * kBlk + (threadIdx.x % kBlk), j = bj * kBlk + (threadIdx.x / kBlk);
+        if (i >= nx || j >= ny) continue;
+        const long cidx = (long)j * nx + i;
+        const uint2 r = crange[cidx];
+        double acc = 0.0, cov = 0.0;
+        for (uint32_t p = r.x; p < r.x + r.y; p++) { acc += pacc[p]; cov += pcov[p]; }
+        double unc = 1.0 - cov;
+        if (unc < 0.0) unc = 0.0;
+        H[cidx] = acc + unc * H[cidx];
+    }
 }
 
 // Irrotational face force F = f_face (H_ij - H_nb) / h on the x-face left of
@@ -1174,7 +1189,8 @@ k_band_sum(int nx, int ny, int bnx, const uint32_t *__restrict__ bactive,
 constexpr int kIrrT = 2 * kBT;  // one thread per face of the block
 constexpr int kNear = 8;        // survivors listed per face
 __global__ void __launch_bounds__(kIrrT)
-k_spread_irrot(int nx, int ny, double ih, int bnx, const uint32_t *__restrict__ bactive,
+k_spread_irrot(int nx, int ny, double ih, int bnx, const uint32_t *__restrict__ blist,
+               const uint32_t *__restrict__ nact,
                const uint32_t *__restrict__ cell_start, const uint32_t *__restrict__ ids,
                const int32_t *__restrict__ next, const double *__restrict__ gx,
                const double *__restrict__ gy, const double *__restrict__ sinv,
@@ -1189,92 +1205,94 @@ k_spread_irrot(int nx, int ny, double ih, int bnx, const uint32_t *__restrict__ 
     __shared__ double wdH[kIrrT];
     __shared__ uint16_t near_q[kNear][kIrrT];  // survivors of the FP32 screen, per face
     __shared__ int nwork;
-    const int bi = blockIdx.x, bj = blockIdx.y;
-    if (!bactive[bj * bnx + bi]) return;
-    const int n = gather_candidates(bi, bj, nx, ny, cell_start, ids, cand, tmp, flags);
-    for (int q = threadIdx.x; q < n; q += blockDim.x) {
-        const int m = (int)cand[q], nm = next[m];
-        const float ax = gxf[m], ay = gyf[m], ex = gxf[nm] - ax, ey = gyf[nm] - ay;
-        seg[q] = make_float4(ax, ay, ex, ey);
-        seg_il[q] = 1.0f / (ex * ex + ey * ey);
-    }
-    if (threadIdx.x == 0) nwork = 0;
-    __syncthreads();
-    // face f: dir = f / 64 (0: x-face left of the cell, 1: y-face below), cell f % 64
-    auto face = [&](int f, int &dir, int &i, int &j) {
-        dir = f / kBT;
-        const int c = f - dir * kBT;
-        i = bi * kBlk + (c % kBlk);
-        j = bj * kBlk + (c / kBlk);
-    };
-    {
-        const int f = threadIdx.x;
-        int dir, i, j;
-        face(f, dir, i, j);
-        if (i < nx && j < ny && !(dir == 0 && i == 0) && !(dir == 1 && j == 0)) {
-            const double dH = dir == 0 ? H[(long)j * nx + i] - H[(long)j * nx + i - 1]
-                                       : H[(long)j * nx + i] - H[(long)(j - 1) * nx + i];
-            if (dH != 0.0) {
-                const int w = atomicAdd(&nwork, 1);
-                work[w] = (uint8_t)f;
-                wdH[w] = dH;
-            } else if (dir == 0) {
-                Fx[(long)j * (nx + 1) + i] = 0.0;
-            } else {
-                Fy[(long)j * nx + i] = 0.0;
+    for (uint32_t ab = blockIdx.x; ab < *nact; ab += gridDim.x) {
+        const int bl = (int)blist[ab], bj = bl / bnx, bi = bl - bj * bnx;
+        __syncthreads();  // the block before is done with the shared arrays
+        const int n = gather_candidates(bi, bj, nx, ny, cell_start, ids, cand, tmp, flags);
+        for (int q = threadIdx.x; q < n; q += blockDim.x) {
+            const int m = (int)cand[q], nm = next[m];
+            const float ax = gxf[m], ay = gyf[m], ex = gxf[nm] - ax, ey = gyf[nm] - ay;
+            seg[q] = make_float4(ax, ay, ex, ey);
+            seg_il[q] = 1.0f / (ex * ex + ey * ey);
+        }
+        if (threadIdx.x == 0) nwork = 0;
+        __syncthreads();
+        // face f: dir = f / 64 (0: x-face left of the cell, 1: y-face below), cell f % 64
+        auto face = [&](int f, int &dir, int &i, int &j) {
+            dir = f / kBT;
+            const int c = f - dir * kBT;
+            i = bi * kBlk + (c % kBlk);
+            j = bj * kBlk + (c / kBlk);
+        };
+        {
+            const int f = threadIdx.x;
+            int dir, i, j;
+            face(f, dir, i, j);
+            if (i < nx && j < ny && !(dir == 0 && i == 0) && !(dir == 1 && j == 0)) {
+                const double dH = dir == 0 ? H[(long)j * nx + i] - H[(long)j * nx + i - 1]
+                                           : H[(long)j * nx + i] - H[(long)(j - 1) * nx + i];
+                if (dH != 0.0) {
+                    const int w = atomicAdd(&nwork, 1);
+                    work[w] = (uint8_t)f;
+                    wdH[w] = dH;
+                } else if (dir == 0) {
+                    Fx[(long)j * (nx + 1) + i] = 0.0;
+                } else {
+                    Fy[(long)j * nx + i] = 0.0;
+                }
             }
         }
-    }
-    __syncthreads();
-    if ((int)threadIdx.x >= nwork) return;
-    int dir, i, j;
-    face(work[threadIdx.x], dir, i, j);
-    const double dH = wdH[threadIdx.x];
-    const double qx = dir == 0 ? (double)i : (double)i + 0.5;
-    const double qy = dir == 0 ? (double)j + 0.5 : (double)j;
-    // FP32 screen: for faces within the band (distance below ~4 cells) and
-    // coordinates below 2^12 cells the FP32 squared distances carry an error
-    // below 2e-3 (grid units), so the exact nearest segment is among those
-    // within best + 0.01 of the FP32 minimum.
-    const float fqx = d2f_rn(qx), fqy = d2f_rn(qy);
-    auto d2f = [&](int q) {
-        const float4 sg = seg[q];
-        float t = ((fqx - sg.x) * sg.z + (fqy - sg.y) * sg.w) * seg_il[q];
-        t = fminf(fmaxf(t, 0.0f), 1.0f);
-        const float dx = sg.x + t * sg.z - fqx, dy = sg.y + t * sg.w - fqy;
-        return dx * dx + dy * dy;
-    };
-    float best32 = INFINITY;
-    for (int q = 0; q < n; q++) best32 = fminf(best32, d2f(q));
-    const float lim = best32 + 0.01f;
-    static_assert(kMaxCand <= 65536, "candidate index in 16 bits");
-    int cnt = 0;
-    for (int q = 0; q < n; q++)
-        if (!(d2f(q) > lim)) {
-            if (cnt < kNear) near_q[cnt][threadIdx.x] = (uint16_t)q;
-            cnt++;
-        }
-    double best = INFINITY, fb = 0.0;
-    auto eval = [&](int q) {
-        const int m = (int)cand[q], nm = next[m];
-        const double ax = gx[m], ay = gy[m];
-        const double ex = gx[nm] - ax, ey = gy[nm] - ay;
-        double t = ((qx - ax) * ex + (qy - ay) * ey) * sinv[m];
-        if (t < 0.0) t = 0.0;
-        if (t > 1.0) t = 1.0;
-        const double dx = ax + t * ex - qx, dy = ay + t * ey - qy;
-        const double d2 = dx * dx + dy * dy;
-        if (d2 < best) { best = d2; fb = (1.0 - t) * fmag[m] + t * fmag[nm]; }
-    };
-    if (cnt <= kNear) {
-        for (int k = 0; k < cnt; k++) eval(near_q[k][threadIdx.x]);
-    } else {
+        __syncthreads();
+        if ((int)threadIdx.x >= nwork) continue;
+        int dir, i, j;
+        face(work[threadIdx.x], dir, i, j);
+        const double dH = wdH[threadIdx.x];
+        const double qx = dir == 0 ? (double)i : (double)i + 0.5;
+        const double qy = dir == 0 ? (double)j + 0.5 : (double)j;
+        // FP32 screen: for faces within the band (distance below ~4 cells) and
+        // coordinates below 2^12 cells the FP32 squared distances carry an error
+        // below 2e-3 (grid units), so the exact nearest segment is among those
+        // within best + 0.01 of the FP32 minimum.
+        const float fqx = d2f_rn(qx), fqy = d2f_rn(qy);
+        auto d2f = [&](int q) {
+            const float4 sg = seg[q];
+            float t = ((fqx - sg.x) * sg.z + (fqy - sg.y) * sg.w) * seg_il[q];
+            t = fminf(fmaxf(t, 0.0f), 1.0f);
+            const float dx = sg.x + t * sg.z - fqx, dy = sg.y + t * sg.w - fqy;
+            return dx * dx + dy * dy;
+        };
+        float best32 = INFINITY;
+        for (int q = 0; q < n; q++) best32 = fminf(best32, d2f(q));
+        const float lim = best32 + 0.01f;
+        static_assert(kMaxCand <= 65536, "candidate index in 16 bits");
+        int cnt = 0;
         for (int q = 0; q < n; q++)
-            if (!(d2f(q) > lim)) eval(q);
+            if (!(d2f(q) > lim)) {
+                if (cnt < kNear) near_q[cnt][threadIdx.x] = (uint16_t)q;
+                cnt++;
+            }
+        double best = INFINITY, fb = 0.0;
+        auto eval = [&](int q) {
+            const int m = (int)cand[q], nm = next[m];
+            const double ax = gx[m], ay = gy[m];
+            const double ex = gx[nm] - ax, ey = gy[nm] - ay;
+            double t = ((qx - ax) * ex + (qy - ay) * ey) * sinv[m];
+            if (t < 0.0) t = 0.0;
+            if (t > 1.0) t = 1.0;
+            const double dx = ax + t * ex - qx, dy = ay + t * ey - qy;
+            const double d2 = dx * dx + dy * dy;
+            if (d2 < best) { best = d2; fb = (1.0 - t) * fmag[m] + t * fmag[nm]; }
+        };
+        if (cnt <= kNear) {
+            for (int k = 0; k < cnt; k++) eval(near_q[k][threadIdx.x]);
+        } else {
+            for (int q = 0; q < n; q++)
+                if (!(d2f(q) > lim)) eval(q);
+        }
+        const double F = fb * dH * ih;
+        if (dir == 0) Fx[(long)j * (nx + 1) + i] = F;
+        else Fy[(long)j * nx + i] = F;
     }
-    const double F = fb * dH * ih;
-    if (dir == 0) Fx[(long)j * (nx + 1) + i] = F;
-    else Fy[(long)j * nx + i] = F;
 }
 
 // ------------------------------------------------------------ B-spline
@@ -1806,7 +1824,7 @@ cudaError_t markers_alloc(Markers &mk, int M, int ndrops, int nx, int ny, double
                    al((size_t)M * 24 * 8) + al((size_t)M * kSegLine * 8) + al((size_t)M * 8 * 16) + al((size_t)M * 5 * 16) + al(M * 8) + al(M) + al(M * 8) +
                    al(64) + al(pair_cap * 4) * 2 + al(pair_cap * 8) * 2 + al(ncell * 8) +
                    al((ndrops + 1) * 4) + al(M * 4) * 5 + al(ncell * 4) +
-                   al((ncell + 1) * 4) + al(nparts * 4) + al(nb * 4) * 2 + al(64) +
+                   al((ncell + 1) * 4) + al(nparts * 4) + al((nb + 1) * 4) + al(nb * 4) + al(64) +
                    al((size_t)nx * 8) + al((size_t)kClipCap * 4) + al((size_t)M * kTab * 8);
     cudaError_t e = cudaMalloc(&mk.mem, bytes);
     if (e != cudaSuccess) { mk.mem = nullptr; return e; }
@@ -1842,7 +1860,8 @@ cudaError_t markers_alloc(Markers &mk, int M, int ndrops, int nx, int ny, double
     mk.cell_count = (uint32_t *)take(ncell * 4);
     mk.cell_start = (uint32_t *)take((ncell + 1) * 4);
     mk.scan_part = (uint32_t *)take(nparts * 4);
-    mk.bcount = (uint32_t *)take(nb * 4); mk.bactive = (uint32_t *)take(nb * 4);
+    mk.bcount = (uint32_t *)take((nb + 1) * 4); mk.blist = (uint32_t *)take(nb * 4);
+    mk.nact = mk.bcount + nb;
     mk.flags = (uint32_t *)take(64);
     mk.colkey = (unsigned long long *)take((size_t)nx * 8);
     mk.clip_list = (uint32_t *)take((size_t)kClipCap * 4);
@@ -1903,7 +1922,7 @@ void launch_sort(Markers &mk, cudaStream_t s)
 {
     long ncell = (long)mk.nx * mk.ny;
     cudaMemsetAsync(mk.cell_count, 0, ncell * 4, s);
-    cudaMemsetAsync(mk.bcount, 0, (size_t)mk.bnx * mk.bny * 4, s);
+    cudaMemsetAsync(mk.bcount, 0, ((size_t)mk.bnx * mk.bny + 1) * 4, s);  // and *nact
     note_launch();
     k_keys<<<cdiv(mk.M, kT), kT, 0, s>>>(mk.M, mk.X, mk.Y, mk.x0, mk.y0, mk.h, mk.nx, mk.ny,
                                         mk.bnx, mk.key, mk.cell_count, mk.bcount);
@@ -1921,7 +1940,7 @@ void launch_sort(Markers &mk, cudaStream_t s)
     k_rerank<<<cdiv(mk.M, kT), kT, 0, s>>>(mk.M, mk.key, mk.cell_start, mk.tmp_ids, mk.ids);
     int nb = mk.bnx * mk.bny;
     note_launch();
-    k_block_active<<<cdiv(nb, kT), kT, 0, s>>>(mk.bnx, mk.bny, mk.bcount, mk.bactive);
+    k_block_active<<<cdiv(nb, kT), kT, 0, s>>>(mk.bnx, mk.bny, mk.bcount, mk.blist, mk.nact);
 }
 
 void launch_interp(const Markers &mk, int kernel, const double *u, const double *v,
@@ -1930,6 +1949,25 @@ void launch_interp(const Markers &mk, int kernel, const double *u, const double 
     note_launch();
     k_interp<<<cdiv(8L * mk.M, 128), 128, 0, s>>>(mk.M, kernel, mk.nx, mk.ny, 1.0 / mk.h, mk.x0, mk.y0, u, v,
                                             mk.X, mk.Y, U, V, dt_move);
+}
+
+// Multiprocessors of the device (the same on every device this runs on).
+static int sm_count()
+{
+    static int sms = 0;
+    if (!sms) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (sms <= 0) sms = 152;
+    }
+    return sms;
+}
+
+// Grid of the kernels over active blocks: per CTAs an SM, or one per block.
+static int block_grid(const Markers &mk, int per)
+{
+    return (int)std::min((long)mk.bnx * mk.bny, (long)per * sm_count());
 }
 
 void launch_spread_conv(const Markers &mk, int kernel, const double *fmag, double *Fx,
@@ -1941,23 +1979,13 @@ void launch_spread_conv(const Markers &mk, int kernel, const double *fmag, doubl
     k_spread_tab<<<cdiv(2L * mk.M, 128), 128, 0, s>>>(mk.M, kernel, 1.0 / mk.h, mk.x0, mk.y0, mk.X, mk.Y, fmag,
                                                       mk.nxm, mk.nym, mk.ds, mk.stab);
     note_launch();
-    k_spread_conv<<<dim3(mk.bnx, mk.bny), 2 * kBlk * kBlk, 0, s>>>(mk.nx, mk.ny, mk.bnx, mk.bactive,
-                                                                  mk.cell_start, mk.ids, mk.stab, Fx, Fy);
+    k_spread_conv<<<block_grid(mk, 16), 2 * kBlk * kBlk, 0, s>>>(mk.nx, mk.ny, mk.bnx, mk.blist, mk.nact,
+                                                                mk.cell_start, mk.ids, mk.stab, Fx, Fy);
 }
 
 // Grid of the strip-area kernel: kClipBlocks clip blocks, then 8 CTAs of
 // 256 threads per SM for the flat pair loop (grid-stride).
-int band_area_grid()
-{
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 152;
-    }
-    return kClipBlocks + 8 * sms;
-}
+int band_area_grid() { return kClipBlocks + 8 * sm_count(); }
 
 // Strip areas of the current band pair list (idempotent: pacc, pcov only).
 void launch_band_area(const Markers &mk, cudaStream_t s)
@@ -1984,16 +2012,16 @@ void launch_heaviside(const Markers &mk, double *H, cudaStream_t s, cudaStream_t
     k_rows_inside<<<mk.ny, kT, 0, sr>>>(mk.ndrops, mk.nx, mk.h, mk.x0, mk.y0, mk.X, mk.Y, mk.ykey,
                                         mk.colkey, mk.next, mk.drop_start, mk.dyk, H, mk.flags);
     if (side) cudaEventRecord(ev_join, side);
-    dim3 g(mk.bnx, mk.bny);
     cudaMemsetAsync(mk.npairs, 0, 2 * sizeof(uint32_t), s);  // pairs, listed clip pairs
     note_launch();
-    k_band_pairs<<<g, kPairT, 0, s>>>(mk.nx, mk.ny, mk.bnx, mk.bactive, mk.cell_start, mk.ids, mk.slf,
-                                   mk.scvx, mk.sbox, mk.pair_cap, mk.npairs, mk.pseg, mk.pcell,
+    k_band_pairs<<<block_grid(mk, 7), kPairT, 0, s>>>(mk.nx, mk.ny, mk.bnx, mk.blist, mk.nact,
+                                   mk.cell_start, mk.ids, mk.slf, mk.scvx, mk.sbox, mk.pair_cap, mk.npairs, mk.pseg, mk.pcell,
                                    mk.crange, mk.clip_list, mk.flags);
     launch_band_area(mk, s);
     if (side) cudaStreamWaitEvent(s, ev_join, 0);
     note_launch();
-    k_band_sum<<<g, kBT, 0, s>>>(mk.nx, mk.ny, mk.bnx, mk.bactive, mk.crange, mk.pacc, mk.pcov, H);
+    k_band_sum<<<block_grid(mk, 32), kBT, 0, s>>>(mk.nx, mk.ny, mk.bnx, mk.blist, mk.nact, mk.crange,
+                                                  mk.pacc, mk.pcov, H);
 }
 
 void launch_spread_irrot(const Markers &mk, const double *fmag, const double *H, double *Fx,
@@ -2001,10 +2029,9 @@ void launch_spread_irrot(const Markers &mk, const double *fmag, const double *H,
 {
     cudaMemsetAsync(Fx, 0, (size_t)(mk.nx + 1) * mk.ny * 8, s);
     cudaMemsetAsync(Fy, 0, (size_t)mk.nx * (mk.ny + 1) * 8, s);
-    dim3 g(mk.bnx, mk.bny);
     note_launch();
-    k_spread_irrot<<<g, kIrrT, 0, s>>>(mk.nx, mk.ny, 1.0 / mk.h, mk.bnx, mk.bactive, mk.cell_start,
-                                       mk.ids, mk.next, mk.gx, mk.gy, mk.sinv, mk.gxf, mk.gyf, fmag,
+    k_spread_irrot<<<block_grid(mk, 7), kIrrT, 0, s>>>(mk.nx, mk.ny, 1.0 / mk.h, mk.bnx, mk.blist, mk.nact,
+                                       mk.cell_start, mk.ids, mk.next, mk.gx, mk.gy, mk.sinv, mk.gxf, mk.gyf, fmag,
                                        H, Fx, Fy, mk.flags);
 }
 
