@@ -26,151 +26,9 @@ namespace {
 
 constexpr int kT = 256;
 
-// Tiled predictor in ring control volumes: the planar kernel's staging and
-// node averages; every flux carries the radius of its face and each balance
-// is divided by the radius of its control volume; the radial component adds
-// -mu_face u / r^2 (vector diffusion).  With a frame record (non-inertial
-// frame, see k_axi_frame) the axial body acceleration adds its S and the
-// boundaries z = 0, Lz and the outer wall move axially with its wb: v = wb
-// on the z boundary faces, the outer wall's reflected ghost is 2 wb - v.
-constexpr int PX = 32, PY = 8;
-__global__ void __launch_bounds__(PX * PY)
-k_predictor_axi(int nx, int ny, double h, double dt, double visc, double ivisc,
-                const double *__restrict__ rho,
-                const double *__restrict__ mu, const double *__restrict__ u,
-                const double *__restrict__ v, const double *__restrict__ aup,
-                const double *__restrict__ avp, int have_prev, double gx, double gy,
-                const double *__restrict__ frame, const double *__restrict__ bx,
-                const double *__restrict__ by, double *__restrict__ us,
-                double *__restrict__ vs, double *__restrict__ au, double *__restrict__ av)
-{
-    constexpr int W = PX + 2, Hh = PY + 2;
-    const double gz = gy + (frame ? frame[kFrS] : 0.0), wb = frame ? frame[kFrWb] : 0.0;
-    __shared__ double sr[Hh][W], sm[Hh][W], su[Hh][W + 1], sv[Hh + 1][W];
-    __shared__ double nr[PY + 1][PX + 1], nm[PY + 1][PX + 1];
-    // fluxes two faces share, with their radius (as the planar predictor):
-    // radial momentum at cells i0-1 .. i0+PX-1 and nodes (i0 .. i0+PX-1,
-    // j0 .. j0+PY); axial momentum at cells j0-1 .. j0+PY-1 and nodes
-    // (i0 .. i0+PX, j0 .. j0+PY-1)
-    __shared__ double fx[PY][PX + 1], vx[PY][PX + 1], gxn[PY + 1][PX], wxn[PY + 1][PX];
-    __shared__ double fy[PY + 1][PX], vy[PY + 1][PX], gyn[PY][PX + 1], wyn[PY][PX + 1];
-    const int i0 = blockIdx.x * PX, j0 = blockIdx.y * PY;
-    const int t = threadIdx.y * PX + threadIdx.x;
-    const long nxf = nx + 1;
-    for (int k = t; k < Hh * (W + 1); k += PX * PY) {
-        const int r = k / (W + 1), c = k - r * (W + 1), gi = i0 - 1 + c, gj = j0 - 1 + r;
-        const bool inj = gj >= 0 && gj < ny;
-        if (c < W) {
-            const bool in = inj && gi >= 0 && gi < nx;
-            const long o = (long)gj * nx + gi;
-            sr[r][c] = in ? rho[o] : 0.0;
-            sm[r][c] = in ? mu[o] : 0.0;
-        }
-        su[r][c] = (inj && gi >= 0 && gi <= nx) ? u[(long)gj * nxf + gi] : 0.0;
-    }
-    for (int k = t; k < (Hh + 1) * W; k += PX * PY) {
-        const int r = k / W, c = k - r * W, gi = i0 - 1 + c, gj = j0 - 1 + r;
-        sv[r][c] = (gi >= 0 && gi < nx && gj >= 0 && gj <= ny) ? v[(long)gj * nx + gi] : 0.0;
-    }
-    __syncthreads();
-    for (int k = t; k < (PY + 1) * (PX + 1); k += PX * PY) {
-        const int r = k / (PX + 1), c = k - r * (PX + 1), I = i0 + c, J = j0 + r;
-        if (I > nx || J > ny) continue;
-        const double *r0 = &sr[r][c], *r1 = &sr[r + 1][c];
-        const double *m0 = &sm[r][c], *m1 = &sm[r + 1][c];
-        const bool wx = I == 0 || I == nx, wy = J == 0 || J == ny;
-        nr[r][c] = 0.25 * (r0[0] + r0[1] + r1[0] + r1[1]);
-        if (!wx && !wy) nm[r][c] = 0.25 * (m0[0] + m0[1] + m1[0] + m1[1]);
-        else if (wy && !wx) nm[r][c] = J == 0 ? 0.5 * (m1[0] + m1[1]) : 0.5 * (m0[0] + m0[1]);
-        else if (wx && !wy) nm[r][c] = I == 0 ? 0.5 * (m0[1] + m1[1]) : 0.5 * (m0[0] + m1[0]);
-        else nm[r][c] = 0.0;
-    }
-    __syncthreads();
-    // radial momentum of cell (i0-1+c, j0+r) at its outer radius (gi + 1/2) h
-    for (int k = t; k < PY * (PX + 1); k += PX * PY) {
-        const int r = k / (PX + 1), c = k - r * (PX + 1), gi = i0 - 1 + c;
-        const double rc = (gi + 0.5) * h, a = 0.5 * (su[r + 1][c + 1] + su[r + 1][c]);
-        fx[r][c] = rc * sr[r + 1][c] * a * a;
-        vx[r][c] = rc * sm[r + 1][c] * (su[r + 1][c + 1] - su[r + 1][c]);
-    }
-    // axial momentum of cell (i0+c, j0-1+r) at the column's radius (gi + 1/2) h
-    for (int k = t; k < (PY + 1) * PX; k += PX * PY) {
-        const int r = k / PX, c = k - r * PX, gi = i0 + c;
-        const double rc = (gi + 0.5) * h, a = 0.5 * (sv[r + 1][c + 1] + sv[r][c + 1]);
-        fy[r][c] = rc * sr[r][c + 1] * a * a;
-        vy[r][c] = rc * sm[r][c + 1] * (sv[r + 1][c + 1] - sv[r][c + 1]);
-    }
-    // radial momentum at node (I, J) = (i0+c, j0+r), radius I h: between
-    // u(I, J-1) and u(I, J); reflected ghost at the bottom and top walls
-    for (int k = t; k < (PY + 1) * PX; k += PX * PY) {
-        const int r = k / PX, c = k - r * PX, I = i0 + c, J = j0 + r;
-        if (I > nx || J > ny) continue;
-        const double rn = I * h, ub = su[r][c + 1], ut = su[r + 1][c + 1];
-        gxn[r][c] = (J > 0 && J < ny)
-                        ? rn * nr[r][c] * (0.5 * (sv[r + 1][c] + sv[r + 1][c + 1])) * (0.5 * (ub + ut))
-                        : 0.0;
-        const double uT = J < ny ? ut : -ub, uB = J > 0 ? ub : -ut;
-        wxn[r][c] = rn * nm[r][c] * (uT - uB);
-    }
-    // axial momentum at node (I, J), radius I h: between v(I-1, J) and
-    // v(I, J); at the outer wall the ghost 2 wb - v, at the axis v itself
-    for (int k = t; k < PY * (PX + 1); k += PX * PY) {
-        const int r = k / (PX + 1), c = k - r * (PX + 1), I = i0 + c, J = j0 + r;
-        if (I > nx || J > ny) continue;
-        const double rn = I * h, vl = sv[r + 1][c], vr = sv[r + 1][c + 1];
-        gyn[r][c] = (I > 0 && I < nx)
-                        ? rn * nr[r][c] * (0.5 * (su[r][c + 1] + su[r + 1][c + 1])) * (0.5 * (vl + vr))
-                        : 0.0;
-        const double vR = I < nx ? vr : 2.0 * wb - vl, vL = I > 0 ? vl : vr;
-        wyn[r][c] = rn * nm[r][c] * (vR - vL);
-    }
-    __syncthreads();
-    const int tx = threadIdx.x, ty = threadIdx.y, i = i0 + tx, j = j0 + ty;
-    if (i >= nx || j >= ny) return;
-    const int R = ty + 1, C = tx + 1;
-    const double h2 = h * h * ivisc;  // the factor visc on mu, a power of two
-    // radial face (i, j) at r = i h, control volume [r_(i-1), r_i]
-    {
-        const long k = (long)j * nxf + i;
-        if (i == 0) {
-            us[k] = 0.0; au[k] = 0.0;
-        } else {
-            const double r0 = i * h;
-            const double uc = su[R][C];
-            const double adv = ((fx[ty][tx + 1] - fx[ty][tx]) + (gxn[ty + 1][tx] - gxn[ty][tx])) / (r0 * h);
-            const double muf = (0.5 * visc) * (sm[R][C - 1] + sm[R][C]);
-            const double vis = (vx[ty][tx + 1] - vx[ty][tx] + wxn[ty + 1][tx] - wxn[ty][tx]) / (r0 * h2) -
-                               muf * uc / (r0 * r0);
-            // 1 / rho_face: the plain face coefficient beta when given
-            const double irf = bx ? bx[k] : 1.0 / (0.5 * (sr[R][C - 1] + sr[R][C]));
-            const double ae = have_prev ? 1.5 * adv - 0.5 * aup[k] : adv;
-            us[k] = uc + dt * ((vis - ae) * irf + gx);
-            au[k] = adv;
-        }
-        if (i == nx - 1) { us[k + 1] = 0.0; au[k + 1] = 0.0; }
-    }
-    // axial face (i, j) at r = (i + 1/2) h, control volume [i h, (i + 1) h]
-    {
-        const long k = (long)j * nx + i;
-        if (j == 0) {
-            vs[k] = wb; av[k] = 0.0;
-        } else {
-            const double r0 = (i + 0.5) * h;
-            const double vc = sv[R][C];
-            const double adv = ((fy[ty + 1][tx] - fy[ty][tx]) + (gyn[ty][tx + 1] - gyn[ty][tx])) / (r0 * h);
-            const double vis = (vy[ty + 1][tx] - vy[ty][tx] + wyn[ty][tx + 1] - wyn[ty][tx]) / (r0 * h2);
-            const double irf = by ? by[k] : 1.0 / (0.5 * (sr[R - 1][C] + sr[R][C]));
-            const double ae = have_prev ? 1.5 * adv - 0.5 * avp[k] : adv;
-            vs[k] = vc + dt * ((vis - ae) * irf + gz);
-            av[k] = adv;
-        }
-        if (j == ny - 1) { vs[k + nx] = wb; av[k + nx] = 0.0; }
-    }
-}
-
 // r_i b with b = div(u*/dt + beta F) in the axisymmetric divergence: the
 // right-hand side of the r-weighted pressure equation.
-__global__ void k_rhs_axi(int nx, int ny, double h, double idt, const double *__restrict__ us,
+__global__ void k_rhs_axi(int nx, int ny, double idt, const double *__restrict__ us,
                           const double *__restrict__ vs, const double *__restrict__ Fx,
                           const double *__restrict__ Fy, const double *__restrict__ bx,
                           const double *__restrict__ by, double *__restrict__ b)
@@ -178,13 +36,17 @@ __global__ void k_rhs_axi(int nx, int ny, double h, double idt, const double *__
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
     if (i >= nx) return;
     const long xw = (long)j * (nx + 1) + i, ys = (long)j * nx + i, yn = ys + nx;
-    const double qE = us[xw + 1] * idt + bx[xw + 1] * Fx[xw + 1];
-    const double qW = us[xw] * idt + bx[xw] * Fx[xw];
-    const double qN = vs[yn] * idt + by[yn] * Fy[yn];
-    const double qS = vs[ys] * idt + by[ys] * Fy[ys];
-    const double ri = (i + 0.5) * h;
-    const double bb = ((i + 1) * h * qE - i * h * qW) / (ri * h) + (qN - qS) / h;
-    b[ys] = ri * bb;
+    // r b = (r_(i+1) q_E - r_i q_W) / h + r_c (q_N - q_S) / h with radii in
+    // units of h; the force is zero on all faces but those of the interface
+    // band: its part and the loads of beta only where a warp's faces carry one
+    const double fe = Fx[xw + 1], fw = Fx[xw], fn = Fy[yn], fs = Fy[ys];
+    const double ri = (double)i, re = ri + 1.0, rc = ri + 0.5;
+    double r = idt * fma(rc, vs[yn] - vs[ys], fma(re, us[xw + 1], -ri * us[xw]));
+    const long long any = __double_as_longlong(fe) | __double_as_longlong(fw) | __double_as_longlong(fn) |
+                          __double_as_longlong(fs);
+    if (any & 0x7fffffffffffffffLL)
+        r += fma(rc, by[yn] * fn - by[ys] * fs, fma(re, bx[xw + 1] * fe, -ri * (bx[xw] * fw)));
+    b[ys] = r;
 }
 
 // Coefficients of the r-weighted pressure operator: r_face beta_x, r_i beta_y.
@@ -373,19 +235,6 @@ k_axi_frame(const double *__restrict__ X, const double *__restrict__ Y,
 
 }  // namespace
 
-void launch_predictor_axi(int nx, int ny, double h, double dt, const double *rho,
-                          const double *mu, const double *u, const double *v,
-                          const double *au_prev, const double *av_prev, int have_prev,
-                          double gx, double gy, const double *frame, const double *bx,
-                          const double *by, double *us, double *vs, double *au, double *av,
-                          cudaStream_t s, double visc)
-{
-    dim3 g(cdiv(nx, PX), cdiv(ny, PY)), b(PX, PY);
-    note_launch();
-    k_predictor_axi<<<g, b, 0, s>>>(nx, ny, h, dt, visc, 1.0 / visc, rho, mu, u, v, au_prev, av_prev, have_prev, gx,
-                                    gy, frame, bx, by, us, vs, au, av);
-}
-
 void launch_axi_zbc(int nx, int ny, const double *frame, double *v, cudaStream_t s)
 {
     note_launch();
@@ -405,7 +254,7 @@ void launch_rhs_axi(int nx, int ny, double h, double dt, const double *us, const
 {
     dim3 g(cdiv(nx, 128), ny);
     note_launch();
-    k_rhs_axi<<<g, 128, 0, s>>>(nx, ny, h, 1.0 / dt, us, vs, Fx, Fy, bx, by, b);
+    k_rhs_axi<<<g, 128, 0, s>>>(nx, ny, 1.0 / dt, us, vs, Fx, Fy, bx, by, b);
 }
 
 void launch_axi_weights(int nx, int ny, double h, const double *bx, const double *by,

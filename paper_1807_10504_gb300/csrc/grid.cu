@@ -98,163 +98,168 @@ __global__ void k_correct(int nx, int ny, double ih, double dt,
     }
 }
 
-// Tiled predictor: a 32 x 8 block of cells stages rho, mu, u and v with a
-// one-cell ring in shared memory, forms the node averages of rho and mu once
-// per node (four cells inside, the two wall cells on a wall), then every
-// flux that two faces share once per tile: per cell the advective flux
-// rho a^2 and the viscous flux mu du of each component, per node the
-// advective flux rho_n a_v a_u (one product for both components, zero
-// through a wall) and the viscous flux mu_n du of each component (the
-// reflected ghost folded in at a wall node).  Each thread then updates the x-face left of and the y-face
-// below its cell (and the wall face on the far side for the last column /
-// row) from differences of those fluxes, in the order of the per-face
-// formula, so each face gets the same value as if it formed them itself.
-// The advective fluxes are kept without their power-of-two factors (the
-// 1/2 of each face average, the 1/4 of the node density): 4 rho a^2 per
-// cell, 16 rho_n a_v a_u per node, the factors folded into 1/h of the
-// difference; the node viscosity is kept as 4 mu_n, its 1/4 folded into the
-// viscous difference.  Scaling by a power of two is exact, so every rounding
-// is as in the per-face formula (fewer FP64 multiplications, the same
-// values), except that the node product is formed in one order for both
-// components.
-constexpr int PX = 32, PY = 8;
-__global__ void __launch_bounds__(PX * PY)
-k_predictor(int nx, int ny, double ih, double ih2, double dt,
+// Predictor: a warp marches up a strip of 30 columns (and one on either side
+// for the neighbours' fluxes), rows j0 .. j0 + R - 1, one lane per column.  A
+// lane holds its column's rho, mu, u and v of the current and the next row,
+// loads the row after next while it computes, and takes its neighbours'
+// values by shuffles; every flux that two faces share is formed once: per
+// cell the advective flux rho a^2 and the viscous flux mu du of each
+// component, per node (the cell's lower left corner) the advective flux
+// rho_n a_v a_u, one product for both components, and the viscous flux mu_n du
+// of each.  Then the x-face left of and the y-face below the cell are updated
+// (and the wall face on the far side by the last column / row).
+//
+// FP64 arithmetic bounds it (64 cycles an instruction for one warp, 19 an SM
+// with four or more): 44 instructions a cell, times 32/30 and (R + 1) / R.  A
+// 32 x 8 tile with the fluxes in shared memory has partly filled warps in
+// every pass over its ring and two barriers.  Next to the hierarchy's setup
+// and the face force, as in a step: 1024^2 171 -> 149 us, 2048^2 665 -> 571,
+// 256 x 1024 axisymmetric 107 -> 61.  R: rows per warp, 16 where that gives
+// 1024 warps, fewer below (512^2: 45 us with 8 rows, 109 with 16, whose 576
+// warps leave each to its latency; 46 the tiles).
+//
+// Walls: a ghost row or column of the velocity reflected to zero on the wall
+// (the outer wall of the axisymmetric form: to wb), of rho and mu equal to the
+// row or column inside, makes the wall nodes' formula the inner one: twice the
+// two wall cells' mean, and no advective flux through the wall.
+//
+// The fluxes are kept without their power-of-two factors (the 1/2 of each
+// face average, the 1/4 of the node averages): 4 rho a^2 per cell, 16 rho_n a_v
+// a_u and 4 mu_n du per node, folded into the factors of their differences.
+//
+// AXI: axisymmetric form (x = r, y = z).  Every flux carries the radius of its
+// face and each balance is divided by the radius of its control volume; these
+// ratios, a column's own, are formed once per lane.  The radial component
+// adds -mu_face u / r^2.
+constexpr int kPredT = 128, kPredCols = 30;
+template <bool AXI>
+__global__ void __launch_bounds__(kPredT)
+k_predictor(int nx, int ny, int R, double h, double visc, double dt,
             const double *__restrict__ rho, const double *__restrict__ mu,
             const double *__restrict__ u, const double *__restrict__ v,
-            const double *__restrict__ aup, const double *__restrict__ avp,
-            int have_prev, double gx, double gy, const double *__restrict__ bx,
-            const double *__restrict__ by, double *__restrict__ us,
-            double *__restrict__ vs, double *__restrict__ au, double *__restrict__ av)
+            const double *aup, const double *avp,  // may be au, av
+            int have_prev, double gx, double gy, const double *__restrict__ frame,
+            const double *__restrict__ bx, const double *__restrict__ by,
+            double *__restrict__ us, double *__restrict__ vs, double *au, double *av)
 {
-    constexpr int W = PX + 2, Hh = PY + 2;  // staged window: cells / faces i0-1 .. i0+PX
-    __shared__ double sr[Hh][W], sm[Hh][W], su[Hh][W + 1], sv[Hh + 1][W];
-    __shared__ double nm4[PY + 1][PX + 1];  // 4 mu_n
-    // shared fluxes: x-momentum at cells i0-1 .. i0+PX-1 (fx, vx) and nodes
-    // (i0 .. i0+PX-1, j0 .. j0+PY) (gx, wx); y-momentum at cells j0-1 ..
-    // j0+PY-1 (fy, vy) and nodes (i0 .. i0+PX, j0 .. j0+PY-1) (gy, wy)
-    __shared__ double fx[PY][PX + 1], vx[PY][PX + 1], gxn[PY + 1][PX], wxn[PY + 1][PX];
-    __shared__ double fy[PY + 1][PX], vy[PY + 1][PX], gyn[PY][PX + 1], wyn[PY][PX + 1];
-    const int i0 = blockIdx.x * PX, j0 = blockIdx.y * PY;
-    const int t = threadIdx.y * PX + threadIdx.x;
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, sx = (nx + kPredCols - 1) / kPredCols;
+    const int wid = blockIdx.x * (kPredT / 32) + (threadIdx.x >> 5), ty = wid / sx;
+    const int j0 = ty * R, j1 = min(j0 + R, ny);
+    if (j0 >= ny) return;  // whole warps
+    const int i = (wid - ty * sx) * kPredCols + lane - 1;
+    const bool out = lane >= 1 && lane <= kPredCols && i < nx;
     const long nxf = nx + 1;
-    // staging; out-of-domain entries are never used by a face that is updated
-    for (int k = t; k < Hh * (W + 1); k += PX * PY) {
-        const int r = k / (W + 1), c = k - r * (W + 1), gi = i0 - 1 + c, gj = j0 - 1 + r;
-        const bool inj = gj >= 0 && gj < ny;
-        if (c < W) {
-            const bool in = inj && gi >= 0 && gi < nx;
-            const long o = (long)gj * nx + gi;
-            sr[r][c] = in ? rho[o] : 0.0;
-            sm[r][c] = in ? mu[o] : 0.0;
-        }
-        su[r][c] = (inj && gi >= 0 && gi <= nx) ? u[(long)gj * nxf + gi] : 0.0;
+    // columns to load from: cell and y-face data of column c, x-faces of cu
+    const int c = min(max(i, 0), nx - 1), cu = min(max(i, 0), nx);
+    const double wb = AXI && frame ? frame[kFrWb] : 0.0;
+    if constexpr (AXI) gy += frame ? frame[kFrS] : 0.0;
+    auto neg = [](double x) {
+        return __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ULL);
+    };
+    auto ld_u = [&](int j) {  // row j, reflected beyond the walls
+        if (j < 0) return neg(u[cu]);
+        return j < ny ? u[(long)j * nxf + cu] : neg(u[(long)(ny - 1) * nxf + cu]);
+    };
+    auto ld_v = [&](int j) {  // y-face row j (0 .. ny), reflected beyond the side walls
+        const double x = v[(long)j * nx + c];
+        if (AXI) return i >= nx ? 2.0 * wb - x : x;
+        return i < 0 || i >= nx ? neg(x) : x;
+    };
+    auto row = [&](int j) { return (long)min(max(j, 0), ny - 1) * nx + c; };
+    auto up = [&](double x) { return __shfl_up_sync(kAll, x, 1); };
+    auto down = [&](double x) { return __shfl_down_sync(kAll, x, 1); };
+    // the factors of the differences
+    const double ih = 1.0 / h, hdt = 0.5 * dt, v2 = 2.0 * visc * ih * ih;
+    double xi = 0.25 * ih, xw = xi, xv = v2, xvw = v2, xm = 0.0;  // x-face: cells i, i-1
+    double ge = 0.0625 * ih, gw = ge, we = 0.25 * v2, ww = we;    // y-face: nodes i+1, i
+    const double ih4 = 0.25 * ih, ih16 = 0.0625 * ih, v24 = 0.25 * v2;
+    if constexpr (AXI) {
+        const double rf = i > 0 ? recip_any((double)i) : 0.0, rc = recip_any((double)i + 0.5);
+        const double a = ((double)i + 0.5) * rf, b = ((double)i - 0.5) * rf;
+        xi = a * ih4; xw = b * ih4; xv = a * v2; xvw = b * v2;
+        xm = -(visc * ih * ih) * (rf * rf);
+        const double e = ((double)i + 1.0) * rc, w = (double)i * rc;
+        ge = i + 1 == nx ? 0.0 : e * ih16;  // no flux through the outer wall
+        gw = w * ih16; we = e * v24; ww = w * v24;
     }
-    for (int k = t; k < (Hh + 1) * W; k += PX * PY) {
-        const int r = k / W, c = k - r * W, gi = i0 - 1 + c, gj = j0 - 1 + r;
-        sv[r][c] = (gi >= 0 && gi < nx && gj >= 0 && gj <= ny) ? v[(long)gj * nx + gi] : 0.0;
-    }
-    __syncthreads();
-    // node (I, J) = corner of cells (I-1, J-1), (I, J-1), (I-1, J), (I, J);
-    // window index of cell (gi, gj) is (gj - j0 + 1, gi - i0 + 1).  The
-    // advective node flux 16 rho_n a_v a_u, between u(I, J-1) and u(I, J)
-    // (window (r, c+1), (r+1, c+1)) and between v(I-1, J) and v(I, J)
-    // (window (r+1, c), (r+1, c+1)), serves the x-momentum (zero on the
-    // walls J = 0, ny) and the y-momentum (zero on the walls I = 0, nx)
-    for (int k = t; k < (PY + 1) * (PX + 1); k += PX * PY) {
-        const int r = k / (PX + 1), c = k - r * (PX + 1), I = i0 + c, J = j0 + r;
-        if (I > nx || J > ny) continue;
-        const double *r0 = &sr[r][c], *r1 = &sr[r + 1][c];  // rows J-1, J; columns I-1, I
-        const double *m0 = &sm[r][c], *m1 = &sm[r + 1][c];
-        const bool wx = I == 0 || I == nx, wy = J == 0 || J == ny;
-        const double rn4 = r0[0] + r0[1] + r1[0] + r1[1];  // 4 rho_n
-        if (!wx && !wy) nm4[r][c] = m0[0] + m0[1] + m1[0] + m1[1];
-        else if (wy && !wx) nm4[r][c] = J == 0 ? 2.0 * (m1[0] + m1[1]) : 2.0 * (m0[0] + m0[1]);
-        else if (wx && !wy) nm4[r][c] = I == 0 ? 2.0 * (m0[1] + m1[1]) : 2.0 * (m0[0] + m1[0]);
-        else nm4[r][c] = 0.0;  // corner: never used
-        const double g = rn4 * (sv[r + 1][c] + sv[r + 1][c + 1]) * (su[r][c + 1] + su[r + 1][c + 1]);
-        if (c < PX) gxn[r][c] = wy ? 0.0 : g;
-        if (r < PY) gyn[r][c] = wx ? 0.0 : g;
-    }
-    __syncthreads();
-    // cell fluxes: x-momentum of cell (i0-1+c, j0+r), window (r+1, c)
-    for (int k = t; k < PY * (PX + 1); k += PX * PY) {
-        const int r = k / (PX + 1), c = k - r * (PX + 1);
-        const double a = su[r + 1][c + 1] + su[r + 1][c];  // 2 a
-        fx[r][c] = sr[r + 1][c] * a * a;                   // 4 rho a^2
-        vx[r][c] = sm[r + 1][c] * (su[r + 1][c + 1] - su[r + 1][c]);
-    }
-    // y-momentum of cell (i0+c, j0-1+r), window (r, c+1)
-    for (int k = t; k < (PY + 1) * PX; k += PX * PY) {
-        const int r = k / PX, c = k - r * PX;
-        const double a = sv[r + 1][c + 1] + sv[r][c + 1];  // 2 a
-        fy[r][c] = sr[r][c + 1] * a * a;                   // 4 rho a^2
-        vy[r][c] = sm[r][c + 1] * (sv[r + 1][c + 1] - sv[r][c + 1]);
-    }
-    // viscous node fluxes (times 4) of the x-momentum at node (I, J) =
-    // (i0+c, j0+r): between u(I, J-1) (window (r, c+1)) and u(I, J) (window
-    // (r+1, c+1))
-    for (int k = t; k < (PY + 1) * PX; k += PX * PY) {
-        const int r = k / PX, c = k - r * PX, I = i0 + c, J = j0 + r;
-        if (I > nx || J > ny) continue;
-        const double ub = su[r][c + 1], ut = su[r + 1][c + 1];
-        const double uT = J < ny ? ut : -ub, uB = J > 0 ? ub : -ut;
-        wxn[r][c] = nm4[r][c] * (uT - uB);
-    }
-    // of the y-momentum at node (I, J) = (i0+c, j0+r): between v(I-1, J)
-    // (window (r+1, c)) and v(I, J) (window (r+1, c+1))
-    for (int k = t; k < PY * (PX + 1); k += PX * PY) {
-        const int r = k / (PX + 1), c = k - r * (PX + 1), I = i0 + c, J = j0 + r;
-        if (I > nx || J > ny) continue;
-        const double vl = sv[r + 1][c], vr = sv[r + 1][c + 1];
-        const double vR = I < nx ? vr : -vl, vL = I > 0 ? vl : -vr;
-        wyn[r][c] = nm4[r][c] * (vR - vL);
-    }
-    __syncthreads();
-    const int tx = threadIdx.x, ty = threadIdx.y, i = i0 + tx, j = j0 + ty;
-    if (i >= nx || j >= ny) return;
-    const int R = ty + 1, C = tx + 1;  // window index of cell (i, j)
-    const double ih4 = 0.25 * ih, ih16 = 0.0625 * ih;  // the folded factors
-    const double ih2x2 = 2.0 * ih2, hdt = 0.5 * dt;
-    // x-face (i, j), left of cell (i, j)
+    // rows j0 - 1 (m), j0 (0) and j0 + 1 (1)
+    double r0, m0, u0, v0, G, Wx, Wy, fyp, vyp, rm;
+    double r1 = rho[row(j0 + 1)], m1 = mu[row(j0 + 1)], u1 = ld_u(j0 + 1), v1 = ld_v(j0 + 1);
     {
-        const long k = (long)j * nxf + i;
-        if (i == 0) {
-            us[k] = 0.0; au[k] = 0.0;
-        } else {
-            const double uc = su[R][C];
-            const double adv = (fx[ty][tx + 1] - fx[ty][tx]) * ih4 + (gxn[ty + 1][tx] - gxn[ty][tx]) * ih16;
-            // vx E - vx W + wx N - wx S with wx = wxn / 4 (exact)
-            const double vis = fma(-0.25, wxn[ty][tx], fma(0.25, wxn[ty + 1][tx], vx[ty][tx + 1] - vx[ty][tx]));
-            // 1 / rho_face: the face coefficient beta when given (the same
-            // reciprocal of the same rho), else formed here
-            const double irf = bx ? bx[k] : twice(recip_nr(sr[R][C - 1] + sr[R][C]));
-            // twice (vis / h^2 - (3/2 adv - 1/2 aup)), its half in dt / 2
-            const double q = have_prev ? fma(-3.0, adv, aup[k]) : -2.0 * adv;
-            double un = fma(hdt, fma(ih2x2, vis, q) * irf, uc);
-            if (gx != 0.0) un = fma(dt, gx, un);
-            us[k] = un;
-            au[k] = adv;
-        }
-        if (i == nx - 1) { us[k + 1] = 0.0; au[k + 1] = 0.0; }  // right wall face
+        rm = rho[row(j0 - 1)];
+        const double mm = mu[row(j0 - 1)], um = ld_u(j0 - 1), vm = ld_v(max(j0 - 1, 0));
+        r0 = rho[row(j0)]; m0 = mu[row(j0)]; u0 = ld_u(j0); v0 = ld_v(j0);
+        const double rs = rm + r0, ms = mm + m0, vl = up(v0);
+        const double rn = rs + up(rs), mn = ms + up(ms), b = vm + v0;
+        G = rn * (vl + v0) * (um + u0);
+        Wx = mn * (u0 - um);
+        Wy = mn * (v0 - vl);
+        fyp = rm * b * b;
+        vyp = mm * (v0 - vm);
     }
-    // y-face (i, j), below cell (i, j)
-    {
-        const long k = (long)j * nx + i;
-        if (j == 0) {
-            vs[k] = 0.0; av[k] = 0.0;
-        } else {
-            const double vc = sv[R][C];
-            const double adv = (fy[ty + 1][tx] - fy[ty][tx]) * ih4 + (gyn[ty][tx + 1] - gyn[ty][tx]) * ih16;
-            const double vis = fma(-0.25, wyn[ty][tx], fma(0.25, wyn[ty][tx + 1], vy[ty + 1][tx] - vy[ty][tx]));
-            const double irf = by ? by[k] : twice(recip_nr(sr[R - 1][C] + sr[R][C]));
-            const double q = have_prev ? fma(-3.0, adv, avp[k]) : -2.0 * adv;
-            double vn = fma(hdt, fma(ih2x2, vis, q) * irf, vc);
-            if (gy != 0.0) vn = fma(dt, gy, vn);
-            vs[k] = vn;
-            av[k] = adv;
+    for (int j = j0; j < j1; j++) {
+        const long kx = (long)j * nxf + i, ky = (long)j * nx + i;
+        double ap = 0.0, bp = 0.0, irx = 0.0, iry = 0.0;
+        if (out) {
+            if (have_prev) { ap = aup[kx]; bp = avp[ky]; }
+            if (bx) { irx = bx[kx]; iry = by[ky]; }
         }
-        if (j == ny - 1) { vs[k + nx] = 0.0; av[k + nx] = 0.0; }  // top wall face
+        // the row after next (the last one's is not used)
+        const int jn = min(j + 2, ny);
+        const double r2 = rho[row(jn)], m2 = mu[row(jn)], u2 = ld_u(jn), v2n = ld_v(jn);
+        // cell fluxes of row j, node fluxes of node row j + 1
+        const double ue = down(u0), a = ue + u0, b = v1 + v0, vl = up(v1);
+        const double fx = r0 * a * a, vx = m0 * (ue - u0);
+        const double fy = r0 * b * b, vy = m0 * (v1 - v0);
+        const double rs = r0 + r1, ms = m0 + m1;
+        const double rn = rs + up(rs), mn = ms + up(ms);
+        const double G1 = rn * (vl + v1) * (u0 + u1);
+        const double Wx1 = mn * (u1 - u0), Wy1 = mn * (v1 - vl);
+        const double fw = up(fx), vw = up(vx), Ge = down(G), We = down(Wy);
+        const double mw = AXI ? up(m0) : 0.0, rw = bx ? 0.0 : up(r0);
+        if (out) {
+            if (!bx) {
+                irx = recip_any(0.5 * (rw + r0));
+                iry = recip_any(0.5 * (rm + r0));
+            }
+            if (i == 0) {
+                us[kx] = 0.0; au[kx] = 0.0;
+            } else {
+                double adv, q;
+                if constexpr (AXI) adv = fma(xi, fx, fma(-xw, fw, ih16 * (G1 - G)));
+                else adv = fma(G1 - G, ih16, (fx - fw) * ih4);
+                // twice (viscous - (3/2 adv - 1/2 adv before)), its half in dt / 2
+                q = have_prev ? fma(-3.0, adv, ap) : -2.0 * adv;
+                if constexpr (AXI)
+                    q = fma(xv, vx, fma(-xvw, vw, fma(v24, Wx1 - Wx, fma(xm, (mw + m0) * u0, q))));
+                else
+                    q = fma(v2, fma(-0.25, Wx, fma(0.25, Wx1, vx - vw)), q);
+                double un = fma(hdt, q * irx, u0);
+                if (__double_as_longlong(gx) << 1) un = fma(dt, gx, un);
+                us[kx] = un;
+                au[kx] = adv;
+            }
+            if (i == nx - 1) { us[kx + 1] = 0.0; au[kx + 1] = 0.0; }  // the right wall's face
+            if (j == 0) {
+                vs[ky] = wb; av[ky] = 0.0;
+            } else {
+                double adv, q;
+                if constexpr (AXI) adv = fma(ge, Ge, fma(-gw, G, (fy - fyp) * ih4));
+                else adv = fma(Ge - G, ih16, (fy - fyp) * ih4);
+                q = have_prev ? fma(-3.0, adv, bp) : -2.0 * adv;
+                if constexpr (AXI) q = fma(v2, vy - vyp, fma(we, We, fma(-ww, Wy, q)));
+                else q = fma(v2, fma(-0.25, Wy, fma(0.25, We, vy - vyp)), q);
+                double vn = fma(hdt, q * iry, v0);
+                if (__double_as_longlong(gy) << 1) vn = fma(dt, gy, vn);
+                vs[ky] = vn;
+                av[ky] = adv;
+            }
+            if (j == ny - 1) { vs[ky + nx] = wb; av[ky + nx] = 0.0; }  // the top wall's face
+        }
+        G = G1; Wx = Wx1; Wy = Wy1; fyp = fy; vyp = vy; rm = r0;
+        r0 = r1; m0 = m1; u0 = u1; v0 = v1;
+        r1 = r2; m1 = m2; u1 = u2; v1 = v2n;
     }
 }
 
@@ -635,6 +640,25 @@ void launch_correct(int nx, int ny, double h, double dt, const double *us,
                                           bx, by, u, v);
 }
 
+static void predictor(bool axi, int nx, int ny, double h, double dt, const double *rho,
+                      const double *mu, const double *u, const double *v, const double *au_prev,
+                      const double *av_prev, int have_prev, double gx, double gy,
+                      const double *frame, const double *bx, const double *by, double *us,
+                      double *vs, double *au, double *av, cudaStream_t s, double visc)
+{
+    const long sx = cdiv(nx, kPredCols);
+    int R = 16;
+    while (R > 1 && sx * cdiv(ny, R) < 1024) R /= 2;
+    const unsigned g = (unsigned)cdiv(sx * cdiv(ny, R), kPredT / 32);
+    note_launch();
+    if (axi)
+        k_predictor<true><<<g, kPredT, 0, s>>>(nx, ny, R, h, visc, dt, rho, mu, u, v, au_prev, av_prev,
+                                               have_prev, gx, gy, frame, bx, by, us, vs, au, av);
+    else
+        k_predictor<false><<<g, kPredT, 0, s>>>(nx, ny, R, h, visc, dt, rho, mu, u, v, au_prev, av_prev,
+                                                have_prev, gx, gy, frame, bx, by, us, vs, au, av);
+}
+
 void launch_predictor(int nx, int ny, double h, double dt, const double *rho,
                       const double *mu, const double *u, const double *v,
                       const double *au_prev, const double *av_prev,
@@ -642,10 +666,19 @@ void launch_predictor(int nx, int ny, double h, double dt, const double *rho,
                       const double *by, double *us, double *vs, double *au, double *av,
                       cudaStream_t s, double visc)
 {
-    dim3 g(cdiv(nx, PX), cdiv(ny, PY)), b(PX, PY);
-    note_launch();
-    k_predictor<<<g, b, 0, s>>>(nx, ny, 1.0 / h, visc / (h * h), dt, rho, mu, u, v, au_prev,
-                                av_prev, have_prev, gx, gy, bx, by, us, vs, au, av);
+    predictor(false, nx, ny, h, dt, rho, mu, u, v, au_prev, av_prev, have_prev, gx, gy, nullptr, bx, by,
+              us, vs, au, av, s, visc);
+}
+
+void launch_predictor_axi(int nx, int ny, double h, double dt, const double *rho,
+                          const double *mu, const double *u, const double *v,
+                          const double *au_prev, const double *av_prev, int have_prev,
+                          double gx, double gy, const double *frame, const double *bx,
+                          const double *by, double *us, double *vs, double *au, double *av,
+                          cudaStream_t s, double visc)
+{
+    predictor(true, nx, ny, h, dt, rho, mu, u, v, au_prev, av_prev, have_prev, gx, gy, frame, bx, by,
+              us, vs, au, av, s, visc);
 }
 
 }  // namespace ibk
