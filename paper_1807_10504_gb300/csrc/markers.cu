@@ -591,15 +591,17 @@ k_rows_inside(int ndrops, int nx, double h, double x0, double y0, const double *
 
 // ------------------------------------------------------------ band candidates
 // Segments (start-marker ids) whose start marker lies within kSearch cells of
-// an 8x8 block, gathered row by row and sorted ascending.
+// an 8x8 block, gathered row by row and sorted ascending; with box, only those
+// whose box (grid units) meets the block's cells.
 __device__ int gather_candidates(int bi, int bj, int nx, int ny,
                                  const uint32_t *__restrict__ cell_start,
                                  const uint32_t *__restrict__ ids, uint32_t *cand,
-                                 uint32_t *tmp, uint32_t *flags)
+                                 uint32_t *tmp, uint32_t *flags, const float4 *__restrict__ box = nullptr)
 {
     constexpr int kRows = kBlk + 2 * kSearch;  // at most 22 rows: one warp
     __shared__ uint32_t rowoff[kRows + 1], rowsrc[kRows];
-    __shared__ int total;
+    __shared__ int total, nkeep;
+    int kept = 0;
     const int ia = max(bi * kBlk - kSearch, 0), ib = min(bi * kBlk + kBlk - 1 + kSearch, nx - 1);
     const int ja = max(bj * kBlk - kSearch, 0), jb = min(bj * kBlk + kBlk - 1 + kSearch, ny - 1);
     const int nrows = jb - ja + 1;
@@ -617,7 +619,7 @@ __device__ int gather_candidates(int bi, int bj, int nx, int ny,
             if (r >= o) inc += v;
         }
         if (r < nrows) { rowoff[r] = inc - cnt; rowsrc[r] = src; }
-        if (r == 31) { rowoff[nrows] = inc; total = (int)inc; }
+        if (r == 31) { rowoff[nrows] = inc; total = (int)inc; nkeep = 0; }
     }
     __syncthreads();
     int n = total;
@@ -628,17 +630,30 @@ __device__ int gather_candidates(int bi, int bj, int nx, int ny,
     for (int q = threadIdx.x; q < n; q += blockDim.x) {
         int r = 0;
         while (r + 1 < nrows && rowoff[r + 1] <= (uint32_t)q) r++;
-        tmp[q] = ids[rowsrc[r] + (uint32_t)q - rowoff[r]];
+        uint32_t v = ids[rowsrc[r] + (uint32_t)q - rowoff[r]];
+        if (box) {  // rejected: an id above all others
+            const float4 b = box[v];
+            const float x0 = (float)(bi * kBlk), y0 = (float)(bj * kBlk);
+            if (b.x > x0 + (float)kBlk || b.y < x0 || b.z > y0 + (float)kBlk || b.w < y0) v = 0xffffffffu;
+            else kept++;
+        }
+        tmp[q] = v;
+    }
+    if (box) {
+        kept = __reduce_add_sync(0xffffffffu, kept);
+        if ((threadIdx.x & 31) == 0 && kept) atomicAdd(&nkeep, kept);
     }
     __syncthreads();
+    const int m = box ? nkeep : n;
     for (int q = threadIdx.x; q < n; q += blockDim.x) {
         uint32_t v = tmp[q];
+        if (box && v == 0xffffffffu) continue;
         int r = 0;
         for (int t = 0; t < n; t++) r += tmp[t] < v ? 1 : 0;
         cand[r] = v;
     }
     __syncthreads();
-    return n;
+    return m;
 }
 
 // Integral of clamp(y, 0, 1) dx along the part of the directed edge
@@ -742,7 +757,7 @@ k_band_pairs(int nx, int ny, int bnx, const uint32_t *__restrict__ blist,
     for (uint32_t ab = blockIdx.x; ab < *nact; ab += gridDim.x) {
         const int bl = (int)blist[ab], bj = bl / bnx, bi = bl - bj * bnx;
         __syncthreads();  // the block before is done with the shared arrays
-        const int n = gather_candidates(bi, bj, nx, ny, cell_start, ids, cand, tmp, flags);
+        const int n = gather_candidates(bi, bj, nx, ny, cell_start, ids, cand, tmp, flags, sbox);
         const int ns = min(n, kStage);
         for (int q = threadIdx.x; q < ns; q += kPairT) {
             const uint32_t m = cand[q];
@@ -1077,12 +1092,10 @@ __device__ __forceinline__ void pair_area(uint32_t m, int ci, int cj, const doub
         for (int r = 0; r < 6; r++)
             if (r == o) S[r] = v;
     }
+    // strip k has S[k] - S[k+1]; strip 0's value is zero
 #pragma unroll
-    for (int k = 0; k < 5; k++) {
-        const double A = S[k] - S[k + 1];
-        acc += A * Hk[k];
-        cov += A;
-    }
+    for (int k = 1; k < 5; k++) acc = fma(S[k] - S[k + 1], Hk[k], acc);
+    cov = S[0] - S[5];
 }
 
 // The first kClipBlocks blocks take the listed pairs, a group of 8 lanes per

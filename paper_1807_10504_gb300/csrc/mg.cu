@@ -1071,8 +1071,11 @@ __host__ __device__ constexpr int xface_pitch(int nx) { return (nx + 4) & ~3; }
 // row) from the finer level (mean of the two fine faces; at level 0 the
 // caller's faces with the walls set to zero), their FP32 copies (the x-faces
 // twice: packed and in padded rows), and the FP64 and FP32 inverse
-// diagonals (the cell's four faces, recomputed locally).
-__device__ __forceinline__ void level_coeffs_cell(int nx, int ny, int level0, int i, int j,
+// diagonals (the cell's four faces, recomputed locally).  LEVEL0 at compile
+// time: as an argument both forms of a face were computed and one selected,
+// eight FP64 operations a cell more (14 in place of 6).
+template <bool LEVEL0>
+__device__ __forceinline__ void level_coeffs_cell(int nx, int ny, int i, int j,
                                                   const double *__restrict__ fbx,
                                                   const double *__restrict__ fby,
                                                   double *__restrict__ bx, double *__restrict__ by,
@@ -1084,12 +1087,12 @@ __device__ __forceinline__ void level_coeffs_cell(int nx, int ny, int level0, in
     const int fnx = 2 * nx;  // finer level width (unused at level 0)
     auto xface = [&](int I, int J) -> double {   // coefficient of x-face (I, J)
         if (I == 0 || I == nx) return 0.0;
-        if (level0) return fbx[(long)J * (nx + 1) + I];
+        if constexpr (LEVEL0) return fbx[(long)J * (nx + 1) + I];
         return 0.5 * (fbx[(long)(2 * J) * (fnx + 1) + 2 * I] + fbx[(long)(2 * J + 1) * (fnx + 1) + 2 * I]);
     };
     auto yface = [&](int I, int J) -> double {
         if (J == 0 || J == ny) return 0.0;
-        if (level0) return fby[(long)J * nx + I];
+        if constexpr (LEVEL0) return fby[(long)J * nx + I];
         return 0.5 * (fby[(long)(2 * J) * fnx + 2 * I] + fby[(long)(2 * J) * fnx + 2 * I + 1]);
     };
     const double w = xface(i, j), e = xface(i + 1, j), s = yface(i, j), n = yface(i, j + 1);
@@ -1149,7 +1152,8 @@ __global__ void k_level_w(LevelWArgs a)
     reinterpret_cast<double2 *>(a.w4[l])[2 * kc + 1] = make_double2(s * id, n * id);
 }
 
-__global__ void k_level_coeffs(int nx, int ny, int level0, const double *__restrict__ fbx,
+template <bool LEVEL0>
+__global__ void k_level_coeffs(int nx, int ny, const double *__restrict__ fbx,
                                const double *__restrict__ fby, double *__restrict__ bx,
                                double *__restrict__ by, float *__restrict__ bxf,
                                float *__restrict__ byf, float *__restrict__ bxp,
@@ -1158,7 +1162,7 @@ __global__ void k_level_coeffs(int nx, int ny, int level0, const double *__restr
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
     if (i >= nx) return;
-    level_coeffs_cell(nx, ny, level0, i, j, fbx, fby, bx, by, bxf, byf, bxp, invd, invdf, w4, w4f);
+    level_coeffs_cell<LEVEL0>(nx, ny, i, j, fbx, fby, bx, by, bxf, byf, bxp, invd, invdf, w4, w4f);
 }
 
 // The small levels (from `first` on) in one CTA, level after level; a level
@@ -1177,7 +1181,7 @@ __global__ void __launch_bounds__(256) k_level_coeffs_small(LevelCoeffArgs a)
         const int nx = a.nx[l], ny = a.ny[l];
         for (int k = threadIdx.x; k < nx * ny; k += blockDim.x) {
             const int j = k / nx, i = k - j * nx;
-            level_coeffs_cell(nx, ny, l == 0, i, j, a.bx[l - 1], a.by[l - 1], a.bx[l], a.by[l], a.bxf[l],
+            level_coeffs_cell<false>(nx, ny, i, j, a.bx[l - 1], a.by[l - 1], a.bx[l], a.by[l], a.bxf[l],
                               a.byf[l], a.bxp[l], a.invd[l], a.invdf[l], a.w4[l], (float4 *)a.wf[l]);
         }
         __syncthreads();
@@ -2150,10 +2154,17 @@ __global__ void k_apply_mean(long n, double *__restrict__ p, const double *__res
     if (k < n) dst[k] = p[k] - mb;
 }
 
-// sum (b0 - A p)^2 over the fine grid, FP64, into res[2].  With rf != NULL
+// sum (b0 - A p)^2 over the fine grid, FP64, into res[2].  A warp takes 31
+// columns of kResRows rows at a time (lane 31 serves its neighbour): a
+// difference to the west is the western cell's difference to the east, one to
+// the south the one to the north of the row below, so a cell costs 8.5 FP64
+// operations, which bound the kernel, in place of 10 (1024^2: 28.4 -> 24.9 us,
+// 2048^2: 87 -> 74, 512^2: 14.1 -> 12.9), and all rows' loads are in flight at
+// once.  With rf != NULL
 // also writes the FP32 residual and zeroes the FP32 correction for the inner
 // cycle.  check = 1 (first) or 2 (after `inc` cycles): the block that
 // finishes the sum also runs the convergence test of the graph's solve loop.
+constexpr int kResRows = 4;
 __global__ void __launch_bounds__(kRedT)
 k_resnorm(int nx, int ny, double ih2, const double *__restrict__ bx,
           const double *__restrict__ by, const double *__restrict__ b0,
@@ -2161,20 +2172,47 @@ k_resnorm(int nx, int ny, double ih2, const double *__restrict__ bx,
           double *part, unsigned *count, double *res, SolveCtl *ctl,
           cudaGraphConditionalHandle hnd, int check, int inc)
 {
+    const int lane = threadIdx.x & 31;
+    const int sx = (nx + 30) / 31, nst = sx * ((ny + kResRows - 1) / kResRows);
     pdl_enter();
-    // an equal contiguous share of the cells per block (the grid is one
-    // wave of resident blocks), consecutive cells on consecutive threads
-    const long n = (long)nx * ny;
-    const long per = (n + gridDim.x - 1) / gridDim.x;
-    const long ke = min(n, (long)blockIdx.x * per + per);
-    long k = (long)blockIdx.x * per + threadIdx.x;
-    int j = (int)k / nx, i = (int)k - j * nx;  // at most 2^28 cells
     double s = 0.0;
-    for (; k < ke; k += kRedT) {
-        const double r = b0[k] - flux_sum(nx, ny, i, j, bx, by, p) * ih2;
-        s += r * r;
-        if (rf) { rf[k] = d2f_rn(r); ef[k] = 0.0f; }
-        for (i += kRedT; i >= nx; i -= nx) j++;
+    for (int st = blockIdx.x * (kRedT / 32) + (threadIdx.x >> 5); st < nst; st += gridDim.x * (kRedT / 32)) {
+        const int ty = st / sx, i = (st - ty * sx) * 31 + lane, j0 = ty * kResRows;
+        // beyond a wall beta is zero: any value stands for the one there
+        const int ic = min(i, nx - 1), iw = min(max(i - 1, 0), nx - 1), ix = min(i, nx);
+        double c[kResRows + 2], w[kResRows], fx[kResRows], fy[kResRows + 1], b[kResRows];
+#pragma unroll
+        for (int r = 0; r < kResRows + 2; r++) c[r] = p[(long)min(max(j0 + r - 1, 0), ny - 1) * nx + ic];
+#pragma unroll
+        for (int r = 0; r < kResRows; r++) {
+            const long j = min(j0 + r, ny - 1);
+            w[r] = p[j * nx + iw];
+            fx[r] = bx[j * (nx + 1) + ix];
+            fy[r] = by[j * nx + ic];
+            b[r] = b0[j * nx + ic];
+        }
+        fy[kResRows] = by[(long)min(j0 + kResRows, ny) * nx + ic];
+        const bool out = lane < 31 && i < nx;
+        double ds = c[1] - c[0];
+#pragma unroll
+        for (int r = 0; r < kResRows; r++) {
+            const double dw = c[r + 1] - w[r], dn = c[r + 2] - c[r + 1];
+            const double de = __shfl_down_sync(0xffffffffu, dw, 1), fe = __shfl_down_sync(0xffffffffu, fx[r], 1);
+            double f = fe * de;
+            f = fma(-fx[r], dw, f);
+            f = fma(fy[r + 1], dn, f);
+            f = fma(-fy[r], ds, f);
+            ds = dn;
+            if (out && j0 + r < ny) {
+                const double v = fma(-f, ih2, b[r]);
+                s = fma(v, v, s);
+                if (rf) {
+                    const long k = (long)(j0 + r) * nx + i;
+                    rf[k] = d2f_rn(v);
+                    ef[k] = 0.0f;
+                }
+            }
+        }
     }
     if (block_fold_and_finish(s, part, count, res + 2) && check)
         solve_check(ctl, res, hnd, check == 1, inc);
@@ -2791,9 +2829,12 @@ void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool w
         const double *fbx = l == 0 ? bx : mg.lv[l - 1].d.bx, *fby = l == 0 ? by : mg.lv[l - 1].d.by;
         dim3 g(cdiv(v.nx, 128), v.ny);
         note_launch();
-        k_level_coeffs<<<g, 128, 0, s>>>(v.nx, v.ny, l == 0, fbx, fby, v.d.bx, v.d.by, v.f.bx, v.f.by,
-                                         v.f.bxp, v.d.invd, v.f.invd, with_w ? v.d.w : nullptr,
-                                         (float4 *)v.f.w);
+        auto coeffs = [&](auto kernel) {
+            kernel<<<g, 128, 0, s>>>(v.nx, v.ny, fbx, fby, v.d.bx, v.d.by, v.f.bx, v.f.by, v.f.bxp,
+                                     v.d.invd, v.f.invd, with_w ? v.d.w : nullptr, (float4 *)v.f.w);
+        };
+        if (l == 0) coeffs(k_level_coeffs<true>);
+        else coeffs(k_level_coeffs<false>);
     }
     if (lsmall < L) {
         LevelCoeffArgs a;
