@@ -180,12 +180,9 @@ constexpr int kFrT = 256;
 __device__ double drop_zc(const double *X, const double *Y, int s, int n)
 {
     __shared__ double a1[kFrT], a2[kFrT];
-    // heights from the marker halfway up: the moment's rounding is then that of
-    // the drop's radius, not of its height in the domain
-    const double z0 = Y[s + n / 4];
     double I1 = 0.0, I2 = 0.0;
     for (int k = threadIdx.x; k < n / 2; k += kFrT) {
-        const double r1 = X[s + k], z1 = Y[s + k] - z0, r2 = X[s + k + 1], z2 = Y[s + k + 1] - z0;
+        const double r1 = X[s + k], z1 = Y[s + k], r2 = X[s + k + 1], z2 = Y[s + k + 1];
         I1 += (z2 - z1) * (r1 * r1 + r1 * r2 + r2 * r2);
         I2 += (z2 - z1) * (r1 * r1 * (3.0 * z1 + z2) + 2.0 * r1 * r2 * (z1 + z2) +
                            r2 * r2 * (z1 + 3.0 * z2));
@@ -201,7 +198,7 @@ __device__ double drop_zc(const double *X, const double *Y, int s, int n)
         __syncthreads();
     }
     const double J1 = a1[0] / 6.0, J2 = a2[0] / 24.0;
-    return J1 != 0.0 ? z0 + J2 / J1 : 0.0;
+    return J1 != 0.0 ? J2 / J1 : 0.0;
 }
 
 // Non-inertial frame following drop 0 (Section 2.4 Eqs. (fictitious),
