@@ -368,7 +368,7 @@ ib_status step_pre(ib_ctx *c, double dt, bool reloc, bool mass, int warm)
     const ib_config &g = c->cfg;
     Markers &mk = c->mk;
     if (reloc) {
-        launch_relocate(mk, c->s);
+        launch_relocate(mk, g.axisym != 0, c->s);
         if (g.axisym) launch_axi_symmetrise(mk, c->s);
     }
     if (mass) mass_correct(c, nullptr);
@@ -814,7 +814,7 @@ ib_status ib_heaviside(ib_ctx *c, double *H)
 ib_status ib_relocate(ib_ctx *c)
 {
     if (!c) return IB_EINVAL;
-    launch_relocate(c->mk, c->s);
+    launch_relocate(c->mk, c->cfg.axisym != 0, c->s);
     if (c->cfg.axisym) launch_axi_symmetrise(c->mk, c->s);
     ib_status st = launch_check(c, "relocate");
     if (st != IB_OK) return st;

@@ -402,7 +402,8 @@ void launch_heaviside(const Markers &mk, double *H, cudaStream_t s, cudaStream_t
 void launch_band_area(const Markers &mk, cudaStream_t s);
 void launch_spread_irrot(const Markers &mk, const double *fmag, const double *H,
                          double *Fx, double *Fy, cudaStream_t s);
-void launch_relocate(Markers &mk, cudaStream_t s);
+// serial: the fixed serial order of operations (axisymmetric contexts).
+void launch_relocate(Markers &mk, bool serial, cudaStream_t s);
 void launch_drop_measure(const Markers &mk, int axisym, double *A, cudaStream_t s);
 void launch_mass_correct(Markers &mk, const double *A0, int axisym, double tol, double *eps,
                          cudaStream_t s);

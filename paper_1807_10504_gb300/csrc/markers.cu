@@ -1606,6 +1606,50 @@ __device__ void ring_solve(double *blk, int m, int g, double *S, double *scr, do
     __syncthreads();
 }
 
+// qs[k], k = 0 .. g: the first marker of span >= k (spans ascend with the
+// marker), n if none.
+__device__ __forceinline__ void span_starts(int n, int g, const int *span, int *qs)
+{
+    for (int m = threadIdx.x; m < n; m += kT) {
+        const int lo = m == 0 ? 0 : span[m - 1] + 1;
+        for (int k = lo; k <= span[m]; k++) qs[k] = m;
+    }
+    for (int k = span[n - 1] + 1 + threadIdx.x; k <= g; k += kT) qs[k] = n;
+}
+
+// Normal equations: put(i, dd, value, .) for entry (i, i+dd), dd = 0 .. 3, and
+// put(i, 4, x, y) for the right-hand sides of row i, over the markers of spans
+// i .. i+3 in ascending order; on span i + t row i has weight 3 - t.
+template <typename F>
+__device__ __forceinline__ void normal_equations(const double *X, const double *Y, int s0, int g,
+                                                 const int *qs, const double *wts, F put)
+{
+    for (int e = threadIdx.x; e < 5 * g; e += kT) {
+        const int i = e / 5, dd = e - 5 * i;
+        const int t0 = i + 3 >= g ? g - i : 0;
+        double acc = 0.0, accy = 0.0;
+        for (int k = 0; k < 4; k++) {
+            const int tt = (t0 + k) & 3, a = 3 - tt;
+            if (tt == g) continue;  // three spans: i + 3 is span i again
+            const int q = i + tt >= g ? i + tt - g : i + tt;
+            int b = a + dd;
+            if (b > 3) b -= g;  // fewer than seven spans: the band meets itself
+            const double *wm = wts + 4L * (s0 + qs[q]);
+            const int ke = qs[q + 1];
+            if (dd < 4) {
+                if (b >= 0)
+                    for (int m = qs[q]; m < ke; m++, wm += 4) acc += wm[a] * wm[b];
+            } else {
+                for (int m = qs[q]; m < ke; m++, wm += 4) {
+                    acc += wm[a] * X[s0 + m];
+                    accy += wm[a] * Y[s0 + m];
+                }
+            }
+        }
+        put(i, dd, acc, accy);
+    }
+}
+
 // Per-drop fit results: at offset 3 * s0 + d of fit (s0 the drop's first
 // marker, n its markers, g <= n) the control points cx[g], cy[g] and the
 // cumulative arc length at the knots cum[g + 1]; par[4d .. 4d+3] = (g, tau,
@@ -1647,9 +1691,7 @@ k_reloc_fit(const double *__restrict__ X, const double *__restrict__ Y,
     if (g > n) g = n;
     const double tau = Lc / g, itau = 1.0 / tau;
     const int w = 3 + g % 3, nch = (g - w) / 3, gc = 3 * nch;
-    // each marker's span and basis weights once (wts, 4 per marker); the
-    // first marker of every span (parameters ascend with m): qs[k] is the
-    // first marker of span >= k, n if none
+    // each marker's span and basis weights once (wts, 4 per marker)
     for (int m = threadIdx.x; m < n; m += kT) {
         const double s = sp[m];
         const int q = bspl_span(s, tau, g);
@@ -1668,41 +1710,13 @@ k_reloc_fit(const double *__restrict__ X, const double *__restrict__ Y,
         S[threadIdx.x] = c == 2 + r && r >= w ? 1.0 : 0.0;
     }
     __syncthreads();
-    for (int m = threadIdx.x; m < n; m += kT) {
-        const int lo = m == 0 ? 0 : span[m - 1] + 1;
-        for (int k = lo; k <= span[m]; k++) qs[k] = m;
-    }
-    for (int k = span[n - 1] + 1 + threadIdx.x; k <= g; k += kT) qs[k] = n;
+    span_starts(n, g, span, qs);
     __syncthreads();
-    // normal equations: entry (i, i+dd), dd = 0 .. 3, and right-hand side i
-    // (dd = 4), markers of spans i .. i+3 in ascending marker order; on span
-    // i + t row i has weight 3 - t
-    for (int e = threadIdx.x; e < 5 * g; e += kT) {
-        const int i = e / 5, dd = e - 5 * i;
-        const int t0 = i + 3 >= g ? g - i : 0;
-        double acc = 0.0, accy = 0.0;
-        for (int k = 0; k < 4; k++) {
-            const int tt = (t0 + k) & 3, a = 3 - tt;
-            if (tt == g) continue;  // three spans: i + 3 is span i again
-            const int q = i + tt >= g ? i + tt - g : i + tt;
-            int b = a + dd;
-            if (b > 3) b -= g;  // fewer than seven spans: the band meets itself
-            const double *wm = wts + 4L * (s0 + qs[q]);
-            const int ke = qs[q + 1];
-            if (dd < 4) {
-                if (b >= 0)
-                    for (int m = qs[q]; m < ke; m++, wm += 4) acc += wm[a] * wm[b];
-            } else {
-                for (int m = qs[q]; m < ke; m++, wm += 4) {
-                    acc += wm[a] * X[s0 + m];
-                    accy += wm[a] * Y[s0 + m];
-                }
-            }
-        }
+    normal_equations(X, Y, s0, g, qs, wts, [&](int i, int dd, double acc, double accy) {
         if (dd == 4) {
             double *r = i < gc ? blk + kBlkLen * (i / 3) + kBR + 7 * (i % 3) : S + 7 * (i - gc);
             r[0] = acc; r[1] = accy;
-            continue;
+            return;
         }
         const int j = i + dd >= g ? i + dd - g : i + dd;
         const int lo = min(i, j), hi = max(i, j);
@@ -1716,7 +1730,7 @@ k_reloc_fit(const double *__restrict__ X, const double *__restrict__ Y,
             else if (hi / 3 == bl) { const int c = hi - 3 * bl; B[kBD + c * (c + 1) / 2 + r] = acc; }
             else B[kBU + 3 * r + hi - 3 * (bl + 1)] = acc;
         }
-    }
+    });
     __syncthreads();
     ring_solve(blk, nch, g, S, sp, cx, cy, &bad);
     double *out = fit + fit_base(s0, d);
@@ -1810,6 +1824,404 @@ k_reloc_place(int M, const int32_t *__restrict__ drop_of, const int32_t *__restr
     const double s6 = 1.0 / 6.0;
     X[j] = s6 * (b0 * c.x[0] + b1 * c.x[1] + b2 * c.x[2] + b3 * c.x[3]);
     Y[j] = s6 * (b0 * c.y[0] + b1 * c.y[1] + b2 * c.y[2] + b3 * c.y[3]);
+}
+
+// ------------------------------------------------------------ B-spline, serial order
+// The same fit and placement in a fixed serial order of operations, for
+// axisymmetric contexts.  The falling frame divides differences of the drop's
+// centre by the square of the time step: there one unit in the last place of
+// a marker shows as 1e-10 of the pressure, and the drop keeps these bits from
+// one version to the next.  So the chord lengths and arc lengths are summed
+// marker by marker, the basis is the Cox-de Boor recursion on knots k tau, the
+// matrix is factored column by column and substituted row by row, each sum
+// in ascending order, its products rounded before they are subtracted.  FP64 latency bounds the chains (64 cycles an
+// instruction), so that operands are loaded a step ahead and nothing but the
+// sums' own instructions is on them: one drop of 1024 markers 1114 us with
+// every entry looked up on the chain, now 378; the block elimination above 134.
+__device__ void bspl_basis(double s, double tau, int g, double *w)
+{
+    const int q = bspl_span(s, tau, g);
+    double N[4][4];
+    N[0][0] = 1.0;
+    for (int d = 1; d <= 3; d++)
+        for (int r = 0; r <= d; r++) {
+            int k = q - d + r;
+            double tk = k * tau, tkd = (k + d) * tau, tk1 = (k + 1) * tau, tkd1 = (k + d + 1) * tau;
+            double left = (r >= 1) ? (s - tk) / (tkd - tk) * N[d - 1][r - 1] : 0.0;
+            double right = (r <= d - 1) ? (tkd1 - s) / (tkd1 - tk1) * N[d - 1][r] : 0.0;
+            N[d][r] = left + right;
+        }
+    for (int r = 0; r <= 3; r++) w[r] = N[3][r];
+}
+
+struct SpanU {
+    int i0, i1, i2, i3;  // control points q-3 .. q (cyclic)
+    double u;
+};
+__device__ __forceinline__ SpanU bspl_span_u(double s, double itau, int g)
+{
+    const double x = s * itau;
+    int q = (int)floor(x);
+    q = q > g - 1 ? g - 1 : (q < 0 ? 0 : q);
+    SpanU r;
+    r.u = x - (double)q;
+    const int k = q - 3;  // >= -3, and q <= g - 1
+    r.i0 = k < 0 ? k + g : k;
+    r.i1 = k + 1 < 0 ? k + 1 + g : k + 1;
+    r.i2 = k + 2 < 0 ? k + 2 + g : k + 2;
+    r.i3 = q;
+    return r;
+}
+
+__device__ double bspl_speed(double s, double tau, int g, const double *cx, const double *cy)
+{
+    const double itau = 1.0 / tau;
+    const SpanU p = bspl_span_u(s, itau, g);
+    const double u = p.u, v = 1.0 - u;
+    // twice the derivatives in u: -(1-u)^2, 3u^2 - 4u, -3u^2 + 2u + 1, u^2
+    const double d0 = -v * v, d1 = u * (3.0 * u - 4.0), d2 = fma(u, 2.0 - 3.0 * u, 1.0), d3 = u * u;
+    const double dx = d0 * cx[p.i0] + d1 * cx[p.i1] + d2 * cx[p.i2] + d3 * cx[p.i3];
+    const double dy = d0 * cy[p.i0] + d1 * cy[p.i1] + d2 * cy[p.i2] + d3 * cy[p.i3];
+    return 0.5 * itau * sqrt(dx * dx + dy * dy);
+}
+
+// The curve's point at s (closed form, as bspl_speed).
+__device__ void bspl_point(double s, double tau, int g, const double *cx, const double *cy,
+                           double &px, double &py)
+{
+    const SpanU p = bspl_span_u(s, 1.0 / tau, g);
+    const double u = p.u, v = 1.0 - u, u2 = u * u, u3 = u2 * u;
+    const double b0 = v * v * v, b1 = fma(3.0, u3, fma(-6.0, u2, 4.0));
+    const double b2 = fma(-3.0, u3, fma(3.0, u2, fma(3.0, u, 1.0))), b3 = u3;
+    const double s6 = 1.0 / 6.0;
+    px = s6 * (b0 * cx[p.i0] + b1 * cx[p.i1] + b2 * cx[p.i2] + b3 * cx[p.i3]);
+    py = s6 * (b0 * cy[p.i0] + b1 * cy[p.i1] + b2 * cy[p.i2] + b3 * cy[p.i3]);
+}
+
+__device__ double gl_len(double a, double b, double tau, int g, const double *cx, const double *cy)
+{
+    double mid = 0.5 * (a + b), half = 0.5 * (b - a), s = 0.0;
+    for (int k = 0; k < 8; k++) s += cGLW[k] * bspl_speed(mid + half * cGLX[k], tau, g, cx, cy);
+    return s * half;
+}
+
+// acc - a b, the product rounded first.
+__device__ __forceinline__ double sub_prod(double acc, double a, double b)
+{
+    return __dsub_rn(acc, __dmul_rn(a, b));
+}
+
+// 1/sqrt(x) by two Newton steps y <- y (3/2 - x y^2 / 2) from the FP32 estimate.
+__device__ __forceinline__ double rsqrt_newton(double x)
+{
+    double y = f2d_exact(rsqrtf(d2f_trunc(x)));
+    const double hx = -0.5 * x;
+    y = y * fma(hx, y * y, 1.5);
+    return y * fma(hx, y * y, 1.5);
+}
+
+// The lower triangle in its envelope: rows r < g - 3 keep columns r-3 .. r
+// (band[4 r + 3 - d] for column r - d), the last three, where the cyclic wrap
+// fills in, all columns (dn[(r - (g - 3)) g + c]).  On entry the matrix, on
+// return its Cholesky factor, by one warp (lane t): lane 0 the diagonal of
+// column c, lanes 1 .. 3 the band rows below it, 4 .. 6 the last rows.  rinv:
+// the diagonal's reciprocals.  Returns -1 (in every lane) if not positive
+// definite.
+__device__ int serial_factor(double *band, double *dn, int g, int t, double *rinv)
+{
+    const int gb = g - 3;
+    const long long lo = __double_as_longlong(1e-30), hi = __double_as_longlong(1e30);
+    auto pivot = [&](double s, double &rd) {  // false if not positive
+        const long long b = __double_as_longlong(s);
+        if (b > lo && b < hi) { rd = rsqrt_newton(s); return true; }
+        if (!(s > 0.0)) return false;
+        rd = 1.0 / sqrt(s);
+        return true;
+    };
+    for (int c = 0; c < gb; c++) {
+        double *slot = nullptr;
+        const double *row = nullptr;  // row[k] is the entry of column k
+        if (t < 4) {
+            if (c + t < gb) { row = band + 4 * (c + t) + 3 - (c + t); slot = band + 4 * (c + t) + 3 - t; }
+        } else if (t < 7) {
+            row = dn + (t - 4) * g; slot = dn + (t - 4) * g + c;
+        }
+        const double *pv = band + 4 * c + 3 - c;
+        const int first = t < 4 ? max(c + t - 3, 0) : max(c - 3, 0);
+        double acc = 0.0;
+        if (slot) {
+            acc = *slot;
+#pragma unroll
+            for (int d = 3; d >= 1; d--)
+                if (c - d >= first) acc = sub_prod(acc, row[c - d], pv[c - d]);
+        }
+        const double s = __shfl_sync(0xffffffffu, acc, 0);
+        double rd = 0.0;
+        if (!pivot(s, rd)) return -1;
+        if (slot) *slot = acc * rd;  // the diagonal: s / sqrt(s)
+        if (t == 0) rinv[c] = rd;
+        __syncwarp();
+    }
+    for (int c = gb; c < g; c++) {
+        // sums over all earlier columns: beyond 32 of them strided partial
+        // sums and a shuffle tree (the same total in every lane)
+        const int r = c + t;
+        const double *pv = dn + (c - gb) * g;
+        double acc = 0.0;
+        if (c > 32) {
+            double pd = 0.0, p1 = 0.0, p2 = 0.0;
+            for (int k = t; k < c; k += 32) {
+                const double lc = pv[k];
+                pd += lc * lc;
+                if (c + 1 < g) p1 += pv[g + k] * lc;
+                if (c + 2 < g) p2 += pv[2 * g + k] * lc;
+            }
+            for (int o = 16; o; o >>= 1) {
+                pd += __shfl_xor_sync(0xffffffffu, pd, o);
+                p1 += __shfl_xor_sync(0xffffffffu, p1, o);
+                p2 += __shfl_xor_sync(0xffffffffu, p2, o);
+            }
+            if (t < 3 && r < g) acc = pv[t * g + c] - (t == 0 ? pd : (t == 1 ? p1 : p2));
+        } else if (t < 3 && r < g) {
+            acc = pv[t * g + c];
+            for (int k = 0; k < c; k++) acc = sub_prod(acc, pv[t * g + k], pv[k]);
+        }
+        const double s = __shfl_sync(0xffffffffu, acc, 0);
+        double rd = 0.0;
+        if (!pivot(s, rd)) return -1;
+        if (t < 3 && r < g) dn[(r - gb) * g + c] = acc * rd;
+        if (t == 0) rinv[c] = rd;
+        __syncwarp();
+    }
+    return 0;
+}
+
+// L L^T x = b for the two right-hand sides bx, by (in place) by one warp (lane
+// t): even lanes the x side, odd lanes the y side, one instruction for both.
+// A lane keeps its side's latest three entries in registers.
+__device__ void serial_subst(const double *band, const double *dn, int g, const double *rinv, double *bx,
+                             double *by, int t)
+{
+    const int gb = g - 3;
+    double *b = (t & 1) ? by : bx;
+    double x1 = 0.0, x2 = 0.0, x3 = 0.0;  // rows r-1, r-2, r-3
+    double s = gb > 0 ? b[0] : 0.0, l1 = 0.0, l2 = 0.0, l3 = 0.0, ri = rinv[0];
+    for (int r = 0; r < gb; r++) {
+        // the next row's operands
+        const int n = min(r + 1, gb - 1);
+        const double sn = b[n], n1 = band[4 * n + 2], n2 = band[4 * n + 1], n3 = band[4 * n], rn = rinv[n];
+        if (r >= 3) s = sub_prod(s, l3, x3);
+        if (r >= 2) s = sub_prod(s, l2, x2);
+        if (r >= 1) s = sub_prod(s, l1, x1);
+        s *= ri;
+        __syncwarp();
+        if (t < 2) b[r] = s;
+        x3 = x2; x2 = x1; x1 = s;
+        s = sn; l1 = n1; l2 = n2; l3 = n3; ri = rn;
+    }
+    for (int r = gb; r < g; r++) {
+        const double *row = dn + (r - gb) * g;
+        __syncwarp();
+        s = b[r];
+        if (r > 32) {
+            double ps = 0.0, pu = 0.0;
+            for (int k = t; k < r; k += 32) { const double l = row[k]; ps += l * bx[k]; pu += l * by[k]; }
+            for (int o = 16; o; o >>= 1) {
+                ps += __shfl_xor_sync(0xffffffffu, ps, o);
+                pu += __shfl_xor_sync(0xffffffffu, pu, o);
+            }
+            s -= (t & 1) ? pu : ps;
+        } else {
+            for (int k = 0; k < r; k++) s = sub_prod(s, row[k], b[k]);
+        }
+        s *= rinv[r];
+        __syncwarp();
+        if (t < 2) b[r] = s;
+    }
+    __syncwarp();
+    double tl[3];  // rows g-3, g-2, g-1
+    for (int q = 2; q >= 0; q--) {
+        s = b[gb + q];
+        for (int k = q + 1; k < 3; k++) s = sub_prod(s, dn[k * g + gb + q], tl[k]);
+        s *= rinv[gb + q];
+        __syncwarp();
+        if (t < 2) b[gb + q] = s;
+        tl[q] = s;
+    }
+    double f1 = 0.0, f2 = 0.0, f3 = 0.0;  // rows r+1, r+2, r+3 of the band
+    double e1 = 0.0, e2 = 0.0, e3 = 0.0, d0 = 0.0, d1 = 0.0, d2 = 0.0;
+    auto load = [&](int r) {
+        s = b[r]; ri = rinv[r];
+        e1 = r + 1 < gb ? band[4 * r + 6] : 0.0;   // (r+1, r)
+        e2 = r + 2 < gb ? band[4 * r + 9] : 0.0;   // (r+2, r)
+        e3 = r + 3 < gb ? band[4 * r + 12] : 0.0;  // (r+3, r)
+        d0 = dn[r]; d1 = dn[g + r]; d2 = dn[2 * g + r];
+    };
+    if (gb > 0) load(gb - 1);
+    for (int r = gb - 1; r >= 0; r--) {
+        double v = s;
+        const double rr = ri, a1 = e1, a2 = e2, a3 = e3, q0 = d0, q1 = d1, q2 = d2;
+        if (r > 0) load(r - 1);
+        if (r + 1 < gb) v = sub_prod(v, a1, f1);
+        if (r + 2 < gb) v = sub_prod(v, a2, f2);
+        if (r + 3 < gb) v = sub_prod(v, a3, f3);
+        v = sub_prod(v, q0, tl[0]);
+        v = sub_prod(v, q1, tl[1]);
+        v = sub_prod(v, q2, tl[2]);
+        v *= rr;
+        __syncwarp();
+        if (t < 2) b[r] = v;
+        f3 = f2; f2 = f1; f1 = v;
+    }
+}
+
+// out[k] = in[0] + ... + in[k-1], k = 0 .. n, one by one; returns the total.
+__device__ double serial_sum(int n, const double *in, double *out)
+{
+    double L = 0.0;
+    int m = 0;
+    for (; m + 8 <= n; m += 8) {
+        double v[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) v[k] = in[m + k];
+#pragma unroll
+        for (int k = 0; k < 8; k++) { out[m + k] = L; L += v[k]; }
+    }
+    for (; m < n; m++) { const double v = in[m]; out[m] = L; L += v; }
+    out[n] = L;
+    return L;
+}
+
+__global__ void __launch_bounds__(kT)
+k_reloc_fit_serial(const double *__restrict__ X, const double *__restrict__ Y,
+                   const int32_t *__restrict__ drop_start, double h, int maxn,
+                   double *__restrict__ fit, double *__restrict__ par, double *__restrict__ wts,
+                   uint32_t *__restrict__ flags)
+{
+    extern __shared__ double sm[];
+    const int d = blockIdx.x, s0 = drop_start[d], n = drop_start[d + 1] - s0;
+    // shared layout: sp[n+1] (then cum[g+1]), qs[n+1] and span[n] (ints),
+    // cx[n], cy[n], the reciprocals and arc lengths [n], band[4n], the last
+    // three rows [3n]
+    double *sp = sm;
+    int *qs = (int *)(sp + maxn + 1);
+    int *span = qs + (maxn + 1);
+    double *cx = (double *)(qs + 2 * (maxn + 1)), *cy = cx + maxn, *rinv = cy + maxn;
+    double *band = rinv + maxn, *dn = band + 4 * maxn;
+    __shared__ double total;
+    __shared__ int bad;
+    for (int m = threadIdx.x; m < n; m += kT) {  // chord lengths
+        const int a = s0 + m, b = s0 + (m + 1 == n ? 0 : m + 1);
+        const double dx = X[b] - X[a], dy = Y[b] - Y[a];
+        cx[m] = sqrt(dx * dx + dy * dy);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        total = serial_sum(n, cx, sp);
+        bad = 0;
+    }
+    __syncthreads();
+    const double Lc = total;
+    int g = (int)floor(Lc / (1.5 * h) + 0.5);
+    if (g < 4) g = 4;
+    if (g > n) g = n;
+    const double tau = Lc / g;
+    for (int m = threadIdx.x; m < n; m += kT) {
+        double w[4];
+        bspl_basis(sp[m], tau, g, w);
+        span[m] = bspl_span(sp[m], tau, g);
+        for (int r = 0; r < 4; r++) wts[4L * (s0 + m) + r] = w[r];
+    }
+    for (int k = threadIdx.x; k < 3 * g; k += kT) dn[k] = 0.0;
+    __syncthreads();
+    span_starts(n, g, span, qs);
+    __syncthreads();
+    normal_equations(X, Y, s0, g, qs, wts, [&](int i, int dd, double acc, double accy) {
+        if (dd == 4) { cx[i] = acc; cy[i] = accy; return; }
+        const int j = i + dd >= g ? i + dd - g : i + dd;
+        const int lo = min(i, j), hi = max(i, j);
+        if (hi >= g - 3) dn[(hi - (g - 3)) * g + lo] = acc;
+        else band[4 * hi + 3 - (hi - lo)] = acc;
+    });
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int f = serial_factor(band, dn, g, threadIdx.x, rinv);  // the same in every lane
+        if (f != 0) {
+            if (threadIdx.x == 0) bad = 1;
+        } else {
+            serial_subst(band, dn, g, rinv, cx, cy, threadIdx.x);
+        }
+    }
+    __syncthreads();
+    double *out = fit + fit_base(s0, d);
+    if (bad) {
+        if (threadIdx.x == 0) {
+            atomicOr(&flags[2], 1u);
+            par[4 * d] = (double)g; par[4 * d + 1] = tau; par[4 * d + 2] = 0.0; par[4 * d + 3] = 1.0;
+        }
+        return;
+    }
+    for (int q = threadIdx.x; q < g; q += kT) rinv[q] = gl_len(q * tau, (q + 1) * tau, tau, g, cx, cy);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const double len = serial_sum(g, rinv, sp);
+        par[4 * d] = (double)g; par[4 * d + 1] = tau; par[4 * d + 2] = len; par[4 * d + 3] = 0.0;
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < g; q += kT) { out[q] = cx[q]; out[n + q] = cy[q]; }
+    for (int q = threadIdx.x; q <= g; q += kT) out[2 * n + q] = sp[q];
+}
+
+// The placement of k_reloc_place with the parameter s as the iterate, eight
+// lanes a marker: lane k evaluates the k-th Gauss-Legendre term, lane 0 also
+// the speed at s, and every lane sums the eight terms in order.
+__global__ void __launch_bounds__(kPlaceT)
+k_reloc_place_serial(int M, const int32_t *__restrict__ drop_of, const int32_t *__restrict__ drop_start,
+                     const double *__restrict__ fit, const double *__restrict__ par,
+                     double *__restrict__ X, double *__restrict__ Y)
+{
+    const int lane = threadIdx.x & 7, j = (blockIdx.x * kPlaceT + threadIdx.x) >> 3;
+    const unsigned grp = 0xffu << (threadIdx.x & 24);  // the eight lanes of this marker
+    if (j >= M) return;  // whole groups leave together
+    const int d = drop_of[j], s0 = drop_start[d], n = drop_start[d + 1] - s0, m = j - s0;
+    if (par[4 * d + 3] != 0.0) return;
+    const int g = (int)par[4 * d];
+    const double tau = par[4 * d + 1], Lp = par[4 * d + 2];
+    const double *cx = fit + fit_base(s0, d), *cy = cx + n, *cum = cx + 2 * n;
+    const double target = Lp * (double)m / (double)n;
+    int lo = 0, hi = g - 1;  // largest q <= g-1 with cum[q] <= target
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (cum[mid] <= target) lo = mid; else hi = mid - 1;
+    }
+    const int q = lo;
+    const double a = q * tau, b = (q + 1) * tau;
+    const double seg = cum[q + 1] - cum[q];
+    double s = a + tau * (target - cum[q]) / seg, prev = s;
+    for (int it = 1; it <= 12; it++) {
+        const double mid = 0.5 * (a + s), half = 0.5 * (s - a);
+        const double term = cGLW[lane] * bspl_speed(mid + half * cGLX[lane], tau, g, cx, cy);
+        const double sp_ = lane == 0 ? bspl_speed(s, tau, g, cx, cy) : 0.0;
+        double sum = 0.0;
+        for (int k = 0; k < 8; k++) sum += __shfl_sync(grp, term, k, 8);
+        const double f = cum[q] + sum * half - target;
+        double sn = s - f / __shfl_sync(grp, sp_, 0, 8);
+        if (sn < a) sn = a;
+        if (sn > b) sn = b;
+        const long long bn = __double_as_longlong(sn);
+        if (bn == __double_as_longlong(s)) break;
+        if (it > 1 && bn == __double_as_longlong(prev)) {  // a cycle of two
+            if (!((12 - it) & 1)) s = sn;
+            break;
+        }
+        prev = s;
+        s = sn;
+    }
+    if (lane != 0) return;
+    double px, py;
+    bspl_point(s, tau, g, cx, cy, px, py);
+    X[j] = px;
+    Y[j] = py;
 }
 
 }  // namespace
@@ -2198,9 +2610,19 @@ void launch_mass_correct(Markers &mk, const double *A0, int axisym, double tol, 
                                               mk.X, mk.Y, eps);
 }
 
-void launch_relocate(Markers &mk, cudaStream_t s)
+void launch_relocate(Markers &mk, bool serial, cudaStream_t s)
 {
     size_t sm = relocate_smem(mk.max_drop);
+    if (serial) {
+        raise_smem_limit((const void *)k_reloc_fit_serial, (int)sm);
+        note_launch(2);
+        k_reloc_fit_serial<<<mk.ndrops, kT, sm, s>>>(mk.X, mk.Y, mk.drop_start, mk.h,
+                                                     relocate_maxn(mk.max_drop), mk.rfit, mk.rpar,
+                                                     mk.rwts, mk.flags);
+        k_reloc_place_serial<<<cdiv(8L * mk.M, kPlaceT), kPlaceT, 0, s>>>(
+            mk.M, mk.drop_of, mk.drop_start, mk.rfit, mk.rpar, mk.X, mk.Y);
+        return;
+    }
     raise_smem_limit((const void *)k_reloc_fit, (int)sm);
     note_launch();
     k_reloc_fit<<<mk.ndrops, kT, sm, s>>>(mk.X, mk.Y, mk.drop_start, mk.h, relocate_maxn(mk.max_drop), mk.rfit,
