@@ -1196,6 +1196,11 @@ struct Cnn {
          *gup = nullptr;
     float *y32 = nullptr, *t = nullptr, *lsum = nullptr, *part = nullptr;
     double *stats = nullptr, *rpart = nullptr;
+    // the weight gradients' streams (see cnn_backward), one event per layer's
+    // output gradient and one per weight gradient
+    static constexpr int kSide = 3;
+    cudaStream_t side[kSide] = {};
+    cudaEvent_t ev_gy[9] = {}, ev_dw[9] = {};
     // coarse-grid inference: restricted inputs and prolongated outputs
     double *cbuf = nullptr;
     size_t cbuf_cap = 0;
@@ -1327,6 +1332,12 @@ Cnn *cnn_new(int c1, int c2, unsigned long long seed, cudaStream_t s, cudaError_
     }
     *err = cudaMemcpy(n->w, h.data(), off * 4, cudaMemcpyHostToDevice);
     if (*err == cudaSuccess) *err = cudaMemset(n->m, 0, off * 4 * 3);
+    for (auto &q : n->side)
+        if (*err == cudaSuccess) *err = cudaStreamCreateWithFlags(&q, cudaStreamNonBlocking);
+    for (int k = 0; k < kLayers; k++) {
+        if (*err == cudaSuccess) *err = cudaEventCreateWithFlags(&n->ev_gy[k], cudaEventDisableTiming);
+        if (*err == cudaSuccess) *err = cudaEventCreateWithFlags(&n->ev_dw[k], cudaEventDisableTiming);
+    }
     if (*err != cudaSuccess) { cnn_free(n); return nullptr; }
     return n;
 }
@@ -1337,6 +1348,12 @@ void cnn_free(Cnn *n)
     if (n->wmem) cudaFree(n->wmem);
     if (n->amem) cudaFree(n->amem);
     if (n->cbuf) cudaFree(n->cbuf);
+    for (auto &q : n->side)
+        if (q) cudaStreamDestroy(q);
+    for (int k = 0; k < kLayers; k++) {
+        if (n->ev_gy[k]) cudaEventDestroy(n->ev_gy[k]);
+        if (n->ev_dw[k]) cudaEventDestroy(n->ev_dw[k]);
+    }
     delete n;
 }
 
@@ -1427,7 +1444,15 @@ void cnn_forward(Cnn &n, int B, int N, double h, const double *rhs, const double
     conv_launch<16, 16>(B, N, N, n.a5, nullptr, nullptr, L[8].wf, bias(8), 0, tc == 2 ? n.y : nullptr, nullptr, n.y32, s, tc);
 }
 
-// Loss and gradients of every parameter (into n.g, master layout).
+// Loss and gradients of every parameter (into n.g, master layout).  A layer's
+// weight gradient waits only for its output gradient, and nothing but the
+// final reduction waits for it: the weight gradients (192 CTAs of a few warps,
+// bound by latency) run on side streams next to the chain of input gradients
+// and to one another (8 x 256^2, the whole call: 750 us one after another, 621
+// so).  A buffer that a
+// weight gradient may still be reading is not written again: where the chain
+// needs one more it takes the target's or the output's (read by the loss
+// alone), t4's or a5's (after the weight gradients that read them) or gup's.
 void cnn_backward(Cnn &n, int B, int N, cudaStream_t s)
 {
     const int N2 = N * N, H2 = N / 2, H4 = N / 4;
@@ -1442,40 +1467,52 @@ void cnn_backward(Cnn &n, int B, int N, cudaStream_t s)
     k_loss_sums<<<gl, 256, 0, s>>>(N2, sc, n.y32, n.t, means, sums);
     k_loss_grad<<<gl, 256, 0, s>>>(N2, B, sc, n.y32, n.t, means, sums, n.gbig, n.lsum);
     ReduceArgs ra;
+    // layer k's weight gradient, from the output gradient that s has just formed
+    auto side = [&](int k, auto launch) {
+        cudaStream_t q = n.side[k % Cnn::kSide];
+        cudaEventRecord(n.ev_gy[k], s);
+        cudaStreamWaitEvent(q, n.ev_gy[k], 0);
+        launch(q);
+        cudaEventRecord(n.ev_dw[k], q);
+    };
     // a layer's input gradient: convolution with the flipped weights
     const bf16 *none = nullptr;
+    bf16 *gp2 = (bf16 *)n.t, *ga2 = n.t4, *gp1 = n.gup, *gs1 = n.y, *ga1 = n.a5;
     // c6 (linear): input a5, grad gbig (channel 0 of two stored)
-    conv_dw<16, 16, 0, 16, 2>(n, ra, 8, B, N, N, n.a5, n.gbig, s);
+    side(8, [&](cudaStream_t q) { conv_dw<16, 16, 0, 16, 2>(n, ra, 8, B, N, N, n.a5, n.gbig, q); });
     conv_launch<16, 16, 0, 2>(B, N, N, n.gbig, none, n.a5, L[8].wb, nullptr, 0, n.gbig2, nullptr, nullptr, s);  // grad a5, masked
     // c5: in up2(t4) ++ s1; the input gradient split into grad t4 (masked) and s1's skip part
-    conv_dw<48, 16, 32>(n, ra, 7, B, N, N, n.s1, n.gbig2, s, n.t4);
+    side(7, [&](cudaStream_t q) { conv_dw<48, 16, 32>(n, ra, 7, B, N, N, n.s1, n.gbig2, q, n.t4); });
     conv_launch<16, 48, 0, 16, kEpiSplit>(B, N, N, n.gbig2, none, n.t4, L[7].wb, nullptr, 0, n.gcat, n.gmid, nullptr, s);
     // c4: in up2(t3) ++ s2
-    conv_dw<64, 32, 32>(n, ra, 6, B, H2, H2, n.s2, n.gmid, s, n.t3);
+    side(6, [&](cudaStream_t q) { conv_dw<64, 32, 32>(n, ra, 6, B, H2, H2, n.s2, n.gmid, q, n.t3); });
     conv_launch<32, 64, 0, 32, kEpiSplit>(B, H2, H2, n.gmid, none, n.t3, L[6].wb, nullptr, 0, n.gup, n.gsmall, nullptr, s);
     // c3b: in a3
-    conv_dw<32, 32>(n, ra, 5, B, H4, H4, n.a3, n.gsmall, s);
+    side(5, [&](cudaStream_t q) { conv_dw<32, 32>(n, ra, 5, B, H4, H4, n.a3, n.gsmall, q); });
     conv_launch<32, 32>(B, H4, H4, n.gsmall, none, n.a3, L[5].wb, nullptr, 0, n.gsmall2, nullptr, nullptr, s);  // grad a3, masked
     // c3a: in p2
-    conv_dw<32, 32>(n, ra, 4, B, H4, H4, n.p2, n.gsmall2, s);
-    conv_launch<32, 32>(B, H4, H4, n.gsmall2, none, nullptr, L[4].wb, nullptr, 0, n.gsmall, nullptr, nullptr, s);  // grad p2
+    side(4, [&](cudaStream_t q) { conv_dw<32, 32>(n, ra, 4, B, H4, H4, n.p2, n.gsmall2, q); });
+    conv_launch<32, 32>(B, H4, H4, n.gsmall2, none, nullptr, L[4].wb, nullptr, 0, gp2, nullptr, nullptr, s);  // grad p2
     // grad s2 = skip part of the c4 input grad + pool2 backward, masked
     note_launch();
-    k_skip_grad<<<cdiv((long)B * H2 * H2 * 4, 256), 256, 0, s>>>(B * H2 * H2 * 4, H2, H2, 32, n.gup, n.gsmall, n.s2, n.gmid2);
+    k_skip_grad<<<cdiv((long)B * H2 * H2 * 4, 256), 256, 0, s>>>(B * H2 * H2 * 4, H2, H2, 32, n.gup, gp2, n.s2, n.gmid2);
     // c2b: in a2
-    conv_dw<32, 32>(n, ra, 3, B, H2, H2, n.a2, n.gmid2, s);
-    conv_launch<32, 32>(B, H2, H2, n.gmid2, none, n.a2, L[3].wb, nullptr, 0, n.gmid, nullptr, nullptr, s);   // grad a2, masked
+    side(3, [&](cudaStream_t q) { conv_dw<32, 32>(n, ra, 3, B, H2, H2, n.a2, n.gmid2, q); });
+    cudaStreamWaitEvent(s, n.ev_dw[7], 0);  // which reads t4
+    conv_launch<32, 32>(B, H2, H2, n.gmid2, none, n.a2, L[3].wb, nullptr, 0, ga2, nullptr, nullptr, s);   // grad a2, masked
     // c2a: in p1
-    conv_dw<16, 32>(n, ra, 2, B, H2, H2, n.p1, n.gmid, s);
-    conv_launch<32, 16>(B, H2, H2, n.gmid, none, nullptr, L[2].wb, nullptr, 0, n.gmid2, nullptr, nullptr, s);  // grad p1
+    side(2, [&](cudaStream_t q) { conv_dw<16, 32>(n, ra, 2, B, H2, H2, n.p1, ga2, q); });
+    conv_launch<32, 16>(B, H2, H2, ga2, none, nullptr, L[2].wb, nullptr, 0, gp1, nullptr, nullptr, s);  // grad p1
     // grad s1 = skip part of the c5 input grad + pool2 backward, masked
     note_launch();
-    k_skip_grad<<<cdiv(P * 2, 256), 256, 0, s>>>((int)(P * 2), N, N, 16, n.gcat, n.gmid2, n.s1, n.gbig);
+    k_skip_grad<<<cdiv(P * 2, 256), 256, 0, s>>>((int)(P * 2), N, N, 16, n.gcat, gp1, n.s1, gs1);
     // c1b: in a1
-    conv_dw<16, 16>(n, ra, 1, B, N, N, n.a1, n.gbig, s);
-    conv_launch<16, 16>(B, N, N, n.gbig, none, n.a1, L[1].wb, nullptr, 0, n.gbig2, nullptr, nullptr, s);     // grad a1, masked
+    side(1, [&](cudaStream_t q) { conv_dw<16, 16>(n, ra, 1, B, N, N, n.a1, gs1, q); });
+    cudaStreamWaitEvent(s, n.ev_dw[8], 0);  // which reads a5
+    conv_launch<16, 16>(B, N, N, gs1, none, n.a1, L[1].wb, nullptr, 0, ga1, nullptr, nullptr, s);     // grad a1, masked
     // c1a: in x
-    conv_dw<16, 16, 0, 2, 16>(n, ra, 0, B, N, N, n.x, n.gbig2, s);
+    side(0, [&](cudaStream_t q) { conv_dw<16, 16, 0, 2, 16>(n, ra, 0, B, N, N, n.x, ga1, q); });
+    for (int k = 0; k < kLayers; k++) cudaStreamWaitEvent(s, n.ev_dw[k], 0);
     int ctas = 0;
     for (int k = 0; k < kLayers; k++) {
         ra.gw[k] = n.g + L[k].woff; ra.gb[k] = n.g + L[k].boff;
