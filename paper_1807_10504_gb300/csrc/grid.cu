@@ -113,8 +113,8 @@ __global__ void k_correct(int nx, int ny, double ih, double dt,
 // with four or more): 44 instructions a cell, times 32/30 and (R + 1) / R.  A
 // 32 x 8 tile with the fluxes in shared memory has partly filled warps in
 // every pass over its ring and two barriers.  Next to the hierarchy's setup
-// and the face force, as in a step: 1024^2 171 -> 149 us, 2048^2 665 -> 571,
-// 256 x 1024 axisymmetric 107 -> 61.  R: rows per warp, 16 where that gives
+// and the face force, as in a step: 1024^2 171 -> 135 us, 2048^2 665 -> 571,
+// 256 x 1024 axisymmetric 107 -> 55.  R: rows per warp, 16 where that gives
 // 1024 warps, fewer below (512^2: 45 us with 8 rows, 109 with 16, whose 576
 // warps leave each to its latency; 46 the tiles).
 //
@@ -134,7 +134,7 @@ __global__ void k_correct(int nx, int ny, double ih, double dt,
 constexpr int kPredT = 128, kPredCols = 30;
 template <bool AXI>
 __global__ void __launch_bounds__(kPredT)
-k_predictor(int nx, int ny, int R, double h, double visc, double dt,
+k_predictor(int nx, int ny, int R, double ih, double visc, double dt,
             const double *__restrict__ rho, const double *__restrict__ mu,
             const double *__restrict__ u, const double *__restrict__ v,
             const double *aup, const double *avp,  // may be au, av
@@ -170,7 +170,8 @@ k_predictor(int nx, int ny, int R, double h, double visc, double dt,
     auto up = [&](double x) { return __shfl_up_sync(kAll, x, 1); };
     auto down = [&](double x) { return __shfl_down_sync(kAll, x, 1); };
     // the factors of the differences
-    const double ih = 1.0 / h, hdt = 0.5 * dt, v2 = 2.0 * visc * ih * ih;
+    const double hdt = 0.5 * dt, v2 = 2.0 * visc * ih * ih;
+    const double gx2 = 2.0 * gx, gy2 = 2.0 * gy, ca = have_prev ? -3.0 : -2.0;
     double xi = 0.25 * ih, xw = xi, xv = v2, xvw = v2, xm = 0.0;  // x-face: cells i, i-1
     double ge = 0.0625 * ih, gw = ge, we = 0.25 * v2, ww = we;    // y-face: nodes i+1, i
     const double ih4 = 0.25 * ih, ih16 = 0.0625 * ih, v24 = 0.25 * v2;
@@ -229,15 +230,14 @@ k_predictor(int nx, int ny, int R, double h, double visc, double dt,
                 double adv, q;
                 if constexpr (AXI) adv = fma(xi, fx, fma(-xw, fw, ih16 * (G1 - G)));
                 else adv = fma(G1 - G, ih16, (fx - fw) * ih4);
-                // twice (viscous - (3/2 adv - 1/2 adv before)), its half in dt / 2
-                q = have_prev ? fma(-3.0, adv, ap) : -2.0 * adv;
+                // twice (viscous - (3/2 adv - 1/2 adv before)), or - adv in the
+                // first step; its half in dt / 2
+                q = fma(ca, adv, ap);
                 if constexpr (AXI)
                     q = fma(xv, vx, fma(-xvw, vw, fma(v24, Wx1 - Wx, fma(xm, (mw + m0) * u0, q))));
                 else
                     q = fma(v2, fma(-0.25, Wx, fma(0.25, Wx1, vx - vw)), q);
-                double un = fma(hdt, q * irx, u0);
-                if (__double_as_longlong(gx) << 1) un = fma(dt, gx, un);
-                us[kx] = un;
+                us[kx] = fma(hdt, fma(q, irx, gx2), u0);
                 au[kx] = adv;
             }
             if (i == nx - 1) { us[kx + 1] = 0.0; au[kx + 1] = 0.0; }  // the right wall's face
@@ -247,12 +247,10 @@ k_predictor(int nx, int ny, int R, double h, double visc, double dt,
                 double adv, q;
                 if constexpr (AXI) adv = fma(ge, Ge, fma(-gw, G, (fy - fyp) * ih4));
                 else adv = fma(Ge - G, ih16, (fy - fyp) * ih4);
-                q = have_prev ? fma(-3.0, adv, bp) : -2.0 * adv;
+                q = fma(ca, adv, bp);
                 if constexpr (AXI) q = fma(v2, vy - vyp, fma(we, We, fma(-ww, Wy, q)));
                 else q = fma(v2, fma(-0.25, Wy, fma(0.25, We, vy - vyp)), q);
-                double vn = fma(hdt, q * iry, v0);
-                if (__double_as_longlong(gy) << 1) vn = fma(dt, gy, vn);
-                vs[ky] = vn;
+                vs[ky] = fma(hdt, fma(q, iry, gy2), v0);
                 av[ky] = adv;
             }
             if (j == ny - 1) { vs[ky + nx] = wb; av[ky + nx] = 0.0; }  // the top wall's face
@@ -652,10 +650,10 @@ static void predictor(bool axi, int nx, int ny, double h, double dt, const doubl
     const unsigned g = (unsigned)cdiv(sx * cdiv(ny, R), kPredT / 32);
     note_launch();
     if (axi)
-        k_predictor<true><<<g, kPredT, 0, s>>>(nx, ny, R, h, visc, dt, rho, mu, u, v, au_prev, av_prev,
+        k_predictor<true><<<g, kPredT, 0, s>>>(nx, ny, R, 1.0 / h, visc, dt, rho, mu, u, v, au_prev, av_prev,
                                                have_prev, gx, gy, frame, bx, by, us, vs, au, av);
     else
-        k_predictor<false><<<g, kPredT, 0, s>>>(nx, ny, R, h, visc, dt, rho, mu, u, v, au_prev, av_prev,
+        k_predictor<false><<<g, kPredT, 0, s>>>(nx, ny, R, 1.0 / h, visc, dt, rho, mu, u, v, au_prev, av_prev,
                                                 have_prev, gx, gy, frame, bx, by, us, vs, au, av);
 }
 

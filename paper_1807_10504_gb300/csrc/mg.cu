@@ -2155,16 +2155,17 @@ __global__ void k_apply_mean(long n, double *__restrict__ p, const double *__res
 }
 
 // sum (b0 - A p)^2 over the fine grid, FP64, into res[2].  A warp takes 31
-// columns of kResRows rows at a time (lane 31 serves its neighbour): a
+// columns of ROWS rows at a time (lane 31 serves its neighbour): a
 // difference to the west is the western cell's difference to the east, one to
 // the south the one to the north of the row below, so a cell costs 8.5 FP64
 // operations, which bound the kernel, in place of 10 (1024^2: 28.4 -> 24.9 us,
 // 2048^2: 87 -> 74, 512^2: 14.1 -> 12.9), and all rows' loads are in flight at
-// once.  With rf != NULL
-// also writes the FP32 residual and zeroes the FP32 correction for the inner
+// once.  ROWS: 4 from 2^17 cells up, 1 below, where one warp's latency counts
+// (256^2: 7.2 us with 4 and 6.5 with one cell a thread; 64^2 6.6 and 5.2).  With
+// rf != NULL also writes the FP32 residual and zeroes the FP32 correction for the inner
 // cycle.  check = 1 (first) or 2 (after `inc` cycles): the block that
 // finishes the sum also runs the convergence test of the graph's solve loop.
-constexpr int kResRows = 4;
+template <int ROWS>
 __global__ void __launch_bounds__(kRedT)
 k_resnorm(int nx, int ny, double ih2, const double *__restrict__ bx,
           const double *__restrict__ by, const double *__restrict__ b0,
@@ -2173,29 +2174,29 @@ k_resnorm(int nx, int ny, double ih2, const double *__restrict__ bx,
           cudaGraphConditionalHandle hnd, int check, int inc)
 {
     const int lane = threadIdx.x & 31;
-    const int sx = (nx + 30) / 31, nst = sx * ((ny + kResRows - 1) / kResRows);
+    const int sx = (nx + 30) / 31, nst = sx * ((ny + ROWS - 1) / ROWS);
     pdl_enter();
     double s = 0.0;
     for (int st = blockIdx.x * (kRedT / 32) + (threadIdx.x >> 5); st < nst; st += gridDim.x * (kRedT / 32)) {
-        const int ty = st / sx, i = (st - ty * sx) * 31 + lane, j0 = ty * kResRows;
+        const int ty = st / sx, i = (st - ty * sx) * 31 + lane, j0 = ty * ROWS;
         // beyond a wall beta is zero: any value stands for the one there
         const int ic = min(i, nx - 1), iw = min(max(i - 1, 0), nx - 1), ix = min(i, nx);
-        double c[kResRows + 2], w[kResRows], fx[kResRows], fy[kResRows + 1], b[kResRows];
+        double c[ROWS + 2], w[ROWS], fx[ROWS], fy[ROWS + 1], b[ROWS];
 #pragma unroll
-        for (int r = 0; r < kResRows + 2; r++) c[r] = p[(long)min(max(j0 + r - 1, 0), ny - 1) * nx + ic];
+        for (int r = 0; r < ROWS + 2; r++) c[r] = p[(long)min(max(j0 + r - 1, 0), ny - 1) * nx + ic];
 #pragma unroll
-        for (int r = 0; r < kResRows; r++) {
+        for (int r = 0; r < ROWS; r++) {
             const long j = min(j0 + r, ny - 1);
             w[r] = p[j * nx + iw];
             fx[r] = bx[j * (nx + 1) + ix];
             fy[r] = by[j * nx + ic];
             b[r] = b0[j * nx + ic];
         }
-        fy[kResRows] = by[(long)min(j0 + kResRows, ny) * nx + ic];
+        fy[ROWS] = by[(long)min(j0 + ROWS, ny) * nx + ic];
         const bool out = lane < 31 && i < nx;
         double ds = c[1] - c[0];
 #pragma unroll
-        for (int r = 0; r < kResRows; r++) {
+        for (int r = 0; r < ROWS; r++) {
             const double dw = c[r + 1] - w[r], dn = c[r + 2] - c[r + 1];
             const double de = __shfl_down_sync(0xffffffffu, dw, 1), fe = __shfl_down_sync(0xffffffffu, fx[r], 1);
             double f = fe * de;
@@ -2644,7 +2645,7 @@ static int resident_red_blocks()
         int dev = 0, sms = 0, per = 0;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_resnorm, kRedT, 0) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_resnorm<4>, kRedT, 0) != cudaSuccess ||
             sms <= 0 || per <= 0) {
             cudaGetLastError();
             return 8 * 152;
@@ -2657,6 +2658,7 @@ static int resident_red_blocks()
 // Blocks of a reduction over n cells: one wave, but none without a cell a
 // thread (1216 blocks on 64^2 cells left 3 threads a block with work and
 // 1216 partials to fold: 11 us).
+static auto resnorm_kernel(long n) { return n >= (1L << 17) ? k_resnorm<4> : k_resnorm<1>; }
 static int red_grid(const MG &mg, long n) { return std::min(mg.red_blocks, (int)cdiv(n, kRedT)); }
 
 size_t mg_layout(MG &mg, int nx, int ny, double h, char *base)
@@ -2788,7 +2790,7 @@ long mg_bench_op(MG &mg, int op, int level, cudaStream_t s)
     case 6: {
         Level &v0 = mg.lv[0];
         note_launch();
-        launch_pdl(k_resnorm, red_grid(mg, (long)v0.nx * v0.ny), kRedT, 0, s, v0.nx, v0.ny, 1.0 / (v0.h * v0.h), v0.d.bx,
+        launch_pdl(resnorm_kernel((long)v0.nx * v0.ny), red_grid(mg, (long)v0.nx * v0.ny), kRedT, 0, s, v0.nx, v0.ny, 1.0 / (v0.h * v0.h), v0.d.bx,
                    v0.d.by, (const double *)v0.d.r, (const double *)v0.d.e, v0.f.r, v0.f.e,
                    mg.red + 8, mg.red_count, mg.red, (SolveCtl *)nullptr,
                    (cudaGraphConditionalHandle)0, 0, 0);
@@ -2918,7 +2920,7 @@ ib_status mg_run_direct(MG &mg, const double *rhs, double *p, int precision, dou
         const bool pr = prof_on(kProfResnorm);
         if (pr) prof_mark(s, true);
         note_launch();
-        k_resnorm<<<RB, kRedT, 0, s>>>(v0.nx, v0.ny, ih2, v0.d.bx, v0.d.by, b0, e0,
+        resnorm_kernel(n)<<<RB, kRedT, 0, s>>>(v0.nx, v0.ny, ih2, v0.d.bx, v0.d.by, b0, e0,
                                        precision ? v0.f.r : nullptr,
                                        precision ? v0.f.e : nullptr, part, mg.red_count,
                                        res, nullptr, (cudaGraphConditionalHandle)0, 0, 0);
@@ -3008,7 +3010,7 @@ static cudaError_t build_solve_graph(MG &mg, SolveGraph &sg)
     // residual norm + convergence test (check 1: before the loop, 2: in its body)
     auto resnorm = [&](cudaStream_t st, int check) {
         note_launch();
-        launch_pdl(k_resnorm, RB, kRedT, 0, st, v0.nx, v0.ny, ih2, v0.d.bx, v0.d.by, b0, e0,
+        launch_pdl(resnorm_kernel(n), RB, kRedT, 0, st, v0.nx, v0.ny, ih2, v0.d.bx, v0.d.by, b0, e0,
                    sg.precision ? v0.f.r : nullptr, sg.precision ? v0.f.e : nullptr, part,
                    mg.red_count, res, mg.ctl, hnd, check, sg.precision == 2 ? 2 : 1);
     };
