@@ -1,0 +1,214 @@
+"""GPU parity of the kernels' separate paths at the sizes where they change or
+end: strips and tiles that do not divide the grid, chains and rings of a few
+spans, coarsest levels on either side of the one-block inverse, lists that
+overflow, drops larger than a register-held share."""
+import numpy as np
+import pytest
+
+import workloads as W
+from oracle import cnn as OC
+from test_gpu_cnn import batch, bf16, dict_of, flat_of, oracle_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def T():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    return torch
+
+
+@pytest.fixture(scope="module")
+def ib():
+    import paper_1807_10504_gb300 as ib
+    ib.lib()
+    return ib
+
+
+# One column and one row short of, at and past a strip of 30 columns and a
+# march of 16 rows; the smallest grid.  About fifty operations a face on
+# operands whose magnitudes sum to at most a few hundred times the result's
+# largest: 1e-12 of it.
+@pytest.mark.parametrize("axisym", [0, 1])
+@pytest.mark.parametrize("nx,ny", [(2, 2), (29, 17), (30, 16), (31, 33), (61, 1100)])
+def test_predictor_strips(T, ib, O, nx, ny, axisym):
+    h, dt = 1.0 / 32, 2e-4
+    rho, mu, bx, by = O.coeffs(W.random_H(nx, ny, 3), 1e-3, 1.0, 1e-4, 1e-2)
+    u, v = W.random_faces(nx, ny, 4)
+    aup, avp = W.random_faces(nx, ny, 5)
+    d = lambda a: T.from_numpy(np.ascontiguousarray(a)).cuda()
+    if axisym:
+        got = ib.ib_op_predictor_axi(d(rho), d(mu), d(u), d(v), h, dt, d(aup), d(avp), gy=-9.81,
+                                     S=0.37, wb=0.21)
+        ref = O.predictor_axi(rho, mu, u, v, h, dt, aup, avp, (0.0, -9.81 + 0.37), 0.21)
+    else:
+        got = ib.ib_op_predictor(d(rho), d(mu), d(u), d(v), h, dt, d(aup), d(avp), g=(0.1, -9.8))
+        ref = O.predictor(rho, mu, u, v, h, dt, aup, avp, g=(0.1, -9.8))
+    for a, b in zip(got, ref):
+        assert np.abs(a.cpu().numpy() - b).max() <= 1e-12 * max(np.abs(b).max(), 1.0)
+
+
+# Rings of 4 .. 20 spans (border of 3, 4 and 5 rows, chains of none to five
+# blocks, last rows shorter and longer than the others), and a marker count
+# that takes four lanes a marker.  The spline's matrix has a condition number
+# below 1e3, so rounding moves a marker by less than 1e-12.
+@pytest.mark.parametrize("case", ["rings", "four_lanes", "axisym_small", "axisym"])
+def test_relocation_sizes(T, ib, O, case):
+    axisym = case.startswith("axisym")
+    if case == "rings":
+        n, h = 96, 1.0 / 96
+        mk = W.join([W.circle((12 + 18 * (k % 5)) * h, (12 + 24 * (k // 5)) * h, g * 1.5 * h / (2 * np.pi),
+                              24 + k, theta0=0.1 * k)
+                     for k, g in enumerate((4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 16, 20))])
+        shape = (n, n)
+    elif case == "four_lanes":
+        n, h = 256, 1.0 / 256
+        mk = W.multidrop(n, ndrops=20, rmin=0.03, rmax=0.06, n_per_drop=256, seed=5, gap_cells=8)
+        assert 4096 <= mk.X.size < 8192
+        shape = (n, n)
+    elif case == "axisym_small":
+        h, shape = 1.0 / 32, (32, 64)
+        mk = W.axi_elliptic_drop(1.0, 0.06, 1.2, 16)
+    else:
+        h, shape = 1.0 / 64, (64, 128)
+        mk = W.axi_elliptic_drop(1.0, 0.4, 1.1, 300)
+    ctx = ib.Context(ib.Config(nx=shape[0], ny=shape[1], h=h, axisym=int(axisym)), mk.X, mk.Y, mk.drop_start)
+    ctx.relocate()
+    X, Y = (a.cpu().numpy() for a in ctx.markers())
+    oX, oY = O.bspline_relocate(mk.X, mk.Y, mk.drop_start, h)
+    if axisym:
+        oX, oY = O.symmetrise(oX, oY, mk.drop_start)
+    assert np.abs(X - oX).max() <= 1e-12 and np.abs(Y - oY).max() <= 1e-12
+
+
+# Coarsest levels of 65, 80, 143 and 1023 cells: past the one-block inverse,
+# whole blocks of 16, a remainder, the largest; rows and columns that do not
+# divide the residual norm's strips of 31 x 4.  The residual is reduced by
+# 1e12 (1e11 in mixed precision) on systems whose solution is at most about
+# 1e2 times the scaled right-hand side.
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("nx,ny", [(26, 10), (32, 10), (26, 22), (62, 66), (124, 132)])
+def test_coarsest_sizes(T, ib, O, nx, ny, precision):
+    n = min(nx, ny)
+    h = 1.0 / n
+    X, Y = W.circle(0.5 * nx / n, 0.5 * ny / n, min(0.2, 0.45 - 3.0 / n), 16)
+    ctx = ib.Context(ib.Config(nx=nx, ny=ny, h=h), X, Y, [0, 16])
+    rho, mu, bx, by = O.coeffs(W.random_H(nx, ny, 3), 1e-3, 1.0, 1e-4, 1e-2)
+    b = W.random_cells(nx, ny, 4)
+    d = lambda a: T.from_numpy(np.ascontiguousarray(a)).cuda()
+    ctx.mg_setup(d(bx), d(by))
+    p = T.zeros((ny, nx), dtype=T.float64, device="cuda")
+    tol = 1e-12 if precision == 0 else 1e-11
+    st, cyc, rr = ctx.mg_solve(d(b), p, precision, tol, 200)
+    o = O.mg_solve(bx, by, b, h, precision=0, tol=1e-12, max_cycles=200)
+    assert st == 0 and rr <= tol
+    assert np.abs(p.cpu().numpy() - o.p).max() <= 100 * tol * np.abs(o.p).max()
+
+
+# The coefficient tables' sweeps, two a launch: one launch, whole launches, an
+# odd sweep left, and an odd number of launches (the buffers then end swapped).
+# As the steps of twenty sweeps: p within 1e-10 of its largest value, u and v
+# within 1e-10 of the inertial-capillary velocity.
+@pytest.mark.parametrize("axisym", [0, 1])
+@pytest.mark.parametrize("sweeps", [1, 2, 3, 6])
+def test_cn_sweep_counts(T, ib, O, sweeps, axisym):
+    if axisym:
+        nx, ny, h = 24, 72, 1 / 24
+        mk = W.axi_elliptic_drop(1.5, 0.25, 1.1, 64)
+        kw = dict(axisym=1, frame=1, gy=-1.0)
+    else:
+        nx, ny, h = 40, 56, 1 / 40
+        mk = W.elliptic_drop(0.5, 0.7, 0.22, 1.15, 96)
+        kw = {}
+    kw.update(spread=1, relocate_every=0, viscous=1, cn_sweeps=sweeps, tol=1e-11)
+    ctx = ib.Context(ib.Config(nx=nx, ny=ny, h=h, **kw), mk.X, mk.Y, mk.drop_start)
+    ocfg = O.Config(nx=nx, ny=ny, h=h, **kw)
+    st = O.init_state(ocfg, mk.X, mk.Y, mk.drop_start)
+    dt = W.capillary_dt(h, 1.0, 1e-3, 1.0, 1e-2, 1e-4)
+    for _ in range(2):
+        ctx.ns_step(dt, 1, 1)
+        O.ns_step(ocfg, st, dt)
+    assert np.abs(ctx.get("p").cpu().numpy() - st.p).max() <= 1e-10 * np.abs(st.p).max()
+    for name, ref in (("u", st.u), ("v", st.v)):
+        assert np.abs(ctx.get(name).cpu().numpy() - ref).max() <= 1e-10 * 2.0, name
+
+
+# A drop of more markers than the block's threads hold in registers: the same
+# bisection decisions as the oracle's, so eps to 1e-13 h.
+def test_measure_correction_large_drop(T, ib, O):
+    n, h = 256, 1.0 / 256
+    X, Y = W.circle(0.5, 0.5, 0.3, 2500)
+    start = np.array([0, 2500], np.int32)
+    ctx = ib.Context(ib.Config(nx=n, ny=n, h=h), X, Y, start)
+    A0 = O.drop_measures(X, Y, start, 0)
+    k, nxm, nym, ds = O.curvature(X, Y, start)
+    Xs, Ys = X + 0.31 * h * nxm, Y + 0.31 * h * nym
+    ctx.set_markers_host(Xs, Ys)
+    eps = ctx.mass_correct()
+    Xo, Yo, eo = O.mass_correct(Xs, Ys, start, A0, h, 0)
+    Xg, Yg = (a.cpu().numpy() for a in ctx.markers())
+    assert np.abs(eps - eo).max() <= 1e-13 * h
+    assert np.abs(Xg - Xo).max() <= 1e-14 and np.abs(Yg - Yo).max() <= 1e-14
+
+
+def tilted_box(cx, cy, a, tilt, m):
+    """A square of half-edge a, turned by tilt, m markers an edge."""
+    t = np.linspace(-1.0, 1.0, m, endpoint=False)
+    o = np.ones_like(t)
+    x = a * np.concatenate([t, o, -t, -o])
+    y = a * np.concatenate([-o, t, o, -t])
+    c, s = np.cos(tilt), np.sin(tilt)
+    return cx + c * x - s * y, cy + s * x + c * y
+
+
+# Squares turned by less than 0.001 rad: every segment takes the edge
+# integrals.  One small square (a few listed pairs) and four large ones, whose
+# pairs overflow the list (the rest is integrated in place).  A cell sums a
+# handful of integrals of coordinates up to n cells, each with a few roundings.
+@pytest.mark.parametrize("n,ndrops", [(32, 1), (320, 4)])
+def test_heaviside_along_the_axes(T, ib, O, n, ndrops):
+    h = 1.0 / n
+    if ndrops == 1:
+        mk = W.join([tilted_box(0.5, 0.5, 0.2, 5e-4, 10)])
+    else:
+        mk = W.join([tilted_box(0.27 + 0.46 * (k % 2), 0.27 + 0.46 * (k // 2), 0.19, 4e-4 + 1e-4 * k, 150)
+                     for k in range(4)])
+    ctx = ib.Context(ib.Config(nx=n, ny=n, h=h), mk.X, mk.Y, mk.drop_start)
+    H = ctx.heaviside().cpu().numpy()
+    oH = O.heaviside(mk.X, mk.Y, mk.drop_start, n, n, h)
+    assert np.abs(H - oH).max() <= 1e-13 + 8 * n * 2.0 ** -53
+
+
+# Images that are not whole tiles at any of the three resolutions, down to one
+# pixel at the coarsest; the weight gradients' streams give the same bits on
+# every call and on another stream.  Bounds as for whole tiles: the loss within
+# 1e-2, gradients within 5e-3 of the layer's largest.
+@pytest.mark.parametrize("B,N", [(3, 20), (1, 44), (2, 4)])
+def test_gradient_ragged_tiles(T, B, N):
+    import paper_1807_10504_gb300 as ib
+    P = OC.init_params(seed=4)
+    Pq = {k: (bf16(v) if k.endswith(".w") else v) for k, v in P.items()}
+    net = ib.Net(seed=0)
+    net.set_params(flat_of(P))
+    rhs, rho, p = batch(B, N, 8)
+    d = lambda a: T.from_numpy(np.ascontiguousarray(a)).cuda()
+    c = net.fit_scale(d(rhs), d(p))
+    loss, g = net.grad(d(rhs), d(rho), d(p))
+    x, s, t = oracle_inputs(rhs, rho, p, c)
+    y, cache = OC.forward(Pq, x, keep=True, bf16=True)
+    L, gy = OC.loss(y, t)
+    G, _ = OC.backward(Pq, cache, gy, bf16=True)
+    assert abs(loss - L) <= 1e-2 * L, (loss, L)
+    Gg = dict_of(g, P)
+    for n, _, _, _ in OC.LAYERS:
+        for k in (".w", ".b"):
+            if n + k != "c6.b":
+                a, ref = Gg[n + k].ravel(), G[n + k].ravel()
+                assert np.abs(a - ref).max() <= 5e-3 * np.abs(ref).max(), n + k
+    side = T.cuda.Stream()
+    side.wait_stream(T.cuda.current_stream())
+    with T.cuda.stream(side):
+        loss2, g2 = net.grad(d(rhs), d(rho), d(p))
+    assert loss2 == loss and np.array_equal(g, g2)
