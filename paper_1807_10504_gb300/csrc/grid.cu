@@ -17,40 +17,60 @@ namespace {
 
 constexpr int kT = 256;
 
-__global__ void k_cells_props(int n, double rho_g, double drho, double mu_g,
-                              double dmu, const double *__restrict__ H,
-                              double *__restrict__ rho, double *__restrict__ mu)
-{
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    double hk = H[k];
-    rho[k] = rho_g + drho * hk;
-    mu[k] = mu_g + dmu * hk;
-}
-
 // 2 x for a normal x (an addition to the exponent, no FP64 operation).
 __device__ __forceinline__ double twice(double x)
 {
     return __longlong_as_double(__double_as_longlong(x) + (1LL << 52));
 }
 
-// beta = 1 / (two-cell mean of rho) on x-faces and y-faces.
-__global__ void k_face_beta(int nx, int ny, const double *__restrict__ rho,
-                            double *__restrict__ bx, double *__restrict__ by)
+// rho and mu of the cells and beta = 1 / (two-cell mean of rho) on the faces.
+// A warp takes 31 columns (lane 0 serves its neighbour) of ROWS rows;
+// where a row of H equals the one below in all its lanes, as it does off the
+// interface, rho, mu and beta are those of the row below, and no FP64
+// operation is needed (ten a cell bound the two kernels that this one replaces;
+// next to the face force 8 + 41 us at 1024^2, now 15, and 85 + 64 at 2048^2,
+// now 49).  ROWS: 8 from 2^18 cells up, 1 below (64^2: 6.6 us with 8 rows,
+// 4.1 the two kernels).
+template <int ROWS>
+__global__ void __launch_bounds__(256)
+k_coeffs(int nx, int ny, double rho_g, double drho, double mu_g, double dmu,
+         const double *__restrict__ H, double *__restrict__ rho, double *__restrict__ mu,
+         double *__restrict__ bx, double *__restrict__ by)
 {
-    // one row of x-faces (j < ny) and of y-faces (j <= ny) per blockIdx.y
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-    if (j < ny && i <= nx) {
-        const long k = (long)j * (nx + 1) + i;
-        bx[k] = (i == 0 || i == nx)
-                    ? 0.0
-                    : twice(recip_nr(rho[(long)j * nx + i - 1] + rho[(long)j * nx + i]));
-    }
-    if (i < nx) {
-        const long k = (long)j * nx + i;
-        by[k] = (j == 0 || j == ny)
-                    ? 0.0
-                    : twice(recip_nr(rho[(long)(j - 1) * nx + i] + rho[(long)j * nx + i]));
+    const int lane = threadIdx.x & 31, sx = (nx + 30) / 31;
+    const int wid = blockIdx.x * (256 / 32) + (threadIdx.x >> 5), ty = wid / sx, j0 = ty * ROWS;
+    if (j0 >= ny) return;  // whole warps
+    const int i = (wid - ty * sx) * 31 + lane - 1, c = min(max(i, 0), nx - 1);
+    const bool out = lane >= 1 && i < nx;
+    double h[ROWS];
+#pragma unroll
+    for (int r = 0; r < ROWS; r++) h[r] = H[(long)min(j0 + r, ny - 1) * nx + c];
+    double rc = rho_g + drho * H[(long)max(j0 - 1, 0) * nx + c], mc = 0.0, xv = 0.0, yv = 0.0;
+    bool steady = false;  // yv is the face between two equal rows
+#pragma unroll
+    for (int r = 0; r < ROWS; r++) {
+        const int j = j0 + r;
+        if (j >= ny) break;
+        if (r > 0 && __all_sync(0xffffffffu, __double_as_longlong(h[r]) == __double_as_longlong(h[r - 1]))) {
+            if (!steady) yv = twice(recip_nr(rc + rc));
+            steady = true;
+        } else {
+            const double rn = rho_g + drho * h[r];
+            mc = mu_g + dmu * h[r];
+            xv = twice(recip_nr(__shfl_up_sync(0xffffffffu, rn, 1) + rn));
+            yv = twice(recip_nr(rc + rn));
+            rc = rn;
+            steady = false;
+        }
+        if (out) {
+            const long k = (long)j * nx + i, kx = (long)j * (nx + 1) + i;
+            rho[k] = rc;
+            mu[k] = mc;
+            bx[kx] = i == 0 ? 0.0 : xv;
+            by[k] = j == 0 ? 0.0 : yv;
+            if (i == nx - 1) bx[kx + 1] = 0.0;
+            if (j == ny - 1) by[k + nx] = 0.0;
+        }
     }
 }
 
@@ -110,11 +130,12 @@ __global__ void k_correct(int nx, int ny, double ih, double dt,
 // (and the wall face on the far side by the last column / row).
 //
 // FP64 arithmetic bounds it (64 cycles an instruction for one warp, 19 an SM
-// with four or more): 44 instructions a cell, times 32/30 and (R + 1) / R.  A
+// with four or more): 44 instructions a cell (40 off the interface), times
+// 32/30 and (R + 1) / R.  A
 // 32 x 8 tile with the fluxes in shared memory has partly filled warps in
 // every pass over its ring and two barriers.  Next to the hierarchy's setup
-// and the face force, as in a step: 1024^2 171 -> 135 us, 2048^2 665 -> 571,
-// 256 x 1024 axisymmetric 107 -> 55.  R: rows per warp, 16 where that gives
+// and the face force, as in a step: 1024^2 171 -> 127 us, 2048^2 665 -> 429,
+// 256 x 1024 axisymmetric 107 -> 52.  R: rows per warp, 16 where that gives
 // 1024 warps, fewer below (512^2: 45 us with 8 rows, 109 with 16, whose 576
 // warps leave each to its latency; 46 the tiles).
 //
@@ -185,17 +206,18 @@ k_predictor(int nx, int ny, int R, double ih, double visc, double dt,
         gw = w * ih16; we = e * v24; ww = w * v24;
     }
     // rows j0 - 1 (m), j0 (0) and j0 + 1 (1)
-    double r0, m0, u0, v0, G, Wx, Wy, fyp, vyp, rm;
+    double r0, m0, u0, v0, G, Wx, Wy, fyp, vyp, rm, rn = 0.0, mn = 0.0;
+    bool steady = false;
     double r1 = rho[row(j0 + 1)], m1 = mu[row(j0 + 1)], u1 = ld_u(j0 + 1), v1 = ld_v(j0 + 1);
     {
         rm = rho[row(j0 - 1)];
         const double mm = mu[row(j0 - 1)], um = ld_u(j0 - 1), vm = ld_v(max(j0 - 1, 0));
         r0 = rho[row(j0)]; m0 = mu[row(j0)]; u0 = ld_u(j0); v0 = ld_v(j0);
         const double rs = rm + r0, ms = mm + m0, vl = up(v0);
-        const double rn = rs + up(rs), mn = ms + up(ms), b = vm + v0;
-        G = rn * (vl + v0) * (um + u0);
-        Wx = mn * (u0 - um);
-        Wy = mn * (v0 - vl);
+        const double rb = rs + up(rs), mb = ms + up(ms), b = vm + v0;
+        G = rb * (vl + v0) * (um + u0);
+        Wx = mb * (u0 - um);
+        Wy = mb * (v0 - vl);
         fyp = rm * b * b;
         vyp = mm * (v0 - vm);
     }
@@ -213,8 +235,16 @@ k_predictor(int nx, int ny, int R, double ih, double visc, double dt,
         const double ue = down(u0), a = ue + u0, b = v1 + v0, vl = up(v1);
         const double fx = r0 * a * a, vx = m0 * (ue - u0);
         const double fy = r0 * b * b, vy = m0 * (v1 - v0);
-        const double rs = r0 + r1, ms = m0 + m1;
-        const double rn = rs + up(rs), mn = ms + up(ms);
+        // rows j and j + 1 alike in all lanes, as rows j - 1 and j were: the
+        // nodes' rho and mu are those of the row below
+        const bool eq = __all_sync(kAll, __double_as_longlong(r1) == __double_as_longlong(r0) &&
+                                             __double_as_longlong(m1) == __double_as_longlong(m0));
+        if (!(eq && steady)) {
+            const double rs = r0 + r1, ms = m0 + m1;
+            rn = rs + up(rs);
+            mn = ms + up(ms);
+        }
+        steady = eq;
         const double G1 = rn * (vl + v1) * (u0 + u1);
         const double Wx1 = mn * (u1 - u0), Wy1 = mn * (v1 - vl);
         const double fw = up(fx), vw = up(vx), Ge = down(G), We = down(Wy);
@@ -610,13 +640,14 @@ void launch_coeffs(int nx, int ny, double rho_g, double rho_l, double mu_g,
                    double mu_l, const double *H, double *rho, double *mu,
                    double *bx, double *by, cudaStream_t s)
 {
-    long n = (long)nx * ny;
+    auto launch = [&](auto kernel, int rows) {
+        const long warps = (long)cdiv(nx, 31) * cdiv(ny, rows);
+        kernel<<<cdiv(warps, 256 / 32), 256, 0, s>>>(nx, ny, rho_g, rho_l - rho_g, mu_g, mu_l - mu_g, H, rho,
+                                                     mu, bx, by);
+    };
     note_launch();
-    k_cells_props<<<cdiv(n, kT), kT, 0, s>>>((int)n, rho_g, rho_l - rho_g, mu_g,
-                                             mu_l - mu_g, H, rho, mu);
-    dim3 gb(cdiv(nx + 1, 128), ny + 1);
-    note_launch();
-    k_face_beta<<<gb, 128, 0, s>>>(nx, ny, rho, bx, by);
+    if ((long)nx * ny >= 1L << 18) launch(k_coeffs<8>, 8);
+    else launch(k_coeffs<1>, 1);
 }
 
 void launch_rhs(int nx, int ny, double h, double dt, const double *us,

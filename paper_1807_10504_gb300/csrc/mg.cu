@@ -1066,62 +1066,53 @@ __global__ void k_coarsen_beta(int nx, int ny, const double *__restrict__ bx,
 // multiple of 4 values (16 bytes).
 __host__ __device__ constexpr int xface_pitch(int nx) { return (nx + 4) & ~3; }
 
-// Coefficients of one level in one pass, one thread per cell: the cell's
-// west and south faces (and the east / north wall faces of the last column /
-// row) from the finer level (mean of the two fine faces; at level 0 the
-// caller's faces with the walls set to zero), their FP32 copies (the x-faces
-// twice: packed and in padded rows), and the FP64 and FP32 inverse
-// diagonals (the cell's four faces, recomputed locally).  LEVEL0 at compile
-// time: as an argument both forms of a face were computed and one selected,
-// eight FP64 operations a cell more (14 in place of 6).
-template <bool LEVEL0>
-__device__ __forceinline__ void level_coeffs_cell(int nx, int ny, int i, int j,
-                                                  const double *__restrict__ fbx,
-                                                  const double *__restrict__ fby,
-                                                  double *__restrict__ bx, double *__restrict__ by,
-                                                  float *__restrict__ bxf, float *__restrict__ byf,
-                                                  float *__restrict__ bxp,
-                                                  double *__restrict__ invd, float *__restrict__ invdf,
-                                                  double *__restrict__ w4, float4 *__restrict__ w4f)
+// Coefficients of one level in one pass: every cell's west and south faces
+// (and the east / north wall faces of the last column / row) from the finer
+// level (mean of the two fine faces; at level 0 the caller's faces with the
+// walls set to zero), their FP32 copies (the x-faces twice: packed and in
+// padded rows), and the FP64 and FP32 inverse diagonals (from the cell's four
+// faces).
+struct LevelOut {
+    double *bx, *by, *invd, *w4;
+    float *bxf, *byf, *bxp, *invdf;
+    float4 *w4f;
+};
+struct CellCoeffs {
+    double w, e, s, n, id;
+    float wf, sf, idf;
+};
+// From the cell's four faces.  FP32 by d2f_rn: (float) on integer instructions.
+__device__ __forceinline__ void cell_coeffs(CellCoeffs &c)
 {
-    const int fnx = 2 * nx;  // finer level width (unused at level 0)
-    auto xface = [&](int I, int J) -> double {   // coefficient of x-face (I, J)
-        if (I == 0 || I == nx) return 0.0;
-        if constexpr (LEVEL0) return fbx[(long)J * (nx + 1) + I];
-        return 0.5 * (fbx[(long)(2 * J) * (fnx + 1) + 2 * I] + fbx[(long)(2 * J + 1) * (fnx + 1) + 2 * I]);
-    };
-    auto yface = [&](int I, int J) -> double {
-        if (J == 0 || J == ny) return 0.0;
-        if constexpr (LEVEL0) return fby[(long)J * nx + I];
-        return 0.5 * (fby[(long)(2 * J) * fnx + 2 * I] + fby[(long)(2 * J) * fnx + 2 * I + 1]);
-    };
-    const double w = xface(i, j), e = xface(i + 1, j), s = yface(i, j), n = yface(i, j + 1);
-    const long kx = (long)j * (nx + 1) + i, kc = (long)j * nx + i;
-    // FP32 copies by d2f_rn: (float) on integer instructions
-    const float wf = d2f_rn(w);
-    bx[kx] = w; bxf[kx] = wf;
-    by[kc] = s; byf[kc] = d2f_rn(s);
-    if (i == nx - 1) { bx[kx + 1] = e; bxf[kx + 1] = d2f_rn(e); }
-    if (j == ny - 1) { by[kc + nx] = n; byf[kc + nx] = d2f_rn(n); }
-    const int xp = xface_pitch(nx);
-    float *rowp = bxp + (long)j * xp;
-    rowp[i] = wf;
-    if (i == nx - 1) {
-        rowp[nx] = d2f_rn(e);
-        for (int t = nx + 1; t < xp; t++) rowp[t] = 0.0f;  // padding
-    }
-    const double d = e + w + n + s;
+    c.wf = d2f_rn(c.w);
+    c.sf = d2f_rn(c.s);
+    const double d = c.e + c.w + c.n + c.s;
     // d > 0 on its bit pattern (an FP64 compare costs an FP64 operation)
-    const double id = __double_as_longlong(d) > 0 ? recip_nr(d) : 0.0;
-    invd[kc] = id;
-    invdf[kc] = d2f_rn(id);
-    if (w4 || w4f) {
-        const double ww = w * id, we = e * id, ws = s * id, wn = n * id;
-        if (w4) {
-            reinterpret_cast<double2 *>(w4)[2 * kc] = make_double2(ww, we);
-            reinterpret_cast<double2 *>(w4)[2 * kc + 1] = make_double2(ws, wn);
+    c.id = __double_as_longlong(d) > 0 ? recip_nr(d) : 0.0;
+    c.idf = d2f_rn(c.id);
+}
+__device__ __forceinline__ void store_coeffs(int nx, int ny, int i, int j, const CellCoeffs &c,
+                                             const LevelOut &o)
+{
+    const long kx = (long)j * (nx + 1) + i, kc = (long)j * nx + i;
+    o.bx[kx] = c.w; o.bxf[kx] = c.wf;
+    o.by[kc] = c.s; o.byf[kc] = c.sf;
+    if (i == nx - 1) { o.bx[kx + 1] = 0.0; o.bxf[kx + 1] = 0.0f; }
+    if (j == ny - 1) { o.by[kc + nx] = 0.0; o.byf[kc + nx] = 0.0f; }
+    const int xp = xface_pitch(nx);
+    float *rowp = o.bxp + (long)j * xp;
+    rowp[i] = c.wf;
+    if (i == nx - 1)
+        for (int t = nx; t < xp; t++) rowp[t] = 0.0f;  // the wall face and the padding
+    o.invd[kc] = c.id;
+    o.invdf[kc] = c.idf;
+    if (o.w4 || o.w4f) {
+        const double ww = c.w * c.id, we = c.e * c.id, ws = c.s * c.id, wn = c.n * c.id;
+        if (o.w4) {
+            reinterpret_cast<double2 *>(o.w4)[2 * kc] = make_double2(ww, we);
+            reinterpret_cast<double2 *>(o.w4)[2 * kc + 1] = make_double2(ws, wn);
         }
-        if (w4f) w4f[kc] = make_float4(d2f_rn(ww), d2f_rn(we), d2f_rn(ws), d2f_rn(wn));
+        if (o.w4f) o.w4f[kc] = make_float4(d2f_rn(ww), d2f_rn(we), d2f_rn(ws), d2f_rn(wn));
     }
 }
 
@@ -1152,17 +1143,66 @@ __global__ void k_level_w(LevelWArgs a)
     reinterpret_cast<double2 *>(a.w4[l])[2 * kc + 1] = make_double2(s * id, n * id);
 }
 
-template <bool LEVEL0>
-__global__ void k_level_coeffs(int nx, int ny, const double *__restrict__ fbx,
-                               const double *__restrict__ fby, double *__restrict__ bx,
-                               double *__restrict__ by, float *__restrict__ bxf,
-                               float *__restrict__ byf, float *__restrict__ bxp,
-                               double *__restrict__ invd, float *__restrict__ invdf,
-                               double *__restrict__ w4, float4 *__restrict__ w4f)
+// A warp takes 31 columns (lane 31 serves its neighbour with the east face) of
+// ROWS rows.  Where a row's finer faces equal those of the row below in all
+// lanes, as off the interface, its coefficients are those of the row below: no
+// FP64 operation and no conversion (next to the predictor: 1024^2 67 -> 38 us,
+// 2048^2 178 -> 85).  ROWS = 1, where every cell's work is in flight at once,
+// below 2^20 cells (256^2 under a 512^2 grid: 23 us with 8 rows, 5 with one).  LEVEL0 at compile time: as an argument both forms of a face
+// were computed and one selected.
+template <bool LEVEL0, int ROWS>
+__global__ void __launch_bounds__(256)
+k_level_coeffs(int nx, int ny, const double *__restrict__ fbx, const double *__restrict__ fby, LevelOut o)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
-    if (i >= nx) return;
-    level_coeffs_cell<LEVEL0>(nx, ny, i, j, fbx, fby, bx, by, bxf, byf, bxp, invd, invdf, w4, w4f);
+    const int lane = threadIdx.x & 31, sx = (nx + 30) / 31;
+    const int wid = blockIdx.x * (256 / 32) + (threadIdx.x >> 5), ty = wid / sx, j0 = ty * ROWS;
+    if (j0 >= ny) return;  // whole warps
+    const int i = (wid - ty * sx) * 31 + lane, ic = min(i, nx - 1);
+    const bool out = lane < 31 && i < nx, wall = i == 0 || i >= nx;
+    const int fnx = 2 * nx;  // finer level width
+    // the finer faces: one (level 0) or two per face
+    double xa[ROWS], xb[ROWS], ya[ROWS + 1], yb[ROWS + 1];
+#pragma unroll
+    for (int r = 0; r <= ROWS; r++) {
+        const long J = min(j0 + r, ny);
+        if constexpr (LEVEL0) {
+            ya[r] = fby[J * nx + ic];
+            yb[r] = 0.0;
+            if (r < ROWS) { xa[r] = fbx[min(J, (long)ny - 1) * (nx + 1) + ic]; xb[r] = 0.0; }
+        } else {
+            ya[r] = fby[2 * J * fnx + 2 * ic];
+            yb[r] = fby[2 * J * fnx + 2 * ic + 1];
+            if (r < ROWS) {
+                const long K = 2 * min(J, (long)ny - 1);
+                xa[r] = fbx[K * (fnx + 1) + 2 * ic];
+                xb[r] = fbx[(K + 1) * (fnx + 1) + 2 * ic];
+            }
+        }
+    }
+    auto face = [](double a, double b) {
+        if constexpr (LEVEL0) return a;
+        return 0.5 * (a + b);
+    };
+    auto same = [](double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); };
+    CellCoeffs c;
+    c.n = j0 == 0 ? 0.0 : face(ya[0], yb[0]);
+#pragma unroll
+    for (int r = 0; r < ROWS; r++) {
+        const int j = j0 + r;
+        if (j >= ny) break;
+        // rows j - 1 and j alike, with the faces above and below them
+        const bool eq = r > 0 && j > 1 && j < ny - 1 && same(xa[r], xa[max(r - 1, 0)]) &&
+                        same(xb[r], xb[max(r - 1, 0)]) && same(ya[r], ya[max(r - 1, 0)]) &&
+                        same(yb[r], yb[max(r - 1, 0)]) && same(ya[r + 1], ya[r]) && same(yb[r + 1], yb[r]);
+        if (!__all_sync(0xffffffffu, eq)) {
+            c.w = wall ? 0.0 : face(xa[r], xb[r]);
+            c.e = __shfl_down_sync(0xffffffffu, c.w, 1);
+            c.s = c.n;
+            c.n = j == ny - 1 ? 0.0 : face(ya[r + 1], yb[r + 1]);
+            cell_coeffs(c);
+        }
+        if (out) store_coeffs(nx, ny, i, j, c, o);
+    }
 }
 
 // The small levels (from `first` on) in one CTA, level after level; a level
@@ -1180,9 +1220,24 @@ __global__ void __launch_bounds__(256) k_level_coeffs_small(LevelCoeffArgs a)
     for (int l = a.first; l < a.nl; l++) {
         const int nx = a.nx[l], ny = a.ny[l];
         for (int k = threadIdx.x; k < nx * ny; k += blockDim.x) {
-            const int j = k / nx, i = k - j * nx;
-            level_coeffs_cell<false>(nx, ny, i, j, a.bx[l - 1], a.by[l - 1], a.bx[l], a.by[l], a.bxf[l],
-                              a.byf[l], a.bxp[l], a.invd[l], a.invdf[l], a.w4[l], (float4 *)a.wf[l]);
+            const int j = k / nx, i = k - j * nx, fnx = 2 * nx;
+            const double *fbx = a.bx[l - 1], *fby = a.by[l - 1];
+            auto xface = [&](int I) {
+                return I == 0 || I == nx ? 0.0
+                                         : 0.5 * (fbx[(long)(2 * j) * (fnx + 1) + 2 * I] +
+                                                  fbx[(long)(2 * j + 1) * (fnx + 1) + 2 * I]);
+            };
+            auto yface = [&](int J) {
+                return J == 0 || J == ny
+                           ? 0.0
+                           : 0.5 * (fby[(long)(2 * J) * fnx + 2 * i] + fby[(long)(2 * J) * fnx + 2 * i + 1]);
+            };
+            CellCoeffs c;
+            c.w = xface(i); c.e = xface(i + 1); c.s = yface(j); c.n = yface(j + 1);
+            cell_coeffs(c);
+            store_coeffs(nx, ny, i, j, c,
+                         LevelOut{a.bx[l], a.by[l], a.invd[l], a.w4[l], a.bxf[l], a.byf[l], a.bxp[l],
+                                  a.invdf[l], (float4 *)a.wf[l]});
         }
         __syncthreads();
     }
@@ -2817,6 +2872,8 @@ void ensure_fp64_w(MG &mg, cudaStream_t s)
     mg.fp64_w = true;
 }
 
+constexpr int kCoefRows = 8;            // rows a warp of k_level_coeffs
+constexpr long kCoefCells = 1L << 20;  // levels from this size on; below one row
 void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool with_w)
 {
     const int L = mg.L;
@@ -2829,14 +2886,18 @@ void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool w
     for (int l = 0; l < lsmall; l++) {
         Level &v = mg.lv[l];
         const double *fbx = l == 0 ? bx : mg.lv[l - 1].d.bx, *fby = l == 0 ? by : mg.lv[l - 1].d.by;
-        dim3 g(cdiv(v.nx, 128), v.ny);
+        const LevelOut o{v.d.bx, v.d.by, v.d.invd, with_w ? v.d.w : nullptr, v.f.bx, v.f.by, v.f.bxp,
+                         v.f.invd, (float4 *)v.f.w};
+        const bool rows = (long)v.nx * v.ny >= kCoefCells;
+        const unsigned g = (unsigned)cdiv(cdiv(v.nx, 31) * cdiv(v.ny, rows ? kCoefRows : 1), 256 / 32);
         note_launch();
-        auto coeffs = [&](auto kernel) {
-            kernel<<<g, 128, 0, s>>>(v.nx, v.ny, fbx, fby, v.d.bx, v.d.by, v.f.bx, v.f.by, v.f.bxp,
-                                     v.d.invd, v.f.invd, with_w ? v.d.w : nullptr, (float4 *)v.f.w);
-        };
-        if (l == 0) coeffs(k_level_coeffs<true>);
-        else coeffs(k_level_coeffs<false>);
+        if (l == 0) {
+            if (rows) k_level_coeffs<true, kCoefRows><<<g, 256, 0, s>>>(v.nx, v.ny, fbx, fby, o);
+            else k_level_coeffs<true, 1><<<g, 256, 0, s>>>(v.nx, v.ny, fbx, fby, o);
+        } else {
+            if (rows) k_level_coeffs<false, kCoefRows><<<g, 256, 0, s>>>(v.nx, v.ny, fbx, fby, o);
+            else k_level_coeffs<false, 1><<<g, 256, 0, s>>>(v.nx, v.ny, fbx, fby, o);
+        }
     }
     if (lsmall < L) {
         LevelCoeffArgs a;

@@ -212,3 +212,45 @@ def test_gradient_ragged_tiles(T, B, N):
     with T.cuda.stream(side):
         loss2, g2 = net.grad(d(rhs), d(rho), d(p))
     assert loss2 == loss and np.array_equal(g, g2)
+
+
+def layered_H(nx, ny, seed):
+    """Rows that repeat the row below, rows that differ in one column only and
+    a band of distinct rows, at odd places."""
+    rng = np.random.default_rng(seed)
+    H = np.zeros((ny, nx))
+    H[ny // 3:ny // 3 + 37] = rng.uniform(0.0, 1.0, (37, nx))
+    H[ny // 3 + 37:] = 1.0
+    H[5:11] = rng.uniform(0.0, 1.0, nx)
+    H[11, nx - 1] = H[14, 0] = H[17, nx // 2] = 0.5
+    return H
+
+
+# The coefficients' kernel that passes on a row equal to the one below, from
+# 2^18 cells up, with a ragged last strip and last rows: the oracle's formulas
+# to a rounding or two.
+def test_coefficients_of_repeated_rows(T, ib, O):
+    nx, ny = 523, 517
+    H = layered_H(nx, ny, 6)
+    got = ib.ib_op_coeffs(T.from_numpy(H).cuda(), 1e-3, 1.0, 1e-4, 1e-2)
+    for a, b in zip(got, O.coeffs(H, 1e-3, 1.0, 1e-4, 1e-2)):
+        assert np.abs(a.cpu().numpy() - b).max() <= 1e-15 * np.abs(b).max()
+
+
+# The hierarchy's kernel does the same from 2^20 cells up: the solve on such
+# coefficients reaches the tolerance by the oracle's residual.
+@pytest.mark.parametrize("precision", [0, 2])
+def test_solve_on_repeated_rows(T, ib, O, precision):
+    nx, ny = 1088, 1024
+    h = 1.0 / ny
+    H = layered_H(nx, ny, 7)
+    rho, mu, bx, by = ib.ib_op_coeffs(T.from_numpy(H).cuda(), 1e-1, 1.0, 1e-4, 1e-2)
+    X, Y = W.circle(0.5, 0.5, 0.1, 32)
+    ctx = ib.Context(ib.Config(nx=nx, ny=ny, h=h), X, Y, [0, 32])
+    ctx.mg_setup(bx, by)
+    b = W.random_cells(nx, ny, 8)
+    b -= b.mean()
+    p = T.zeros((ny, nx), dtype=T.float64, device="cuda")
+    st, cyc, rr = ctx.mg_solve(T.from_numpy(b).cuda(), p, precision, 1e-10, 200)
+    r = O.residual(bx.cpu().numpy(), by.cpu().numpy(), b, p.cpu().numpy(), h)
+    assert st == 0 and np.linalg.norm(r) <= 1.001e-10 * np.linalg.norm(b)
