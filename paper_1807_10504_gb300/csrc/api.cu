@@ -310,16 +310,24 @@ void interp_into(ib_ctx *c, const double *u, const double *v, double *U, double 
     if (dt_move != 0.0) launch_axi_symmetrise(c->mk, c->s);
 }
 
-ib_status read_flags(ib_ctx *c)
+// Waits for c->s; the status that the flag words on the host give.
+ib_status wait_flags(ib_ctx *c)
 {
-    cudaError_t e = cudaMemcpyAsync(c->flags_host, c->mk.flags, 3 * sizeof(uint32_t),
-                                    cudaMemcpyDeviceToHost, c->s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->s);
+    const cudaError_t e = cudaStreamSynchronize(c->s);
     if (e != cudaSuccess) return cuda_check(c, e, "flags");
     ib_status st = IB_OK;
     if (c->flags_host[0]) st = fail(c, IB_EMARKER, "a marker left the domain or came within 3 cells of a wall");
     else if (c->flags_host[1]) st = fail(c, IB_EINVAL, "too many interface segments near a cell block or row");
     else if (c->flags_host[2]) st = fail(c, IB_EINVAL, "B-spline normal equations not positive definite");
+    return st;
+}
+
+ib_status read_flags(ib_ctx *c)
+{
+    const cudaError_t e = cudaMemcpyAsync(c->flags_host, c->mk.flags, 3 * sizeof(uint32_t),
+                                          cudaMemcpyDeviceToHost, c->s);
+    if (e != cudaSuccess) return cuda_check(c, e, "flags");
+    const ib_status st = wait_flags(c);
     cudaMemsetAsync(c->mk.flags, 0, 3 * sizeof(uint32_t), c->s);
     return st;
 }
@@ -455,7 +463,7 @@ ib_status step_post(ib_ctx *c, double dt)
     if (g.frame) launch_axi_zbc(g.nx, g.ny, c->frame, c->v, c->s);
     interp_into(c, c->u, c->v, mk.U, mk.V, dt);
     if (g.frame) launch_axi_frame(mk, dt, g.c1, g.c2, 0, c->frame, c->s);
-    launch_validate(mk, c->s);
+    launch_validate(mk, c->flags_host, c->s);
     return launch_check(c, "step");
 }
 
@@ -703,7 +711,7 @@ ib_status ib_set_markers(ib_ctx *c, const double *X, const double *Y, int where)
     if (e == cudaSuccess) e = cudaMemcpyAsync(c->mk.Y, Y, (size_t)M * 8, k, c->s);
     if (e != cudaSuccess) return cuda_check(c, e, "set markers");
     if (where) {
-        launch_validate(c->mk, c->s);
+        launch_validate(c->mk, nullptr, c->s);
         return read_flags(c);
     }
     return IB_OK;
@@ -911,7 +919,7 @@ ib_status step_one(ib_ctx *c, double dt, int warm, F before_flags)
     c->have_prev = 1;
     c->step++;
     before_flags();
-    ib_status fs = read_flags(c);
+    ib_status fs = wait_flags(c);  // the last launch has moved them
     if (pend.pending) {
         // a failed solve is reported ahead of the flags (its message wins)
         const ib_status ss = mg_run_finish(c->mg, pend, &c->last_cycles, &c->last_relres, c->err);

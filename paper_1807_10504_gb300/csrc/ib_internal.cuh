@@ -386,7 +386,8 @@ cudaError_t markers_alloc(Markers &mk, int M, int ndrops, int nx, int ny,
 void markers_free(Markers &mk);
 // flags[0]: bad marker (outside / too near a wall); flags[1]: candidate,
 // crossing or band pair list overflow; flags[2]: B-spline system not positive definite.
-void launch_validate(Markers &mk, cudaStream_t s);
+// flags_host: page-locked place for the flag words, which are then cleared.
+void launch_validate(Markers &mk, uint32_t *flags_host, cudaStream_t s);
 void launch_geometry(Markers &mk, double sigma, cudaStream_t s);
 // Segment records and the drops' Y ranges of the Heaviside (after
 // launch_geometry, whose normals they take).

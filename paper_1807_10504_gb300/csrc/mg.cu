@@ -2169,8 +2169,16 @@ __device__ void solve_check(SolveCtl *ctl, const double *res, cudaGraphCondition
 }
 
 __global__ void __launch_bounds__(kRedT)
-k_sum(long n, const double *__restrict__ a, double *part, unsigned *count, double *out)
+k_sum(long n, const double *__restrict__ a, double *part, unsigned *count, double *out,
+      SolveCtl *ctl, const SolveCtl *in)
 {
+    // the graph's first kernel: the solve's settings from the host's block
+    if (ctl && blockIdx.x == 0 && threadIdx.x == 0) {
+        const volatile SolveCtl *h = in;
+        ctl->tol = h->tol;
+        ctl->max_cycles = h->max_cycles;
+        ctl->fault = 0;
+    }
     double s = 0.0;
     for (long k = (long)blockIdx.x * kRedT + threadIdx.x; k < n; k += (long)gridDim.x * kRedT)
         s += a[k];
@@ -2178,11 +2186,12 @@ k_sum(long n, const double *__restrict__ a, double *part, unsigned *count, doubl
 }
 
 // r0 = b - sum/n; accumulates sum r0^2.  With bt, also the right-hand side
-// of the pre-scaled FP64 sweep, h^2 r0 / diag.
+// of the pre-scaled FP64 sweep, h^2 r0 / diag; with e0, a copy of p there.
 __global__ void __launch_bounds__(kRedT)
 k_sub_mean(long n, const double *__restrict__ b, const double *__restrict__ sum,
            double *__restrict__ r0, double h2, const double *__restrict__ invd,
-           double *__restrict__ bt, double *part, unsigned *count, double *out)
+           double *__restrict__ bt, const double *__restrict__ p, double *__restrict__ e0,
+           double *part, unsigned *count, double *out)
 {
     // the mean once per block (one FP64 division, the same value everywhere)
     __shared__ double mb;
@@ -2194,6 +2203,7 @@ k_sub_mean(long n, const double *__restrict__ b, const double *__restrict__ sum,
         double v = b[k] - m;
         r0[k] = v;
         if (bt) bt[k] = v * h2 * invd[k];
+        if (e0) e0[k] = p[k];
         s += v * v;
     }
     block_fold_and_finish(s, part, count, out);
@@ -2282,10 +2292,12 @@ __global__ void k_add_f32(long n, const float *__restrict__ e, double *__restric
 }
 
 __global__ void k_finalize(long n, const double *__restrict__ e0, const double *__restrict__ sum,
-                           const SolveCtl *__restrict__ ctl, double *__restrict__ p)
+                           const SolveCtl *__restrict__ ctl, double *__restrict__ p,
+                           SolveCtl *host)
 {
     __shared__ double mb;  // the mean once per block
     if (threadIdx.x == 0) mb = *sum / (double)n;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *host = *ctl;  // page-locked memory
     __syncthreads();
     long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k < n) p[k] = ctl->zero_p ? 0.0 : e0[k] - mb;
@@ -2973,10 +2985,10 @@ ib_status mg_run_direct(MG &mg, const double *rhs, double *p, int precision, dou
     cudaMemsetAsync(&mg.ctl->fault, 0, sizeof(int), s);  // fault word of this solve
     cudaMemcpyAsync(e0, p, n * 8, cudaMemcpyDeviceToDevice, s);
     note_launch();
-    k_sum<<<RB, kRedT, 0, s>>>(n, rhs, part, mg.red_count, res + 0);
+    k_sum<<<RB, kRedT, 0, s>>>(n, rhs, part, mg.red_count, res + 0, nullptr, nullptr);
     note_launch();
     k_sub_mean<<<RB, kRedT, 0, s>>>(n, rhs, res + 0, b0, v0.h * v0.h, v0.d.invd,
-                                    precision ? nullptr : v0.d.bt, part, mg.red_count, res + 1);
+                                    precision ? nullptr : v0.d.bt, nullptr, nullptr, part, mg.red_count, res + 1);
     auto resnorm = [&]() {
         const bool pr = prof_on(kProfResnorm);
         if (pr) prof_mark(s, true);
@@ -3021,7 +3033,7 @@ ib_status mg_run_direct(MG &mg, const double *rhs, double *p, int precision, dou
             rr = sqrt(mg.red_host[2]) / nb;
         }
         note_launch();
-        k_sum<<<RB, kRedT, 0, s>>>(n, e0, part, mg.red_count, res + 3);
+        k_sum<<<RB, kRedT, 0, s>>>(n, e0, part, mg.red_count, res + 3, nullptr, nullptr);
         note_launch();
         k_apply_mean<<<cdiv(n, 256), 256, 0, s>>>(n, e0, res + 3, p);
         int fault = 0;  // pageable landing (the no-allocation solve has no pinned control block)
@@ -3041,7 +3053,11 @@ ib_status mg_run_direct(MG &mg, const double *rhs, double *p, int precision, dou
 // residual, convergence test), a device-side WHILE node whose body is one
 // cycle + FP64 residual + convergence test, and an epilogue (mean removal,
 // control block to the host).  One graph launch and one host synchronisation
-// per solve; the loop is bounded by max_cycles on the device.
+// per solve; the loop is bounded by max_cycles on the device.  The settings
+// and the results pass through page-locked memory that the first and the last
+// kernel read and write: with a copy node at the end the next launch began 20
+// us after the last kernel, now 3 (a 64^2 step 514 -> 482 us with the flag words'
+// copy gone as well).
 static cudaError_t build_solve_graph(MG &mg, SolveGraph &sg)
 {
     Level &v0 = mg.lv[0];
@@ -3054,13 +3070,11 @@ static cudaError_t build_solve_graph(MG &mg, SolveGraph &sg)
     const unsigned long long k0 = launch_count();
     cudaError_t e = cudaStreamBeginCapture(c, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    cudaMemsetAsync(&mg.ctl->fault, 0, sizeof(int), c);  // fault word of this solve
-    if (sg.p != e0) cudaMemcpyAsync(e0, sg.p, n * 8, cudaMemcpyDeviceToDevice, c);
     note_launch();
-    k_sum<<<RB, kRedT, 0, c>>>(n, sg.rhs, part, mg.red_count, res + 0);
+    k_sum<<<RB, kRedT, 0, c>>>(n, sg.rhs, part, mg.red_count, res + 0, mg.ctl, mg.ctl_host);
     note_launch();
     k_sub_mean<<<RB, kRedT, 0, c>>>(n, sg.rhs, res + 0, b0, v0.h * v0.h, v0.d.invd,
-                                    sg.precision ? nullptr : v0.d.bt, part, mg.red_count, res + 1);
+                                    sg.precision ? nullptr : v0.d.bt, sg.p, sg.p != e0 ? e0 : nullptr, part, mg.red_count, res + 1);
     cudaStreamCaptureStatus cs;
     cudaGraph_t g;
     const cudaGraphNode_t *deps;
@@ -3116,10 +3130,9 @@ static cudaError_t build_solve_graph(MG &mg, SolveGraph &sg)
     }
     if (e == cudaSuccess) {
         note_launch();
-        k_sum<<<RB, kRedT, 0, c>>>(n, e0, part, mg.red_count, res + 3);
+        k_sum<<<RB, kRedT, 0, c>>>(n, e0, part, mg.red_count, res + 3, nullptr, nullptr);
         note_launch();
-        k_finalize<<<cdiv(n, 256), 256, 0, c>>>(n, e0, res + 3, mg.ctl, sg.p);
-        cudaMemcpyAsync(mg.ctl_host, mg.ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, c);
+        k_finalize<<<cdiv(n, 256), 256, 0, c>>>(n, e0, res + 3, mg.ctl, sg.p, mg.ctl_host);
     }
     cudaGraph_t full = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(c, &full);
@@ -3167,8 +3180,7 @@ ib_status mg_run_launch(MG &mg, const double *rhs, double *p, int precision, dou
     }
     mg.ctl_host->tol = tol;
     mg.ctl_host->max_cycles = max_cycles;
-    cudaError_t e = cudaMemcpyAsync(mg.ctl, mg.ctl_host, 2 * sizeof(double), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaGraphLaunch(sg->exec, s);
+    const cudaError_t e = cudaGraphLaunch(sg->exec, s);
     if (e != cudaSuccess) { err = cudaGetErrorString(e); return IB_ECUDA; }
     pend.pending = true;
     pend.tol = tol;
