@@ -18,6 +18,7 @@ struct StepGraph {
     int key = 0;
     cudaGraphExec_t exec = nullptr;
     unsigned long long kernels = 0;
+    ibk::MgPending solve;  // the kernel counts of a solve within it
 };
 
 struct ib_ctx {
@@ -471,51 +472,67 @@ ib_status step_post(ib_ctx *c, double dt)
 // (dt, key) is seen: recorded on the private stream c->cap (c->s points at
 // it meanwhile), then replayed on c->s.  Direct launches while graphs are
 // off or per-kernel timing is active, and for good if recording fails.
+StepGraph *find_recorded(ib_ctx *c, double dt, int key)
+{
+    for (auto &q : c->sgraphs)
+        if (q.dt == dt && q.key == key) return &q;
+    return nullptr;
+}
+
+// Records fn's launches (see run_recorded); NULL if that fails, and then no
+// graph is recorded any more.
+template <typename F>
+StepGraph *record(ib_ctx *c, double dt, int key, F fn)
+{
+    if (c->sgraphs.size() >= 16) {
+        cudaGraphExecDestroy(c->sgraphs.front().exec);
+        c->sgraphs.erase(c->sgraphs.begin());
+    }
+    cudaStream_t user = c->s;
+    c->s = c->cap;
+    const unsigned long long k0 = launch_count();
+    cudaError_t e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
+    ib_status st = IB_OK;
+    cudaGraph_t gr = nullptr;
+    StepGraph q;
+    q.dt = dt;
+    q.key = key;
+    if (e == cudaSuccess) {
+        st = fn(q.solve);
+        e = cudaStreamEndCapture(c->cap, &gr);
+    }
+    c->s = user;
+    q.kernels = launch_count() - k0;
+    note_launch(-(int)q.kernels);  // recording launches nothing
+    // per-node priorities: the side streams' launches (hierarchy, face
+    // force) keep their higher priority inside the replayed graph, so
+    // their blocks take free SM slots ahead of the predictor's
+    if (e == cudaSuccess && st == IB_OK)
+        e = cudaGraphInstantiate(&q.exec, gr, cudaGraphInstantiateFlagUseNodePriority);
+    if (gr) cudaGraphDestroy(gr);
+    if (e != cudaSuccess || st != IB_OK || !q.exec) {
+        cudaGetLastError();
+        c->err.clear();
+        c->step_graphs_off = true;
+        return nullptr;
+    }
+    c->sgraphs.push_back(q);
+    return &c->sgraphs.back();
+}
+
+ib_status launch_recorded(ib_ctx *c, const StepGraph *sg)
+{
+    note_launch((int)sg->kernels);
+    return cuda_check(c, cudaGraphLaunch(sg->exec, c->s), "step graph");
+}
+
 template <typename F>
 ib_status run_recorded(ib_ctx *c, double dt, int key, F fn)
 {
     if (!c->mg.use_graphs || profiling_active() || c->step_graphs_off) return fn();
-    StepGraph *sg = nullptr;
-    for (auto &q : c->sgraphs)
-        if (q.dt == dt && q.key == key) sg = &q;
-    if (!sg) {
-        if (c->sgraphs.size() >= 16) {
-            cudaGraphExecDestroy(c->sgraphs.front().exec);
-            c->sgraphs.erase(c->sgraphs.begin());
-        }
-        cudaStream_t user = c->s;
-        c->s = c->cap;
-        const unsigned long long k0 = launch_count();
-        cudaError_t e = cudaStreamBeginCapture(c->cap, cudaStreamCaptureModeThreadLocal);
-        ib_status st = IB_OK;
-        cudaGraph_t gr = nullptr;
-        if (e == cudaSuccess) {
-            st = fn();
-            e = cudaStreamEndCapture(c->cap, &gr);
-        }
-        c->s = user;
-        StepGraph q;
-        q.dt = dt;
-        q.key = key;
-        q.kernels = launch_count() - k0;
-        note_launch(-(int)q.kernels);  // recording launches nothing
-        // per-node priorities: the side streams' launches (hierarchy, face
-        // force) keep their higher priority inside the replayed graph, so
-        // their blocks take free SM slots ahead of the predictor's
-        if (e == cudaSuccess && st == IB_OK)
-            e = cudaGraphInstantiate(&q.exec, gr, cudaGraphInstantiateFlagUseNodePriority);
-        if (gr) cudaGraphDestroy(gr);
-        if (e != cudaSuccess || st != IB_OK || !q.exec) {
-            cudaGetLastError();
-            c->err.clear();
-            c->step_graphs_off = true;
-            return fn();
-        }
-        c->sgraphs.push_back(q);
-        sg = &c->sgraphs.back();
-    }
-    note_launch((int)sg->kernels);
-    return cuda_check(c, cudaGraphLaunch(sg->exec, c->s), "step graph");
+    StepGraph *sg = find_recorded(c, dt, key);
+    if (!sg) sg = record(c, dt, key, [&](MgPending &) { return fn(); });
+    return sg ? launch_recorded(c, sg) : fn();
 }
 
 }  // namespace
@@ -867,6 +884,25 @@ ib_status step_args(ib_ctx *c, double dt, int nsteps, int warm)
     return IB_OK;
 }
 
+// The end of a time step whose launches are queued: the step's one host
+// synchronisation, the status of a pending solve (else st) and the flags.
+template <typename F>
+ib_status step_end(ib_ctx *c, const MgPending &pend, ib_status st, F before_flags)
+{
+    c->have_prev = 1;
+    c->step++;
+    before_flags();
+    ib_status fs = wait_flags(c);  // the last launch has moved them
+    if (pend.pending) {
+        // a failed solve is reported ahead of the flags (its message wins)
+        const ib_status ss = mg_run_finish(c->mg, pend, &c->last_cycles, &c->last_relres, c->err);
+        if (ss != IB_OK && ss != IB_ENOTCONV) return ss;
+        st = ss;
+    }
+    if (fs != IB_OK) return fs;
+    return st;
+}
+
 // One time step; before_flags enqueues work on c->s ahead of the step's
 // final host synchronisation (the marker flags read).
 template <typename F>
@@ -881,6 +917,29 @@ ib_status step_one(ib_ctx *c, double dt, int warm, F before_flags)
     const bool rec = c->have_prev && !g.indicator && warm != 2;
     const int key = (reloc ? 1 : 0) | (mass ? 2 : 0) | (warm == 0 ? 4 : 0);
     const bool t_pre = prof_on(kProfPre), t_solve = prof_on(kProfSolve), t_post = prof_on(kProfPost);
+    // From the third step of the same shape on, one graph for the launches
+    // before, in and after the solve: a graph's first kernel starts about 20
+    // us after the graph before it (ten steps at 1024^2 12.03 -> 11.81 ms).  Not the
+    // first time: a program that changes dt at every step would record it at
+    // every step.
+    if (rec && warm <= 1 && !t_pre && !t_solve && !t_post && c->mg.use_graphs && !profiling_active() &&
+        !c->step_graphs_off) {
+        StepGraph *sg = find_recorded(c, dt, key | 128);
+        if (!sg && find_recorded(c, dt, key))
+            sg = record(c, dt, key | 128, [&](MgPending &solve) {
+                ib_status st = step_pre(c, dt, reloc, mass, warm);
+                if (st == IB_OK) st = mg_record(c->mg, c->b, c->p, g.precision, g.nu1, g.nu2, c->s, solve);
+                return st == IB_OK ? step_post(c, dt) : st;
+            });
+        if (sg) {
+            c->mg.fp64_w = g.precision == 0;
+            c->have_pprev = false;
+            MgPending pend = sg->solve;
+            mg_settings(c->mg, g.tol, g.max_cycles, pend);
+            const ib_status st = launch_recorded(c, sg);
+            return st == IB_OK ? step_end(c, pend, IB_OK, before_flags) : st;
+        }
+    }
     if (t_pre) prof_mark(c->s, true);
     ib_status st = rec ? run_recorded(c, dt, key, [&] { return step_pre(c, dt, reloc, mass, warm); })
                        : step_pre(c, dt, reloc, mass, warm);
@@ -916,18 +975,7 @@ ib_status step_one(ib_ctx *c, double dt, int warm, F before_flags)
                              : step_post(c, dt);
     if (t_post) prof_mark(c->s, false);
     if (sp != IB_OK) return sp;
-    c->have_prev = 1;
-    c->step++;
-    before_flags();
-    ib_status fs = wait_flags(c);  // the last launch has moved them
-    if (pend.pending) {
-        // a failed solve is reported ahead of the flags (its message wins)
-        const ib_status ss = mg_run_finish(c->mg, pend, &c->last_cycles, &c->last_relres, c->err);
-        if (ss != IB_OK && ss != IB_ENOTCONV) return ss;
-        st = ss;
-    }
-    if (fs != IB_OK) return fs;
-    return st;
+    return step_end(c, pend, st, before_flags);
 }
 
 }  // namespace

@@ -317,6 +317,9 @@ struct MgPending {
 ib_status mg_run_launch(MG &mg, const double *rhs, double *p, int precision, double tol,
                         int max_cycles, int nu1, int nu2, int *cycles, double *relres,
                         cudaStream_t s, std::string &err, MgPending &pend);
+ib_status mg_record(MG &mg, const double *rhs, double *p, int precision, int nu1, int nu2,
+                    cudaStream_t c, MgPending &pend);
+void mg_settings(MG &mg, double tol, int max_cycles, MgPending &pend);
 ib_status mg_run_finish(MG &mg, const MgPending &pend, int *cycles, double *relres, std::string &err);
 
 // The same solve with one launch per kernel and a host read of the residual

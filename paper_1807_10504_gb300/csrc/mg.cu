@@ -3058,7 +3058,9 @@ ib_status mg_run_direct(MG &mg, const double *rhs, double *p, int precision, dou
 // kernel read and write: with a copy node at the end the next launch began 20
 // us after the last kernel, now 3 (a 64^2 step 514 -> 482 us with the flag words'
 // copy gone as well).
-static cudaError_t build_solve_graph(MG &mg, SolveGraph &sg)
+//
+// Records those launches on c, which is capturing; sets sg's kernel counts.
+static cudaError_t record_solve(MG &mg, SolveGraph &sg, cudaStream_t c)
 {
     Level &v0 = mg.lv[0];
     const long n = (long)v0.nx * v0.ny;
@@ -3066,10 +3068,8 @@ static cudaError_t build_solve_graph(MG &mg, SolveGraph &sg)
     double *part = mg.red + 8, *res = mg.red;
     double *e0 = v0.d.e, *b0 = v0.d.r;
     const double ih2 = 1.0 / (v0.h * v0.h);
-    cudaStream_t c = mg.cap, cb = mg.cap_body;
+    cudaStream_t cb = mg.cap_body;
     const unsigned long long k0 = launch_count();
-    cudaError_t e = cudaStreamBeginCapture(c, cudaStreamCaptureModeThreadLocal);
-    if (e != cudaSuccess) return e;
     note_launch();
     k_sum<<<RB, kRedT, 0, c>>>(n, sg.rhs, part, mg.red_count, res + 0, mg.ctl, mg.ctl_host);
     note_launch();
@@ -3089,7 +3089,7 @@ static cudaError_t build_solve_graph(MG &mg, SolveGraph &sg)
                    sg.precision ? v0.f.r : nullptr, sg.precision ? v0.f.e : nullptr, part,
                    mg.red_count, res, mg.ctl, hnd, check, sg.precision == 2 ? 2 : 1);
     };
-    e = cudaStreamGetCaptureInfo(c, &cs, nullptr, &g, &deps, &ed, &nd);
+    cudaError_t e = cudaStreamGetCaptureInfo(c, &cs, nullptr, &g, &deps, &ed, &nd);
     if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&hnd, g, 0, cudaGraphCondAssignDefault);
     if (e == cudaSuccess) {
         resnorm(c, 1);
@@ -3134,17 +3134,47 @@ static cudaError_t build_solve_graph(MG &mg, SolveGraph &sg)
         note_launch();
         k_finalize<<<cdiv(n, 256), 256, 0, c>>>(n, e0, res + 3, mg.ctl, sg.p, mg.ctl_host);
     }
-    cudaGraph_t full = nullptr;
-    cudaError_t e2 = cudaStreamEndCapture(c, &full);
-    if (e == cudaSuccess) e = e2;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&sg.exec, full, 0);
-    if (full) cudaGraphDestroy(full);
     const unsigned long long kall = launch_count() - k0;
     sg.body_kernels = kb1 - kb0;
     sg.outer_kernels = kall - sg.body_kernels;
     note_launch(-(int)kall);  // capture issues no kernel; executions are counted per launch
+    return e;
+}
+
+static cudaError_t build_solve_graph(MG &mg, SolveGraph &sg)
+{
+    cudaError_t e = cudaStreamBeginCapture(mg.cap, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    e = record_solve(mg, sg, mg.cap);
+    cudaGraph_t full = nullptr;
+    const cudaError_t e2 = cudaStreamEndCapture(mg.cap, &full);
+    if (e == cudaSuccess) e = e2;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&sg.exec, full, 0);
+    if (full) cudaGraphDestroy(full);
     cudaGetLastError();
     return e;
+}
+
+// The solve as part of a caller's graph: its launches on the capturing stream
+// c, and before every launch of that graph the settings.
+ib_status mg_record(MG &mg, const double *rhs, double *p, int precision, int nu1, int nu2,
+                    cudaStream_t c, MgPending &pend)
+{
+    SolveGraph sg;
+    sg.rhs = rhs; sg.p = p; sg.precision = precision; sg.nu1 = nu1; sg.nu2 = nu2;
+    if (precision == 0) ensure_fp64_w(mg, c);
+    if (record_solve(mg, sg, c) != cudaSuccess) return IB_ECUDA;
+    pend.outer_kernels = sg.outer_kernels;
+    pend.body_kernels = sg.body_kernels;
+    return IB_OK;
+}
+
+void mg_settings(MG &mg, double tol, int max_cycles, MgPending &pend)
+{
+    mg.ctl_host->tol = tol;
+    mg.ctl_host->max_cycles = max_cycles;
+    pend.pending = true;
+    pend.tol = tol;
 }
 
 static bool prof_active();
@@ -3178,12 +3208,9 @@ ib_status mg_run_launch(MG &mg, const double *rhs, double *p, int precision, dou
         mg.graphs.push_back(ng);
         sg = &mg.graphs.back();
     }
-    mg.ctl_host->tol = tol;
-    mg.ctl_host->max_cycles = max_cycles;
+    mg_settings(mg, tol, max_cycles, pend);
     const cudaError_t e = cudaGraphLaunch(sg->exec, s);
-    if (e != cudaSuccess) { err = cudaGetErrorString(e); return IB_ECUDA; }
-    pend.pending = true;
-    pend.tol = tol;
+    if (e != cudaSuccess) { pend.pending = false; err = cudaGetErrorString(e); return IB_ECUDA; }
     pend.outer_kernels = sg->outer_kernels;
     pend.body_kernels = sg->body_kernels;
     return IB_OK;
