@@ -276,7 +276,8 @@ struct MG {
     int *piv = nullptr;           // coarsest row permutation
     double *red = nullptr;        // reduction partials + results (device)
     unsigned *red_count = nullptr;
-    double *red_host = nullptr;   // pinned mirror of the results
+    double *red_host = nullptr;   // host mirror of the results
+    bool red_direct = false;      // kernels may write red_host
     int red_blocks = 0;
     // the FP64 sweep weights (LevelT<double>::w) match the coefficients: the
     // build leaves them out (only FP64 cycles read them), ensure_fp64_w forms

@@ -2236,7 +2236,7 @@ k_resnorm(int nx, int ny, double ih2, const double *__restrict__ bx,
           const double *__restrict__ by, const double *__restrict__ b0,
           const double *__restrict__ p, float *__restrict__ rf, float *__restrict__ ef,
           double *part, unsigned *count, double *res, SolveCtl *ctl,
-          cudaGraphConditionalHandle hnd, int check, int inc)
+          cudaGraphConditionalHandle hnd, int check, int inc, double *host)
 {
     const int lane = threadIdx.x & 31;
     const int sx = (nx + 30) / 31, nst = sx * ((ny + ROWS - 1) / ROWS);
@@ -2280,8 +2280,10 @@ k_resnorm(int nx, int ny, double ih2, const double *__restrict__ bx,
             }
         }
     }
-    if (block_fold_and_finish(s, part, count, res + 2) && check)
-        solve_check(ctl, res, hnd, check == 1, inc);
+    if (block_fold_and_finish(s, part, count, res + 2)) {
+        if (check) solve_check(ctl, res, hnd, check == 1, inc);
+        if (host) { host[1] = res[1]; host[2] = res[2]; }
+    }
 }
 
 __global__ void k_add_f32(long n, const float *__restrict__ e, double *__restrict__ p)
@@ -2787,6 +2789,7 @@ cudaError_t mg_alloc(MG &mg, int nx, int ny, double h)
     mg_layout(mg, nx, ny, h, (char *)mg.mem);
     mg.bytes = bytes;
     e = cudaMallocHost((void **)&mg.red_host, 16 * sizeof(double));
+    mg.red_direct = true;  // page-locked
     if (e == cudaSuccess) e = cudaMallocHost((void **)&mg.ctl_host, sizeof(SolveCtl));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&mg.cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&mg.cap_body, cudaStreamNonBlocking);
@@ -2860,7 +2863,7 @@ long mg_bench_op(MG &mg, int op, int level, cudaStream_t s)
         launch_pdl(resnorm_kernel((long)v0.nx * v0.ny), red_grid(mg, (long)v0.nx * v0.ny), kRedT, 0, s, v0.nx, v0.ny, 1.0 / (v0.h * v0.h), v0.d.bx,
                    v0.d.by, (const double *)v0.d.r, (const double *)v0.d.e, v0.f.r, v0.f.e,
                    mg.red + 8, mg.red_count, mg.red, (SolveCtl *)nullptr,
-                   (cudaGraphConditionalHandle)0, 0, 0);
+                   (cudaGraphConditionalHandle)0, 0, 0, (double *)nullptr);
         return (long)v0.nx * v0.ny;
     }
     default: return -1;
@@ -2996,9 +2999,11 @@ ib_status mg_run_direct(MG &mg, const double *rhs, double *p, int precision, dou
         resnorm_kernel(n)<<<RB, kRedT, 0, s>>>(v0.nx, v0.ny, ih2, v0.d.bx, v0.d.by, b0, e0,
                                        precision ? v0.f.r : nullptr,
                                        precision ? v0.f.e : nullptr, part, mg.red_count,
-                                       res, nullptr, (cudaGraphConditionalHandle)0, 0, 0);
+                                       res, nullptr, (cudaGraphConditionalHandle)0, 0, 0,
+                                       mg.red_direct ? mg.red_host : nullptr);
         if (pr) prof_mark(s, false);
-        cudaMemcpyAsync(mg.red_host, res, 4 * sizeof(double), cudaMemcpyDeviceToHost, s);
+        if (!mg.red_direct)
+            cudaMemcpyAsync(mg.red_host, res, 4 * sizeof(double), cudaMemcpyDeviceToHost, s);
         return cudaStreamSynchronize(s);
     };
     cudaError_t ce = resnorm();
@@ -3087,7 +3092,7 @@ static cudaError_t record_solve(MG &mg, SolveGraph &sg, cudaStream_t c)
         note_launch();
         launch_pdl(resnorm_kernel(n), RB, kRedT, 0, st, v0.nx, v0.ny, ih2, v0.d.bx, v0.d.by, b0, e0,
                    sg.precision ? v0.f.r : nullptr, sg.precision ? v0.f.e : nullptr, part,
-                   mg.red_count, res, mg.ctl, hnd, check, sg.precision == 2 ? 2 : 1);
+                   mg.red_count, res, mg.ctl, hnd, check, sg.precision == 2 ? 2 : 1, (double *)nullptr);
     };
     cudaError_t e = cudaStreamGetCaptureInfo(c, &cs, nullptr, &g, &deps, &ed, &nd);
     if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&hnd, g, 0, cudaGraphCondAssignDefault);
