@@ -923,13 +923,17 @@ __device__ __forceinline__ double dmax0(double x)
     return (b > 0 && b <= 0x7ff0000000000000LL) ? x : 0.0;
 }
 
-// Narrow [lo, hi] to the s with alpha + beta s >= 0 (rbeta = 1 / beta).
-__device__ __forceinline__ void narrow(double alpha, double beta, double rbeta, double &lo, double &hi)
+// Narrow [lo, hi] to the s with alpha + beta s >= 0, rbeta = 1 / beta (0 for
+// beta = 0), which has beta's sign; q = -alpha rbeta where that is known.
+__device__ __forceinline__ void narrow(double alpha, double rbeta, double q, double &lo, double &hi)
 {
-    const double q = -alpha * rbeta;
-    if (dpos(beta)) { if (dkey(q) > dkey(lo)) lo = q; }
-    else if (dneg(beta)) { if (dkey(q) < dkey(hi)) hi = q; }
+    if (dpos(rbeta)) { if (dkey(q) > dkey(lo)) lo = q; }
+    else if (dneg(rbeta)) { if (dkey(q) < dkey(hi)) hi = q; }
     else if (dneg(alpha)) hi = -INFINITY;
+}
+__device__ __forceinline__ void narrow(double alpha, double rbeta, double &lo, double &hi)
+{
+    narrow(alpha, rbeta, -alpha * rbeta, lo, hi);
 }
 
 // Areas of the unit square cut by half-planes, by Green's theorem: area =
@@ -954,28 +958,36 @@ __device__ __forceinline__ bool on_edge(const CellLine &L)
     return (dzero(L.a) && dneg(L.b) && dzero(L.b - L.c)) || (dzero(L.b) && dneg(L.a) && dzero(L.a - L.c));
 }
 
-// Interval of line L's own piece inside the unit square.
-__device__ __forceinline__ void square_piece(const CellLine &L, double &lo, double &hi)
+// Interval of line L's own piece inside the unit square; (px, py) = c (a, b).
+// The FP64 pipe bounds the areas, so the far side's crossing comes from the
+// near one's ((1 - px) / b = 1 / b - px / b) and a determinant's sign from its
+// reciprocal (170k pairs at 1024^2: 1.19 -> 0.97 million FP64 warp
+// instructions, 106 -> 88 us).
+__device__ __forceinline__ void square_piece(const CellLine &L, double px, double py, double &lo,
+                                             double &hi)
 {
-    const double px = L.c * L.a, py = L.c * L.b;
     lo = -INFINITY; hi = INFINITY;
-    narrow(px, L.b, L.rb, lo, hi);              // x >= 0
-    narrow(1.0 - px, -L.b, -L.rb, lo, hi);      // x <= 1
-    narrow(py, -L.a, -L.ra, lo, hi);            // y >= 0
-    narrow(1.0 - py, L.a, L.ra, lo, hi);        // y <= 1
+    const double qx = -px * L.rb, qy = py * L.ra;
+    narrow(px, L.rb, qx, lo, hi);                                       // x >= 0
+    if (dzero(L.rb)) narrow(1.0 - px, 0.0, 0.0, lo, hi);
+    else narrow(0.0, -L.rb, qx + L.rb, lo, hi);                         // x <= 1
+    narrow(py, -L.ra, qy, lo, hi);                                      // y >= 0
+    if (dzero(L.ra)) narrow(1.0 - py, 0.0, 0.0, lo, hi);
+    else narrow(0.0, L.ra, qy - L.ra, lo, hi);                          // y <= 1
 }
 
-// Narrow line J's piece by half-plane I (rIJ = 1 / (a_I b_J - b_I a_J)).
-__device__ __forceinline__ void cross_narrow(const CellLine &I, const CellLine &J, double rIJ,
+// Narrow line J's piece, through (px, py), by half-plane I (rIJ = 1 / (a_I b_J
+// - b_I a_J)).
+__device__ __forceinline__ void cross_narrow(const CellLine &I, double px, double py, double rIJ,
                                              double &lo, double &hi)
 {
-    const double px = J.c * J.a, py = J.c * J.b;
-    narrow(I.a * px + I.b * py - I.c, I.a * J.b - I.b * J.a, rIJ, lo, hi);
+    narrow(fma(I.a, px, fma(I.b, py, -I.c)), rIJ, lo, hi);
 }
 
 struct RailCut {
     double Rlo, Rhi, Tlo, Thi;  // right edge (y) and top edge (x) inside both normal edges
     double Plo[2], Phi[2];      // normal-edge pieces (s)
+    double px[2], py[2];        // c (a, b) of the normal edges
     bool piece[2];              // normal edge j cuts the cell and has a piece of its own
 };
 
@@ -985,16 +997,18 @@ __device__ __forceinline__ void rail_cut(const CellLine *L, double r01, RailCut 
     rc.Rlo = 0.0; rc.Rhi = 1.0; rc.Tlo = 0.0; rc.Thi = 1.0;
 #pragma unroll
     for (int j = 0; j < 2; j++) {
-        narrow(L[j].a - L[j].c, L[j].b, L[j].rb, rc.Rlo, rc.Rhi);  // x = 1
-        narrow(L[j].b - L[j].c, L[j].a, L[j].ra, rc.Tlo, rc.Thi);  // y = 1
+        narrow(L[j].a - L[j].c, L[j].rb, rc.Rlo, rc.Rhi);  // x = 1
+        narrow(L[j].b - L[j].c, L[j].ra, rc.Tlo, rc.Thi);  // y = 1
     }
 #pragma unroll
     for (int j = 0; j < 2; j++) {
         rc.piece[j] = L[j].on && !on_edge(L[j]);
         rc.Plo[j] = 0.0; rc.Phi[j] = 0.0;
         if (!rc.piece[j]) continue;
-        square_piece(L[j], rc.Plo[j], rc.Phi[j]);
-        if (L[1 - j].on) cross_narrow(L[1 - j], L[j], j == 1 ? r01 : -r01, rc.Plo[j], rc.Phi[j]);
+        rc.px[j] = L[j].c * L[j].a; rc.py[j] = L[j].c * L[j].b;
+        square_piece(L[j], rc.px[j], rc.py[j], rc.Plo[j], rc.Phi[j]);
+        if (L[1 - j].on)
+            cross_narrow(L[1 - j], rc.px[j], rc.py[j], j == 1 ? r01 : -r01, rc.Plo[j], rc.Phi[j]);
     }
 }
 
@@ -1015,23 +1029,24 @@ __device__ __forceinline__ double rail_line_area(const CellLine *L, const RailCu
                                                  const CellLine &O, double r0O, double r1O)
 {
     double lo = rc.Rlo, hi = rc.Rhi, acc;
-    narrow(O.a - O.c, O.b, O.rb, lo, hi);
+    narrow(O.a - O.c, O.rb, lo, hi);
     acc = dmax0(hi - lo);
     lo = rc.Tlo; hi = rc.Thi;
-    narrow(O.b - O.c, O.a, O.ra, lo, hi);
+    narrow(O.b - O.c, O.ra, lo, hi);
     acc += dmax0(hi - lo);
 #pragma unroll
     for (int j = 0; j < 2; j++) {
         if (!rc.piece[j]) continue;
         lo = rc.Plo[j]; hi = rc.Phi[j];
-        cross_narrow(O, L[j], j == 0 ? -r0O : -r1O, lo, hi);  // D_Oj = -D_jO
+        cross_narrow(O, rc.px[j], rc.py[j], j == 0 ? -r0O : -r1O, lo, hi);  // D_Oj = -D_jO
         acc -= L[j].c * dmax0(hi - lo);
     }
     if (!on_edge(O)) {
-        square_piece(O, lo, hi);
+        const double px = O.c * O.a, py = O.c * O.b;
+        square_piece(O, px, py, lo, hi);
 #pragma unroll
         for (int i = 0; i < 2; i++)
-            if (L[i].on) cross_narrow(L[i], O, i == 0 ? r0O : r1O, lo, hi);
+            if (L[i].on) cross_narrow(L[i], px, py, i == 0 ? r0O : r1O, lo, hi);
         acc -= O.c * dmax0(hi - lo);
     }
     return 0.5 * acc;
@@ -1117,7 +1132,7 @@ __device__ __forceinline__ void pair_area(uint32_t m, int ci, int cj, const doub
 // chains overlap the rest.  The other blocks take one pair per thread (flat
 // over the list), skipping the listed ones.  (Strips clipped side by side of
 // the square, 1024 pairs listed: 42 us for one drop of 128 markers, 125 us for
-// 64 of 256; now 20 and 104.)
+// 64 of 256; then 20 and 104, and 88 with the rule at square_piece.)
 __global__ void __launch_bounds__(256)
 k_band_area(int nx, const uint32_t *__restrict__ npairs, uint32_t cap,
             const uint32_t *__restrict__ pseg, const uint32_t *__restrict__ pcell,

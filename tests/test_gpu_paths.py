@@ -254,3 +254,31 @@ def test_solve_on_repeated_rows(T, ib, O, precision):
     st, cyc, rr = ctx.mg_solve(T.from_numpy(b).cuda(), p, precision, 1e-10, 200)
     r = O.residual(bx.cpu().numpy(), by.cpu().numpy(), b, p.cpu().numpy(), h)
     assert st == 0 and np.linalg.norm(r) <= 1.001e-10 * np.linalg.norm(b)
+
+
+# One graph for the whole step (from the third step of a shape on), separate
+# graphs before that, and direct launches run the same kernels on the same
+# data: the same bits, also after a step of another size in between.
+@pytest.mark.parametrize("kw", [dict(precision=2, spread=1, relocate_every=2),
+                                dict(precision=0, spread=0, relocate_every=0),
+                                dict(precision=1, viscous=1, mass_every=2),
+                                dict(precision=2, axisym=1, frame=1, gy=-1.0, relocate_every=3)])
+def test_step_graphs_match_direct_launches(T, ib, kw):
+    if kw.get("axisym"):
+        nx, ny, h = 32, 96, 1 / 32
+        mk = W.axi_elliptic_drop(1.5, 0.25, 1.1, 96)
+    else:
+        nx, ny, h = 64, 48, 1 / 64
+        mk = W.elliptic_drop(0.5, 0.375, 0.2, 1.15, 128)
+    dt = W.capillary_dt(h, 1.0, 1e-3, 1.0, 1e-2, 1e-4)
+    got = []
+    for graphs in (True, False):
+        ctx = ib.Context(ib.Config(nx=nx, ny=ny, h=h, tol=1e-10, **kw), mk.X, mk.Y, mk.drop_start)
+        ctx.use_graphs(graphs)
+        for step in [dt] * 5 + [0.5 * dt] + [dt] * 2:
+            ctx.ns_step(step, 1, 1)
+        got.append([ctx.get(f).cpu().numpy() for f in ("u", "v", "p")] +
+                   [a.cpu().numpy() for a in ctx.markers()])
+        ctx.close()
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
