@@ -423,11 +423,11 @@ __global__ void k_block_active(int bnx, int bny, const uint32_t *__restrict__ bc
 
 // ------------------------------------------------------------ interpolation
 // Eight lanes per marker: lanes 0-3 the rows of u's 4 x 4 stencil, 4-7 those
-// of v's.  A lane forms its component's factors along x and its row's along
-// y, sums its row, and the four rows meet in a fixed order.  The kernel is
-// bound by the latency of one thread's chain of FP64 operations and loads
-// not by their number: one thread per marker took 21 us for 512 and 24 us for
-// 16384 markers, here 6 and 9.
+// of v's.  The even lanes form their component's factors along x, the odd
+// ones those along y, passed on by shuffles; a lane sums its row, and the four
+// rows meet in a fixed order.  Few markers are bound by the latency of one
+// lane's chain (512: 21 us with one thread per marker, here 6), many by the FP64
+// pipe (16384: 25 us with both factors in every lane, 17 so).
 __global__ void __launch_bounds__(128)
 k_interp(int M, int kernel, int nx, int ny, double ih, double x0, double y0,
          const double *__restrict__ u, const double *__restrict__ v,
@@ -442,9 +442,19 @@ k_interp(int M, int kernel, int nx, int ny, double ih, double x0, double y0,
     const double sx = (Xm - x0) * ih - (isv ? 0.5 : 0.0), sy = (Ym - y0) * ih - (isv ? 0.0 : 0.5);
     const double fx = floor(sx), fy = floor(sy);
     const int i0 = (int)fx - 1, j = (int)fy - 1 + b;
-    double px[4], py[4];
-    phi4(kernel, sx - fx, px);
-    phi4(kernel, sy - fy, py);
+    // the factors along x by the even lanes, those along y by the odd ones
+    double q[4], px[4], py;
+    phi4(kernel, b & 1 ? sy - fy : sx - fx, q);
+    {
+        const int e = threadIdx.x & 31 & ~3;  // the component's first lane
+        double w[4];
+#pragma unroll
+        for (int a = 0; a < 4; a++) {
+            px[a] = __shfl_sync(0xffffffffu, q[a], e);
+            w[a] = __shfl_sync(0xffffffffu, q[a], e + 1);
+        }
+        py = b == 0 ? w[0] : (b == 1 ? w[1] : (b == 2 ? w[2] : w[3]));
+    }
     const int W = isv ? nx : nx + 1, H = isv ? ny + 1 : ny;
     const double *f = isv ? v : u;
     double acc = 0.0;
@@ -454,7 +464,7 @@ k_interp(int M, int kernel, int nx, int ny, double ih, double x0, double y0,
             const int i = i0 + a;
             if (i >= 0 && i < W) acc += f[(long)j * W + i] * px[a];
         }
-    acc *= b == 0 ? py[0] : (b == 1 ? py[1] : (b == 2 ? py[2] : py[3]));
+    acc *= py;
     // rows (0 + 1) + (2 + 3), in every lane of the component
     acc += __shfl_xor_sync(0xffffffffu, acc, 1);
     acc += __shfl_xor_sync(0xffffffffu, acc, 2);
