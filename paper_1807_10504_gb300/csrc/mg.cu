@@ -2345,7 +2345,10 @@ void launch_smooth2(const Level &v, const LevelT<float> &a, const float *pin, fl
 // leave room (dynamic shared memory) for two blocks an SM only, so that the
 // scheduler hands the rest to the SMs that finish first instead of placing
 // all at once (1024^2: FP64 cycle 246 -> 222 us; 2048^2, with 13 tiles an SM,
-// would lose a tenth).
+// would lose a tenth).  Levels that 16 x 8 tiles cover with at most one block an
+// SM (up to 128^2) take those: a block's FP64 work, not the halo's share of it,
+// then sets the launch's time (FP64 cycle at 64^2 40.1 -> 36.9 us, 128^2 52.0 ->
+// 44.3, 256^2 69.4 -> 60.1, 1024^2 211 -> 200).
 template <int MODE>
 void launch_smooth2_f64(const Level &v, const LevelT<double> &a, const double *pin, double *p,
                         double *rc, double *ecz, double h2c, const double *invdc, double *btc,
@@ -2359,9 +2362,14 @@ void launch_smooth2_f64(const Level &v, const LevelT<double> &a, const double *p
         launch_pdl(k_smooth2_f64<MODE, 64, 32>, g, 256, pad, s, v.nx, v.ny, ih2, (const double2 *)a.w,
                    (const double *)a.bt, (const double *)a.bx, (const double *)a.by, pin, p, rc,
                    ecz, h2c, invdc, btc, ecp);
-    } else {
+    } else if ((long)cdiv(v.nx, 16) * cdiv(v.ny, 8) > 152) {
         dim3 g(cdiv(v.nx, 32), cdiv(v.ny, 16));
         launch_pdl(k_smooth2_f64<MODE, 32, 16>, g, 256, 0, s, v.nx, v.ny, ih2, (const double2 *)a.w,
+                   (const double *)a.bt, (const double *)a.bx, (const double *)a.by, pin, p, rc,
+                   ecz, h2c, invdc, btc, ecp);
+    } else {
+        dim3 g(cdiv(v.nx, 16), cdiv(v.ny, 8));
+        launch_pdl(k_smooth2_f64<MODE, 16, 8>, g, 256, 0, s, v.nx, v.ny, ih2, (const double2 *)a.w,
                    (const double *)a.bt, (const double *)a.bx, (const double *)a.by, pin, p, rc,
                    ecz, h2c, invdc, btc, ecp);
     }
