@@ -183,7 +183,7 @@ struct ConvCfg {
 // reads, two buffers and separate pooling and folding launches the layers
 // took (us) 25.5 (16 -> 16, 8 x 256^2), 44.9 (48 -> 16), 33.1 (64 -> 32, half
 // resolution), 12.6 (32 -> 32, half and quarter) in all; now
-// 15.5, 40, 28 and 10.
+// 13, 41, 26 and 10.
 template <int CIN, int COUT, int CUP, int CST, int EPI>
 __global__ void __launch_bounds__(128)
 k_conv_fwd(int B, int H, int W, const bf16 *__restrict__ x, const bf16 *__restrict__ xu,
@@ -655,8 +655,7 @@ struct DwSplit {
 // What bounds it is that chain and the fragment loads (four a 16-pixel step
 // for six products).  One CTA per tap with element-wise fragment reads took
 // 325 us (16 -> 16), 528 us (48 -> 16) and 260 us (64 -> 32, half resolution)
-// at 8 x 256^2; this takes 58, 83 and
-// 42 us.
+// at 8 x 256^2; this takes 45, 71 and 39 us.
 template <int CIN, int COUT, int CUP, int CSX, int CSG>
 __global__ void __launch_bounds__(128)
 k_conv_dw(int B, int H, int W, int tiles_per_chunk, const bf16 *__restrict__ x,

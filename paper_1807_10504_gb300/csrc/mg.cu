@@ -21,9 +21,9 @@
 //  * kernels of the cycle use programmatic dependent launch: the next grid is
 //    scheduled while the previous one drains and waits (griddepcontrol) for
 //    its results.
-//  * levels with <= 1024 cells run as one single-CTA kernel (the whole lower
-//    V-cycle and the coarsest solve) with its data in shared memory, since
-//    launches dominate there.
+//  * levels with <= 256 cells (FP64) / <= 1024 cells (FP32) run as one
+//    single-CTA kernel (the whole lower V-cycle and the coarsest solve) with
+//    its data in shared memory, since launches dominate there.
 //  * norms are deterministic two-stage reductions (fixed per-thread order,
 //    fixed tree, last-block fold) with no floating-point atomics.
 //  * the FP32 instantiations of the same kernels form the inner cycle of the
@@ -2348,7 +2348,8 @@ void launch_smooth2(const Level &v, const LevelT<float> &a, const float *pin, fl
 // would lose a tenth).  Levels that 16 x 8 tiles cover with at most one block an
 // SM (up to 128^2) take those: a block's FP64 work, not the halo's share of it,
 // then sets the launch's time (FP64 cycle at 64^2 40.1 -> 36.9 us, 128^2 52.0 ->
-// 44.3, 256^2 69.4 -> 60.1, 1024^2 211 -> 200).
+// 44.3, 256^2 69.4 -> 60.1, 1024^2 211 -> 200), up to 64^2 those of 8 x 8 (36.9 ->
+// 36.5, 44.3 -> 43.2, 60.3 -> 59.5).
 template <int MODE>
 void launch_smooth2_f64(const Level &v, const LevelT<double> &a, const double *pin, double *p,
                         double *rc, double *ecz, double h2c, const double *invdc, double *btc,
@@ -2365,6 +2366,11 @@ void launch_smooth2_f64(const Level &v, const LevelT<double> &a, const double *p
     } else if ((long)cdiv(v.nx, 16) * cdiv(v.ny, 8) > 152) {
         dim3 g(cdiv(v.nx, 32), cdiv(v.ny, 16));
         launch_pdl(k_smooth2_f64<MODE, 32, 16>, g, 256, 0, s, v.nx, v.ny, ih2, (const double2 *)a.w,
+                   (const double *)a.bt, (const double *)a.bx, (const double *)a.by, pin, p, rc,
+                   ecz, h2c, invdc, btc, ecp);
+    } else if ((long)v.nx * v.ny <= 4096) {
+        dim3 g(cdiv(v.nx, 8), cdiv(v.ny, 8));
+        launch_pdl(k_smooth2_f64<MODE, 8, 8>, g, 256, 0, s, v.nx, v.ny, ih2, (const double2 *)a.w,
                    (const double *)a.bt, (const double *)a.bx, (const double *)a.by, pin, p, rc,
                    ecz, h2c, invdc, btc, ecp);
     } else {
