@@ -14,7 +14,8 @@ namespace ibk {
 // Levels with at most this many cells run in one CTA, in the FP64 and in the
 // FP32 cycle.  FP64: with 1024 a cycle took 36.9 us at 64^2, 60.3 at 256^2 and
 // 200 at 1024^2 (the FP64 work of a 32^2 level on one SM: 7 us, against two
-// launches of 3.5), with 256 33.9, 59.0 and 198.  FP32: with 4096 78.9 us at
+// launches of 3.5), with 256 33.9, 59.0 and 198, and 31.6, 56.8 and 195 with the
+// smoother's 8 x 8 tiles as well.  FP32: with 4096 78.9 us at
 // 1024^2, 52.7 at 512^2, 25.9 at 64^2 (a level of 64^2 costs one CTA 11 us, its
 // two launches 7.5), with 1024 76.4, 49.9 and 22.9, with 256 78.7, 52.6 and 24.5.
 constexpr int kTailCells = 256;
