@@ -114,6 +114,35 @@ __device__ __forceinline__ double recip_any(double x)
     return (a > lo && a < hi) ? recip_nr(x) : 1.0 / x;
 }
 
+// Programmatic dependent launch: kernels of the V-cycle and of the network's
+// forward pass are launched with programmatic stream serialisation, so the
+// next grid is scheduled while the previous one drains.  Each such kernel
+// first waits until the grid before it has completed and its writes are
+// visible (griddepcontrol.wait), then lets the next grid launch
+// (griddepcontrol.launch_dependents); before the wait nothing is written, and
+// read only what was complete before the grid before it began.
+__device__ __forceinline__ void pdl_enter()
+{
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
+template <typename... KArgs, typename... Args>
+inline void launch_pdl(void (*kern)(KArgs...), dim3 g, dim3 b, size_t smem, cudaStream_t s, Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = g;
+    cfg.blockDim = b;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, ((KArgs)args)...);
+}
+
 // Raises a kernel's dynamic shared-memory limit to at least `bytes` (one
 // host call the first time a larger value is needed, none afterwards, so
 // that launches recorded into a CUDA graph make no such call).

@@ -48,34 +48,6 @@ namespace {
 constexpr int TW = 64, TH = 16, TT = 256;
 constexpr int kRedT = 256;
 
-// Programmatic dependent launch: kernels of the V-cycle are launched with
-// programmatic stream serialisation, so the next grid is scheduled while the
-// previous one drains.  Each such kernel first waits until the grid before
-// it has completed and its writes are visible (griddepcontrol.wait), then
-// lets the next grid launch (griddepcontrol.launch_dependents); nothing is
-// read or written before the wait.
-__device__ __forceinline__ void pdl_enter()
-{
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-}
-
-template <typename... KArgs, typename... Args>
-void launch_pdl(void (*kern)(KArgs...), dim3 g, dim3 b, size_t smem, cudaStream_t s, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = g;
-    cfg.blockDim = b;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kern, ((KArgs)args)...);
-}
-
 // ------------------------------------------------------------------ sweeps
 template <typename T>
 __global__ void __launch_bounds__(TT)
