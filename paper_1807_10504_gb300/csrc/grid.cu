@@ -95,7 +95,8 @@ __global__ void k_rhs(int nx, int ny, double ih, double ihdt,
     b[ys] = v;
 }
 
-// One row of x-faces (j < ny) and of y-faces (j <= ny) per blockIdx.y.
+// One row of x-faces (j < ny) and of y-faces (j <= ny) per blockIdx.y, and
+// further ones where a grid has more rows than a launch may have (65,535).
 __global__ void k_correct(int nx, int ny, double ih, double dt,
                           const double *__restrict__ us, const double *__restrict__ vs,
                           const double *__restrict__ p, const double *__restrict__ Fx,
@@ -103,18 +104,20 @@ __global__ void k_correct(int nx, int ny, double ih, double dt,
                           const double *__restrict__ by, double *__restrict__ u,
                           double *__restrict__ v)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i > nx) return;
-    const long c = (long)j * nx + i;
-    const double pc = (i < nx && j < ny) ? p[c] : 0.0;
-    if (j < ny) {
-        const long k = (long)j * (nx + 1) + i;
-        if (i == 0 || i == nx) u[k] = 0.0;
-        else u[k] = fma(dt, bx[k] * fma(-ih, pc - p[c - 1], Fx[k]), us[k]);
-    }
-    if (i < nx) {
-        if (j == 0 || j == ny) v[c] = 0.0;
-        else v[c] = fma(dt, by[c] * fma(-ih, pc - p[c - nx], Fy[c]), vs[c]);
+    for (int j = blockIdx.y; j <= ny; j += gridDim.y) {
+        const long c = (long)j * nx + i;
+        const double pc = (i < nx && j < ny) ? p[c] : 0.0;
+        if (j < ny) {
+            const long k = (long)j * (nx + 1) + i;
+            if (i == 0 || i == nx) u[k] = 0.0;
+            else u[k] = fma(dt, bx[k] * fma(-ih, pc - p[c - 1], Fx[k]), us[k]);
+        }
+        if (i < nx) {
+            if (j == 0 || j == ny) v[c] = 0.0;
+            else v[c] = fma(dt, by[c] * fma(-ih, pc - p[c - nx], Fy[c]), vs[c]);
+        }
     }
 }
 
@@ -665,7 +668,7 @@ void launch_correct(int nx, int ny, double h, double dt, const double *us,
                     double *u, double *v, cudaStream_t s)
 {
     note_launch();
-    k_correct<<<dim3(cdiv(nx + 1, 128), ny + 1), 128, 0, s>>>(nx, ny, 1.0 / h, dt, us, vs, p, Fx, Fy,
+    k_correct<<<dim3(cdiv(nx + 1, 128), std::min(ny + 1, 65535)), 128, 0, s>>>(nx, ny, 1.0 / h, dt, us, vs, p, Fx, Fy,
                                           bx, by, u, v);
 }
 

@@ -282,3 +282,21 @@ def test_step_graphs_match_direct_launches(T, ib, kw):
         ctx.close()
     for a, b in zip(*got):
         assert np.array_equal(a, b)
+
+
+# The correction takes one row a block up to the most rows of a launch, and
+# further ones in turn above that.  Two fused multiply-adds a face: within a few
+# ulps of the operands' sizes.
+@pytest.mark.parametrize("ny", [65533, 65534, 65535, 131075])
+def test_correct_tall_grids(T, ib, O, ny):
+    nx, h, dt = 3, 0.01, 1e-3
+    rng = np.random.default_rng(ny)
+    f = lambda *n: rng.standard_normal(n)
+    us, vs, p = f(ny, nx + 1), f(ny + 1, nx), f(ny, nx)
+    Fx, Fy = f(ny, nx + 1), f(ny + 1, nx)
+    bx, by = np.abs(f(ny, nx + 1)), np.abs(f(ny + 1, nx))
+    d = lambda a: T.from_numpy(a).cuda()
+    gu, gv = ib.ib_op_correct(d(us), d(vs), d(p), d(Fx), d(Fy), d(bx), d(by), h, dt)
+    ou, ov = O.correct(us, vs, p, Fx, Fy, bx, by, h, dt)
+    for g, o in ((gu, ou), (gv, ov)):
+        assert np.abs(g.cpu().numpy() - o).max() <= 1e-14 * max(np.abs(o).max(), 1.0)
