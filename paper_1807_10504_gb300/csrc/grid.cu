@@ -362,68 +362,113 @@ __global__ void k_cn_sweep(int nx, int ny, double h, double dt, const double *__
 //
 // k_cn_coeffs: per face the update u <- r + W u_W + E u_E + S u_S + N u_N of
 // k_cn_sweep, u = (u_e + tau nb) / (1 + tau (cs + ex)), as four weights and a
-// right-hand side (w[2k], w[2k + 1], r[k]; x-faces then y-faces).  Boundary
-// faces get zero weights and their own value.
-__global__ void k_cn_coeffs(int nx, int ny, double h, double dt, const double *__restrict__ rho,
-                            const double *__restrict__ mu, int axisym,
-                            const double *__restrict__ frame, const double *__restrict__ ue,
-                            const double *__restrict__ ve, double2 *__restrict__ w,
-                            double *__restrict__ r)
+// right-hand side (w[2k], w[2k + 1], r[k]; x-faces then y-faces, blockIdx.z).
+// Boundary faces get zero weights and their own value.  Bound by the FP64 pipe,
+// some 45 instructions a face.  So a thread takes a column's ROWS rows, and where
+// the cells that a face's coefficients depend on equal those of the face below,
+// as off the interface, it keeps that face's: one product is left.  Single-warp
+// blocks spread the warps along an interface over the SMs (512^2: 52 us with a
+// face a thread; 8 rows 43 us in blocks of 128 and 33 in blocks of 32; 16 rows
+// 43, 4 rows 36, 2 rows 49).  A thread's 8 rows take 21 us whatever the size, so
+// small grids have one row a thread: 160 x 480 cells 22 us with 8 and 21 with 1,
+// 320^2 24 and 27, 1024^2 68 and 231.
+constexpr int kCnT = 32;
+constexpr long kCnRowCells = 90000;  // 8 rows a thread from here up
+template <int ROWS>
+__global__ void __launch_bounds__(kCnT)
+k_cn_coeffs(int nx, int ny, double h, double dt, const double *__restrict__ rho,
+            const double *__restrict__ mu, int axisym, const double *__restrict__ frame,
+            const double *__restrict__ ue, const double *__restrict__ ve, double2 *__restrict__ w,
+            double *__restrict__ r)
 {
     const long nxf = nx + 1, nu = nxf * ny;
-    const long f = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    auto M = [&](int i, int j) { return mu[(long)j * nx + i]; };
-    if (f < nu) {
-        const int j = (int)(f / nxf), i = (int)(f - (long)j * nxf);
-        if (i == 0 || i == nx) {
-            w[2 * f] = make_double2(0.0, 0.0); w[2 * f + 1] = make_double2(0.0, 0.0);
-            r[f] = ue[f];
-            return;
-        }
+    const int i = blockIdx.x * kCnT + threadIdx.x, j0 = blockIdx.y * ROWS;
+    auto M = [&](int a, int j) { return mu[(long)j * nx + a]; };
+    auto same = [](double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); };
+    const double2 zero = make_double2(0.0, 0.0);
+    double2 we = zero, sn = zero;  // the weights, (W, E) and (S, N)
+    double g = 0.0, ghost = 0.0;   // of the right-hand side; of the moving outer wall
+    double p0 = 0.0, p1 = 0.0, p2 = 0.0, q0 = 0.0, q1 = 0.0;  // the face below's mu, rho
+    bool even = false;             // its cells were alike along y
+    if (blockIdx.z == 0) {
+        if (i > nx) return;
         const double r0 = axisym ? i * h : 1.0, rE = axisym ? (i + 0.5) * h : 1.0,
                      rW = axisym ? (i - 0.5) * h : 1.0;
-        const double s = axisym ? recip_any(r0 * h * h) : recip_any(h * h);
-        const double m0 = M(i - 1, j), m1 = M(i, j), m = m0 + m1;
-        const double muN = (j + 1 < ny) ? 0.25 * (m + (M(i - 1, j + 1) + M(i, j + 1))) : 0.5 * m;
-        const double muS = (j > 0) ? 0.25 * ((M(i - 1, j - 1) + M(i, j - 1)) + m) : 0.5 * m;
-        const double cE = rE * m1 * s, cW = rW * m0 * s, cN = r0 * muN * s, cS = r0 * muS * s;
-        const bool n = j + 1 < ny, b = j > 0;
-        // a wall's reflected ghost: twice its weight on the diagonal
-        double d = (cE + cW) + (n ? cN : 2.0 * cN) + (b ? cS : 2.0 * cS);
-        if (axisym) d += 0.5 * m * recip_any(r0 * r0);
-        const double tau = dt * recip_any(rho[(long)j * nx + i - 1] + rho[(long)j * nx + i]);
-        const double g = recip_any(1.0 + tau * d), tg = tau * g;
-        w[2 * f] = make_double2(cW * tg, cE * tg);
-        w[2 * f + 1] = make_double2(b ? cS * tg : 0.0, n ? cN * tg : 0.0);
-        r[f] = ue[f] * g;
+#pragma unroll 1
+        for (int j = j0; j < min(j0 + ROWS, ny); j++) {
+            const long f = (long)j * nxf + i;
+            if (i == 0 || i == nx) {
+                w[2 * f] = zero; w[2 * f + 1] = zero;
+                r[f] = ue[f];
+                continue;
+            }
+            const bool n = j + 1 < ny, b = j > 0;
+            const double m0 = M(i - 1, j), m1 = M(i, j);
+            const double n0 = n ? M(i - 1, j + 1) : 0.0, n1 = n ? M(i, j + 1) : 0.0;
+            const double s0 = b ? M(i - 1, j - 1) : 0.0, s1 = b ? M(i, j - 1) : 0.0;
+            const double d0 = rho[(long)j * nx + i - 1], d1 = rho[(long)j * nx + i];
+            const bool ev = n && b && same(n0, m0) && same(n1, m1) && same(s0, m0) && same(s1, m1);
+            if (!(ROWS > 1 && ev && even && same(m0, p0) && same(m1, p1) && same(d0, q0) && same(d1, q1))) {
+                const double s = axisym ? recip_any(r0 * h * h) : recip_any(h * h);
+                const double m = m0 + m1;
+                const double muN = n ? 0.25 * (m + (n0 + n1)) : 0.5 * m;
+                const double muS = b ? 0.25 * ((s0 + s1) + m) : 0.5 * m;
+                const double cE = rE * m1 * s, cW = rW * m0 * s, cN = r0 * muN * s, cS = r0 * muS * s;
+                // a wall's reflected ghost: twice its weight on the diagonal
+                double d = (cE + cW) + (n ? cN : 2.0 * cN) + (b ? cS : 2.0 * cS);
+                if (axisym) d += 0.5 * m * recip_any(r0 * r0);
+                const double tau = dt * recip_any(d0 + d1);
+                g = recip_any(1.0 + tau * d);
+                const double tg = tau * g;
+                we = make_double2(cW * tg, cE * tg);
+                sn = make_double2(b ? cS * tg : 0.0, n ? cN * tg : 0.0);
+            }
+            even = ev; p0 = m0; p1 = m1; q0 = d0; q1 = d1;
+            w[2 * f] = we; w[2 * f + 1] = sn;
+            r[f] = ue[f] * g;
+        }
         return;
     }
-    const long k = f - nu;
-    if (k >= (long)nx * (ny + 1)) return;
-    const int j = (int)(k / nx), i = (int)(k - (long)j * nx);
-    if (j == 0 || j == ny) {
-        w[2 * f] = make_double2(0.0, 0.0); w[2 * f + 1] = make_double2(0.0, 0.0);
-        r[f] = ve[k];
-        return;
-    }
+    if (i >= nx) return;
     const double r0 = axisym ? (i + 0.5) * h : 1.0, rE = axisym ? (i + 1) * h : 1.0,
                  rW = axisym ? i * h : 1.0;
-    const double s = axisym ? recip_any(r0 * h * h) : recip_any(h * h);
-    const double m0 = M(i, j - 1), m1 = M(i, j), m = m0 + m1;
-    const double muE = (i + 1 < nx) ? 0.25 * (m + (M(i + 1, j - 1) + M(i + 1, j))) : 0.5 * m;
-    const double muW = (i > 0) ? 0.25 * ((M(i - 1, j - 1) + M(i - 1, j)) + m) : 0.5 * m;
-    const double cN = r0 * m1 * s, cS = r0 * m0 * s, cE = rE * muE * s, cW = rW * muW * s;
     const bool e = i + 1 < nx, b = i > 0;
-    double d = (cN + cS) + (e ? cE : 2.0 * cE);
-    if (b) d += cW;
-    else if (!axisym) d += 2.0 * cW;
-    const double tau = dt * recip_any(rho[(long)(j - 1) * nx + i] + rho[(long)j * nx + i]);
-    const double g = recip_any(1.0 + tau * d), tg = tau * g;
-    w[2 * f] = make_double2(b ? cW * tg : 0.0, e ? cE * tg : 0.0);
-    w[2 * f + 1] = make_double2(cS * tg, cN * tg);
-    double v = ve[k] * g;
-    if (!e && frame) v += 2.0 * cE * tg * frame[kFrWb];  // the outer wall moves with the frame
-    r[f] = v;
+#pragma unroll 1
+    for (int j = j0; j < min(j0 + ROWS, ny + 1); j++) {
+        const long k = (long)j * nx + i, f = nu + k;
+        if (j == 0 || j == ny) {
+            w[2 * f] = zero; w[2 * f + 1] = zero;
+            r[f] = ve[k];
+            continue;
+        }
+        const double m0 = M(i, j - 1), m1 = M(i, j);
+        const double e0 = e ? M(i + 1, j - 1) : 0.0, e1 = e ? M(i + 1, j) : 0.0;
+        const double w0 = b ? M(i - 1, j - 1) : 0.0, w1 = b ? M(i - 1, j) : 0.0;
+        const double d0 = rho[(long)(j - 1) * nx + i], d1 = rho[(long)j * nx + i];
+        const bool ev = same(m0, m1) && same(e0, e1) && same(w0, w1);
+        if (!(ROWS > 1 && ev && even && same(m1, p0) && same(e1, p1) && same(w1, p2) && same(d0, q0) &&
+              same(d1, q1))) {
+            const double s = axisym ? recip_any(r0 * h * h) : recip_any(h * h);
+            const double m = m0 + m1;
+            const double muE = e ? 0.25 * (m + (e0 + e1)) : 0.5 * m;
+            const double muW = b ? 0.25 * ((w0 + w1) + m) : 0.5 * m;
+            const double cN = r0 * m1 * s, cS = r0 * m0 * s, cE = rE * muE * s, cW = rW * muW * s;
+            double d = (cN + cS) + (e ? cE : 2.0 * cE);
+            if (b) d += cW;
+            else if (!axisym) d += 2.0 * cW;
+            const double tau = dt * recip_any(d0 + d1);
+            g = recip_any(1.0 + tau * d);
+            const double tg = tau * g;
+            we = make_double2(b ? cW * tg : 0.0, e ? cE * tg : 0.0);
+            sn = make_double2(cS * tg, cN * tg);
+            ghost = 2.0 * cE * tg;
+        }
+        even = ev; p0 = m1; p1 = e1; p2 = w1; q0 = d0; q1 = d1;
+        w[2 * f] = we; w[2 * f + 1] = sn;
+        double v = ve[k] * g;
+        if (!e && frame) v += ghost * frame[kFrWb];  // the outer wall moves with the frame
+        r[f] = v;
+    }
 }
 
 // NS red-black sweeps of both components in one launch, out of place: a block
@@ -582,8 +627,12 @@ void launch_cn_solve_tab(int nx, int ny, double h, double dt, const double *rho,
 {
     const long nf = (long)(nx + 1) * ny + (long)nx * (ny + 1);
     note_launch();
-    k_cn_coeffs<<<cdiv(nf, 128), 128, 0, s>>>(nx, ny, h, dt, rho, mu, axisym, frame, ua, va,
-                                              (double2 *)w, r);
+    auto coeffs = [&](auto kern, int rows) {
+        kern<<<dim3(cdiv(nx + 1, kCnT), cdiv(ny + 1, rows), 2), kCnT, 0, s>>>(nx, ny, h, dt, rho, mu, axisym, frame,
+                                                                           ua, va, (double2 *)w, r);
+    };
+    if ((long)nx * ny >= kCnRowCells) coeffs(k_cn_coeffs<8>, 8);
+    else coeffs(k_cn_coeffs<1>, 1);
     auto go = [&](auto kern, int dw, int dh) {
         const int nbu = (int)(cdiv(nx + 1, dw) * cdiv(ny, dh)), nbv = (int)(cdiv(nx, dw) * cdiv(ny + 1, dh));
         note_launch();

@@ -135,6 +135,33 @@ def test_cn_sweep_counts(T, ib, O, sweeps, axisym):
         assert np.abs(ctx.get(name).cpu().numpy() - ref).max() <= 1e-10 * 2.0, name
 
 
+# The coefficients formed several rows a thread, from 90,000 cells up: a last strip
+# of one row, and rows that repeat above and below those of the drop.  Pressure
+# within 100 of the solver's tolerances, u and v within 1e-10 of the
+# inertial-capillary velocity.
+@pytest.mark.parametrize("axisym", [0, 1])
+def test_cn_rows_in_strips(T, ib, O, axisym):
+    if axisym:
+        nx, ny, h = 224, 672, 1 / 224
+        mk = W.axi_elliptic_drop(1.5, 0.25, 1.1, 512)
+        kw = dict(axisym=1, gy=-1.0)
+    else:
+        nx, ny, h = 320, 416, 1 / 320
+        mk = W.elliptic_drop(0.5, 0.65, 0.22, 1.15, 512)
+        kw = {}
+    kw.update(spread=1, relocate_every=0, viscous=1, cn_sweeps=2, tol=1e-12)
+    ctx = ib.Context(ib.Config(nx=nx, ny=ny, h=h, **kw), mk.X, mk.Y, mk.drop_start)
+    ocfg = O.Config(nx=nx, ny=ny, h=h, **kw)
+    st = O.init_state(ocfg, mk.X, mk.Y, mk.drop_start)
+    dt = W.capillary_dt(h, 1.0, 1e-3, 1.0, 1e-2, 1e-4)
+    for _ in range(2):
+        ctx.ns_step(dt, 1, 1)
+        O.ns_step(ocfg, st, dt)
+    assert np.abs(ctx.get("p").cpu().numpy() - st.p).max() <= 1e-10 * np.abs(st.p).max()
+    for name, ref in (("u", st.u), ("v", st.v)):
+        assert np.abs(ctx.get(name).cpu().numpy() - ref).max() <= 1e-10 * 2.0, name
+
+
 # A drop of more markers than the block's threads hold in registers: the same
 # bisection decisions as the oracle's, so eps to 1e-13 h.
 def test_measure_correction_large_drop(T, ib, O):
