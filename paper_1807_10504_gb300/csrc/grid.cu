@@ -17,9 +17,12 @@ namespace {
 
 constexpr int kT = 256;
 
-// 2 x for a normal x (an addition to the exponent, no FP64 operation).
+// x + x: an addition to the exponent, no FP64 operation, for a normal x whose
+// double is normal too; the sum for all others (zeros, infinities, NaN).
 __device__ __forceinline__ double twice(double x)
 {
+    const unsigned e = (unsigned)__double2hiint(x) & 0x7ff00000u;
+    if (e - 0x00100000u >= 0x7fd00000u) return x + x;
     return __longlong_as_double(__double_as_longlong(x) + (1LL << 52));
 }
 
