@@ -720,6 +720,21 @@ __device__ __forceinline__ double edge_integral(double x0, double y0, double x1,
     return dx * fma(v - u, fma(0.5 * (u + v), dy, y0), above);
 }
 
+// The two integrals of which a strip's area is made, in the frame of cell
+// (di, dj): along its inner offset line, v the line's corner at the segment's
+// first marker (the one at the next marker 12 values on), and the difference of
+// those along its sides on the normals, next marker less first.  Strip k has
+// line(k + 1) - line(k) - rails(k), to the bit wherever a pair's area is formed.
+__device__ __forceinline__ double line_integral(const double *v, double di, double dj)
+{
+    return edge_integral(v[0] - di, v[1] - dj, v[12] - di, v[13] - dj);
+}
+__device__ __forceinline__ double rail_integral(const double *v, double di, double dj)
+{
+    return edge_integral(v[12] - di, v[13] - dj, v[14] - di, v[15] - dj) -
+           edge_integral(v[0] - di, v[1] - dj, v[2] - di, v[3] - dj);
+}
+
 __device__ __forceinline__ double strip_value(int k)
 {
     // integral of the cosine kernel from -2 to the strip centre r = k - 2:
@@ -753,7 +768,8 @@ __device__ __forceinline__ int cell_side(float4 l, float fi, float fj)
 //  k_band_sum (one CTA per active block): every cell sums its pairs in order,
 //    H = sum A_k H_k + max(0, 1 - sum A_k) chi.
 // Pair ranges are claimed with an atomic counter, so their place in the list
-// varies from run to run, but each cell's pairs and their order do not: H is
+// varies from run to run, but each cell's pairs and their order do not, and a
+// pair's area has the same bits on every route through k_band_area: H is
 // deterministic.
 constexpr int kPairT = 256, kPairSub = kPairT / kBT;  // 4 threads per cell
 // Pairs of non-convex strips or strips along a grid axis (edge integrals, more
@@ -1083,18 +1099,20 @@ __device__ __forceinline__ void pair_area(uint32_t m, int ci, int cj, const doub
     cov = 0.0;
     if (!scvx[m]) {
         const double *v = sv + (long)m * 24;
-        for (int k = 0; k < 5; k++) {
+        double line = 0.0;
+        bool have = false;  // line is the strip's inner one
+        for (int k = 0; k < 5; k++, v += 2) {
             const float4 b = sb5[(long)m * 5 + k];
-            if (b.x > gi + 1.0f || b.y < gi || b.z > gj + 1.0f || b.w < gj) continue;
-            double qx[4], qy[4];
-            qx[0] = v[2 * k] - di;            qy[0] = v[2 * k + 1] - dj;
-            qx[1] = v[12 + 2 * k] - di;       qy[1] = v[12 + 2 * k + 1] - dj;
-            qx[2] = v[12 + 2 * k + 2] - di;   qy[2] = v[12 + 2 * k + 3] - dj;
-            qx[3] = v[2 * k + 2] - di;        qy[3] = v[2 * k + 3] - dj;
-            double A = 0.0;
-            for (int e = 0; e < 4; e++) A -= edge_integral(qx[e], qy[e], qx[(e + 1) & 3], qy[(e + 1) & 3]);
-            acc += A * Hk[k];
-            cov += A;
+            const bool hit = !(b.x > gi + 1.0f || b.y < gi || b.z > gj + 1.0f || b.w < gj);
+            if (hit) {
+                if (!have) line = line_integral(v, di, dj);
+                const double next = line_integral(v + 2, di, dj);
+                const double A = next - line - rail_integral(v, di, dj);
+                acc += A * Hk[k];
+                cov += A;
+                line = next;
+            }
+            have = hit;
         }
         return;
     }
@@ -1171,11 +1189,9 @@ k_band_area(int nx, const uint32_t *__restrict__ npairs, uint32_t cap,
             bool hit = false;
             if (live && k < 6) {
                 const double *v = sv + (long)m * 24 + 2 * k;
-                const double ax = v[0] - di, ay = v[1] - dj, bx = v[12] - di, by = v[13] - dj;
-                line = edge_integral(ax, ay, bx, by);
+                line = line_integral(v, di, dj);
                 if (k < 5) {
-                    rails = edge_integral(bx, by, v[14] - di, v[15] - dj) -
-                            edge_integral(ax, ay, v[2] - di, v[3] - dj);
+                    rails = rail_integral(v, di, dj);
                     const float4 bb = sb5[(long)m * 5 + k];
                     hit = !(bb.x > gi + 1.0f || bb.y < gi || bb.z > gj + 1.0f || bb.w < gj);
                 }
