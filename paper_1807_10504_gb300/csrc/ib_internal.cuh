@@ -321,8 +321,10 @@ struct MG {
 bool mg_levels(int nx, int ny, std::vector<int> &nxs, std::vector<int> &nys);
 // Places the hierarchy (levels, coarsest LU, reduction partials, control
 // block) at `base` (or only measures it when base is NULL); returns its bytes.
-// Allocates nothing.
-size_t mg_layout(MG &mg, int nx, int ny, double h, char *base);
+// Allocates nothing.  shared_w: the small levels' FP32 sweep weights take the
+// place of their FP64 ones, for a hierarchy that runs cycles of one precision
+// (the caller keeps the pointers of that one and builds no others).
+size_t mg_layout(MG &mg, int nx, int ny, double h, char *base, bool shared_w = false);
 cudaError_t mg_alloc(MG &mg, int nx, int ny, double h);
 void mg_free(MG &mg);
 // One launch of one cycle kernel on the hierarchy's current data, for timing.

@@ -2716,7 +2716,7 @@ static int resident_red_blocks()
 static auto resnorm_kernel(long n) { return n >= (1L << 17) ? k_resnorm<4> : k_resnorm<1>; }
 static int red_grid(const MG &mg, long n) { return std::min(mg.red_blocks, (int)cdiv(n, kRedT)); }
 
-size_t mg_layout(MG &mg, int nx, int ny, double h, char *base)
+size_t mg_layout(MG &mg, int nx, int ny, double h, char *base, bool shared_w)
 {
     int nxs[16], nys[16], L = 0;
     nxs[0] = nx; nys[0] = ny; L = 1;
@@ -2746,7 +2746,8 @@ size_t mg_layout(MG &mg, int nx, int ny, double h, char *base)
         v.f.r = (float *)take(n * 4); v.f.invd = (float *)take(n * 4);
         v.f.bx = (float *)take(fx * 4); v.f.by = (float *)take(fy * 4);
         v.f.bxp = (float *)take((size_t)xface_pitch(v.nx) * v.ny * 4);
-        v.f.w = n <= (size_t)kTailCellsF32 ? (float *)take(n * 16) : nullptr;
+        v.f.w = nullptr;
+        if (n <= (size_t)kTailCellsF32) v.f.w = shared_w ? (float *)v.d.w : (float *)take(n * 16);
     }
     mg.lu = (double *)take((size_t)nc * nc * 8 * 2);  // A' and its transposed inverse
     mg.piv = (int *)take((size_t)nc * 4);

@@ -44,7 +44,7 @@ extern "C" ib_status mg_solve_noalloc(int32_t nx, int32_t ny, double h, const do
         g_err = "the grid does not coarsen to a small enough coarsest level";
         return IB_EINVAL;
     }
-    const size_t need = ibk::mg_layout(g_mg, nx, ny, h, nullptr);
+    const size_t need = ibk::mg_layout(g_mg, nx, ny, h, nullptr, true);
     if (need > (size_t)IB_NOALLOC_SCRATCH_BYTES) {
         g_err = "the multigrid hierarchy does not fit the scratch array";
         return IB_EINVAL;
@@ -65,7 +65,11 @@ extern "C" ib_status mg_solve_noalloc(int32_t nx, int32_t ny, double h, const do
         g_scratch_dev[dev] = ptr;
     }
     cudaStream_t s = (cudaStream_t)stream;
-    ibk::mg_layout(g_mg, nx, ny, h, (char *)g_scratch_dev[dev]);
+    // a solve has one precision, so the scratch array holds one set of the small
+    // levels' sweep weights: FP32 ones by mg_build, or FP64 ones, by the solve
+    ibk::mg_layout(g_mg, nx, ny, h, (char *)g_scratch_dev[dev], true);
+    if (precision == 0)
+        for (int l = 0; l < g_mg.L; l++) g_mg.lv[l].f.w = nullptr;
     g_mg.red_host = g_read_back;
     // where the device reaches pageable host memory, the residual norm's kernel
     // writes its results there: a copy to pageable memory fewer on every outer
