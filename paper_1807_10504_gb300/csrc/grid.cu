@@ -257,8 +257,8 @@ k_predictor(int nx, int ny, int R, double ih, double visc, double dt,
         const double mw = AXI ? up(m0) : 0.0, rw = bx ? 0.0 : up(r0);
         if (out) {
             if (!bx) {
-                irx = recip_any(0.5 * (rw + r0));
-                iry = recip_any(0.5 * (rm + r0));
+                irx = recip_div(0.5 * (rw + r0));
+                iry = recip_div(0.5 * (rm + r0));
             }
             if (i == 0) {
                 us[kx] = 0.0; au[kx] = 0.0;
@@ -420,8 +420,8 @@ k_cn_coeffs(int nx, int ny, double h, double dt, const double *__restrict__ rho,
                 // a wall's reflected ghost: twice its weight on the diagonal
                 double d = (cE + cW) + (n ? cN : 2.0 * cN) + (b ? cS : 2.0 * cS);
                 if (axisym) d += 0.5 * m * recip_any(r0 * r0);
-                const double tau = dt * recip_any(d0 + d1);
-                g = recip_any(1.0 + tau * d);
+                const double tau = dt * recip_div(d0 + d1);
+                g = recip_div(1.0 + tau * d);
                 const double tg = tau * g;
                 we = make_double2(cW * tg, cE * tg);
                 sn = make_double2(b ? cS * tg : 0.0, n ? cN * tg : 0.0);
@@ -459,8 +459,8 @@ k_cn_coeffs(int nx, int ny, double h, double dt, const double *__restrict__ rho,
             double d = (cN + cS) + (e ? cE : 2.0 * cE);
             if (b) d += cW;
             else if (!axisym) d += 2.0 * cW;
-            const double tau = dt * recip_any(d0 + d1);
-            g = recip_any(1.0 + tau * d);
+            const double tau = dt * recip_div(d0 + d1);
+            g = recip_div(1.0 + tau * d);
             const double tg = tau * g;
             we = make_double2(b ? cW * tg : 0.0, e ? cE * tg : 0.0);
             sn = make_double2(cS * tg, cN * tg);

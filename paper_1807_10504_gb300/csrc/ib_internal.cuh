@@ -101,17 +101,22 @@ __device__ __forceinline__ double recip_nr(double x)
     return fma(r, fma(e, e, e), r);
 }
 
-// 1/x for any nonzero finite x of either sign (0 for x = 0): recip_nr where
-// |x| lies well inside the FP32 normal range, the FP64 division elsewhere.
-__device__ __forceinline__ double recip_any(double x)
+// 1.0 / x, within one unit in the last place: recip_nr where |x| lies well
+// inside the FP32 normal range, the FP64 division elsewhere (zeros, infinities
+// and NaN as the division has them).
+__device__ __forceinline__ double recip_div(double x)
 {
     // the tests on |x|'s bit pattern (ordered like the value), in integer
     // instructions
     const unsigned long long a = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffULL;
-    if (a == 0) return 0.0;
     const unsigned long long lo = (unsigned long long)__double_as_longlong(1e-30),
                              hi = (unsigned long long)__double_as_longlong(1e30);
     return (a > lo && a < hi) ? recip_nr(x) : 1.0 / x;
+}
+// The same, but 0 for x = 0: for components of a direction that may vanish.
+__device__ __forceinline__ double recip_any(double x)
+{
+    return (__double_as_longlong(x) & 0x7fffffffffffffffLL) == 0 ? 0.0 : recip_div(x);
 }
 
 // Programmatic dependent launch: kernels of the V-cycle and of the network's

@@ -1226,7 +1226,7 @@ __global__ void __launch_bounds__(256) k_level_coeffs_small(LevelCoeffArgs a)
 // SM's FP64 pipe: the size of the coarsest level decides its cost).  One
 // CTA, for at most kCoarseOneCta cells; A' lies in two shared-memory buffers,
 // a column step reading one and writing the other behind one barrier, and the
-// thread that forms the next pivot also forms its reciprocal (recip_any: a
+// thread that forms the next pivot also forms its reciprocal (recip_div: a
 // division is a chain of ~1.5 k cycles on this part).  With four barriers and
 // a division a column 16 cells took 15.7 us, now CI_TIMES.
 constexpr int kCoarseOneCta = 64;  // larger coarsest levels: k_coarse_step
@@ -1269,7 +1269,7 @@ k_coarse_inv(int nx, int ny, double ihh, const double *__restrict__ bx,
         const int r = k / n;
         const double v = coarse_entry(nx, ny, ihh, bx, by, r, k - r * n) + s0;
         cinv_sm[k] = v;
-        if (k == 0) ip_s[0] = recip_any(v);
+        if (k == 0) ip_s[0] = recip_div(v);
     }
     for (int c = 0; c < n; c++) {
         __syncthreads();
@@ -1283,7 +1283,7 @@ k_coarse_inv(int nx, int ny, double ihh, const double *__restrict__ bx,
             const double f = src[r * n + c], dp = (q == c ? 1.0 : src[c * n + q]) * ip;
             const double v = r == c ? dp : fma(-f, dp, q == c ? 0.0 : src[k]);
             dst[k] = v;
-            if (k == (c + 1) * (n + 1)) ip_s[(c + 1) & 1] = recip_any(v);
+            if (k == (c + 1) * (n + 1)) ip_s[(c + 1) & 1] = recip_div(v);
         }
     }
     __syncthreads();
@@ -1330,7 +1330,7 @@ k_coarse_step(int n, int K, const double *__restrict__ A, double *__restrict__ o
         __syncthreads();
         // every thread its own entry: row p scaled by the pivot's reciprocal,
         // eliminated from the others
-        const double ip = recip_any(D[p][p]);
+        const double ip = recip_div(D[p][p]);
         const double dp = D[p][c], f = D[r][p];
         __syncthreads();
         if (r == p) d = c == p ? ip : dp * ip;

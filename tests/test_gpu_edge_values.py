@@ -65,3 +65,31 @@ def test_solve_on_coefficients_of_a_bad_cell(T, ib, n, precision):
     p = T.zeros((n, n), dtype=T.float64, device="cuda")
     st, _, _ = ctx.mg_solve(T.from_numpy(b - b.mean()).cuda(), p, precision, 1e-8, 50, check=False)
     assert st == ib.IB_ENAN
+
+
+# Without any coefficient there is no solution: the coarsest level's inverse does
+# not exist, and the solve says so (one block's inverse at 64^2, blocks of 16 at
+# 104^2, whose coarsest level has 169 cells).
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("n", [64, 104])
+def test_solve_without_coefficients(T, ib, n, precision):
+    ctx = context(ib, n)
+    ctx.mg_setup(T.zeros((n, n + 1), dtype=T.float64, device="cuda"),
+                 T.zeros((n + 1, n), dtype=T.float64, device="cuda"))
+    b = W.random_cells(n, n, 4)
+    p = T.zeros((n, n), dtype=T.float64, device="cuda")
+    st, _, _ = ctx.mg_solve(T.from_numpy(b - b.mean()).cuda(), p, precision, 1e-8, 20, check=False)
+    assert st == ib.IB_ENAN
+
+
+# Two massless cells next to each other: their face has no finite acceleration
+# (axisymmetric predictor: as by the division).
+def test_predictor_of_massless_cells(T, ib):
+    nx, ny, h, dt = 40, 24, 1.0 / 32, 1e-3
+    u, v = W.random_faces(nx, ny, 5)
+    rho = np.full((ny, nx), 0.7)
+    rho[9, 12:14] = 0.0
+    d = lambda a: T.from_numpy(np.ascontiguousarray(a)).cuda()
+    us, vs, _, _ = ib.ib_op_predictor_axi(d(rho), d(np.full_like(rho, 0.1)), d(u), d(v), h, dt)
+    bad = ~np.isfinite(us.cpu().numpy())
+    assert bad[9, 13] and bad.sum() == 1 and np.isfinite(vs.cpu().numpy()).all()
