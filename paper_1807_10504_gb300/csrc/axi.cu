@@ -37,15 +37,13 @@ __global__ void k_rhs_axi(int nx, int ny, double idt, const double *__restrict__
     if (i >= nx) return;
     const long xw = (long)j * (nx + 1) + i, ys = (long)j * nx + i, yn = ys + nx;
     // r b = (r_(i+1) q_E - r_i q_W) / h + r_c (q_N - q_S) / h with radii in
-    // units of h; the force is zero on all faces but those of the interface
-    // band: its part and the loads of beta only where a warp's faces carry one
+    // units of h; the force's part as in k_rhs
     const double fe = Fx[xw + 1], fw = Fx[xw], fn = Fy[yn], fs = Fy[ys];
+    const double be = bx[xw + 1], bw = bx[xw], bn = by[yn], bs = by[ys];
     const double ri = (double)i, re = ri + 1.0, rc = ri + 0.5;
     double r = idt * fma(rc, vs[yn] - vs[ys], fma(re, us[xw + 1], -ri * us[xw]));
-    const long long any = __double_as_longlong(fe) | __double_as_longlong(fw) | __double_as_longlong(fn) |
-                          __double_as_longlong(fs);
-    if (any & 0x7fffffffffffffffLL)
-        r += fma(rc, by[yn] * fn - by[ys] * fs, fma(re, bx[xw + 1] * fe, -ri * (bx[xw] * fw)));
+    if (any_force(fe, fw, fn, fs) || any_unbounded(be, bw, bn, bs))
+        r += fma(rc, bn * fn - bs * fs, fma(re, be * fe, -ri * (bw * fw)));
     b[ys] = r;
 }
 

@@ -78,8 +78,9 @@ k_coeffs(int nx, int ny, double rho_g, double drho, double mu_g, double dmu,
 }
 
 // The force is zero on all faces but those of the interface band: where a
-// warp's faces carry none, its part and the loads of beta are skipped (12
-// FP64 operations a cell to 4; 1024^2: 22 -> 13 us).
+// warp's faces carry none, its part is skipped (12 FP64 operations a cell to 4;
+// 1024^2 21.1 -> 10.0 us, 19.0 with a force everywhere), unless a coefficient is infinite or
+// NaN, which reaches b whatever the force.
 __global__ void k_rhs(int nx, int ny, double ih, double ihdt,
                       const double *__restrict__ us, const double *__restrict__ vs,
                       const double *__restrict__ Fx, const double *__restrict__ Fy,
@@ -90,11 +91,10 @@ __global__ void k_rhs(int nx, int ny, double ih, double ihdt,
     if (i >= nx) return;
     const long xw = (long)j * (nx + 1) + i, ys = (long)j * nx + i, yn = ys + nx;
     const double fe = Fx[xw + 1], fw = Fx[xw], fn = Fy[yn], fs = Fy[ys];
+    const double be = bx[xw + 1], bw = bx[xw], bn = by[yn], bs = by[ys];
     double v = ((us[xw + 1] - us[xw]) + (vs[yn] - vs[ys])) * ihdt;
-    const long long any = __double_as_longlong(fe) | __double_as_longlong(fw) | __double_as_longlong(fn) |
-                          __double_as_longlong(fs);
-    if (any & 0x7fffffffffffffffLL)
-        v = fma(bx[xw + 1] * fe - bx[xw] * fw + by[yn] * fn - by[ys] * fs, ih, v);
+    if (any_force(fe, fw, fn, fs) || any_unbounded(be, bw, bn, bs))
+        v = fma(be * fe - bw * fw + bn * fn - bs * fs, ih, v);
     b[ys] = v;
 }
 

@@ -119,6 +119,19 @@ __device__ __forceinline__ double recip_any(double x)
     return (__double_as_longlong(x) & 0x7fffffffffffffffLL) == 0 ? 0.0 : recip_div(x);
 }
 
+// Whether one of four values is not zero, and whether one is infinite or NaN, on
+// the bit patterns.
+__device__ __forceinline__ bool any_force(double a, double b, double c, double d)
+{
+    return ((__double_as_longlong(a) | __double_as_longlong(b) | __double_as_longlong(c) |
+             __double_as_longlong(d)) & 0x7fffffffffffffffLL) != 0;
+}
+__device__ __forceinline__ bool any_unbounded(double a, double b, double c, double d)
+{
+    auto top = [](double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; };
+    return max(max(top(a), top(b)), max(top(c), top(d))) >= 0x7ff00000u;
+}
+
 // Programmatic dependent launch: kernels of the V-cycle and of the network's
 // forward pass are launched with programmatic stream serialisation, so the
 // next grid is scheduled while the previous one drains.  Each such kernel

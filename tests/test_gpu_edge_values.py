@@ -93,3 +93,21 @@ def test_predictor_of_massless_cells(T, ib):
     us, vs, _, _ = ib.ib_op_predictor_axi(d(rho), d(np.full_like(rho, 0.1)), d(u), d(v), h, dt)
     bad = ~np.isfinite(us.cpu().numpy())
     assert bad[9, 13] and bad.sum() == 1 and np.isfinite(vs.cpu().numpy()).all()
+
+
+# A coefficient that is not finite, at a face without force: b of the cells on
+# either side of it.
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("axisym", [0, 1])
+def test_rhs_of_a_bad_coefficient(T, ib, bad, axisym):
+    nx, ny, h, dt = 70, 33, 1.0 / 64, 1e-3
+    us, vs = W.random_faces(nx, ny, 5)
+    bx, by = (np.abs(a) + 0.5 for a in W.random_faces(nx, ny, 6))
+    bx[7, 30] = by[20, 41] = bad
+    d = lambda a: T.from_numpy(np.ascontiguousarray(a)).cuda()
+    rhs = ib.ib_op_rhs_axi if axisym else ib.ib_op_rhs
+    zx, zy = np.zeros_like(us), np.zeros_like(vs)
+    b = rhs(d(us), d(vs), d(zx), d(zy), d(bx), d(by), h, dt).cpu().numpy()
+    hit = np.zeros((ny, nx), bool)
+    hit[7, 29:31] = hit[19:21, 41] = True
+    assert np.array_equal(np.isnan(b), hit)
