@@ -479,12 +479,13 @@ StepGraph *find_recorded(ib_ctx *c, double dt, int key)
     return nullptr;
 }
 
-// Records fn's launches (see run_recorded); NULL if that fails, and then no
-// graph is recorded any more.
+// Records fn's launches (see run_recorded), in the slot `old` (which then
+// holds them instead) or in a new one, for which the oldest of sixteen goes;
+// NULL if that fails, and then no graph is recorded any more.
 template <typename F>
-StepGraph *record(ib_ctx *c, double dt, int key, F fn)
+StepGraph *record(ib_ctx *c, double dt, int key, StepGraph *old, F fn)
 {
-    if (c->sgraphs.size() >= 16) {
+    if (!old && c->sgraphs.size() >= 16) {
         cudaGraphExecDestroy(c->sgraphs.front().exec);
         c->sgraphs.erase(c->sgraphs.begin());
     }
@@ -516,6 +517,11 @@ StepGraph *record(ib_ctx *c, double dt, int key, F fn)
         c->step_graphs_off = true;
         return nullptr;
     }
+    if (old) {
+        cudaGraphExecDestroy(old->exec);
+        *old = q;
+        return old;
+    }
     c->sgraphs.push_back(q);
     return &c->sgraphs.back();
 }
@@ -531,7 +537,7 @@ ib_status run_recorded(ib_ctx *c, double dt, int key, F fn)
 {
     if (!c->mg.use_graphs || profiling_active() || c->step_graphs_off) return fn();
     StepGraph *sg = find_recorded(c, dt, key);
-    if (!sg) sg = record(c, dt, key, [&](MgPending &) { return fn(); });
+    if (!sg) sg = record(c, dt, key, nullptr, [&](MgPending &) { return fn(); });
     return sg ? launch_recorded(c, sg) : fn();
 }
 
@@ -933,12 +939,15 @@ ib_status step_one(ib_ctx *c, double dt, int warm, F before_flags)
     // before, in and after the solve: a graph's first kernel starts about 20
     // us after the graph before it (ten steps at 1024^2 12.03 -> 11.81 ms).  Not the
     // first time: a program that changes dt at every step would record it at
-    // every step.
+    // every step.  It takes the slot of the shape's separate graph, which no
+    // step of the shape launches again, so that a time step of n shapes holds n
+    // slots and the one of the launches after the solve.
     if (rec && warm <= 1 && !t_pre && !t_solve && !t_post && c->mg.use_graphs && !profiling_active() &&
         !c->step_graphs_off) {
         StepGraph *sg = find_recorded(c, dt, key | 128);
-        if (!sg && find_recorded(c, dt, key))
-            sg = record(c, dt, key | 128, [&](MgPending &solve) {
+        StepGraph *pre = sg ? nullptr : find_recorded(c, dt, key);
+        if (pre)
+            sg = record(c, dt, key | 128, pre, [&](MgPending &solve) {
                 ib_status st = step_pre(c, dt, reloc, mass, warm);
                 if (st == IB_OK) st = mg_record(c->mg, c->b, c->p, g.precision, g.nu1, g.nu2, c->s, solve);
                 return st == IB_OK ? step_post(c, dt) : st;
