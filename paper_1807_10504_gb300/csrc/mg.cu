@@ -2419,6 +2419,33 @@ void launch_tail_w(MG &mg, T *e, bool zero, cudaStream_t s)
     launch_pdl(nco > kTailWarpSolve ? k_tail_w<T, true> : k_tail_w<T, false>, 1, 1024, tailw_bytes<T>(mg, lt), s, a);
 }
 
+// The tail from level lt on, its iterate in e, of any sweep counts; the coarsest
+// solve alone where lt is the coarsest level.
+template <typename T>
+void launch_tail(MG &mg, int lt, T *e, int nu1, int nu2, cudaStream_t s)
+{
+    const int L = mg.L;
+    TailArgs<T> ta;
+    ta.lt = lt;
+    ta.nl = L;
+    for (int l = lt; l < L; l++) {
+        Level &v = mg.lv[l];
+        LevelT<T> *a;
+        if constexpr (sizeof(T) == 8) a = &v.d; else a = &v.f;
+        ta.nx[l] = v.nx; ta.ny[l] = v.ny;
+        ta.h2[l] = (T)(v.h * v.h); ta.ih2[l] = (T)(1.0 / (v.h * v.h));
+        ta.e[l] = a->e; ta.r[l] = a->r; ta.bx[l] = a->bx; ta.by[l] = a->by; ta.invd[l] = a->invd;
+    }
+    ta.e[lt] = e;
+    const size_t nco = (size_t)mg.lv[L - 1].nx * mg.lv[L - 1].ny;
+    ta.ainvT = mg.lu + nco * nco;
+    ta.nu1 = nu1;
+    ta.nu2 = nu2;
+    note_launch();
+    const size_t smem = tail_prepare(ta);
+    launch_pdl(nco > kTailWarpSolve ? k_tail<T, true> : k_tail<T, false>, 1, 1024, smem, s, ta);
+}
+
 // One V(nu1, nu2) cycle on the level-0 data of precision T.  Every level's
 // iterate moves between its two buffers (cur[l]); the coarse corrections
 // start in the canonical buffer, which the restriction zeroes, and level 0
@@ -2473,24 +2500,7 @@ bool vcycle(MG &mg, int nu1, int nu2, cudaStream_t s, double *add64 = nullptr)
     if (fused && lt < L - 1) {
         launch_tail_w<T>(mg, cur[lt], lt > 0, s);
     } else {
-    TailArgs<T> ta;
-    ta.lt = lt;
-    ta.nl = L;
-    for (int l = lt; l < L; l++) {
-        Level &v = mg.lv[l];
-        LevelT<T> &a = lvT(l);
-        ta.nx[l] = v.nx; ta.ny[l] = v.ny;
-        ta.h2[l] = (T)(v.h * v.h); ta.ih2[l] = (T)(1.0 / (v.h * v.h));
-        ta.e[l] = a.e; ta.r[l] = a.r; ta.bx[l] = a.bx; ta.by[l] = a.by; ta.invd[l] = a.invd;
-    }
-    ta.e[lt] = cur[lt];
-    ta.ainvT = mg.lu + (size_t)mg.lv[mg.L - 1].nx * mg.lv[mg.L - 1].ny * mg.lv[mg.L - 1].nx * mg.lv[mg.L - 1].ny;
-    ta.nu1 = nu1;
-    ta.nu2 = nu2;
-    note_launch();
-    const size_t smem = tail_prepare(ta);
-    const bool big = ta.nx[L - 1] * ta.ny[L - 1] > kTailWarpSolve;
-    launch_pdl(big ? k_tail<T, true> : k_tail<T, false>, 1, 1024, smem, s, ta);
+        launch_tail<T>(mg, lt, cur[lt], nu1, nu2, s);
     }
     for (int l = lt - 1; l >= 0; l--) {
         Level &v = mg.lv[l];
@@ -2828,8 +2838,8 @@ long mg_bench_op(MG &mg, int op, int level, cudaStream_t s)
                           level == 0 ? v.d.e : nullptr);
         return cells;
     case 5:
-        if (mg.tail_f >= mg.L - 1) return -1;
-        launch_tail_w<float>(mg, mg.lv[mg.tail_f].f.e2, mg.tail_f > 0, s);
+        if (mg.tail_f < mg.L - 1) launch_tail_w<float>(mg, mg.lv[mg.tail_f].f.e2, mg.tail_f > 0, s);
+        else launch_tail<float>(mg, mg.tail_f, mg.lv[mg.tail_f].f.e2, 2, 2, s);
         return (long)mg.lv[mg.tail_f].nx * mg.lv[mg.tail_f].ny;
     case 7:
     case 8: {  // the fused FP64 smoothers (7: sweeps + restriction, 8: prolongation + sweeps)

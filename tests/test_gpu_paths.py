@@ -376,3 +376,17 @@ def test_step_graphs_of_several_time_steps(T, ib):
 
     same = cycle_time([1.0] * 4)
     assert cycle_time([1.0, 0.9, 0.8, 0.7]) <= 1.3 * same
+
+
+# The lower cycle is timed also where it is the coarsest level alone (25 x 25,
+# under 50 x 50, which is launched for itself).
+def test_timing_of_a_coarsest_level_alone(T, ib):
+    n = 200
+    X, Y = W.circle(0.5, 0.5, 0.2, 16)
+    ctx = ib.Context(ib.Config(nx=n, ny=n, h=1.0 / n), X, Y, [0, 16])
+    one = T.ones((n, n + 1), dtype=T.float64, device="cuda")
+    ctx.mg_setup(one, T.ones((n + 1, n), dtype=T.float64, device="cuda"))
+    p = T.zeros((n, n), dtype=T.float64, device="cuda")
+    ctx.mg_solve(T.from_numpy(W.random_cells(n, n, 4)).cuda(), p, 1, 1e-8, 100)
+    us, units = ctx.bench_kernel(5)
+    assert us > 0.0 and units == 25 * 25
