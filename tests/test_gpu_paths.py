@@ -390,3 +390,22 @@ def test_timing_of_a_coarsest_level_alone(T, ib):
     ctx.mg_solve(T.from_numpy(W.random_cells(n, n, 4)).cuda(), p, 1, 1e-8, 100)
     us, units = ctx.bench_kernel(5)
     assert us > 0.0 and units == 25 * 25
+
+
+# Markers on grid lines and cell centres, and one unit in the last place to either
+# side, where a factor of the delta functions vanishes or the stencil moves on:
+# sums of sixteen products of factors below 1/2 and values below 1.
+@pytest.mark.parametrize("kernel", [0, 1])
+def test_delta_factors_on_grid_lines(T, ib, O, kernel):
+    n, h = 32, 1.0 / 32
+    X, Y = W.circle(0.5, 0.5, 0.3, 48)
+    X, Y = np.round(X * 2 * n) / (2 * n), np.round(Y * 2 * n) / (2 * n)
+    X[1::3], Y[2::3] = np.nextafter(X[1::3], 0.0), np.nextafter(Y[2::3], 1.0)
+    X[2::4], Y[3::4] = np.nextafter(X[2::4], 1.0), np.nextafter(Y[3::4], 0.0)
+    start = np.array([0, 48], np.int32)
+    ctx = ib.Context(ib.Config(nx=n, ny=n, h=h, kernel=kernel), X, Y, start)
+    u, v = W.random_faces(n, n, 9)
+    d = lambda a: T.from_numpy(np.ascontiguousarray(a)).cuda()
+    U, V = (a.cpu().numpy() for a in ctx.interp(d(u), d(v)))
+    oU, oV = O.interp(u, v, X, Y, h, kernel=kernel)
+    assert np.abs(U - oU).max() <= 1e-14 and np.abs(V - oV).max() <= 1e-14
