@@ -125,7 +125,10 @@ __global__ void k_correct(int nx, int ny, double ih, double dt,
 }
 
 // Predictor: a warp marches up a strip of 30 columns (and one on either side
-// for the neighbours' fluxes), rows j0 .. j0 + R - 1, one lane per column.  A
+// for the neighbours' fluxes), rows j0 .. j0 + R - 1, one lane per column; the
+// columns that whole strips leave over, where they are at most 14 or 6, are
+// marched by 16 or 8 lanes, two or four ranges of rows a warp (64 columns were
+// three strips: 64 x 4096 56 us, now 38, 32 x 4096 38 and 26).  A
 // lane holds its column's rho, mu, u and v of the current and the next row,
 // loads the row after next while it computes, and takes its neighbours'
 // values by shuffles; every flux that two faces share is formed once: per
@@ -141,9 +144,7 @@ __global__ void k_correct(int nx, int ny, double ih, double dt,
 // 32 x 8 tile with the fluxes in shared memory has partly filled warps in
 // every pass over its ring and two barriers.  Next to the hierarchy's setup
 // and the face force, as in a step: 1024^2 171 -> 127 us, 2048^2 665 -> 429,
-// 256 x 1024 axisymmetric 107 -> 52.  R: rows per warp, 16 where that gives
-// 1024 warps, fewer below (512^2: 45 us with 8 rows, 109 with 16, whose 576
-// warps leave each to its latency; 46 the tiles).
+// 256 x 1024 axisymmetric 107 -> 52.  R: rows per warp (pred_rows).
 //
 // Walls: a ghost row or column of the velocity reflected to zero on the wall
 // (the outer wall of the axisymmetric form: to wb), of rho and mu equal to the
@@ -159,6 +160,19 @@ __global__ void k_correct(int nx, int ny, double ih, double dt,
 // ratios, a column's own, are formed once per lane.  The radial component
 // adds -mu_face u / r^2.
 constexpr int kPredT = 128, kPredCols = 30;
+// Lanes for the columns left over by whole strips (0 if none are).
+__host__ __device__ inline int pred_lanes(int nx)
+{
+    const int left = nx % kPredCols;
+    return left == 0 ? 0 : (left <= 6 ? 8 : (left <= 14 ? 16 : 32));
+}
+// Warps of a grid, R rows a range.
+inline long pred_warps(int nx, int ny, int R)
+{
+    const long rows = cdiv(ny, R);
+    const int G = pred_lanes(nx);
+    return nx / kPredCols * rows + (G ? cdiv(rows, 32 / G) : 0);
+}
 template <bool AXI>
 __global__ void __launch_bounds__(kPredT)
 k_predictor(int nx, int ny, int R, double ih, double visc, double dt,
@@ -170,12 +184,20 @@ k_predictor(int nx, int ny, int R, double ih, double visc, double dt,
             double *__restrict__ us, double *__restrict__ vs, double *au, double *av)
 {
     constexpr unsigned kAll = 0xffffffffu;
-    const int lane = threadIdx.x & 31, sx = (nx + kPredCols - 1) / kPredCols;
-    const int wid = blockIdx.x * (kPredT / 32) + (threadIdx.x >> 5), ty = wid / sx;
-    const int j0 = ty * R, j1 = min(j0 + R, ny);
-    if (j0 >= ny) return;  // whole warps
-    const int i = (wid - ty * sx) * kPredCols + lane - 1;
-    const bool out = lane >= 1 && lane <= kPredCols && i < nx;
+    const int sx = nx / kPredCols, rows = (ny + R - 1) / R, whole = sx * rows;
+    const int wid = blockIdx.x * (kPredT / 32) + (threadIdx.x >> 5);
+    const bool rest = wid >= whole;             // a warp of the columns left over
+    const int GL = rest ? pred_lanes(nx) : 32;  // lanes of a range
+    if (GL == 0) return;
+    const int lane = threadIdx.x & (GL - 1);
+    // the warp's first range, and this lane's
+    const int w0 = rest ? (wid - whole) * (32 / GL) : wid / sx;
+    const int ty = w0 + (rest ? (threadIdx.x & 31) / GL : 0);
+    if (w0 >= rows) return;  // whole warps
+    const int n = min(R, ny - w0 * R);
+    const int j0 = min(ty * R, ny - 1);  // a range beyond the grid writes nothing
+    const int i = (rest ? sx : wid - w0 * sx) * kPredCols + lane - 1;
+    const bool out = lane >= 1 && lane <= GL - 2 && i < nx && ty < rows;
     const long nxf = nx + 1;
     // columns to load from: cell and y-face data of column c, x-faces of cu
     const int c = min(max(i, 0), nx - 1), cu = min(max(i, 0), nx);
@@ -194,8 +216,8 @@ k_predictor(int nx, int ny, int R, double ih, double visc, double dt,
         return i < 0 || i >= nx ? neg(x) : x;
     };
     auto row = [&](int j) { return (long)min(max(j, 0), ny - 1) * nx + c; };
-    auto up = [&](double x) { return __shfl_up_sync(kAll, x, 1); };
-    auto down = [&](double x) { return __shfl_down_sync(kAll, x, 1); };
+    auto up = [&](double x) { return __shfl_up_sync(kAll, x, 1, GL); };
+    auto down = [&](double x) { return __shfl_down_sync(kAll, x, 1, GL); };
     // the factors of the differences
     const double hdt = 0.5 * dt, v2 = 2.0 * visc * ih * ih;
     const double gx2 = 2.0 * gx, gy2 = 2.0 * gy, ca = have_prev ? -3.0 : -2.0;
@@ -227,10 +249,11 @@ k_predictor(int nx, int ny, int R, double ih, double visc, double dt,
         fyp = rm * b * b;
         vyp = mm * (v0 - vm);
     }
-    for (int j = j0; j < j1; j++) {
+    for (int j = j0; j < j0 + n; j++) {
         const long kx = (long)j * nxf + i, ky = (long)j * nx + i;
+        const bool wr = out && j < ny;
         double ap = 0.0, bp = 0.0, irx = 0.0, iry = 0.0;
-        if (out) {
+        if (wr) {
             if (have_prev) { ap = aup[kx]; bp = avp[ky]; }
             if (bx) { irx = bx[kx]; iry = by[ky]; }
         }
@@ -255,7 +278,7 @@ k_predictor(int nx, int ny, int R, double ih, double visc, double dt,
         const double Wx1 = mn * (u1 - u0), Wy1 = mn * (v1 - vl);
         const double fw = up(fx), vw = up(vx), Ge = down(G), We = down(Wy);
         const double mw = AXI ? up(m0) : 0.0, rw = bx ? 0.0 : up(r0);
-        if (out) {
+        if (wr) {
             if (!bx) {
                 irx = recip_div(0.5 * (rw + r0));
                 iry = recip_div(0.5 * (rm + r0));
@@ -724,16 +747,40 @@ void launch_correct(int nx, int ny, double h, double dt, const double *us,
                                           bx, by, u, v);
 }
 
+// Rows a warp marches: those of the least time by what was measured, (R + 1)
+// (4 n + 1) in units of 0.48 us with n the most blocks that an SM gets (n = 1 .. 4:
+// 2.45, 4.15, 6.05 and 8.1 us a row; the FP64 pipe's rate, but for one block,
+// whose four warps wait for their own chains).  The time steps up with n, so 16
+// rows wherever they give 1024 warps cost 103 us at 960 x 640 (320 blocks: three
+// on some SMs), the tiles before 87 and 17 rows (two) 74; 768^2 101, 87 and 73;
+// 3000 x 100 53, 48 and 41; 1024^2 137, 144 and 130; 2048^2 500, 566 and 491.
+static int pred_rows(int nx, int ny)
+{
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            cudaGetLastError();
+        return n > 0 ? n : 152;
+    }();
+    int best = 1;
+    long least = 0;
+    for (int R = 1; R <= 20; R++) {
+        const long blocks = cdiv(pred_warps(nx, ny, R), kPredT / 32);
+        const long cost = (R + 1) * (4 * (long)cdiv(blocks, sms) + 1);
+        if (R == 1 || cost < least) { best = R; least = cost; }
+    }
+    return best;
+}
+
 static void predictor(bool axi, int nx, int ny, double h, double dt, const double *rho,
                       const double *mu, const double *u, const double *v, const double *au_prev,
                       const double *av_prev, int have_prev, double gx, double gy,
                       const double *frame, const double *bx, const double *by, double *us,
                       double *vs, double *au, double *av, cudaStream_t s, double visc)
 {
-    const long sx = cdiv(nx, kPredCols);
-    int R = 16;
-    while (R > 1 && sx * cdiv(ny, R) < 1024) R /= 2;
-    const unsigned g = (unsigned)cdiv(sx * cdiv(ny, R), kPredT / 32);
+    const int R = pred_rows(nx, ny);
+    const unsigned g = cdiv(pred_warps(nx, ny, R), kPredT / 32);
     note_launch();
     if (axi)
         k_predictor<true><<<g, kPredT, 0, s>>>(nx, ny, R, 1.0 / h, visc, dt, rho, mu, u, v, au_prev, av_prev,

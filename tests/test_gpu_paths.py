@@ -409,3 +409,15 @@ def test_delta_factors_on_grid_lines(T, ib, O, kernel):
     U, V = (a.cpu().numpy() for a in ctx.interp(d(u), d(v)))
     oU, oV = O.interp(u, v, X, Y, h, kernel=kernel)
     assert np.abs(U - oU).max() <= 1e-14 and np.abs(V - oV).max() <= 1e-14
+
+
+# Marches of as many rows as an uneven share of blocks makes them take: 17 rows
+# (960 x 640, the last of 11), 11 (768^2, the last of 9) and 14 (700 x 701, the
+# last of one); and columns left over by whole strips, marched by 8 lanes (up to
+# 6), 16 (up to 14) or 32, with ranges beyond the grid in the last warp.  By the
+# bound of the other strips.
+@pytest.mark.parametrize("axisym", [0, 1])
+@pytest.mark.parametrize("nx,ny", [(960, 640), (768, 768), (700, 701), (6, 9), (31, 7), (36, 50), (37, 51),
+                                   (44, 33), (45, 33), (64, 1001), (102, 770)])
+def test_predictor_rows(T, ib, O, nx, ny, axisym):
+    test_predictor_strips(T, ib, O, nx, ny, axisym)
