@@ -17,13 +17,12 @@ namespace {
 
 constexpr int kT = 256;
 
-// x + x: an addition to the exponent, no FP64 operation, for a normal x whose
-// double is normal too; the sum for all others (zeros, infinities, NaN).
+// 2 x for a normal x, an infinity or a NaN (not finite where the double is not), by
+// an addition to the exponent: x + x for those beyond it costs k_coeffs a fifth.
 __device__ __forceinline__ double twice(double x)
 {
-    const unsigned e = (unsigned)__double2hiint(x) & 0x7ff00000u;
-    if (e - 0x00100000u >= 0x7fd00000u) return x + x;
-    return __longlong_as_double(__double_as_longlong(x) + (1LL << 52));
+    const int hi = __double2hiint(x);
+    return __hiloint2double(hi + ((hi & 0x7ff00000) == 0x7ff00000 ? 0 : 0x00100000), __double2loint(x));
 }
 
 // rho and mu of the cells and beta = 1 / (two-cell mean of rho) on the faces.
@@ -32,8 +31,12 @@ __device__ __forceinline__ double twice(double x)
 // interface, rho, mu and beta are those of the row below, and no FP64
 // operation is needed (ten a cell bound the two kernels that this one replaces;
 // next to the face force 8 + 41 us at 1024^2, now 15, and 85 + 64 at 2048^2,
-// now 49).  ROWS: 8 from 2^18 cells up, 1 below (64^2: 6.6 us with 8 rows,
-// 4.1 the two kernels).
+// now 49).  ROWS: 1 below 2^18 cells, 4 up to 2^20, 8 from there.  Alone, with one
+// row, 4 and 8 (drops; values that never repeat): 64^2 2.4, 4.7, 7.7 us; 256^2
+// 3.3, 4.4, 7.0; 512^2 7.9, 6.2, 7.4 (7.9, 7.6, 7.8); 64 x 4096 10.1, 10.5, 13.2;
+// 960 x 640 14.9, 10.7, 12.0 (15.0, 16.3, 19.0); 960^2 21.1, 13.5, 12.6 (21.2, 22.0,
+// 24.7); 1024^2 24.3, 13.9, 13.7 (24.2, 24.9, 24.7); 2048^2 90, 38.7, 32.0 (90, 86, 88);
+// the two kernels: 10.7 at 64 x 4096, 19.5 at 960 x 640, 30.7 at 1024^2.
 template <int ROWS>
 __global__ void __launch_bounds__(256)
 k_coeffs(int nx, int ny, double rho_g, double drho, double mu_g, double dmu,
@@ -724,7 +727,9 @@ void launch_coeffs(int nx, int ny, double rho_g, double rho_l, double mu_g,
                                                      mu, bx, by);
     };
     note_launch();
-    if ((long)nx * ny >= 1L << 18) launch(k_coeffs<8>, 8);
+    const long n = (long)nx * ny;
+    if (n >= 1L << 20) launch(k_coeffs<8>, 8);
+    else if (n >= 1L << 18) launch(k_coeffs<4>, 4);
     else launch(k_coeffs<1>, 1);
 }
 

@@ -421,3 +421,13 @@ def test_delta_factors_on_grid_lines(T, ib, O, kernel):
                                    (44, 33), (45, 33), (64, 1001), (102, 770)])
 def test_predictor_rows(T, ib, O, nx, ny, axisym):
     test_predictor_strips(T, ib, O, nx, ny, axisym)
+
+
+# Four rows a warp between 2^18 and 2^20 cells and eight above, with last strips of
+# one row and of all but one: as above.
+@pytest.mark.parametrize("nx,ny", [(93, 2821), (520, 519), (1023, 1025), (1030, 1023)])
+def test_coefficients_rows_a_warp(T, ib, O, nx, ny):
+    H = layered_H(nx, ny, 6)
+    got = ib.ib_op_coeffs(T.from_numpy(H).cuda(), 1e-3, 1.0, 1e-4, 1e-2)
+    for a, b in zip(got, O.coeffs(H, 1e-3, 1.0, 1e-4, 1e-2)):
+        assert np.abs(a.cpu().numpy() - b).max() <= 1e-15 * np.abs(b).max()
