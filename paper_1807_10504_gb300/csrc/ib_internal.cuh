@@ -12,14 +12,25 @@
 namespace ibk {
 
 // Levels with at most this many cells run in one CTA, in the FP64 and in the
-// FP32 cycle.  FP64: with 1024 a cycle took 36.9 us at 64^2, 60.3 at 256^2 and
-// 200 at 1024^2 (the FP64 work of a 32^2 level on one SM: 7 us, against two
-// launches of 3.5), with 256 33.9, 59.0 and 198, and 31.6, 56.8 and 195 with the
-// smoother's 8 x 8 tiles as well.  FP32: with 4096 78.9 us at
-// 1024^2, 52.7 at 512^2, 25.9 at 64^2 (a level of 64^2 costs one CTA 11 us, its
-// two launches 7.5), with 1024 76.4, 49.9 and 22.9, with 256 78.7, 52.6 and 24.5.
+// FP32 V(2,2) cycle, whose larger levels take two fused launches each.  FP64:
+// with 1024 a cycle took 36.9 us at 64^2, 60.3 at 256^2 and 200 at 1024^2 (the
+// FP64 work of a 32^2 level on one SM: 7 us, against two launches of 3.5), with
+// 256 33.9, 59.0 and 198, and 31.6, 56.8 and 195 with the smoother's 8 x 8 tiles
+// as well.  FP32: with 4096 78.9 us at 1024^2, 52.7 at 512^2, 25.9 at 64^2 (a
+// level of 64^2 costs one CTA 11 us, its two launches 7.5), with 1024 76.4, 49.9
+// and 22.9, with 256 78.7, 52.6 and 24.5.
 constexpr int kTailCells = 256;
 constexpr int kTailCellsF32 = 1024;
+// The same for cycles of other sweep counts, whose larger levels take a launch
+// for each sweep, for the restriction and for the prolongation.  FP64, of
+// V(1,1), V(3,3) and V(6,6): 50.9, 91.3 and 150 us at 64^2 with 1024 (53.8, 101
+// and 171 with 256), 124, 223 and 381 at 256 x 1024 (125, 232 and 400), 208, 362
+// and 604 at 1024^2 (212, 375 and 627).  FP32 the same, where a count is odd:
+// 26.5 and 36.4 (V(1,1), V(3,3)) at 64^2 with 4096 (30.2 and 40.6 with 1024), 103
+// and 151 at 1024^2 (106 and 153); even counts take two sweeps a launch and
+// kTailCellsF32 (V(4,4) 41.0 us at 64^2, 41.6 with 4096; 86.5 and 88.9 at 256 x 1024).
+constexpr int kTailSweepCells = 1024;
+constexpr int kTailSweepCellsF32 = 4096;
 constexpr int kMaxCoarsest = 1024;   // dense LU limit of the coarsest level
 constexpr int kBlk = 8;              // marker-activity block edge (cells)
 constexpr int kSearch = 7;           // marker search radius (cells) around a cell or face
@@ -321,6 +332,7 @@ struct MG {
     bool use_graphs = true;
     int tail = 0;                 // first level handled by the single-CTA tail kernel (FP64)
     int tail_f = 0;               // the same for the FP32 cycle
+    int tail_s = 0, tail_sf = 0;  // the same in cycles of one launch a sweep
     double *lu = nullptr;         // coarsest dense LU (n x n), FP64
     int *piv = nullptr;           // coarsest row permutation
     double *red = nullptr;        // reduction partials + results (device)

@@ -21,9 +21,10 @@
 //  * kernels of the cycle use programmatic dependent launch: the next grid is
 //    scheduled while the previous one drains and waits (griddepcontrol) for
 //    its results.
-//  * levels with <= 256 cells (FP64) / <= 1024 cells (FP32) run as one
-//    single-CTA kernel (the whole lower V-cycle and the coarsest solve) with
-//    its data in shared memory, since launches dominate there.
+//  * levels with <= 256 cells (FP64) / <= 1024 cells (FP32; more in cycles of
+//    other sweep counts) run as one single-CTA kernel (the whole lower V-cycle
+//    and the coarsest solve) with its data in shared memory, since launches
+//    dominate there.
 //  * norms are deterministic two-stage reductions (fixed per-thread order,
 //    fixed tree, last-block fold) with no floating-point atomics.
 //  * the FP32 instantiations of the same kernels form the inner cycle of the
@@ -2462,9 +2463,10 @@ bool vcycle(MG &mg, int nu1, int nu2, cudaStream_t s, double *add64 = nullptr)
     auto lvT = [&](int l) -> LevelT<T> & {
         if constexpr (sizeof(T) == 8) return mg.lv[l].d; else return mg.lv[l].f;
     };
-    const int L = mg.L, lt = sizeof(T) == 8 ? mg.tail : mg.tail_f;
     constexpr bool f32 = sizeof(T) == 4;
     const bool fused = nu1 == 2 && nu2 == 2;
+    const bool single = f32 ? nu1 % 2 || nu2 % 2 : !fused;  // a launch for one sweep
+    const int L = mg.L, lt = f32 ? (single ? mg.tail_sf : mg.tail_f) : (single ? mg.tail_s : mg.tail);
     T *cur[kMaxLv];
     for (int l = 0; l < L; l++) cur[l] = lvT(l).e;
     for (int l = 0; l < lt; l++) {
@@ -2769,12 +2771,15 @@ size_t mg_layout(MG &mg, int nx, int ny, double h, char *base, bool shared_w)
         v.fault = base ? &mg.ctl->fault : nullptr;
         v.tma = base && encode_level_maps(v);
     }
-    int t = 0;
-    while (t < L && (long)nxs[t] * nys[t] > kTailCells) t++;
-    mg.tail = std::min(t, L - 1);
-    t = 0;
-    while (t < L && (long)nxs[t] * nys[t] > kTailCellsF32) t++;
-    mg.tail_f = std::min(t, L - 1);
+    auto first = [&](int cells) {
+        int t = 0;
+        while (t < L && (long)nxs[t] * nys[t] > cells) t++;
+        return std::min(t, L - 1);
+    };
+    mg.tail = first(kTailCells);
+    mg.tail_f = first(kTailCellsF32);
+    mg.tail_s = first(kTailSweepCells);
+    mg.tail_sf = first(kTailSweepCellsF32);
     return off;
 }
 
@@ -2928,8 +2933,8 @@ void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool w
         // shared memory of the single-CTA tail (set here, outside any capture)
         size_t e = 0;
         size_t ef = 0;
-        for (int l = mg.tail; l < L; l++) e += tail_level_elems(mg.lv[l].nx, mg.lv[l].ny, l == L - 1);
-        for (int l = mg.tail_f; l < L; l++) ef += tail_level_elems(mg.lv[l].nx, mg.lv[l].ny, l == L - 1);
+        for (int l = mg.tail_s; l < L; l++) e += tail_level_elems(mg.lv[l].nx, mg.lv[l].ny, l == L - 1);
+        for (int l = mg.tail_sf; l < L; l++) ef += tail_level_elems(mg.lv[l].nx, mg.lv[l].ny, l == L - 1);
         const size_t inv = tail_inv_bytes(mg.lv[L - 1].nx * mg.lv[L - 1].ny);
         raise_smem_limit((const void *)k_smooth2_f64<1, 64, 32>, kTwoBlocks);
         raise_smem_limit((const void *)k_smooth2_f64<2, 64, 32>, kTwoBlocks);

@@ -431,3 +431,25 @@ def test_coefficients_rows_a_warp(T, ib, O, nx, ny):
     got = ib.ib_op_coeffs(T.from_numpy(H).cuda(), 1e-3, 1.0, 1e-4, 1e-2)
     for a, b in zip(got, O.coeffs(H, 1e-3, 1.0, 1e-4, 1e-2)):
         assert np.abs(a.cpu().numpy() - b).max() <= 1e-15 * np.abs(b).max()
+
+
+# Cycles of other sweep counts, whose single-block tail takes more levels: 32^2 and
+# (FP32) 64^2, and a coarsest level of 33 x 17 alone.  The solution to a hundred
+# times the tolerance, as on the coarsest sizes.
+@pytest.mark.parametrize("nu", [(1, 1), (2, 1), (3, 3), (4, 2)])
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("nx,ny", [(64, 64), (128, 128), (132, 68)])
+def test_tails_of_other_sweep_counts(T, ib, O, nx, ny, precision, nu):
+    h = 1.0 / ny
+    X, Y = W.circle(0.5 * nx / ny, 0.5, 0.2, 16)
+    ctx = ib.Context(ib.Config(nx=nx, ny=ny, h=h, nu1=nu[0], nu2=nu[1]), X, Y, [0, 16])
+    rho, mu, bx, by = O.coeffs(W.random_H(nx, ny, 3), 1e-3, 1.0, 1e-4, 1e-2)
+    b = W.random_cells(nx, ny, 4)
+    d = lambda a: T.from_numpy(np.ascontiguousarray(a)).cuda()
+    ctx.mg_setup(d(bx), d(by))
+    p = T.zeros((ny, nx), dtype=T.float64, device="cuda")
+    tol = 1e-12 if precision == 0 else 1e-11
+    st, cyc, rr = ctx.mg_solve(d(b), p, precision, tol, 300)
+    o = O.mg_solve(bx, by, b, h, precision=0, tol=1e-12, max_cycles=300)
+    assert st == 0 and rr <= tol
+    assert np.abs(p.cpu().numpy() - o.p).max() <= 100 * tol * np.abs(o.p).max()
