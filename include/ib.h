@@ -91,7 +91,11 @@ typedef struct ib_config {
                                  off-diagonal / diagonal ratio is at most 2s / (1 + 2s),
                                  s = nu dt / h^2, and a sweep contracts the error by
                                  about its square: 20 sweeps reach ~1e-12 for s <= 0.5;
-                                 larger steps need more) */
+                                 larger steps need more).  Takes 40 more bytes a face
+                                 (336 MB at 2048^2) for tables of the system's
+                                 coefficients; where the device has no room for them,
+                                 every sweep forms them anew (ten times as slow, the
+                                 same values to rounding) */
     int32_t cn_sweeps;
     int32_t indicator;        /* density and viscosity from 0: the polygon Heaviside H;
                                  1: the indicator I of Sec. 2.2 Eq. (ind_psn),

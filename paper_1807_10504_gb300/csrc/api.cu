@@ -46,7 +46,7 @@ struct ib_ctx {
            *bxa = nullptr, *bya = nullptr, *fr = nullptr;
     double *frame = nullptr;   // non-inertial frame record (kFrSlots doubles)
     double *ue = nullptr, *ve = nullptr;  // Crank-Nicolson: the other pair of iterate buffers
-    double *cnw = nullptr, *cnr = nullptr;  // its weights and right-hand sides (cnmem)
+    double *cnw = nullptr, *cnr = nullptr;  // its weights and right-hand sides (cnmem), or NULL
     void *cnmem = nullptr;
     double *mh = nullptr;      // the indicator function
     double *pprev = nullptr;   // the previous step's pressure (warm start 3)
@@ -179,6 +179,8 @@ ib_status launch_check(ib_ctx *c, const char *what)
 }
 
 size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
+
+constexpr size_t kStepRoom = 64u << 20;  // device memory left to a step's graphs
 
 // Orientation and wall distance of host marker arrays.
 // Ghost columns of the axisymmetric marker grid: the mirror half of the
@@ -413,7 +415,7 @@ ib_status step_pre(ib_ctx *c, double dt, bool reloc, bool mass, int warm)
     // half the viscosity into the pair of buffers from which the implicit
     // half's launches end in us, vs
     const double visc = g.viscous ? 0.5 : 1.0;
-    const bool odd = g.viscous && cn_launches(g.cn_sweeps) % 2;
+    const bool odd = g.viscous && c->cnw && cn_launches(g.cn_sweeps) % 2;
     double *pu = odd ? c->ue : c->us, *pv = odd ? c->ve : c->vs;
     // on two side streams, overlapping the predictor: the hierarchy of the
     // pressure coefficients (the r-weighted operator r_face beta in
@@ -436,7 +438,12 @@ ib_status step_pre(ib_ctx *c, double dt, bool reloc, bool mass, int warm)
     else
         launch_predictor(g.nx, g.ny, g.h, dt, c->rho, c->mu, c->u, c->v, c->au, c->av, c->have_prev,
                          g.gx, g.gy, c->bx, c->by, pu, pv, c->au, c->av, c->s, visc);
-    if (g.viscous) {
+    if (g.viscous && !c->cnw) {  // no memory for the tables: the coefficients anew in every sweep
+        cudaMemcpyAsync(c->ue, c->us, (size_t)(g.nx + 1) * g.ny * 8, cudaMemcpyDeviceToDevice, c->s);
+        cudaMemcpyAsync(c->ve, c->vs, (size_t)g.nx * (g.ny + 1) * 8, cudaMemcpyDeviceToDevice, c->s);
+        launch_cn_solve(g.nx, g.ny, g.h, dt, c->rho, c->mu, g.axisym, g.frame ? c->frame : nullptr,
+                        g.cn_sweeps, c->ue, c->ve, c->us, c->vs, c->s);
+    } else if (g.viscous) {
         launch_cn_solve_tab(g.nx, g.ny, g.h, dt, c->rho, c->mu, g.axisym, g.frame ? c->frame : nullptr,
                             g.cn_sweeps, c->cnw, c->cnr, pu, pv, odd ? c->us : c->ue,
                             odd ? c->vs : c->ve, c->s);
@@ -655,15 +662,6 @@ ib_status ib_init(ib_ctx **out, const ib_config *cfg, const double *X, const dou
         launch_axi_frame(c->mk, 1.0, g.c1, g.c2, 1, c->frame, c->s);
         e = cudaStreamSynchronize(c->s);
     }
-    if (e == cudaSuccess && g.viscous) {
-        e = cudaMalloc(&c->cnmem, al((fx + fy) * 32) + al((fx + fy) * 8));
-        if (e == cudaSuccess) {
-            c->cnw = (double *)c->cnmem;
-            c->cnr = (double *)((char *)c->cnmem + al((fx + fy) * 32));
-        } else {
-            c->cnmem = nullptr;
-        }
-    }
     if (e == cudaSuccess && g.indicator) {
         const size_t ib = al(fx * 8) + al(fy * 8) + al(nc * 8) + al(8) + al((size_t)M * 8);
         e = cudaMalloc(&c->imem, ib);
@@ -709,6 +707,21 @@ ib_status ib_init(ib_ctx **out, const ib_config *cfg, const double *X, const dou
         e = cudaStreamSynchronize(c->s);
     } else {
         c->dmem = nullptr;
+    }
+    // the Crank-Nicolson tables last, and only where they leave room for what a
+    // step still takes (its graphs): a context that fits without them is made
+    // without them
+    if (e == cudaSuccess && g.viscous) {
+        const size_t need = al((fx + fy) * 32) + al((fx + fy) * 8);
+        size_t room = 0, all = 0;
+        if (cudaMemGetInfo(&room, &all) == cudaSuccess && room >= need + kStepRoom &&
+            cudaMalloc(&c->cnmem, need) == cudaSuccess) {
+            c->cnw = (double *)c->cnmem;
+            c->cnr = (double *)((char *)c->cnmem + al((fx + fy) * 32));
+        } else {
+            cudaGetLastError();
+            c->cnmem = nullptr;
+        }
     }
     if (e != cudaSuccess) {
         ib_status r = (e == cudaErrorMemoryAllocation) ? IB_ENOMEM : IB_ECUDA;
