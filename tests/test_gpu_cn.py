@@ -108,3 +108,34 @@ def test_cn_without_room_for_its_tables(T, ib):
         T.cuda.empty_cache()
     for a, b in zip(got, ref):
         assert float((a - b).abs().max()) <= 1e-10 * 3.2
+
+
+# The sweeps as a step runs them (from tables, two a launch) against the operator
+# that forms every coefficient in every sweep: tiles of 32 x 16 and, from 1.25
+# million faces up, 64 x 32, widths and heights that they do not divide, an odd
+# sweep left and odd numbers of launches, one row and eight rows a thread.  The
+# operator's bound against the oracle.
+@pytest.mark.parametrize("axisym", [0, 1])
+@pytest.mark.parametrize("nx,ny,sweeps", [(62, 66, 5), (320, 416, 6), (800, 832, 4), (800, 832, 5)])
+def test_step_sweeps_match_operator(T, ib, nx, ny, sweeps, axisym):
+    h = 1.0 / nx
+    if axisym:
+        mk = W.axi_elliptic_drop(0.5, 0.25, 1.1, 4 * (nx // 8))
+    else:
+        mk = W.elliptic_drop(0.5, 0.5, 0.25, 1.1, 4 * (nx // 8))
+    cfg = ib.Config(nx=nx, ny=ny, h=h, mu_g=0.05, mu_l=5.0, relocate_every=0, axisym=axisym, viscous=1,
+                    cn_sweeps=sweeps, precision=1, tol=1e-3)
+    ctx = ib.Context(cfg, mk.X, mk.Y, mk.drop_start)
+    u, v = W.random_faces(nx, ny, 63, scale=1e-3)
+    d = lambda a: T.from_numpy(np.ascontiguousarray(a)).cuda()
+    u, v = d(u), d(v)
+    ctx.set("u", u)
+    ctx.set("v", v)
+    dt = 0.4 * h * h  # s = nu dt / h^2 between 2 and 20
+    ctx.ns_step(dt, 1, 0)
+    rho, mu, us, vs = (ctx.get(f) for f in ("rho", "mu", "us", "vs"))
+    predictor = ib.ib_op_predictor_axi if axisym else ib.ib_op_predictor
+    ue, ve, _, _ = predictor(rho, 0.5 * mu, u, v, h, dt)
+    uo, vo = ib.ib_op_cn_solve(rho, mu, ue, ve, h, dt, sweeps, axisym)
+    for a, b in ((us, uo), (vs, vo)):
+        assert float((a - b).abs().max()) <= 1e-13 * float(b.abs().max())
