@@ -810,8 +810,8 @@ __device__ __forceinline__ T flux_sum(int nx, int ny, int i, int j, const T *bx,
 // while staging, then the sweeps (halo 4).
 // The FP64 pipe bounds these kernels on this part (its instruction rate, not
 // HBM), so the design counts FP64 instructions: fused sweeps, the residual
-// identity, prolongation in FMAs; tiles of 32 x 16 spread the levels below
-// 2^20 cells over the SMs.  With those a block is few warps and every phase
+// identity, prolongation in FMAs; tiles of 32 x 16 spread most levels below
+// 2^21 cells over the SMs.  With those a block is few warps and every phase
 // would wait for its weights from L2, so a thread keeps its (at most two)
 // cells' weights and right-hand sides of the next phase in registers, loaded
 // while the current one runs, the first phase's weights before the wait for
@@ -2310,19 +2310,23 @@ void launch_smooth2(const Level &v, const LevelT<float> &a, const float *pin, fl
     }
 }
 
-// One fused FP64 smoother launch of MODE on level v (pin -> p): 64 x 32 tiles
-// from 2^20 cells up, 32 x 16 below, where more tiles share the FP64 work
-// more evenly (512^2 as 128 tiles of 64 x 32, several of them on one SM while
-// others had none: 22 and 44 us in the cycle; as 512 of 32 x 16 and with
-// their weights prefetched a 512^2 V-cycle went from 139 to 105 us).  Up to four waves of 64 x 32 tiles
-// leave room (dynamic shared memory) for two blocks an SM only, so that the
-// scheduler hands the rest to the SMs that finish first instead of placing
-// all at once (1024^2: FP64 cycle 246 -> 222 us; 2048^2, with 13 tiles an SM,
-// would lose a tenth).  Levels that 16 x 8 tiles cover with at most one block an
-// SM (up to 128^2) take those: a block's FP64 work, not the halo's share of it,
-// then sets the launch's time (FP64 cycle at 64^2 40.1 -> 36.9 us, 128^2 52.0 ->
-// 44.3, 256^2 69.4 -> 60.1, 1024^2 211 -> 200), up to 64^2 those of 8 x 8 (36.9 ->
-// 36.5, 44.3 -> 43.2, 60.3 -> 59.5).
+// One fused FP64 smoother launch of MODE on level v (pin -> p).  Tiles of 64 x 32
+// (15 to 25 % of halo) from 2^21 cells up and where they make one wave of two blocks
+// an SM that leaves none idle (153 to 304 tiles), 32 x 16 otherwise, whose finer
+// grain evens out the last wave.  FP64 V(2,2) cycle with 64 x 32 and with 32 x 16 on
+// the finest level: 512^2 (128 tiles) 101.6 and 96.2 us; 640^2 (200) 115.4, 117.4;
+// 1024 x 512 (256) 124.1, 135.2; 768^2 (288) 126.2, 142.1; 960 x 640 (300) 127.2,
+// 145.1; 1024 x 768 (384) 179.4, 167.0; 896^2 (392) 182.3, 169.5; 960^2 (450) 199.8,
+// 192.4; 1024^2 (512) 203.5, 203.5; 1280 x 1024 (640) 248.2, 239.4; 1536 x 1024 (768)
+// 273.6, 271.5; 2048 x 1024 (1024) 304.9, 307.1.  Up to four tiles an SM, 64 x 32 ones
+// leave room (dynamic shared memory) for two blocks an SM only, so that the scheduler
+// hands the rest to the SMs that finish first instead of placing all at once (1024^2:
+// FP64 cycle 246 -> 222 us; 2048^2, with 13 tiles an SM, would lose a tenth).  Levels
+// that 16 x 8 tiles cover with at most one block an SM (up to 128^2) take those: a
+// block's FP64 work, not the halo's share of it, then sets the launch's time (FP64
+// cycle at 64^2 40.1 -> 36.9 us, 128^2 52.0 -> 44.3, 256^2 69.4 -> 60.1, 1024^2 211 ->
+// 200), up to 64^2 those of 8 x 8 (36.9 -> 36.5, 44.3 -> 43.2, 60.3 -> 59.5; between 64^2
+// and 128^2 the two differ by less than 1 %, 256 x 128 loses 4 % with 8 x 8).
 template <int MODE>
 void launch_smooth2_f64(const Level &v, const LevelT<double> &a, const double *pin, double *p,
                         double *rc, double *ecz, double h2c, const double *invdc, double *btc,
@@ -2330,9 +2334,11 @@ void launch_smooth2_f64(const Level &v, const LevelT<double> &a, const double *p
 {
     const double ih2 = 1.0 / (v.h * v.h);
     note_launch();
-    if ((long)v.nx * v.ny >= (1L << 20)) {
-        dim3 g(cdiv(v.nx, 64), cdiv(v.ny, 32));
-        const int pad = g.x * g.y <= 4 * 152 ? kTwoBlocks : 0;
+    const dim3 g64(cdiv(v.nx, 64), cdiv(v.ny, 32));
+    const long n64 = (long)g64.x * g64.y;
+    if ((long)v.nx * v.ny >= (1L << 21) || (n64 > 152 && n64 <= 2 * 152)) {
+        const dim3 g = g64;
+        const int pad = n64 <= 4 * 152 ? kTwoBlocks : 0;
         launch_pdl(k_smooth2_f64<MODE, 64, 32>, g, 256, pad, s, v.nx, v.ny, ih2, (const double2 *)a.w,
                    (const double *)a.bt, (const double *)a.bx, (const double *)a.by, pin, p, rc,
                    ecz, h2c, invdc, btc, ecp);
