@@ -1121,8 +1121,12 @@ __global__ void k_level_w(LevelWArgs a)
 // lanes, as off the interface, its coefficients are those of the row below: no
 // FP64 operation and no conversion (next to the predictor: 1024^2 67 -> 38 us,
 // 2048^2 178 -> 85).  ROWS = 1, where every cell's work is in flight at once,
-// below 2^20 cells (256^2 under a 512^2 grid: 23 us with 8 rows, 5 with one).  LEVEL0 at compile time: as an argument both forms of a face
-// were computed and one selected.
+// below 2^19 cells (256^2 under a 512^2 grid: 23 us with 8 rows, 5 with one).  A whole
+// mg_setup alone with 8 rows and with one on the finest level (drops; values that
+// never repeat): 512^2 52.9 and 52.8 us (54.8, 52.9); 1024 x 512 57.8, 60.2 (59.9, 60.0);
+// 768^2 57.8, 63.9 (59.9, 63.9); 896^2 148, 154 (152, 154); 1024^2 74.2, 72.6 (84.1, 74.5);
+// 1536 x 1024 80.9, 88.2 (90.9, 88.3); 2048^2 132, 152 (155, 152).  LEVEL0 at compile
+// time: as an argument both forms of a face were computed and one selected.
 template <bool LEVEL0, int ROWS>
 __global__ void __launch_bounds__(256)
 k_level_coeffs(int nx, int ny, const double *__restrict__ fbx, const double *__restrict__ fby, LevelOut o)
@@ -2896,7 +2900,7 @@ void ensure_fp64_w(MG &mg, cudaStream_t s)
 }
 
 constexpr int kCoefRows = 8;            // rows a warp of k_level_coeffs
-constexpr long kCoefCells = 1L << 20;  // levels from this size on; below one row
+constexpr long kCoefCells = 1L << 19;  // levels from this size on; below one row
 void mg_build(MG &mg, const double *bx, const double *by, cudaStream_t s, bool with_w)
 {
     const int L = mg.L;
