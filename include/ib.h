@@ -313,9 +313,10 @@ ib_status cnn_set_coarsen(ib_cnn *net, int32_t levels);   /* 0 .. 6 */
  * for every layer; 1 (default) the fifth-generation tensor cores
  * (tcgen05.mma, FP32 accumulators in tensor memory) for the layer shapes
  * where they measure faster (at present none: the layers are bound by
- * staging and latency, and 1 runs as 0); 2 tcgen05 for every layer whose
- * width is a multiple of 128, the warp-level kernel elsewhere.  The paths
- * accumulate in the same order and agree bit for bit.  The backward pass
+ * staging and latency, and 1 runs as 0); 2 tcgen05 for every layer but the
+ * first (whose input stores two of its sixteen channels) if the width is a
+ * multiple of 128, the warp-level kernel elsewhere.  The paths accumulate in
+ * the same order and agree bit for bit.  The backward pass
  * always uses the warp-level kernel.
  * cnn_grad and cnn_train return IB_ECUDA if a tensor-core completion wait
  * ran out (50 ms).                                                         */
@@ -499,7 +500,10 @@ ib_status ib_op_rhs_axi(int32_t nx, int32_t ny, double h, double dt,
 /* Crank-Nicolson viscous solve (Section 2.1): nsweeps red-black sweeps on
  * u* - dt / (2 rho_f) D(u*) = u_e for both components (planar, or
  * axisymmetric with fixed outer wall), starting from u_e; boundary faces keep
- * u_e's values.  ue, ve: inputs; us, vs: outputs (device face arrays).     */
+ * u_e's values.  ue, ve: inputs; us, vs: outputs (device face arrays).
+ * Allocates nothing, so it forms every coefficient in every sweep, as a step
+ * does whose context found no room for the tables of them that the others
+ * sweep from (see ib_config's viscous); the two agree to rounding.         */
 ib_status ib_op_cn_solve(int32_t nx, int32_t ny, double h, double dt,
                          const double *rho, const double *mu, int32_t axisym,
                          int32_t nsweeps, const double *ue, const double *ve,

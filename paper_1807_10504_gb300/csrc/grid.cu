@@ -6,8 +6,7 @@
 //
 // All kernels are single-pass, one thread per cell or face, coalesced along
 // x.  FP64 arithmetic bounds them on this part before HBM (1.25 TFLOP/s), so
-// they are written for few FP64 operations; divisions of indices are avoided
-// by two-dimensional grids.
+// they are written for few FP64 operations.
 #include <utility>
 
 #include "ib_internal.cuh"
@@ -648,8 +647,11 @@ void launch_cn_solve(int nx, int ny, double h, double dt, const double *rho, con
 int cn_launches(int nsweeps) { return (nsweeps + 1) / 2; }
 
 // Tiles of 64 x 32 faces once they fill the device four times over, 32 x 16
-// below (a small grid's weights come from L2 with too few blocks in flight
-// otherwise).
+// below, where a small grid's weights come from L2 with too few blocks in flight
+// otherwise.  Two sweeps with 32 x 16 and with 64 x 32: 256^2 6.2 and 13.2 us, 384^2
+// 10.4, 14.3, 512^2 15.1, 15.3, 640^2 21.3, 19.8, 768^2 27.5, 30.0, 800^2 (the line) 24.8,
+// 26.0, 960^2 41.0, 38.7, 1024^2 47.7, 44.8, 1280 x 1024 58.5, 63.6, 2048^2 170, 157: from
+// 512^2 on within 9 % either way as the last wave fills.
 void launch_cn_solve_tab(int nx, int ny, double h, double dt, const double *rho, const double *mu,
                          int axisym, const double *frame, int nsweeps, double *w, double *r,
                          double *ua, double *va, double *ub, double *vb, cudaStream_t s)

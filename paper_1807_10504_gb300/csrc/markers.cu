@@ -26,7 +26,7 @@ constexpr int kT = 256;
 // axis: at r = a - 1 - f, a = 0 .. 3, f in [0, 1) the marker's fraction past
 // line 1.  The cosine kernel's four values are 1/4 (1 -+ sin, cos(pi f / 2)) of
 // one angle: one sincospi instead of four cospi.  Peskin's are 1/8 (3 - 2 f -+ q,
-// 1 + 2 f +- q) with q = sqrt(1 + 4 f - 4 f^2), his two branches at 1 + f, f, 1 - f
+// 1 + 2 f +- q) with q = sqrt(1 + 4 f - 4 f^2), the two branches at 1 + f, f, 1 - f
 // and 2 - f: one square root in place of four (the markers' FP64 bounds the
 // interpolation: 16384 markers 30.9 -> 16.4 us, 300,000 465 -> 213; one thread a
 // marker with a root a factor took 22.6 and 265).
@@ -1882,7 +1882,8 @@ k_reloc_place(int M, const int32_t *__restrict__ drop_of, const int32_t *__restr
 // axisymmetric contexts.  The falling frame divides differences of the drop's
 // centre by the square of the time step: there one unit in the last place of
 // a marker shows as 1e-10 of the pressure, and the drop keeps these bits from
-// one version to the next.  So the chord lengths and arc lengths are summed
+// one version to the next.  (Contexts without the frame have no such division;
+// they share the path, at 0.3 ms a relocation.)  So the chord lengths and arc lengths are summed
 // marker by marker, the basis is the Cox-de Boor recursion on knots k tau, the
 // matrix is factored column by column and substituted row by row, each sum
 // in ascending order, its products rounded before they are subtracted.  FP64 latency bounds the chains (64 cycles an

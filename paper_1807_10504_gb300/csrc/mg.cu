@@ -1090,8 +1090,8 @@ __device__ __forceinline__ void store_coeffs(int nx, int ny, int i, int j, const
 }
 
 // The FP64 sweep weights w_f = beta_f / diag of every level from its faces
-// and inverse diagonal (the products level_coeffs_cell forms when given w4),
-// one thread per cell over all levels.
+// and inverse diagonal (the products store_coeffs forms when given w4), one thread
+// per cell over all levels.
 struct LevelWArgs {
     int nl;
     long start[17];  // first flat index of each level
@@ -1233,7 +1233,7 @@ __global__ void __launch_bounds__(256) k_level_coeffs_small(LevelCoeffArgs a)
 // a column step reading one and writing the other behind one barrier, and the
 // thread that forms the next pivot also forms its reciprocal (recip_div: a
 // division is a chain of ~1.5 k cycles on this part).  With four barriers and
-// a division a column 16 cells took 15.7 us, now CI_TIMES.
+// a division a column 16 cells took 18.0 us, now 12.9 (ncu).
 constexpr int kCoarseOneCta = 64;  // larger coarsest levels: k_coarse_step
 
 // Entry (r, c) of A on a grid of nx x ny cells, and its diagonal (r, r).
@@ -1876,11 +1876,12 @@ __global__ void __launch_bounds__(1024) k_tail(const __grid_constant__ TailArgs<
 // FP64: what bounds it is FP64 instructions, each of which occupies its
 // sub-partition for 64 cycles whatever its active lanes: one cell a thread
 // spreads a small level over the four sub-partitions (k_tail's pairs double a
-// warp's chain).  From 32^2 down 31 us a cycle with k_tail<double>, now 18.
+// warp's chain).  From 32^2 down, as the tail ran then, 31 us a cycle with
+// k_tail<double>, 18 so; from 16^2 down, as now, 14 (ncu).
 // FP32: latency (a phase of a small level is one chain of address, loads,
 // FMAs and barrier, 600 cycles in k_tail with its parameter reads in every
-// phase) and issue on the largest level.  From 64^2 down 24.6 us a cycle with
-// k_tail<float>, now 22.5.
+// phase) and issue on the largest level.  From 64^2 down, as the tail ran then,
+// 24.6 us a cycle with k_tail<float>, 22.5 so; from 32^2 down, as now, 10.6.
 // Shared memory per level of n cells (colour-split as in k_tail, without
 // padding): e, bt, h^2 / diag (n each), the weights (W, E, S, N; 4 n), diag /
 // (4 h^2) of the red cells and the last half sweep's changes of the black
@@ -2203,7 +2204,11 @@ __global__ void k_apply_mean(long n, double *__restrict__ p, const double *__res
 // operations, which bound the kernel, in place of 10 (1024^2: 28.4 -> 24.9 us,
 // 2048^2: 87 -> 74, 512^2: 14.1 -> 12.9), and all rows' loads are in flight at
 // once.  ROWS: 4 from 2^17 cells up, 1 below, where one warp's latency counts
-// (256^2: 7.2 us with 4 and 6.5 with one cell a thread; 64^2 6.6 and 5.2).  With
+// (256^2: 7.2 us with 4 and 6.5 with one cell a thread; 64^2 6.6 and 5.2).  A V(2,2)
+// cycle and its norm with 1 and with 4, FP64 (mixed, one cycle a norm): 256^2 59.3 and
+// 59.2 us (45.3, 45.8); 512 x 256 74.2, 74.8 (52.7, 53.4); 384^2 77.4, 75.9 (53.8, 54.1);
+// 512^2 99.7, 94.8 (60.2, 57.9); 768^2 149, 141 (81.4, 74.9); 1024^2 214, 200 (101, 94);
+// 2048^2 538, 501 (265, 214); alone and back to back one row leads up to 512^2.  With
 // rf != NULL also writes the FP32 residual and zeroes the FP32 correction for the inner
 // cycle.  check = 1 (first) or 2 (after `inc` cycles): the block that
 // finishes the sum also runs the convergence test of the graph's solve loop.
@@ -2732,9 +2737,12 @@ static int resident_red_blocks()
     return nb;
 }
 
-// Blocks of a reduction over n cells: one wave, but none without a cell a
-// thread (1216 blocks on 64^2 cells left 3 threads a block with work and
-// 1216 partials to fold: 11 us).
+// Blocks of a reduction over n cells: one wave of the norm's kernel (456: its 75
+// registers leave room for three blocks an SM), but none without a cell a thread
+// (1216 blocks on 64^2 cells left 3 threads a block with work and 1216 partials to
+// fold: 11 us).  The sums before and after a solve take the same number; a solve of no
+// cycle with 304, 456 and 1216 blocks of theirs: 512^2 60, 63 and 68 us, 1024^2 89, 91
+// and 98, 2048^2 208, 204 and 210, 4096^2 676, 648 and 653.
 static auto resnorm_kernel(long n) { return n >= (1L << 17) ? k_resnorm<4> : k_resnorm<1>; }
 static int red_grid(const MG &mg, long n) { return std::min(mg.red_blocks, (int)cdiv(n, kRedT)); }
 
