@@ -16,8 +16,8 @@ namespace {
 
 constexpr int kT = 256;
 
-// 2 x for a normal x, an infinity or a NaN (not finite where the double is not), by
-// an addition to the exponent: x + x for those beyond it costs k_coeffs a fifth.
+// 2 x for a normal x, and not finite for an infinity or a NaN, by an addition to the
+// exponent (x + x where that does not give the double would cost k_coeffs a fifth).
 __device__ __forceinline__ double twice(double x)
 {
     const int hi = __double2hiint(x);
@@ -81,8 +81,8 @@ k_coeffs(int nx, int ny, double rho_g, double drho, double mu_g, double dmu,
 
 // The force is zero on all faces but those of the interface band: where a
 // warp's faces carry none, its part is skipped (12 FP64 operations a cell to 4;
-// 1024^2 21.1 -> 10.0 us, 19.0 with a force everywhere), unless a coefficient is infinite or
-// NaN, which reaches b whatever the force.
+// 1024^2 21.1 -> 10.0 us, 19.0 with a force everywhere), unless a coefficient is
+// infinite or NaN, which reaches b whatever the force.
 __global__ void k_rhs(int nx, int ny, double ih, double ihdt,
                       const double *__restrict__ us, const double *__restrict__ vs,
                       const double *__restrict__ Fx, const double *__restrict__ Fy,

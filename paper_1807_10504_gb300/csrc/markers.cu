@@ -1883,12 +1883,13 @@ k_reloc_place(int M, const int32_t *__restrict__ drop_of, const int32_t *__restr
 // centre by the square of the time step: there one unit in the last place of
 // a marker shows as 1e-10 of the pressure, and the drop keeps these bits from
 // one version to the next.  (Contexts without the frame have no such division;
-// they share the path, at 0.3 ms a relocation.)  So the chord lengths and arc lengths are summed
-// marker by marker, the basis is the Cox-de Boor recursion on knots k tau, the
-// matrix is factored column by column and substituted row by row, each sum
-// in ascending order, its products rounded before they are subtracted.  FP64 latency bounds the chains (64 cycles an
-// instruction), so that operands are loaded a step ahead and nothing but the
-// sums' own instructions is on them: one drop of 1024 markers 1114 us with
+// they share the path, at 0.3 ms a relocation.)  So the chord lengths and arc
+// lengths are summed marker by marker, the basis is the Cox-de Boor recursion on
+// knots k tau, the matrix is factored column by column and substituted row by
+// row, each sum in ascending order, its products rounded before they are
+// subtracted.  FP64 latency bounds the chains (64 cycles an instruction), so that
+// operands are loaded a step ahead and nothing but the sums' own instructions is
+// on them: one drop of 1024 markers 1114 us with
 // every entry looked up on the chain, now 378; the block elimination above 134.
 __device__ void bspl_basis(double s, double tau, int g, double *w)
 {

@@ -2320,18 +2320,18 @@ void launch_smooth2(const Level &v, const LevelT<float> &a, const float *pin, fl
 }
 
 // One fused FP64 smoother launch of MODE on level v (pin -> p).  Tiles of 64 x 32
-// (15 to 25 % of halo) from 2^21 cells up and where they make one wave of two blocks
-// an SM that leaves none idle (153 to 304 tiles), 32 x 16 otherwise, whose finer
-// grain evens out the last wave.  FP64 V(2,2) cycle with 64 x 32 and with 32 x 16 on
-// the finest level: 512^2 (128 tiles) 101.6 and 96.2 us; 640^2 (200) 115.4, 117.4;
-// 1024 x 512 (256) 124.1, 135.2; 768^2 (288) 126.2, 142.1; 960 x 640 (300) 127.2,
-// 145.1; 1024 x 768 (384) 179.4, 167.0; 896^2 (392) 182.3, 169.5; 960^2 (450) 199.8,
-// 192.4; 1024^2 (512) 203.5, 203.5; 1280 x 1024 (640) 248.2, 239.4; 1536 x 1024 (768)
-// 273.6, 271.5; 2048 x 1024 (1024) 304.9, 307.1.  Up to four tiles an SM, 64 x 32 ones
-// leave room (dynamic shared memory) for two blocks an SM only, so that the scheduler
-// hands the rest to the SMs that finish first instead of placing all at once (1024^2:
-// FP64 cycle 246 -> 222 us; 2048^2, with 13 tiles an SM, would lose a tenth).  Levels
-// that 16 x 8 tiles cover with at most one block an SM (up to 128^2) take those: a
+// (15 to 25 % of halo) from 2^21 cells up and where they fill one wave of two blocks
+// an SM more than half or a second one as well (153 to 304 and 457 to 608 tiles), 32 x
+// 16 otherwise, whose finer grain evens out the last wave.  FP64 V(2,2) cycle with 64 x
+// 32 and with 32 x 16 on the finest level: 512^2 (128 tiles) 101.6 and 96.2 us; 640^2
+// (200) 115.4, 117.4; 1024 x 512 (256) 124.1, 135.2; 768^2 (288) 126.2, 142.1; 960 x 640
+// (300) 127.2, 145.1; 1024 x 768 (384) 179.4, 167.0; 896^2 (392) 182.3, 169.5; 960^2 (450)
+// 199.8, 192.4; 1024^2 (512) 203.5, 203.5 (a whole solve 4.62 and 4.64 ms); 1280 x 1024
+// (640) 248.2, 239.4; 1536 x 1024 (768) 273.6, 271.5; 2048 x 1024 (1024) 304.9, 307.1.
+// Up to four tiles an SM, 64 x 32 ones leave room (dynamic shared memory) for two
+// blocks an SM only, so that the scheduler hands the rest to the SMs that finish first
+// instead of placing all at once (1024^2: FP64 cycle 246 -> 222 us; 2048^2, with 13
+// tiles an SM, would lose a tenth).  Levels that 16 x 8 tiles cover with at most one block an SM (up to 128^2) take those: a
 // block's FP64 work, not the halo's share of it, then sets the launch's time (FP64
 // cycle at 64^2 40.1 -> 36.9 us, 128^2 52.0 -> 44.3, 256^2 69.4 -> 60.1, 1024^2 211 ->
 // 200), up to 64^2 those of 8 x 8 (36.9 -> 36.5, 44.3 -> 43.2, 60.3 -> 59.5; between 64^2
@@ -2345,7 +2345,7 @@ void launch_smooth2_f64(const Level &v, const LevelT<double> &a, const double *p
     note_launch();
     const dim3 g64(cdiv(v.nx, 64), cdiv(v.ny, 32));
     const long n64 = (long)g64.x * g64.y;
-    if ((long)v.nx * v.ny >= (1L << 21) || (n64 > 152 && n64 <= 2 * 152)) {
+    if ((long)v.nx * v.ny >= (1L << 21) || (n64 > 152 && n64 <= 304) || (n64 > 456 && n64 <= 608)) {
         const dim3 g = g64;
         const int pad = n64 <= 4 * 152 ? kTwoBlocks : 0;
         launch_pdl(k_smooth2_f64<MODE, 64, 32>, g, 256, pad, s, v.nx, v.ny, ih2, (const double2 *)a.w,
